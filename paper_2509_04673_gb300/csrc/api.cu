@@ -148,8 +148,9 @@ static void continuation(int p, int side, double out[N1MAX][N1MAX]) {
 struct HostTables {
     Tab<double> td[NTABD];  // Bernstein at p, LGL at PMAX + 1 + p
     Tab<float> tf[PMAX + 1];
-    double a2d[2 * A2_TOTAL];
-    float a2f[A2_TOTAL];
+    double a2d[2 * A2_TOTAL];  // semi-norm matrices in the nodal basis (table export)
+    double m2d[2 * A2_TOTAL];  // the same in the modal basis of modal.cuh (device)
+    float m2f[A2_TOTAL];
 };
 
 // ---------------------------------------------------------------------------
@@ -317,6 +318,61 @@ static void build_lgl_tables(int p, Tab<double>& T, double* a2) {
         }
 }
 
+// Modal tables of degree p (modal.cuh).  With P_k the Legendre polynomials on
+// [0, 1] and L[k][a] the P_k coefficient of the basis function a, a line v
+// has the modal coefficients l_k = (sum_a L[k][a] v_a) / L[k][p], so that u =
+// sum_k l_k m_k with m_k = L[k][p] P_k.  mf holds the weights L[k][p - j] /
+// L[k][p] of the pairs (v_j, v_{p-j}), mc the expansion of m_j(x + 1) in m_k,
+// and m2 the semi-norm matrix of eq. (WENO:norm) over the products
+// m_k1 m_k2, off-diagonal entries doubled.  Gauss-Legendre with p + 2 points
+// (exact to degree 2p + 3).
+static void build_modal_tables(int p, Tab<double>& T, double* m2) {
+    const int n = p + 1, nq = p + 2, n2 = n * n;
+    double xg[NQMAX], wg[NQMAX];
+    gauss_legendre(nq, xg, wg);
+    // monomial coefficients of P_k(2x - 1): sum_i (-1)^(k+i) C(k,i) C(k+i,i) x^i
+    double P[N1MAX][N1MAX], L[N1MAX][N1MAX];
+    for (int k = 0; k < n; ++k)
+        for (int i = 0; i < N1MAX; ++i)
+            P[k][i] = i <= k ? ((k + i) % 2 ? -1.0 : 1.0) * binom(k, i) * binom(k + i, i) : 0.0;
+    for (int k = 0; k < n; ++k)
+        for (int a = 0; a < n; ++a) {
+            double s = 0.0;
+            for (int q = 0; q < nq; ++q) s += T.wq[q] * T.Bq[q][a] * poly_eval(p, P[k], T.xq[q]);
+            L[k][a] = (2 * k + 1) * s;
+        }
+    const int pairs = (p + 1) / 2;  // (v_j, v_{p-j}), j < pairs; an even p has the middle value too
+    for (int k = 0; k < n; ++k)
+        for (int j = 1; j < 3; ++j) {
+            const bool used = (k % 2 == 0) ? j < pairs + (p % 2 == 0) : j < pairs;
+            T.mf[k][j - 1] = used ? L[k][p - j] / L[k][p] : 0.0;
+        }
+    for (int k = 0; k < n; ++k)
+        for (int j = 0; j < n; ++j) {
+            double s = 0.0;
+            for (int q = 0; q < nq; ++q) s += T.wq[q] * poly_eval(p, P[j], T.xq[q] + 1.0) * poly_eval(p, P[k], T.xq[q]);
+            T.mc[k][j] = j > k ? (2 * k + 1) * s * L[j][p] / L[k][p] : (j == k ? 1.0 : 0.0);
+        }
+    double S[N1MAX][N1MAX][N1MAX];
+    for (int d = 0; d <= p; ++d)
+        for (int k = 0; k < n; ++k)
+            for (int l = 0; l < n; ++l) {
+                double dk[N1MAX], dl[N1MAX], s = 0.0;
+                poly_deriv(p, P[k], d, dk);
+                poly_deriv(p, P[l], d, dl);
+                for (int q = 0; q < nq; ++q) s += T.wq[q] * poly_eval(p, dk, T.xq[q]) * poly_eval(p, dl, T.xq[q]);
+                S[d][k][l] = s * L[k][p] * L[l][p];
+            }
+    for (int i = 0; i < n2; ++i)
+        for (int j = 0; j < n2; ++j) {
+            double s = 0.0;
+            for (int d1 = 0; d1 <= p; ++d1)
+                for (int d2 = 0; d2 <= p - d1; ++d2)
+                    if (d1 + d2 >= 1) s += S[d1][i % n][j % n] * S[d2][i / n][j / n];
+            m2[i * n2 + j] = i == j ? s : 2.0 * s;
+        }
+}
+
 static void semi_norm_blocks(int p, std::vector<std::vector<double>>& S) {
     // S[k][a*(p+1)+b] = int B_a^(k) B_b^(k), with
     // B_a^(k) = p!/(p-k)! sum_j (-1)^(k-j) C(k,j) B^{p-k}_{a-j}
@@ -384,14 +440,18 @@ static void build_tables(HostTables& H) {
                                 H.a2d[off + (b * n + a) * n2 + d * n + c] +=
                                     S[k1][a * n + c] * S[k2][b * n + d];
             }
+        build_modal_tables(p, T, H.m2d + off);
         // float copies
         Tab<float>& F = H.tf[p];
         const double* src = (const double*)&T;
         float* dst = (float*)&F;
         for (size_t i = 0; i < sizeof(Tab<double>) / sizeof(double); ++i) dst[i] = (float)src[i];
     }
-    for (int i = 0; i < A2_TOTAL; ++i) H.a2f[i] = (float)H.a2d[i];
-    for (int p = 1; p <= PMAX; ++p) build_lgl_tables(p, H.td[PMAX + 1 + p], H.a2d + A2_TOTAL + A2_OFF[p]);
+    for (int i = 0; i < A2_TOTAL; ++i) H.m2f[i] = (float)H.m2d[i];
+    for (int p = 1; p <= PMAX; ++p) {
+        build_lgl_tables(p, H.td[PMAX + 1 + p], H.a2d + A2_TOTAL + A2_OFF[p]);
+        build_modal_tables(p, H.td[PMAX + 1 + p], H.m2d + A2_TOTAL + A2_OFF[p]);
+    }
 }
 
 static const HostTables& host_tables() {
@@ -408,7 +468,7 @@ namespace cgl {
 // copy the host tables into the constant memory of the unit that owns `f`
 cudaError_t upload_host_tables(UploadFn f) {
     const HostTables& H = host_tables();
-    return f(H.td, H.tf, H.a2d, H.a2f);
+    return f(H.td, H.tf, H.m2d, H.m2f);
 }
 }  // namespace cgl
 
@@ -578,7 +638,7 @@ static cgl_status ensure_tables(int dev) {
     const HostTables& H = host_tables();
     UploadFn fns[9] = {upload_adv,   upload_burgers,   upload_kpp,   upload_euler,  upload_adv32,
                        upload_burgers32, upload_kpp32, upload_euler32, upload_batch};
-    for (UploadFn f : fns) CUDA_TRY(f(H.td, H.tf, H.a2d, H.a2f));
+    for (UploadFn f : fns) CUDA_TRY(f(H.td, H.tf, H.m2d, H.m2f));
     g_uploaded.push_back(dev);
     return CGL_OK;
 }
@@ -932,6 +992,9 @@ extern "C" cgl_status cgl_set_problem(cgl_state* S, const cgl_problem* p) {
     d.weno_eps_f = (float)d.weno_eps;
     d.gamma_eps_f = (float)d.gamma_eps;
     d.q_f = (float)d.q;
+    d.rh_f = (float)(0.5 * d.r);
+    d.r2 = d.r == 2.0;
+    d.q1 = d.q == 1.0;
     for (int c = 0; c < 4; ++c) {
         d.ubc_f[c] = (float)d.ubc[c];
         d.ubc_lo_f[c] = (float)(d.ubc[c] - (double)d.ubc_f[c]);
@@ -1467,7 +1530,8 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
     const int lo = S->prob.mode == CGL_MODE_LO;
     int64_t per_stage = 1 + 2 + (lo ? 0 : 3 + (S->prob.k_g + S->prob.k_u));
-    if (S->prec == CGL_FP32_MIXED && S->nc > 1) per_stage += 2;  // k_avg, k_sens
+    if (S->nc > 1) per_stage += 1;                                // k_sens
+    if (S->prec == CGL_FP32_MIXED && S->nc > 1) per_stage += 1;  // k_avg
     if (S->prec == CGL_FP32_MIXED) per_stage += 1;                // k_facet
     if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
     if (S->prec == CGL_FP32_MIXED && !lo && fuse_sweeps(S->mesh->m) && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
@@ -1475,8 +1539,8 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
         per_stage -= (S->prob.k_g >= 1) + (S->prob.k_u >= 1);
     }
     if ((S->prob.options & CGL_OPT_AEC_Q1) && !lo) {
-        // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_avg, k_sens for mixed systems)
-        per_stage = 5 + ((S->prec == CGL_FP32_MIXED && S->nc > 1) ? 2 : 0);
+        // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_sens for systems, k_avg for mixed ones)
+        per_stage = 5 + (S->nc > 1) + (S->prec == CGL_FP32_MIXED && S->nc > 1);
     }
     *kernels = 3 * per_stage + 1;  // + dt finalisation; the time advance rides in the last k_final
     return CGL_OK;

@@ -70,6 +70,8 @@ struct ProbDev {
     float ubc_f[4], ubc_lo_f[4];
     float lo32_f, hi32_f, lo_tol_f, hi_tol_f;
     int opts;              // CGL_OPT_* bits
+    int r2, q1;            // r == 2, q == 1 (the sensor's default exponents)
+    float rh_f;            // r / 2
     float ome_f;           // 1 - pos_eps rounded to float
     float lambda_floor_f;
     SideDev side[4];       // W, E, S, N
@@ -94,6 +96,7 @@ template <> struct PV<double> {
     static DEV double weno_eps(const ProbDev& p) { return p.weno_eps; }
     static DEV double gamma_eps(const ProbDev& p) { return p.gamma_eps; }
     static DEV double q(const ProbDev& p) { return p.q; }
+    static DEV double rh(const ProbDev& p) { return 0.5 * p.r; }
     static DEV double ubc(const ProbDev& p, int c) { return p.ubc[c]; }
     static DEV double side_state(const SideDev& s, int slot, int c) { return s.st[slot][c]; }
     static DEV double lo(const ProbDev& p) { return p.umin; }
@@ -113,6 +116,7 @@ template <> struct PV<float> {
     static DEV float weno_eps(const ProbDev& p) { return p.weno_eps_f; }
     static DEV float gamma_eps(const ProbDev& p) { return p.gamma_eps_f; }
     static DEV float q(const ProbDev& p) { return p.q_f; }
+    static DEV float rh(const ProbDev& p) { return p.rh_f; }
     static DEV float ubc(const ProbDev& p, int c) { return p.ubc_f[c]; }
     static DEV float side_state(const SideDev& s, int slot, int c) { return s.st_f[slot][c]; }
     static DEV float lo(const ProbDev& p) { return p.lo32_f; }
@@ -141,9 +145,15 @@ struct Tab {
     T wl[N1MAX];           // int_0^1 phi_a: 1/(p+1) (Bernstein), the LGL weights
     T iwl[N1MAX];          // 1 / wl[a]
     T xn[N1MAX];           // node positions on [0,1]: a/p, the LGL points
+    // modal coefficients of a 1D coefficient line (modal.cuh): mf[k][j - 1]
+    // weights the j-th even (odd) pair of the line in mode k, mc[k][j] the
+    // mode j > k of the lower neighbour in the continued mode k
+    T mf[N1MAX][2];
+    T mc[N1MAX][N1MAX];
 };
 
-// semi-norm matrices (n2 x n2 for p = 1..4) packed at offsets
+// semi-norm matrices (n2 x n2 for p = 1..4) packed at offsets; on the device
+// in the modal basis of modal.cuh, off-diagonal entries doubled
 constexpr int A2_OFF[PMAX + 1] = {0, 0, 16, 97, 353};
 constexpr int A2_TOTAL = 978;
 

@@ -34,7 +34,7 @@
 // elements writes, and a warp of consecutive nodes reads, contiguous runs.
 #pragma once
 
-#include "common.cuh"
+#include "modal.cuh"
 
 namespace cgl {
 
@@ -425,13 +425,6 @@ DEV void cell_state(const R* __restrict__ u, const MeshDev& m, const ProbDev& pr
     }
 }
 
-// x^e for the exponents other than the defaults r = 2, q = 1 of the sensor
-// (eqs. (WENO:alpha), (stab:WENO)): out of line, so that the sensor's hot
-// code, which the default exponents take, stays small in the instruction
-// cache (the same powf / pow as an inlined call)
-static __device__ __noinline__ float pow_rare(float x, float e) { return powf(x, e); }
-static __device__ __noinline__ double pow_rare(double x, double e) { return pow(x, e); }
-
 // the float64 Appendix-A factor where the float32 certificate of the
 // FP32-mixed form could not show alpha = 1 (rare): out of line, so that the
 // unrolled node loop of the slope limiter carries a call per node instead of
@@ -448,53 +441,7 @@ DEV double euler_alpha_of(const double* ub, const double* f, double m, double ep
     else return euler_alpha<double>(ub, f, m, eps);
 }
 
-// quadratic form of the semi-norm matrix A; A annihilates constants, so the
-// block is shifted by its first coefficient first (exact zeros for constant
-// data, no cancellation for nearly constant data).  a2b: the basis's offset
-// in the packed matrices (a2_base; 0 for Bernstein)
 template <class R, int P>
-DEV R qform(const R (&v)[Dim<P>::N2], int a2b = 0) {
-    constexpr int N2 = Dim<P>::N2;
-    constexpr int off = A2_OFF[P];
-    // d = v - v_0 (d_0 = 0); A symmetric: s = sum_i d_i (A_ii d_i + 2 sum_{j>i} A_ij d_j)
-    R d[N2];
-#pragma unroll
-    for (int i = 0; i < N2; ++i) d[i] = v[i] - v[0];
-    R s = R(0);
-#pragma unroll
-    for (int i = 1; i < N2; ++i) {
-        R t = R(0);
-#pragma unroll
-        for (int j = i + 1; j < N2; ++j) t += TabSel<R>::A2(a2b + off + i * N2 + j) * d[j];
-        s += d[i] * (TabSel<R>::A2(a2b + off + i * N2 + i) * d[i] + R(2) * t);
-    }
-    return s;
-}
-
-// neighbour polynomial continued onto K_e: dir 0 W (Em in x), 1 E (Ep in x),
-// 2 S (Em in y), 3 N (Ep in y)
-template <class R, int P>
-DEV void continue_nb(const Tab<R>& T, int dir, const R (&src)[Dim<P>::N2], R (&dst)[Dim<P>::N2]) {
-    constexpr int N1 = P + 1;
-#pragma unroll
-    for (int b = 0; b < N1; ++b)
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            R s = R(0);
-            if (dir < 2) {
-#pragma unroll
-                for (int c = 0; c < N1; ++c)
-                    s += (dir == 0 ? T.Em[a][c] : T.Ep[a][c]) * src[b * N1 + c];
-            } else {
-#pragma unroll
-                for (int d = 0; d < N1; ++d)
-                    s += (dir == 2 ? T.Em[b][d] : T.Ep[b][d]) * src[d * N1 + a];
-            }
-            dst[b * N1 + a] = s;
-        }
-}
-
-template <class R, int P, class Ph>
 DEV void load_comp(const R* __restrict__ u, const MeshDev& m, int ex, int ey, int c, R (&V)[Dim<P>::N2]) {
     constexpr int N1 = P + 1;
     const ElemNodes<P> en(m, ex, ey);
@@ -505,126 +452,22 @@ DEV void load_comp(const R* __restrict__ u, const MeshDev& m, int ex, int ey, in
         for (int a = 0; a < N1; ++a) V[b * N1 + a] = uc[en(a, b)];
 }
 
-// WENO smoothness sensor gamma_e, eq. (WENO:alpha), minimum over components.
-// Every block is shifted by its first coefficient (constants do not change
-// semi-norms) and u_h^e - u_h^{e,*} is formed as sum_{l>=1} omega_l
-// (u_h^e - u_{h,l}^e), using sum_l omega_l = 1.
-template <class R, int P, class Ph>
-DEV R sensor(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
-             const R (&U)[Ph::NC][Dim<P>::N2], const int (&nb)[4], int ex, int ey) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    const R wl = PV<R>::w_lin(pr), eps = PV<R>::weno_eps(pr), geps = PV<R>::gamma_eps(pr);
-    const bool r2 = (pr.r == 2.0);
-    const R rh = R(0.5 * pr.r);
-    const Tab<R>& T = tab_of<R>(m, P);
-    const int a2b = a2_base<R>(m);
-    int ne = 0;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) ne += (nb[d] >= 0);
-    R gam = R(1);
-#pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
-        R U0[N2];
-#pragma unroll
-        for (int i = 0; i < N2; ++i) U0[i] = U[c][i] - U[c][0];
-        R sig0 = fmax(qform<R, P>(U0, a2b), R(0));
-        R wt[5];
-        wt[0] = (R(1) - R(ne) * wl) / ((r2 ? sig0 : pow_rare(sig0, rh)) + eps);
-#pragma unroll 1
-        for (int d = 0; d < 4; ++d) {
-            wt[d + 1] = R(0);
-            if (nb[d] >= 0) {
-                R V[N2], W[N2];
-                int jx, jy;
-                neighbour_xy(m, ex, ey, d, jx, jy);
-                load_comp<R, P, Ph>(u, m, jx, jy, c, V);
-                const R v0 = V[0];
-#pragma unroll
-                for (int i = 0; i < N2; ++i) V[i] -= v0;
-                continue_nb<R, P>(T, d, V, W);
-                R sg = fmax(qform<R, P>(W, a2b), R(0));
-                wt[d + 1] = wl / ((r2 ? sg : pow_rare(sg, rh)) + eps);
-            }
-        }
-        R tot = (((wt[0] + wt[1]) + wt[2]) + wt[3]) + wt[4];
-        R Dl[N2];
-#pragma unroll
-        for (int i = 0; i < N2; ++i) Dl[i] = R(0);
-#pragma unroll 1
-        for (int d = 0; d < 4; ++d) {
-            if (nb[d] >= 0) {
-                R V[N2], W[N2];
-                int jx, jy;
-                neighbour_xy(m, ex, ey, d, jx, jy);
-                load_comp<R, P, Ph>(u, m, jx, jy, c, V);
-                const R v0 = V[0];
-#pragma unroll
-                for (int i = 0; i < N2; ++i) V[i] -= v0;
-                continue_nb<R, P>(T, d, V, W);
-                R wd = wt[d + 1] / tot;
-#pragma unroll
-                for (int i = 0; i < N2; ++i) Dl[i] += wd * (U0[i] - W[i]);
-            }
-        }
-        R num = sqrt(fmax(qform<R, P>(Dl, a2b), R(0)));
-        R den = sqrt(sig0);
-        R ratio = num / (den + geps);
-        R gc = R(1) - (pr.q == 1.0 ? fmin(R(1), ratio) : pow_rare(fmin(R(1), ratio), PV<R>::q(pr)));
-        gam = fmin(gam, gc);
-    }
-    return gam;
-}
-
-// scalar sensor with the four neighbour blocks already in registers (V[d]
-// holds the raw block of neighbour d when nb[d] >= 0); same arithmetic as
-// sensor() with NC = 1
+// gamma_e of one component whose field is u (modal.cuh) from the element's own
+// block, the neighbours' blocks loaded and transformed by this thread
 template <class R, int P>
-DEV R sensor_scalar(const ProbDev& pr, const R (&U)[Dim<P>::N2], const R (&V)[4][Dim<P>::N2],
-                    const int (&nb)[4]) {
+DEV R sensor_scalar(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, const R (&U)[Dim<P>::N2],
+                    const int (&nb)[4], int ex, int ey) {
     constexpr int N2 = Dim<P>::N2;
-    const R wl = PV<R>::w_lin(pr), eps = PV<R>::weno_eps(pr), geps = PV<R>::gamma_eps(pr);
-    const bool r2 = (pr.r == 2.0);
-    const R rh = R(0.5 * pr.r);
-    int ne = 0;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) ne += (nb[d] >= 0);
-    R U0[N2];
-#pragma unroll
-    for (int i = 0; i < N2; ++i) U0[i] = U[i] - U[0];
-    R sig0 = fmax(qform<R, P>(U0), R(0));
-    R wt[5];
-    wt[0] = (R(1) - R(ne) * wl) / ((r2 ? sig0 : pow_rare(sig0, rh)) + eps);
-    // the continued candidates, each formed once and kept for both passes
-    R W[4][N2];
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        wt[d + 1] = R(0);
-        if (nb[d] >= 0) {
-            R Vc[N2];
-#pragma unroll
-            for (int i = 0; i < N2; ++i) Vc[i] = V[d][i] - V[d][0];
-            continue_nb<R, P>(TabSel<R>::t(P), d, Vc, W[d]);
-            R sg = fmax(qform<R, P>(W[d]), R(0));
-            wt[d + 1] = wl / ((r2 ? sg : pow_rare(sg, rh)) + eps);
-        }
-    }
-    R tot = (((wt[0] + wt[1]) + wt[2]) + wt[3]) + wt[4];
-    const R rtot = R(1) / tot;  // one division for the four weights omega_l
-    R Dl[N2];
-#pragma unroll
-    for (int i = 0; i < N2; ++i) Dl[i] = R(0);
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        if (nb[d] >= 0) {
-            R wd = wt[d + 1] * rtot;
-#pragma unroll
-            for (int i = 0; i < N2; ++i) Dl[i] += wd * (U0[i] - W[d][i]);
-        }
-    }
-    R num = sqrt(fmax(qform<R, P>(Dl), R(0)));
-    R den = sqrt(sig0);
-    R ratio = num / (den + geps);
-    return R(1) - (pr.q == 1.0 ? fmin(R(1), ratio) : pow_rare(fmin(R(1), ratio), PV<R>::q(pr)));
+    const Tab<R>& T = tab_of<R>(m, P);
+    R own[N2];
+    modal_block<R, P>(T, U, own);
+    return modal_sensor<R, P, true>(T, a2_base<R>(m), pr, own, nb, [&](int d, R(&l)[N2]) {
+        int jx, jy;
+        neighbour_xy(m, ex, ey, d, jx, jy);
+        R V[N2];
+        load_comp<R, P>(u, m, jx, jy, 0, V);
+        modal_block<R, P>(T, V, l);
+    });
 }
 
 // float-float mean of N floats: compensated (Neumaier) sum, then a division
@@ -899,10 +742,6 @@ DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __rest
     }
     // neighbours: means, fluxes (and, for scalars, the blocks for the sensor)
     float oh[4][NC], ol[4][NC], ofx[4][NC], ofy[4][NC];
-    // scalars at p <= 2 keep the neighbour blocks for the sensor; at p >= 3
-    // the sensor reloads them (registers, hence occupancy, matter more)
-    constexpr bool keepV = (NC == 1) && (P <= 2);
-    float V1[keepV ? 4 : 1][keepV ? N2 : 1];
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
         if (nb[d] >= 0) {
@@ -929,19 +768,11 @@ DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __rest
                 load_block<float, P, NC>(u, m, jx, jy, B);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) ff_mean<N2>(B[c], oh[d][c], ol[d][c]);
-                if constexpr (keepV) {
-#pragma unroll
-                    for (int i = 0; i < N2; ++i) V1[d][i] = B[0][i];
-                }
             }
             if constexpr (!LO) Ph::template flux<float>(oh[d], ofx[d], ofy[d], pr);
         } else {
 #pragma unroll
             for (int c = 0; c < NC; ++c) oh[d][c] = ol[d][c] = ofx[d][c] = ofy[d][c] = 0.f;
-            if constexpr (keepV) {
-#pragma unroll
-                for (int i = 0; i < N2; ++i) V1[d][i] = 0.f;
-            }
         }
     }
     // canonical facet fluxes F(u^L, u^R; n), n = +x (W, E) or +y (S, N)
@@ -1042,14 +873,7 @@ DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __rest
     } else {
     float gam;
     if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-        if constexpr (keepV) {
-            float U1[N2];
-#pragma unroll
-            for (int i = 0; i < N2; ++i) U1[i] = U[0][i];
-            gam = sensor_scalar<float, P>(pr, U1, V1, nb);
-        } else {
-            gam = sensor<float, P, Ph>(m, pr, u, U, nb, ex, ey);
-        }
+        gam = sensor_scalar<float, P>(m, pr, u, U[0], nb, ex, ey);
     } else {
         gam = (pr.mode == MODE_HO) ? 1.f : 0.f;
     }
@@ -1146,22 +970,24 @@ DEV double pre_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, 
                 q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
             }
         }
-        double gam;
-        if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-            gam = (double)sensor<R, P, Ph>(m, pr, u, U, nb, ex, ey);
-        } else {
-            gam = (pr.mode == MODE_HO) ? 1.0 : 0.0;
-        }
-        gam_out[e] = gam;
-        R lm = R(0);
+        if constexpr (NC == 1) {  // systems: k_sens
+            double gam;
+            if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
+                gam = sensor_scalar<R, P>(m, pr, u, U[0], nb, ex, ey);
+            } else {
+                gam = (pr.mode == MODE_HO) ? 1.0 : 0.0;
+            }
+            gam_out[e] = gam;
+            R lm = R(0);
 #pragma unroll
-        for (int i = 0; i < N2; ++i) {
-            R ui[NC];
+            for (int i = 0; i < N2; ++i) {
+                R ui[NC];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) ui[c] = U[c][i];
-            lm = fmax(lm, Ph::template node_speed<R>(ui, pr));
+                for (int c = 0; c < NC; ++c) ui[c] = U[c][i];
+                lm = fmax(lm, Ph::template node_speed<R>(ui, pr));
+            }
+            nu_out[e] = (double)lm * (m.h * (0.5 / m.p));
         }
-        nu_out[e] = (double)lm * (m.h * (0.5 / m.p));
         if (EV) grad_vectors<R, P, NC>(m, U, PV<R>::h(m), m.E, e, EV);
     }
     return dte;
@@ -1257,89 +1083,102 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_PRE_LO)) k_p
     if (dtbits) block_min_to(dte, dtbits);
 }
 
-// FP32-mixed systems: the WENO sensor gamma_e (eqs. (WENO:alpha),
-// (WENO:norm)) and nu_e (eq. (stab:WENO)) with one thread per element and
-// component.  A block holds K_SENS_TX consecutive elements of one row, one
-// warp per component (threadIdx.y = c): each thread evaluates the scalar
-// sensor of its component (the arithmetic of sensor() for that component),
-// the block takes gamma_e = min over the components and the node speeds of
-// nu_e from the element blocks it stages in shared memory.
-constexpr int K_SENS_TX = 32;
-template <int P, class Ph>
-__global__ void __launch_bounds__(K_SENS_TX * Ph::NC) k_sens(MeshDev m, ProbDev pr, const float* __restrict__ u,
-                                                             double* __restrict__ gam_out,
-                                                             double* __restrict__ nu_out) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2, TX = K_SENS_TX;
-    __shared__ float sU[NC][N2][TX];
-    __shared__ float sG[NC][TX], sL[NC][TX];
+// systems: the WENO sensor gamma_e (eqs. (WENO:alpha), (WENO:norm)) and nu_e
+// (eq. (stab:WENO)).  A block of K_TX x TY threads holds a tile of K_TX x TY
+// elements; component by component it puts the modal coefficients of the tile
+// and its one-element halo in shared memory (modal.cuh), so that each block of
+// coefficients is loaded and transformed 1.3 to 1.6 times instead of five,
+// and one thread per element evaluates the sensor from them.
+constexpr int K_TX = 32;
+// element of position i of a tile's halo rows: false where it does not exist
+// or no sensor of the tile reads it (wrapped once on periodic directions)
+template <int TY>
+DEV bool halo_elem(const MeshDev& m, int ex0, int ey0, int i, int& jx, int& jy) {
+    constexpr int HX = K_TX + 2;
+    const int hy = i / HX, hx = i - hy * HX;
+    jx = ex0 + hx - 1;
+    jy = ey0 + hy - 1;
+    if ((hx == 0 || hx == HX - 1) && (hy == 0 || hy == TY + 1)) return false;
+    if (jx > m.nx || jy > m.ny) return false;
+    if (m.px) jx = jx < 0 ? m.nx - 1 : (jx == m.nx ? 0 : jx);
+    if (m.py) jy = jy < 0 ? m.ny - 1 : (jy == m.ny ? 0 : jy);
+    return jx >= 0 && jx < m.nx && jy >= 0 && jy < m.ny;
+}
+// halo position of the face neighbour d of the tile element (tx, ty)
+DEV int halo_pos(int tx, int ty, int d) {
+    return (ty + 1 + (d == 2 ? -1 : d == 3 ? 1 : 0)) * (K_TX + 2) + tx + 1 + (d == 0 ? -1 : d == 1 ? 1 : 0);
+}
+
+template <class R, int P, class Ph, int TY>
+__global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const R* __restrict__ u,
+                                                    double* __restrict__ gam_out, double* __restrict__ nu_out) {
+    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, HE = (K_TX + 2) * (TY + 2), NT = K_TX * TY;
+    // four continued candidates in registers where they leave two blocks per SM
+    constexpr bool KEEP = (N2 - 1) * sizeof(R) <= 128;
+    __shared__ R sM[N2 - 1][HE];
     pdl_wait_then_trigger();
-    const int tx = threadIdx.x, c = threadIdx.y;
-    const int ex = blockIdx.x * TX + tx, ey = blockIdx.y;
-    const bool valid = ex < m.nx;
-    float gam = 1.f;
-    if (valid) {
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * K_TX + tx;
+    const int ex0 = blockIdx.x * K_TX, ey0 = blockIdx.y * TY;
+    const int ex = ex0 + tx, ey = ey0 + ty;
+    const bool valid = ex < m.nx && ey < m.ny;
+    const Tab<R>& T = tab_of<R>(m, P);
+    R gam = R(1);
+    if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
         int nb[4];
 #pragma unroll
         for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-        const float* uc = u + c * m.NN;
-        float U[1][N2];
-        load_comp<float, P, Ph>(u, m, ex, ey, c, U[0]);
-#pragma unroll
-        for (int i = 0; i < N2; ++i) sU[c][i][tx] = U[0][i];
-        if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-            if constexpr (P <= 2) {
-                float V[4][N2];
-#pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    if (nb[d] >= 0) {
-                        int jx, jy;
-                        neighbour_xy(m, ex, ey, d, jx, jy);
-                        load_comp<float, P, Ph>(u, m, jx, jy, c, V[d]);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < N2; ++i) V[d][i] = 0.f;
-                    }
-                }
-                gam = sensor_scalar<float, P>(pr, U[0], V, nb);
-            } else {
-                // one component as a scalar field (neighbour blocks reloaded,
-                // fewer live registers at p >= 3)
-                gam = sensor<float, P, PhysAdv>(m, pr, uc, U, nb, ex, ey);
-            }
-        } else {
-            gam = (pr.mode == MODE_HO) ? 1.f : 0.f;
-        }
-    }
-    sG[c][tx] = gam;
-    __syncthreads();
-    float lm = 0.f;
-    if (valid) {
-        // the nodes of this component's thread, in a loop that is not
-        // unrolled: one copy of the node-speed code (the unrolled form with a
-        // test per node put nine copies in the instruction cache; measured
-        // k_sens 8.21 -> 7.24 ms per three blast steps with the reciprocal
-        // of the weight sum below)
 #pragma unroll 1
-        for (int i = c; i < N2; i += NC) {
-            float ui[NC];
+        for (int c = 0; c < NC; ++c) {
+            if (c > 0) __syncthreads();  // the previous component is consumed
+#pragma unroll 1
+            for (int i = tid; i < HE; i += NT) {
+                int jx, jy;
+                if (!halo_elem<TY>(m, ex0, ey0, i, jx, jy)) continue;
+                R V[N2], l[N2];
+                load_comp<R, P>(u, m, jx, jy, c, V);
+                modal_block<R, P>(T, V, l);
 #pragma unroll
-            for (int k = 0; k < NC; ++k) ui[k] = sU[k][i][tx];
-            lm = fmaxf(lm, Ph::template node_speed<float>(ui, pr));
+                for (int k = 1; k < N2; ++k) sM[k - 1][i] = l[k];
+            }
+            __syncthreads();
+            if (valid) {
+                R own[N2];
+                const int at = halo_pos(tx, ty, -1);
+                own[0] = R(0);
+#pragma unroll
+                for (int k = 1; k < N2; ++k) own[k] = sM[k - 1][at];
+                const R g = modal_sensor<R, P, KEEP>(T, a2_base<R>(m), pr, own, nb, [&](int d, R(&l)[N2]) {
+                    const int j = halo_pos(tx, ty, d);
+                    l[0] = R(0);
+#pragma unroll
+                    for (int k = 1; k < N2; ++k) l[k] = sM[k - 1][j];
+                });
+                gam = fmin(gam, g);
+            }
+        }
+    } else {
+        gam = (pr.mode == MODE_HO) ? R(1) : R(0);
+    }
+    if (!valid) return;
+    R lm = R(0);
+    const int gxe = (m.px && ex * P + P == m.nnx) ? 0 : ex * P + P;  // the last column may wrap
+#pragma unroll 1
+    for (int b = 0; b < N1; ++b) {
+        int gy = ey * P + b;
+        if (m.py && gy == m.nny) gy = 0;
+        const R* __restrict__ ur = u + (long long)gy * m.nnx;
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+            R ui[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ui[c] = ur[c * m.NN + (a < P ? ex * P + a : gxe)];
+            lm = fmax(lm, Ph::template node_speed<R>(ui, pr));
         }
     }
-    sL[c][tx] = lm;
-    __syncthreads();
-    if (c == 0 && valid) {
-        float g = 1.f, l = 0.f;
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            g = fminf(g, sG[k][tx]);
-            l = fmaxf(l, sL[k][tx]);
-        }
-        const int e = ey * m.nx + ex;
-        gam_out[e] = (double)g;
-        nu_out[e] = (double)(l * (m.h_f * (0.5f / P)));
-    }
+    const int e = ey * m.nx + ex;
+    gam_out[e] = (double)gam;
+    if constexpr (sizeof(R) == 4) nu_out[e] = (double)(lm * (m.h_f * (0.5f / P)));
+    else nu_out[e] = lm * (m.h * (0.5 / m.p));
 }
 
 // global dt from the block minima folded into the bit pattern by k_pre
@@ -1466,13 +1305,6 @@ __global__ void k_gather_init(MeshDev m, const R* __restrict__ EV, R* __restrict
 
 
 
-
-// explicitly rounded multiply-add and multiply (no contraction choices left
-// to the compiler, so the per-node and the tiled stencils give equal bits)
-DEV float fma_r(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-DEV double fma_r(double a, double b, double c) { return __fma_rn(a, b, c); }
-DEV float mul_r(float a, float b) { return __fmul_rn(a, b); }
-DEV double mul_r(double a, double b) { return __dmul_rn(a, b); }
 
 // Richardson update x + (b - h^2 s) / m_i with s = (M (x) M) x at the node
 template <class R>

@@ -119,6 +119,10 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     auto* k_sweep_g = small_tiles ? k_mass_sweep<R, P, 2 * NC, 8> : k_mass_sweep<R, P, 2 * NC, ST_TY>;
     auto* k_sweep_u = small_tiles ? k_mass_sweep<R, P, NC, 8> : k_mass_sweep<R, P, NC, ST_TY>;
     const dim3 gts = small_tiles ? gt8 : gt;
+    // the sensor's element tiles (k_sens): 8 rows of 32 in float, 4 in float64
+    // (24 modes of 340 elements are 65 KB there)
+    constexpr int STY = sizeof(R) == 4 ? 8 : 4;
+    const dim3 bs(K_TX, STY), gs(nblk(m.nx, K_TX), nblk(m.ny, STY));
     // per-launch timing records events between kernels: plain launches then
     const bool pdl = prof == nullptr;
     cudaError_t err = cudaSuccess;
@@ -176,9 +180,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
                 // g_h kernels of the main stream (k_sens is arithmetic-bound,
                 // the fused g_h sweep shared-memory-bound; measured: quadrants
                 // 512^2 Q3 2.368 -> 2.312 ms per step, blast 2048^2 -0.3 %)
-                const dim3 bs(K_SENS_TX, NC), gs(nblk(m.nx, K_SENS_TX), m.ny);
                 CGL_LAUNCH(prof, KID_SENS, s2,
-                           chk(launch(false, k_sens<P, Ph>, gs, bs, s2, m, pr, (const float*)u, B.gam, B.nu)));
+                           chk(launch(false, k_sens<float, P, Ph, STY>, gs, bs, s2, m, pr, (const float*)u, B.gam, B.nu)));
                 chk(cudaEventRecord(B.ev_w, s2));
             }
             CGL_LAUNCH(prof, KID_FACET, s2,
@@ -188,13 +191,12 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
             chk(cudaEventRecord(B.ev_join, s2));
         }
     }
-    if constexpr (use_avg) {
-        if (q1) {
-            // eq. (aecQ1) scales its contributions by gamma_e: the sensor on the main stream
-            const dim3 bs(K_SENS_TX, NC), gs(nblk(m.nx, K_SENS_TX), m.ny);
+    if constexpr (NC > 1) {
+        // the FP64 form, and eq. (aecQ1), which scales its contributions by
+        // gamma_e: the sensor on the main stream
+        if (!split || q1)
             CGL_LAUNCH(prof, KID_SENS, st,
-                       chk(launch(pdl, k_sens<P, Ph>, gs, bs, st, m, pr, (const float*)u, B.gam, B.nu)));
-        }
+                       chk(launch(pdl, k_sens<R, P, Ph, STY>, gs, bs, st, m, pr, (const R*)u, B.gam, B.nu)));
     }
     if (q1) {
         CGL_LAUNCH(prof, KID_Q1F, st,
