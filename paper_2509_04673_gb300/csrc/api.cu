@@ -1534,7 +1534,7 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     if (S->prec == CGL_FP32_MIXED && S->nc > 1) per_stage += 1;  // k_avg
     if (S->prec == CGL_FP32_MIXED) per_stage += 1;                // k_facet
     if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
-    if (S->prec == CGL_FP32_MIXED && !lo && fuse_sweeps(S->mesh->m) && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
+    if (!lo && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
         // the first sweep of each solve runs inside k_grad_sweep / k_udot_sweep
         per_stage -= (S->prob.k_g >= 1) + (S->prob.k_u >= 1);
     }

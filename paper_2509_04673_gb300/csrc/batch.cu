@@ -61,14 +61,23 @@ enum { PH_FACET = 3, PH_UPDATE_EL, PH_RES_W, PH_RES_S };
 enum { PH_GRAD = 0, PH_SWEEP_G, PH_GATHER_R, PH_SWEEP_U, PH_FINAL, PH_GRADF, PH_GATHERF };
 
 constexpr int BT = 128;  // threads per block of the persistent grid
-constexpr int BY = BT / ST_TX;  // node tiles of ST_TX x ST_TY nodes: the block as 32 x BY threads
 
-// shared workspace of the tiled stencils, the largest over the degrees
+// node tiles: the single-state stencils' large tiles, worked by NT threads
+template <int P, int NT>
+using BatchTile = SegTile<float, P, StageTile<float, P, false>::X, StageTile<float, P, false>::Y, NT>;
+static int tile_nx(int p) {
+    return p == 1 ? BatchTile<1, BT>::NX : p == 2 ? BatchTile<2, BT>::NX : p == 3 ? BatchTile<3, BT>::NX : BatchTile<4, BT>::NX;
+}
+static int tile_ny(int p) {
+    return p == 1 ? BatchTile<1, BT>::NY : p == 2 ? BatchTile<2, BT>::NY : p == 3 ? BatchTile<3, BT>::NY : BatchTile<4, BT>::NY;
+}
+
+// shared workspace of the tiled stencils, the largest over the phases
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 template <int P>
 constexpr int ws_deg() {
-    return cmax(cmax(StFields<float, P, 1, 2>::ws, cmax(StFields<float, P, 2, 1>::ws, StFields<float, P, 1, 1>::ws)),
-                cmax(GradSweepWs<P, 1>::size, UdotSweepWs<P, 1>::size));
+    using TL = BatchTile<P, BT>;
+    return cmax(TL::grad_ws, cmax(TL::sweep_ws, TL::udot_ws(1)));
 }
 
 // bounded grid barrier: returns false if it gave up (or another block did)
@@ -155,43 +164,36 @@ DEV void elem_dispatch(int phase, const InstDev& D, int ex, int ey, int e, doubl
     }
 }
 
-// node phases on one ST_TX x ST_TY node tile of an instance: the stencils
-// (g_h right-hand side, Richardson sweeps) with the tiled shared-memory
-// functions of the single-state kernels, the gathers node by node
-// (ST_TY / BY nodes per thread)
-// NT threads per block (the block as 32 x NT/32 threads); inlined, so a
+// node phases on one node tile of an instance: the stencils (g_h right-hand
+// side, Richardson sweeps) with the tiled functions of the single-state
+// kernels, the gathers node by node.  NT threads per block; inlined, so a
 // caller with a compile-time phase carries only that phase's code
 template <int P, int NT>
 DEV void node_phase_body(int phase, const InstDev& D, const MeshDev& m, int gx0, int gy0, float a, float b, int k,
                          float* ws) {
-    constexpr int BYN = NT / ST_TX;
-    const int tx = threadIdx.x % ST_TX, ty = threadIdx.x / ST_TX;
+    using TL = BatchTile<P, NT>;
+    const int tid = threadIdx.x;
     switch (phase) {
         case PH_GRADF:
             // right-hand side and first sweep in one pass (k carries k_g: b is
-            // kept only when more sweeps follow); a block of k_grad_sweep's
-            // shape runs its body (the block's geometry formed once in
-            // registers), the same arithmetic as grad_sweep_tile
-            if constexpr (NT == ST_TX * ST_BY)
-                grad_sweep_block<P, 1>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tx, ty, ws);
-            else
-                grad_sweep_tile<P, 1, NT>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, threadIdx.x, ws);
+            // kept only when more sweeps follow)
+            grad_sweep_seg<float, P, 1, TL>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tid, ws);
             break;
-        case PH_GATHERF: udot_sweep_tile<P, 1, NT>(m, D.ER, D.r, D.ud2, gx0, gy0, threadIdx.x, ws); break;
-        case PH_GRAD: grad_tile<float, P, 1, BYN>(m, D.u, D.bg, D.g, gx0, gy0, tx, ty, ws); break;
+        case PH_GATHERF: udot_sweep_seg<float, P, 1, TL>(m, D.ER, D.r, D.ud2, gx0, gy0, tid, ws); break;
+        case PH_GRAD: grad_sweep_seg<float, P, 1, TL, false>(m, D.u, D.bg, D.g, gx0, gy0, tid, ws); break;
         case PH_SWEEP_G:
-            if (k & 1) sweep_tile<float, P, 2, BYN>(m, D.g2, D.bg, D.g, gx0, gy0, tx, ty, ws);
-            else sweep_tile<float, P, 2, BYN>(m, D.g, D.bg, D.g2, gx0, gy0, tx, ty, ws);
+            if (k & 1) mass_sweep_seg<float, P, 2, TL>(m, D.g2, D.bg, D.g, gx0, gy0, tid, ws);
+            else mass_sweep_seg<float, P, 2, TL>(m, D.g, D.bg, D.g2, gx0, gy0, tid, ws);
             break;
         case PH_SWEEP_U:
-            if (k & 1) sweep_tile<float, P, 1, BYN>(m, D.ud2, D.r, D.ud, gx0, gy0, tx, ty, ws);
-            else sweep_tile<float, P, 1, BYN>(m, D.ud, D.r, D.ud2, gx0, gy0, tx, ty, ws);
+            if (k & 1) mass_sweep_seg<float, P, 1, TL>(m, D.ud2, D.r, D.ud, gx0, gy0, tid, ws);
+            else mass_sweep_seg<float, P, 1, TL>(m, D.ud, D.r, D.ud2, gx0, gy0, tid, ws);
             break;
         default: {
-            const int gx = gx0 + tx, nnx = m.nnx, nny = m.nny;
-#pragma unroll
-            for (int j = 0; j < ST_TY / BYN; ++j) {
-                const int gy = gy0 + ty + j * BYN;
+            const int nnx = m.nnx, nny = m.nny;
+#pragma unroll 2
+            for (int i = tid; i < TL::NX * TL::NY; i += NT) {
+                const int r = i / TL::NX, gx = gx0 + i - r * TL::NX, gy = gy0 + r;
                 if (gx >= nnx || gy >= nny) continue;
                 const long long node = (long long)gy * nnx + gx;
                 if (phase == PH_GATHER_R) gather_init_at<float, P, 1>(m, D.ER, D.r, D.ud, gx, gy, node);
@@ -231,6 +233,7 @@ DEV void node_loop(int phase, const InstDev* __restrict__ I, const Tile* __restr
     for (int t = blockIdx.x; t < nnt; t += gridDim.x) {
         const Tile T = nt[t];
         node_phase<P>(phase, I[T.inst], T.begin, T.count, a, b, k, ws);
+        __syncthreads();  // the workspace is free for the next tile
     }
 }
 
@@ -488,7 +491,6 @@ struct cgl_batch {
     int ninst;
     std::vector<DegreeGroup> groups;  // one per degree present, ascending
     int tile_elems[PMAX + 1];
-    int node_tile;
     int mode_lo, kg, ku;
     long long limit;
     int phantom;
@@ -520,8 +522,8 @@ static cgl_status build_tiles(cgl_batch* B) {
         }
         for (int k = 0; k < (int)G.members.size(); ++k) {
             const MeshDev& m = B->states[G.members[k]]->mesh->m;
-            for (int gy0 = 0; gy0 < m.nny; gy0 += ST_TY)
-                for (int gx0 = 0; gx0 < m.nnx; gx0 += ST_TX) nt.push_back(Tile{k, gx0, gy0, 0});
+            for (int gy0 = 0; gy0 < m.nny; gy0 += tile_ny(G.p))
+                for (int gx0 = 0; gx0 < m.nnx; gx0 += tile_nx(G.p)) nt.push_back(Tile{k, gx0, gy0, 0});
         }
         if (G.d_et) cudaFree(G.d_et);
         if (G.d_nt) cudaFree(G.d_nt);
@@ -692,7 +694,6 @@ extern "C" cgl_status cgl_batch_create(cgl_state* const* states, int32_t n, cgl_
     B->ku = s0->prob.k_u;
     B->limit = 1LL << 22;
     B->phantom = 0;
-    B->node_tile = ST_TX * ST_TY;
     B->use_graph = true;
     B->graph_err = cudaSuccess;
     B->graph = nullptr;

@@ -1,19 +1,30 @@
-// fused.cuh — the first Richardson sweep fused into the kernel that builds
-// its right-hand side (FP32-mixed form).
+// fused.cuh — the separable node stencils of the g_h and udot solves on tiles
+// of whole elements, and the first Richardson sweep fused into the kernel
+// that builds its right-hand side.
 //
 // k_grad_sweep: g_h right-hand side b = int phi_i grad u_h, lumped iterate
 //   g0 = b / m_i and the first sweep g1 = g0 + (b - M_C g0) / m_i (Sec. 2.2,
-//   Richardson reading of the consistent L2 projection) in one pass over a
-//   32 x 16 node tile.
+//   Richardson reading of the consistent L2 projection) in one pass.
 // k_udot_sweep: node gather r_i = sum_e R^e_i, lumped iterate udot0 = r / m_i
-//   and the first sweep (Sec. 4.3, step 2) in one pass over a tile.
+//   and the first sweep (Sec. 4.3, step 2) in one pass.
+// k_mass_sweep: one further sweep.
+// k_grad_rhs: b and g0 alone (no sweeps, CGL_OPT_UNFUSED_SWEEPS).
 //
-// A sweep needs its lumped iterate on the tile plus a halo of p nodes, so
-// each block recomputes the right-hand side there (the grad stencil reads u
-// on a halo of 2p nodes).  The arithmetic is that of grad_tile,
-// gather_init_at and sweep_tile, in the same order with the same explicit
-// roundings, so the fused kernels give the same bits as the separate ones
-// (the batched stage, which keeps them separate, is compared bitwise).
+// What bounds them is the shared-memory pipe and instruction issue, not DRAM,
+// so a thread owns a segment, the vertex v and the p - 1 interior nodes after
+// it, instead of a node: one read of the 2p + 1 values v - p .. v + p gives
+// the p outputs of every 1D operator applied to them (p = 2: 2.5 reads per
+// node in place of 5), the interior nodes skip the p weights that are zero
+// for them, and every weight is a table constant, except the vertex's own,
+// which differs at the ends of a non-periodic mesh.
+//
+// Tiles start at vertices.  A field is staged by local index: plane a holds
+// the nodes of index a of every segment, so the segment reads of a warp along
+// x fall on consecutive words; planes are padded so that a warp running over
+// nodes (along y, and at the global stores) hits distinct banks as well.
+//
+// The sums run over the offsets -p .. p in order with explicit rounding, so
+// the fused and the separate kernels, and every tile size, give the same bits.
 #pragma once
 
 #include "kernels.cuh"
@@ -31,468 +42,482 @@ DEV bool wrap_node(const MeshDev& m, int& gx, int& gy) {
     return in;
 }
 
-template <int P, int NC>
-struct GradSweepWs {
-    static constexpr int HX1 = ST_TX + 2 * P, HY1 = ST_TY + 2 * P;  // tile + p halo
-    static constexpr int HX2 = ST_TX + 4 * P, HY2 = ST_TY + 4 * P;  // tile + 2p halo
-    static constexpr int NW = 2 * P + 1, NCL = P + 2;
-    static constexpr int A = HY2 * HX2;                // u on the 2p halo
-    static constexpr int B = 2 * HY2 * HX1;            // x-pass of the grad stencil; later the sweep's x-pass
-    static constexpr int C = 2 * HY1 * HX1;            // g0 (x and y parts) on the p halo
-    static constexpr int D = 2 * ST_TY * ST_TX;        // b on the tile
-    static constexpr int size = A + B + C + D + 2 * NCL * NW;
+// a tile of TEX x TEY elements (NX x NY nodes) worked by NT threads
+template <class R, int P, int TEX_, int TEY_, int NT_>
+struct SegTile {
+    static constexpr int TEX = TEX_, TEY = TEY_, NT = NT_;
+    static constexpr int NX = TEX * P, NY = TEY * P;
+    // nodes and segments of the tile with one (1) and two (2) elements of halo
+    // on the low side and one, two vertices' reach on the high side
+    static constexpr int W1 = (TEX + 1) * P + 1, H1 = (TEY + 1) * P + 1, S1 = TEX + 2;
+    static constexpr int W2 = (TEX + 3) * P + 1, H2 = (TEY + 3) * P + 1, S2 = TEX + 4;
+    // plane stride: n words or more, congruent to a p-th of the banks
+    static constexpr int plane(int n) {
+        constexpr int B = 128 / (int)sizeof(R), want = P == 1 ? 0 : (B + P - 1) / P;
+        int k = n;
+        while (P > 1 && k % B != want % B) ++k;
+        return k;
+    }
+    static constexpr int PU = plane(H2 * S2);   // u on the two-element halo
+    static constexpr int PT = plane(H2 * S1);   // its x pass
+    static constexpr int PG = plane(H1 * S1);   // an iterate on the one-element halo
+    static constexpr int PS = plane(H1 * TEX);  // its x pass
+    static constexpr int PR = plane(NY * TEX);  // a field on the tile
+    static constexpr int NOWN = NX * TEY, NJ = (NOWN + NT - 1) / NT;  // (column, y segment) items
+    static constexpr int grad_a = P * PU > 2 * P * PG ? P * PU : 2 * P * PG;
+    static constexpr int grad_b = 2 * P * (PT > PS ? PT : PS);
+    static constexpr int grad_ws = grad_a + grad_b;
+    static constexpr int sweep_ws = P * (PG + PS);
+    // fields of a udot sweep staged together: two where they take 32 KB at most
+    static constexpr int udot1 = P * (PG + PS + PR);
+    static constexpr int udot_fields(int nc) { return (nc % 2 == 0 && 2 * udot1 * (int)sizeof(R) <= 32768) ? 2 : 1; }
+    static constexpr int udot_ws(int nc) { return udot_fields(nc) * udot1; }
 };
 
-// The block's geometry (wrapped node indices, node classes, weights, masses)
-// is the same for every component, so it is formed once into registers
-// before the component loop; the halo passes give each thread a fixed
-// column (its x weights stay in registers) and a set of rows.
-// One block of ST_TX x ST_BY threads (thread (tx, ty)) on the tile at (gx0,
-// gy0); ws: GradSweepWs<P, NC>::size floats of shared memory.  k_grad_sweep
-// and the batched stage's phase kernels run it.
-template <int P, int NC>
-DEV void grad_sweep_block(const MeshDev& m, const float* __restrict__ u, float* __restrict__ bout,
-                          float* __restrict__ gout, int gx0, int gy0, int tx, int ty, float* ws) {
-    using WS = GradSweepWs<P, NC>;
-    constexpr int HX1 = WS::HX1, HY1 = WS::HY1, HX2 = WS::HX2, HY2 = WS::HY2, NW = WS::NW, NCL = WS::NCL;
-    constexpr int NT = ST_TX * ST_BY, NJ = ST_TY / ST_BY;
-    constexpr int RG = NT / HX1;                    // row groups of the halo passes
-    constexpr int NA = (HY2 * HX2 + NT - 1) / NT;  // staged values per thread
-    constexpr int NXP = (HY2 + RG - 1) / RG;        // x-pass rows per thread
-    constexpr int NYP = (HY1 + RG - 1) / RG;        // y-pass rows per thread
-    constexpr int NSX = (HY1 + ST_BY - 1) / ST_BY;  // rows of the sweep's x-pass per thread
-    float(*A)[HX2] = reinterpret_cast<float(*)[HX2]>(ws);
-    float(*tC)[HX1] = reinterpret_cast<float(*)[HX1]>(ws + WS::A);
-    float(*tM)[HX1] = reinterpret_cast<float(*)[HX1]>(ws + WS::A + HY2 * HX1);
-    float(*t)[HY1][ST_TX] = reinterpret_cast<float(*)[HY1][ST_TX]>(ws + WS::A);  // after tC, tM are consumed
-    float(*G)[HY1][HX1] = reinterpret_cast<float(*)[HY1][HX1]>(ws + WS::A + WS::B);
-    float(*Bt)[ST_TY][ST_TX] = reinterpret_cast<float(*)[ST_TY][ST_TX]>(ws + WS::A + WS::B + WS::C);
-    float(*WM)[NW] = reinterpret_cast<float(*)[NW]>(ws + WS::A + WS::B + WS::C + WS::D);
-    float(*WC)[NW] = reinterpret_cast<float(*)[NW]>(ws + WS::A + WS::B + WS::C + WS::D + NCL * NW);
-    const Tab<float>& T = TabSel<float>::t(P);
-    const int tid = ty * ST_TX + tx;
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        WM[cls][k] = class_weight<float, P, 0>(T, cls, k - P);
-        WC[cls][k] = class_weight<float, P, 1>(T, cls, k - P);
+// kind of a vertex along a direction of n nodes: 0 shared by two elements, 1
+// and 2 the lower and upper end of a non-periodic mesh
+DEV int vertex_kind(int g, int n, int periodic) { return periodic ? 0 : (g == 0 ? 1 : (g == n - 1 ? 2 : 0)); }
+
+// the vertex's own weight in the assembled operator (WHICH 0 mass, 1
+// derivative on the trial index)
+template <class R, int P, int WHICH>
+DEV R vertex_weight(const Tab<R>& T, int kind) {
+    const R lo = wtab<R, P, WHICH>(T, P, P), hi = wtab<R, P, WHICH>(T, 0, 0);
+    return kind == 0 ? add_r(lo, hi) : (kind == 1 ? hi : lo);
+}
+
+// the 1D operator on a segment: x[k] the value at offset k - P from its vertex
+template <class R, int P, int WHICH>
+DEV void seg_apply(const Tab<R>& T, const R (&x)[2 * P + 1], R w0, R (&out)[P]) {
+    R s = R(0);
+#pragma unroll
+    for (int k = 0; k <= 2 * P; ++k) {
+        const R w = k < P ? wtab<R, P, WHICH>(T, P, k) : (k == P ? w0 : wtab<R, P, WHICH>(T, 0, k - P));
+        s = fma_r(w, x[k], s);
     }
-    const float h = m.h_f, h2 = m.h2_f;
-    // staged values of u: node offsets (-1 outside the mesh)
-    long long aoff[NA];
+    out[0] = s;
+#pragma unroll
+    for (int a = 1; a < P; ++a) {
+        s = R(0);
+#pragma unroll
+        for (int c = 0; c <= P; ++c) s = fma_r(wtab<R, P, WHICH>(T, a, c), x[P + c], s);
+        out[a] = s;
+    }
+}
+
+// a segment's values along x (planes of stride PL, at: its row and segment)
+// and along y (rows of stride S, at: its column, row the vertex's)
+template <class R, int P>
+DEV void seg_x(const R* f, int PL, int at, R (&x)[2 * P + 1]) {
+#pragma unroll
+    for (int k = 0; k <= 2 * P; ++k) x[k] = f[(k % P) * PL + at + k / P - 1];
+}
+template <class R, int P>
+DEV void seg_y(const R* f, int S, int at, int row, R (&x)[2 * P + 1]) {
+#pragma unroll
+    for (int k = 0; k <= 2 * P; ++k) x[k] = f[at + (row + k - P) * S];
+}
+
+// 1 / m_i of node (gx, gy) with local indices a, b in its segments
+template <class R, int P>
+DEV R seg_inv_mass(const MeshDev& m, int a, int kx, int b, int ky) {
+    const int cnt = (a == 0 && kx == 0 ? 2 : 1) * (b == 0 && ky == 0 ? 2 : 1);
+    if (is_lgl<R>(m)) {
+        const int a0 = a != 0 ? a : (kx == 1 ? 0 : P), b0 = b != 0 ? b : (ky == 1 ? 0 : P);
+        return R(inv_lumped_lgl<P>(m, cnt, a0, b0));
+    }
+    return mul_r(PV<R>::inv_me(m), inv_count<R>(cnt));
+}
+
+// Right-hand side of the g_h projection, its lumped iterate and the first
+// sweep on the tile at (gx0, gy0), one component after the other: u on a
+// two-element halo (the next component's loads run under this one's passes),
+// x pass with the derivative and the mass operator, y pass to b and g0 on the
+// one-element halo, then the sweep's x and y passes.  A thread keeps b and g0
+// of its own nodes in registers from the first y pass to the second.  ws:
+// TL::grad_ws values.  All threads of the block call it together.
+// SWEEP false: b and g0 of the tile's nodes only.
+template <class R, int P, int NC, class TL, bool SWEEP = true>
+DEV void grad_sweep_seg(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
+                        int gy0, int tid, R* ws) {
+    constexpr int NT = TL::NT, NJ = TL::NJ, NX = TL::NX, TEX = TL::TEX, TEY = TL::TEY;
+    constexpr int NA = (TL::W2 * TL::H2 + NT - 1) / NT;
+    R* A = ws;                // u, then g0 (x and y parts)
+    R* B = ws + TL::grad_a;   // the x passes
+    const Tab<R>& T = tab_of<R>(m, P);
+    const R h = PV<R>::h(m), h2 = PV<R>::h2(m);
+    // segments and rows that feed nodes of the mesh (ragged tiles stop there)
+    const int ns = min(TL::S1, (m.nnx - gx0 + P - 1) / P + 2), nr = min(TL::H2, m.nny - gy0 + 4 * P);
+    long long off[NA];
+    R next[NA];
 #pragma unroll
     for (int j = 0; j < NA; ++j) {
-        const int i = tid + j * NT;
-        aoff[j] = -1;
-        if (i < HY2 * HX2) {
-            const int r = i / HX2, cc = i - r * HX2;
-            int gx = gx0 - 2 * P + cc, gy = gy0 - 2 * P + r;
-            if (wrap_node(m, gx, gy)) aoff[j] = (long long)gy * m.nnx + gx;
-        }
+        const int i = tid + j * NT, r = i / TL::W2, q = i - r * TL::W2;
+        int gx = gx0 - 2 * P + q, gy = gy0 - 2 * P + r;
+        const bool in = r < nr && wrap_node(m, gx, gy);
+        off[j] = in ? (long long)gy * m.nnx + gx : -1;
+        // through L2 (ld.global.cg): this runs before the kernel launched just
+        // before it has completed
+        next[j] = in ? __ldcg(&u[off[j]]) : R(0);
     }
-    // halo passes: column cx of the p halo, rows rg + RG j
-    const int cx = tid % HX1, rg = tid / HX1;
-    const bool hv = rg < RG;
-    int clx;
-    {
-        int gx = gx0 - P + cx, gy = 0;
-        wrap_node(m, gx, gy);
-        clx = node_class<P>(gx, m.nnx, m.px);
-    }
-    bool yin[NYP];
-    int ycl[NYP];
-    float yinv[NYP];
-#pragma unroll
-    for (int j = 0; j < NYP; ++j) {
-        const int r = rg + RG * j;
-        int gx = gx0 - P + cx, gy = gy0 - P + r;
-        yin[j] = wrap_node(m, gx, gy) && hv && r < HY1;
-        ycl[j] = node_class<P>(gy, m.nny, m.py);
-        const int cnt = (clx == 0 ? 2 : 1) * (ycl[j] == 0 ? 2 : 1);
-        yinv[j] = mul_r(m.inv_me_f, inv_count<float>(cnt));
-    }
-    // the sweep: column tx of the tile, its x class and rows
-    const int gxt = gx0 + tx;
-    const int clxt = node_class<P>(gxt, m.nnx, m.px);
-    __syncthreads();  // weights ready
-    float wcx[NW], wmx[NW], wst[NW];
-#pragma unroll
-    for (int k = 0; k < NW; ++k) {
-        wcx[k] = WC[clx][k];
-        wmx[k] = WM[clx][k];
-        wst[k] = WM[clxt][k];
-    }
+#pragma unroll 1
     for (int c = 0; c < NC; ++c) {
-        if (c > 0) __syncthreads();  // previous component consumed
-        // u of component c on the tile plus a halo of 2p nodes
-        const float* uc = u + (long long)c * m.NN;
 #pragma unroll
         for (int j = 0; j < NA; ++j) {
-            const int i = tid + j * NT;
-            if (i < HY2 * HX2) ws[i] = aoff[j] >= 0 ? __ldcg(&uc[aoff[j]]) : 0.f;
+            const int i = tid + j * NT, r = i / TL::W2, q = i - r * TL::W2;
+            if (i < TL::W2 * TL::H2) A[(q % P) * TL::PU + r * TL::S2 + q / P] = next[j];
         }
         __syncthreads();
-        // grad stencil along x for the columns of the p halo, all 2p-halo rows
-        if (hv) {
+        if (c + 1 < NC) {
+            const R* __restrict__ uc = u + (c + 1) * m.NN;
 #pragma unroll
-            for (int j = 0; j < NXP; ++j) {
-                const int r = rg + RG * j;
-                if (r < HY2) {
-                    float sc = 0.f, sm = 0.f;
+            for (int j = 0; j < NA; ++j)
+                if (off[j] >= 0) next[j] = __ldcg(&uc[off[j]]);
+        }
+        for (int i = tid; i < TL::H2 * TL::S1; i += NT) {
+            const int r = i / TL::S1, s = i - r * TL::S1;
+            if (s >= ns || r >= nr) continue;
+            if (!SWEEP && (s == 0 || s > TEX || r < P || r >= TL::H2 - P)) continue;  // feeds the halo only
+            R x[2 * P + 1], o[P];
+            seg_x<R, P>(A, TL::PU, r * TL::S2 + s + 1, x);
+            const int kind = vertex_kind(gx0 + (s - 1) * P, m.nnx, m.px);
+            seg_apply<R, P, 1>(T, x, vertex_weight<R, P, 1>(T, kind), o);
 #pragma unroll
-                    for (int k = 0; k < NW; ++k) {
-                        const float x = A[r][cx + k];
-                        sc = fma_r(wcx[k], x, sc);
-                        sm = fma_r(wmx[k], x, sm);
-                    }
-                    tC[r][cx] = sc;
-                    tM[r][cx] = sm;
+            for (int a = 0; a < P; ++a) B[a * TL::PT + i] = o[a];
+            seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, kind), o);
+#pragma unroll
+            for (int a = 0; a < P; ++a) B[(P + a) * TL::PT + i] = o[a];
+        }
+        __syncthreads();
+        // b and g0 = b / m_i (zero outside the mesh) on column q of the halo
+        // tile and the rows of y segment sy
+        R ob[NJ][2][P], og[NJ][2][P];
+        auto column = [&](int q, int sy, R(&bx)[P], R(&by)[P], R(&vx)[P], R(&vy)[P]) {
+            const int a = q % P, s = q / P;
+            const int gx = gx0 - P + q, gyv = gy0 + (sy - 1) * P;
+            const int kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
+            R t[2 * P + 1];
+            seg_y<R, P>(B + a * TL::PT, TL::S1, s, (sy + 1) * P, t);
+            seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), bx);
+            seg_y<R, P>(B + (P + a) * TL::PT, TL::S1, s, (sy + 1) * P, t);
+            seg_apply<R, P, 1>(T, t, vertex_weight<R, P, 1>(T, ky), by);
+            const bool inx = m.px || (gx >= 0 && gx < m.nnx);
+#pragma unroll
+            for (int b = 0; b < P; ++b) {
+                const int gy = gyv + b;
+                const bool in = inx && (m.py || (gy >= 0 && gy < m.nny));
+                const R inv = seg_inv_mass<R, P>(m, a, kx, b, ky);
+                bx[b] = mul_r(h, bx[b]);
+                by[b] = mul_r(h, by[b]);
+                vx[b] = in ? mul_r(bx[b], inv) : R(0);
+                vy[b] = in ? mul_r(by[b], inv) : R(0);
+                if (SWEEP && (sy <= TEY || b == 0)) {
+                    const int at = a * TL::PG + (sy * P + b) * TL::S1 + s;
+                    A[at] = vx[b];
+                    A[P * TL::PG + at] = vy[b];
                 }
             }
-        }
-        __syncthreads();
-        // along y: b and g0 = b / m_i on the p halo (zero outside the mesh)
-        if (hv) {
-#pragma unroll
-            for (int j = 0; j < NYP; ++j) {
-                const int r = rg + RG * j;
-                if (r < HY1) {
-                    const int cly = ycl[j];
-                    float sx = 0.f, sy = 0.f;
-#pragma unroll
-                    for (int k = 0; k < NW; ++k) {
-                        sx = fma_r(WM[cly][k], tC[r + k][cx], sx);
-                        sy = fma_r(WC[cly][k], tM[r + k][cx], sy);
-                    }
-                    const float bx = mul_r(h, sx), by = mul_r(h, sy);
-                    G[0][r][cx] = yin[j] ? mul_r(bx, yinv[j]) : 0.f;
-                    G[1][r][cx] = yin[j] ? mul_r(by, yinv[j]) : 0.f;
-                    const int rt = r - P, ct = cx - P;
-                    if (rt >= 0 && rt < ST_TY && ct >= 0 && ct < ST_TX) {
-                        Bt[0][rt][ct] = bx;
-                        Bt[1][rt][ct] = by;
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        // first sweep, along x for every p-halo row (the mass weights)
-#pragma unroll
-        for (int j = 0; j < NSX; ++j) {
-            const int r = ty + ST_BY * j;
-            if (r < HY1) {
-#pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                    float sx = 0.f;
-#pragma unroll
-                    for (int k = 0; k < NW; ++k) sx = fma_r(wst[k], G[f][r][tx + k], sx);
-                    t[f][r][tx] = sx;
-                }
-            }
-        }
-        __syncthreads();
-        // along y and the outputs: g1 (and b where more sweeps follow)
+        };
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-            const int r = ty + j * ST_BY, gy = gy0 + r;
-            if (gxt >= m.nnx || gy >= m.nny) continue;
-            const int cly = node_class<P>(gy, m.nny, m.py);
-            const int cnt = (clxt == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-            const float inv_mi = mul_r(m.inv_me_f, inv_count<float>(cnt));
-            const long long node = (long long)gy * m.nnx + gxt;
+            const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
+            if (i < TL::NOWN && gx0 + q < m.nnx + P && gy0 + sy * P < m.nny + P)
+                column(q + P, sy + 1, ob[j][0], ob[j][1], og[j][0], og[j][1]);
+        }
+        if constexpr (!SWEEP) {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
+                const int gx = gx0 + q, gyv = gy0 + sy * P;
+                if (i >= TL::NOWN || gx >= m.nnx || gyv >= m.nny) continue;
+#pragma unroll
+                for (int f = 0; f < 2; ++f) {
+                    const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + gx;
+#pragma unroll
+                    for (int b = 0; b < P; ++b)
+                        if (gyv + b < m.nny) {
+                            bout[node + (long long)b * m.nnx] = ob[j][f][b];
+                            gout[node + (long long)b * m.nnx] = og[j][f][b];
+                        }
+                }
+            }
+            continue;  // the next staging writes u, which no one reads any more
+        }
+        // the halo: the rows below and above the tile, then its sides
+        constexpr int NROW = 2 * TL::W1, NEXT = NROW + (P + 1) * TEY;
+        for (int i = tid; i < NEXT; i += NT) {
+            int q, sy;
+            if (i < NROW) {
+                sy = i < TL::W1 ? 0 : TEY + 1;
+                q = i < TL::W1 ? i : i - TL::W1;
+            } else {
+                const int k = i - NROW, w = k % (P + 1);
+                sy = k / (P + 1) + 1;
+                q = w < P ? w : TL::W1 - 1;
+            }
+            R b0[P], b1[P], v0[P], v1[P];
+            column(q, sy, b0, b1, v0, v1);
+        }
+        __syncthreads();
+        const int ns0 = ns - 2, nr1 = min(TL::H1, m.nny - gy0 + 2 * P);
+        for (int i = tid; i < 2 * TL::H1 * TEX; i += NT) {
+            const int f = i / (TL::H1 * TEX), k = i - f * (TL::H1 * TEX), r = k / TEX, s = k - r * TEX;
+            if (s >= ns0 || r >= nr1) continue;
+            R x[2 * P + 1], o[P];
+            seg_x<R, P>(A + f * P * TL::PG, TL::PG, r * TL::S1 + s + 1, x);
+            seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, vertex_kind(gx0 + s * P, m.nnx, m.px)), o);
+#pragma unroll
+            for (int a = 0; a < P; ++a) B[(f * P + a) * TL::PS + k] = o[a];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
+            const int gx = gx0 + q, gyv = gy0 + sy * P;
+            if (i >= TL::NOWN || gx >= m.nnx || gyv >= m.nny) continue;
+            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
-                float sy = 0.f;
+                R t[2 * P + 1], o[P];
+                seg_y<R, P>(B + (f * P + a) * TL::PS, TEX, q / P, (sy + 1) * P, t);
+                seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
+                const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + gx;
 #pragma unroll
-                for (int k = 0; k < NW; ++k) sy = fma_r(WM[cly][k], t[f][r + k][tx], sy);
-                const long long k = (long long)(f * NC + c) * m.NN + node;
-                gout[k] = sweep_value(G[f][r + P][tx + P], Bt[f][r][tx], sy, h2, inv_mi);
-                if (bout) bout[k] = Bt[f][r][tx];
+                for (int b = 0; b < P; ++b)
+                    if (gyv + b < m.nny) {
+                        const long long k = node + (long long)b * m.nnx;
+                        gout[k] = sweep_value(og[j][f][b], ob[j][f][b], o[b], h2, seg_inv_mass<R, P>(m, a, kx, b, ky));
+                        if (bout) bout[k] = ob[j][f][b];
+                    }
             }
         }
     }
 }
 
-template <int P, int NC>
-__global__ void __launch_bounds__(ST_TX * ST_BY)
-    k_grad_sweep(MeshDev m, const float* __restrict__ u, float* __restrict__ bout, float* __restrict__ gout) {
+// x pass of a mass sweep for FB iterates staged at X (planes PG), into Y
+template <class R, int P, int FB, class TL>
+DEV void sweep_x(const MeshDev& m, const Tab<R>& T, const R* X, R* Y, int gx0, int gy0, int tid) {
+    constexpr int TEX = TL::TEX;
+    const int ns = (m.nnx - gx0 + P - 1) / P, nr = min(TL::H1, m.nny - gy0 + 2 * P);
+    for (int i = tid; i < FB * TL::H1 * TEX; i += TL::NT) {
+        const int f = i / (TL::H1 * TEX), k = i - f * (TL::H1 * TEX), r = k / TEX, s = k - r * TEX;
+        if (s >= ns || r >= nr) continue;
+        R x[2 * P + 1], o[P];
+        seg_x<R, P>(X + f * P * TL::PG, TL::PG, r * TL::S1 + s + 1, x);
+        seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, vertex_kind(gx0 + s * P, m.nnx, m.px)), o);
+#pragma unroll
+        for (int a = 0; a < P; ++a) Y[(f * P + a) * TL::PS + k] = o[a];
+    }
+}
+
+// one Richardson sweep for NV fields on the tile; ws: TL::sweep_ws values
+template <class R, int P, int NV, class TL>
+DEV void mass_sweep_seg(const MeshDev& m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout,
+                        int gx0, int gy0, int tid, R* ws) {
+    constexpr int NT = TL::NT, NX = TL::NX;
+    constexpr int NA = (TL::W1 * TL::H1 + NT - 1) / NT;
+    R* A = ws;
+    R* B = ws + P * TL::PG;
+    const Tab<R>& T = tab_of<R>(m, P);
+    const R h2 = PV<R>::h2(m);
+    long long off[NA];
+    R next[NA];
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+        const int i = tid + j * NT, r = i / TL::W1, q = i - r * TL::W1;
+        int gx = gx0 - P + q, gy = gy0 - P + r;
+        const bool in = r < TL::H1 && wrap_node(m, gx, gy);
+        off[j] = in ? (long long)gy * m.nnx + gx : -1;
+        next[j] = in ? xin[off[j]] : R(0);
+    }
+#pragma unroll 1
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+        for (int j = 0; j < NA; ++j) {
+            const int i = tid + j * NT, r = i / TL::W1, q = i - r * TL::W1;
+            if (i < TL::W1 * TL::H1) A[(q % P) * TL::PG + r * TL::S1 + q / P] = next[j];
+        }
+        __syncthreads();
+        if (v + 1 < NV) {
+            const R* __restrict__ xv = xin + (v + 1) * m.NN;
+#pragma unroll
+            for (int j = 0; j < NA; ++j)
+                if (off[j] >= 0) next[j] = xv[off[j]];
+        }
+        sweep_x<R, P, 1, TL>(m, T, A, B, gx0, gy0, tid);
+        __syncthreads();
+        for (int i = tid; i < TL::NOWN; i += NT) {
+            const int sy = i / NX, q = i - sy * NX, gx = gx0 + q, gyv = gy0 + sy * P;
+            if (gx >= m.nnx || gyv >= m.nny) continue;
+            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
+            R t[2 * P + 1], o[P];
+            seg_y<R, P>(B + a * TL::PS, TL::TEX, q / P, (sy + 1) * P, t);
+            seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
+            const long long node = v * m.NN + (long long)gyv * m.nnx + gx;
+#pragma unroll
+            for (int c = 0; c < P; ++c)
+                if (gyv + c < m.nny) {
+                    const long long k = node + (long long)c * m.nnx;
+                    xout[k] = sweep_value(A[a * TL::PG + ((sy + 1) * P + c) * TL::S1 + q / P + 1], b[k], o[c], h2,
+                                          seg_inv_mass<R, P>(m, a, kx, c, ky));
+                }
+        }
+        if (v + 1 < NV) __syncthreads();  // the iterate is consumed
+    }
+}
+
+// Gather of the element residuals, lumped iterate and first sweep on the
+// tile.  A thread gathers the p x p nodes of one vertex segment pair: each of
+// the (p+1)^2 element values it needs is read once, a warp's reads of one
+// value are consecutive in the element index, and no lane branches on its
+// node's position in the element.  r = sum over E_i (stored for further sweeps
+// and diagnostics), udot0 = r / m_i, udot1 = udot0 + (r - M_C udot0) / m_i.
+// ws: TL::udot_ws(NC) values.
+template <class R, int P, int NC, class TL>
+DEV void udot_sweep_seg(const MeshDev& m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout, int gx0,
+                        int gy0, int tid, R* ws) {
+    constexpr int NT = TL::NT, NX = TL::NX, TEX = TL::TEX, TEY = TL::TEY, N1 = P + 1;
+    constexpr int FB = TL::udot_fields(NC);
+    R* A = ws;                    // udot0 on the one-element halo
+    R* B = A + FB * P * TL::PG;   // its x pass
+    R* C = B + FB * P * TL::PS;   // r on the tile
+    const Tab<R>& T = tab_of<R>(m, P);
+    const R h2 = PV<R>::h2(m);
+    const int ex0 = gx0 / P, ey0 = gy0 / P;
+    const long long E = m.E;
+#pragma unroll 1
+    for (int v0 = 0; v0 < NC; v0 += FB) {
+        if (v0 > 0) __syncthreads();  // the previous fields are consumed
+        for (int i = tid; i < (TEX + 2) * (TEY + 2); i += NT) {
+            const int sy = i / (TEX + 2), sx = i - sy * (TEX + 2);
+            // the elements before (l) and after (h) the vertex along x and y;
+            // hx, hy false: the segment has its vertex only (or lies outside)
+            int xl = ex0 + sx - 2, xh = xl + 1, yl = ey0 + sy - 2, yh = yl + 1;
+            if (xl > m.nx || yl > m.ny) continue;  // feeds no node of the mesh
+            if (m.px) xl = wrap_periodic(xl, m.nx), xh = wrap_periodic(xh, m.nx);
+            if (m.py) yl = wrap_periodic(yl, m.ny), yh = wrap_periodic(yh, m.ny);
+            const bool lx = xl >= 0 && xl < m.nx, hx = xh >= 0 && xh < m.nx;
+            const bool ly = yl >= 0 && yl < m.ny, hy = yh >= 0 && yh < m.ny;
+            const int kx = m.px ? 0 : (!lx ? 1 : !hx ? 2 : 0), ky = m.py ? 0 : (!ly ? 1 : !hy ? 2 : 0);
+            const bool tile = sx >= 1 && sx <= TEX && sy >= 1 && sy <= TEY;
+            const long long ell = (long long)yl * m.nx + xl, ehl = (long long)yl * m.nx + xh;
+            const long long elh = (long long)yh * m.nx + xl, ehh = (long long)yh * m.nx + xh;
+#pragma unroll
+            for (int f = 0; f < FB; ++f) {
+                const R* __restrict__ Ev = ER + (v0 + f) * E;
+                auto val = [&](bool in, long long e, int a, int b) {
+                    return in ? Ev[(long long)((b * N1 + a) * NC) * E + e] : R(0);
+                };
+#pragma unroll
+                for (int b = 0; b < P; ++b)
+#pragma unroll
+                    for (int a = 0; a < P; ++a) {
+                        // past the last vertex of the halo
+                        if ((a > 0 && sx == TEX + 1) || (b > 0 && sy == TEY + 1)) continue;
+                        R s;
+                        bool in;
+                        if (a == 0 && b == 0) {
+                            s = ((val(lx && ly, ell, P, P) + val(hx && ly, ehl, 0, P)) + val(lx && hy, elh, P, 0)) +
+                                val(hx && hy, ehh, 0, 0);
+                            in = (lx || hx) && (ly || hy);
+                        } else if (b == 0) {
+                            s = val(hx && ly, ehl, a, P) + val(hx && hy, ehh, a, 0);
+                            in = hx && (ly || hy);
+                        } else if (a == 0) {
+                            s = val(lx && hy, elh, P, b) + val(hx && hy, ehh, 0, b);
+                            in = (lx || hx) && hy;
+                        } else {
+                            s = val(hx && hy, ehh, a, b);
+                            in = hx && hy;
+                        }
+                        const int q = sx, row = sy * P + b;
+                        A[(f * P + a) * TL::PG + row * TL::S1 + q] =
+                            in ? mul_r(s, seg_inv_mass<R, P>(m, a, kx, b, ky)) : R(0);
+                        if (tile) C[(f * P + a) * TL::PR + (row - P) * TEX + q - 1] = s;
+                    }
+            }
+        }
+        __syncthreads();
+        sweep_x<R, P, FB, TL>(m, T, A, B, gx0, gy0, tid);
+        __syncthreads();
+        for (int i = tid; i < TL::NOWN; i += NT) {
+            const int sy = i / NX, q = i - sy * NX, gx = gx0 + q, gyv = gy0 + sy * P;
+            if (gx >= m.nnx || gyv >= m.nny) continue;
+            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
+#pragma unroll
+            for (int f = 0; f < FB; ++f) {
+                R t[2 * P + 1], o[P];
+                seg_y<R, P>(B + (f * P + a) * TL::PS, TEX, q / P, (sy + 1) * P, t);
+                seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
+                const long long node = (v0 + f) * m.NN + (long long)gyv * m.nnx + gx;
+#pragma unroll
+                for (int c = 0; c < P; ++c)
+                    if (gyv + c < m.nny) {
+                        const long long k = node + (long long)c * m.nnx;
+                        const R r = C[(f * P + a) * TL::PR + (sy * P + c) * TEX + q / P];
+                        rout[k] = r;
+                        xout[k] = sweep_value(A[(f * P + a) * TL::PG + ((sy + 1) * P + c) * TL::S1 + q / P + 1], r, o[c],
+                                              h2, seg_inv_mass<R, P>(m, a, kx, c, ky));
+                    }
+            }
+        }
+    }
+}
+
+// The tiles of the single-state kernels.  Large: about 1024 nodes and 256
+// threads (float64 with fewer rows at p >= 3, where 48 KB of shared memory
+// ends); small: 4 x 4 elements (8 x 8 at p = 1) and 64 threads, for meshes
+// whose large tiles leave SMs idle.
+template <class R, int P, bool SMALL>
+struct StageTile {
+    static constexpr bool F = sizeof(R) == 4;
+    static constexpr int X = SMALL ? (P == 1 ? 8 : 4) : (P == 1 ? 32 : P == 2 ? 16 : P == 3 ? 12 : 8);
+    static constexpr int Y = SMALL ? (P == 1 ? 8 : 4) : (P <= 2 ? 16 : P == 3 ? (F ? 12 : 7) : (F ? 8 : 6));
+    using type = SegTile<R, P, X, Y, SMALL ? 64 : 256>;
+};
+template <class R, int P, bool SMALL>
+using stage_tile_t = typename StageTile<R, P, SMALL>::type;
+
+template <class R, int P, int NC, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 64 : 256, SMALL ? 1 : (sizeof(R) == 4 ? 3 : 2))
+    k_grad_sweep(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
+    using TL = stage_tile_t<R, P, SMALL>;
     // like k_grad_rhs: runs beside k_pre, waits for it before exiting
     pdl_trigger();
-    __shared__ float ws[GradSweepWs<P, NC>::size];
-    grad_sweep_block<P, NC>(m, u, bout, gout, blockIdx.x * ST_TX, blockIdx.y * ST_TY, threadIdx.x, threadIdx.y, ws);
+    __shared__ R ws[TL::grad_ws];
+    grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
     pdl_wait();
 }
 
+template <class R, int P, int NC, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 64 : 256)
+    k_grad_rhs(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
+    using TL = stage_tile_t<R, P, SMALL>;
+    // needs only u, whose last writer completed before k_pre let this kernel
+    // start (pdl_wait_then_trigger), so it runs beside k_pre and waits for it
+    // only before exiting
+    pdl_trigger();
+    __shared__ R ws[TL::grad_ws];
+    grad_sweep_seg<R, P, NC, TL, false>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
+    pdl_wait();
+}
 
-template <int P, int NC>
-struct UdotSweepWs {
-    static constexpr int HX = ST_TX + 2 * P, HY = ST_TY + 2 * P, NW = 2 * P + 1, NCL = P + 2;
-    static constexpr int size = NC * (HY * HX + HY * ST_TX + ST_TY * ST_TX) + NCL * NW;
-};
-
-// r = sum over E_i of the element residuals (stored for further sweeps and
-// diagnostics), udot0 = r / m_i on the tile plus a p halo, and the first
-// sweep udot1 = udot0 + (r - M_C udot0) / m_i on the tile
-template <int P, int NC>
-__global__ void __launch_bounds__(ST_TX * ST_BY)
-    k_udot_sweep(MeshDev m, const float* __restrict__ ER, float* __restrict__ rout, float* __restrict__ xout) {
+template <class R, int P, int NC, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 64 : 256)
+    k_udot_sweep(MeshDev m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout) {
+    using TL = stage_tile_t<R, P, SMALL>;
     pdl_begin();
-    using WS = UdotSweepWs<P, NC>;
-    constexpr int HX = WS::HX, HY = WS::HY, NW = WS::NW, NCL = WS::NCL;
-    constexpr int NT = ST_TX * ST_BY, NJ = ST_TY / ST_BY;
-    __shared__ float ws[WS::size];
-    float(*xs)[HY][HX] = reinterpret_cast<float(*)[HY][HX]>(ws);
-    float(*t)[HY][ST_TX] = reinterpret_cast<float(*)[HY][ST_TX]>(ws + NC * HY * HX);
-    float(*rt)[ST_TY][ST_TX] = reinterpret_cast<float(*)[ST_TY][ST_TX]>(ws + NC * (HY * HX + HY * ST_TX));
-    float(*W)[NW] = reinterpret_cast<float(*)[NW]>(ws + NC * (HY * HX + HY * ST_TX + ST_TY * ST_TX));
-    const Tab<float>& T = TabSel<float>::t(P);
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * ST_TX + tx;
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        W[cls][k] = class_weight<float, P, 0>(T, cls, k - P);
-    }
-    const int gx0 = blockIdx.x * ST_TX, gy0 = blockIdx.y * ST_TY;
-    // gathers on the tile plus a p halo (gather_init_at's arithmetic)
-    for (int i = tid; i < HY * HX; i += NT) {
-        const int r = i / HX, cc = i - r * HX;
-        int gx = gx0 - P + cc, gy = gy0 - P + r;
-        const bool in = wrap_node(m, gx, gy);
-        float s[NC];
-        float inv_mi = 0.f;
-        if (in) {
-            const NodeC<P> nc = node_c<P>(m, gx, gy);
-            gather_at<float, P, NC>(m, ER, nc, s);
-            inv_mi = PV<float>::inv_me(m) * inv_count<float>(nc.nxc * nc.nyc);
-        }
-        const int rr = r - P, ct = cc - P;
-        const bool tile = rr >= 0 && rr < ST_TY && ct >= 0 && ct < ST_TX;
-        // a node of this tile itself, not a wrapped copy of another tile's
-        const bool own = tile && gx0 + ct < m.nnx && gy0 + rr < m.nny;
-        const long long node = (long long)gy * m.nnx + gx;
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            xs[v][r][cc] = in ? s[v] * inv_mi : 0.f;
-            if (tile) {
-                rt[v][rr][ct] = in ? s[v] : 0.f;
-                if (in && own) rout[v * m.NN + node] = s[v];
-            }
-        }
-    }
-    __syncthreads();
-    const int gx = gx0 + tx;
-    const int clx = node_class<P>(gx, m.nnx, m.px);
-    for (int r = ty; r < HY; r += ST_BY) {
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            float sx = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) sx = fma_r(W[clx][k], xs[v][r][tx + k], sx);
-            t[v][r][tx] = sx;
-        }
-    }
-    __syncthreads();
-    const float h2 = PV<float>::h2(m);
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        const int r = ty + j * ST_BY, gy = gy0 + r;
-        if (gx >= m.nnx || gy >= m.nny) continue;
-        const int cly = node_class<P>(gy, m.nny, m.py);
-        const int cnt = (clx == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-        const float inv_mi = mul_r(PV<float>::inv_me(m), inv_count<float>(cnt));
-        const long long node = (long long)gy * m.nnx + gx;
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            float sy = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) sy = fma_r(W[cly][k], t[v][r + k][tx], sy);
-            xout[v * m.NN + node] = sweep_value(xs[v][r + P][tx + P], rt[v][r][tx], sy, h2, inv_mi);
-        }
-    }
+    __shared__ R ws[TL::udot_ws(NC)];
+    udot_sweep_seg<R, P, NC, TL>(m, ER, rout, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
 }
 
-// ---------------------------------------------------------------------------
-// The two fused sweeps as functions of one ST_TX x ST_TY node tile for a block
-// of NT threads (the batched stage runs them with 128 threads per block),
-// geometry formed per component: the same arithmetic, in the same order, as
-// k_grad_sweep and k_udot_sweep, hence the same bits as the separate
-// stencils.  ws holds GradSweepWs<P, NC>::size or UdotSweepWs<P, NC>::size
-// floats; the block's threads all call them (they synchronise the block).
-// ---------------------------------------------------------------------------
-template <int P, int NC, int NT>
-DEV void grad_sweep_tile(const MeshDev& m, const float* __restrict__ u, float* __restrict__ bout,
-                         float* __restrict__ gout, int gx0, int gy0, int tid, float* ws) {
-    using WS = GradSweepWs<P, NC>;
-    constexpr int HX1 = WS::HX1, HY1 = WS::HY1, HX2 = WS::HX2, HY2 = WS::HY2, NW = WS::NW, NCL = WS::NCL;
-    constexpr int BYT = NT / ST_TX, NJ = ST_TY / BYT;
-    float(*A)[HX2] = reinterpret_cast<float(*)[HX2]>(ws);
-    float(*tC)[HX1] = reinterpret_cast<float(*)[HX1]>(ws + WS::A);
-    float(*tM)[HX1] = reinterpret_cast<float(*)[HX1]>(ws + WS::A + HY2 * HX1);
-    float(*t)[HY1][ST_TX] = reinterpret_cast<float(*)[HY1][ST_TX]>(ws + WS::A);
-    float(*G)[HY1][HX1] = reinterpret_cast<float(*)[HY1][HX1]>(ws + WS::A + WS::B);
-    float(*Bt)[ST_TY][ST_TX] = reinterpret_cast<float(*)[ST_TY][ST_TX]>(ws + WS::A + WS::B + WS::C);
-    float(*WM)[NW] = reinterpret_cast<float(*)[NW]>(ws + WS::A + WS::B + WS::C + WS::D);
-    float(*WC)[NW] = reinterpret_cast<float(*)[NW]>(ws + WS::A + WS::B + WS::C + WS::D + NCL * NW);
-    const Tab<float>& T = TabSel<float>::t(P);
-    const int tx = tid % ST_TX, ty = tid / ST_TX;
-    __syncthreads();  // the previous user of ws is done
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        WM[cls][k] = class_weight<float, P, 0>(T, cls, k - P);
-        WC[cls][k] = class_weight<float, P, 1>(T, cls, k - P);
-    }
-    const float h = m.h_f, h2 = m.h2_f;
-    for (int c = 0; c < NC; ++c) {
-        __syncthreads();
-        for (int i = tid; i < HY2 * HX2; i += NT) {
-            const int r = i / HX2, cc = i - r * HX2;
-            int gx = gx0 - 2 * P + cc, gy = gy0 - 2 * P + r;
-            const bool in = wrap_node(m, gx, gy);
-            A[r][cc] = in ? __ldcg(&u[(long long)c * m.NN + (long long)gy * m.nnx + gx]) : 0.f;
-        }
-        __syncthreads();
-        for (int i = tid; i < HY2 * HX1; i += NT) {
-            const int r = i / HX1, cc = i - r * HX1;
-            int gx = gx0 - P + cc, gy = 0;
-            wrap_node(m, gx, gy);
-            const int clx = node_class<P>(gx, m.nnx, m.px);
-            float sc = 0.f, sm = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                const float x = A[r][cc + k];
-                sc = fma_r(WC[clx][k], x, sc);
-                sm = fma_r(WM[clx][k], x, sm);
-            }
-            tC[r][cc] = sc;
-            tM[r][cc] = sm;
-        }
-        __syncthreads();
-        for (int i = tid; i < HY1 * HX1; i += NT) {
-            const int r = i / HX1, cc = i - r * HX1;
-            int gx = gx0 - P + cc, gy = gy0 - P + r;
-            const bool in = wrap_node(m, gx, gy);
-            const int clx = node_class<P>(gx, m.nnx, m.px), cly = node_class<P>(gy, m.nny, m.py);
-            float sx = 0.f, sy = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                sx = fma_r(WM[cly][k], tC[r + k][cc], sx);
-                sy = fma_r(WC[cly][k], tM[r + k][cc], sy);
-            }
-            const int cnt = (clx == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-            const float inv_mi = mul_r(m.inv_me_f, inv_count<float>(cnt));
-            const float bx = mul_r(h, sx), by = mul_r(h, sy);
-            G[0][r][cc] = in ? mul_r(bx, inv_mi) : 0.f;
-            G[1][r][cc] = in ? mul_r(by, inv_mi) : 0.f;
-            const int rt = r - P, ct = cc - P;
-            if (rt >= 0 && rt < ST_TY && ct >= 0 && ct < ST_TX) {
-                Bt[0][rt][ct] = bx;
-                Bt[1][rt][ct] = by;
-            }
-        }
-        __syncthreads();
-        const int gxt = gx0 + tx;
-        const int clxt = node_class<P>(gxt, m.nnx, m.px);
-        for (int r = ty; r < HY1; r += BYT) {
-#pragma unroll
-            for (int f = 0; f < 2; ++f) {
-                float sx = 0.f;
-#pragma unroll
-                for (int k = 0; k < NW; ++k) sx = fma_r(WM[clxt][k], G[f][r][tx + k], sx);
-                t[f][r][tx] = sx;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int r = ty + j * BYT, gy = gy0 + r;
-            if (gxt >= m.nnx || gy >= m.nny) continue;
-            const int cly = node_class<P>(gy, m.nny, m.py);
-            const int cnt = (clxt == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-            const float inv_mi = mul_r(m.inv_me_f, inv_count<float>(cnt));
-            const long long node = (long long)gy * m.nnx + gxt;
-#pragma unroll
-            for (int f = 0; f < 2; ++f) {
-                float sy = 0.f;
-#pragma unroll
-                for (int k = 0; k < NW; ++k) sy = fma_r(WM[cly][k], t[f][r + k][tx], sy);
-                const long long k = (long long)(f * NC + c) * m.NN + node;
-                gout[k] = sweep_value(G[f][r + P][tx + P], Bt[f][r][tx], sy, h2, inv_mi);
-                if (bout) bout[k] = Bt[f][r][tx];
-            }
-        }
-    }
-}
-
-template <int P, int NC, int NT>
-DEV void udot_sweep_tile(const MeshDev& m, const float* __restrict__ ER, float* __restrict__ rout,
-                         float* __restrict__ xout, int gx0, int gy0, int tid, float* ws) {
-    using WS = UdotSweepWs<P, NC>;
-    constexpr int HX = WS::HX, HY = WS::HY, NW = WS::NW, NCL = WS::NCL;
-    constexpr int BYT = NT / ST_TX, NJ = ST_TY / BYT;
-    float(*xs)[HY][HX] = reinterpret_cast<float(*)[HY][HX]>(ws);
-    float(*t)[HY][ST_TX] = reinterpret_cast<float(*)[HY][ST_TX]>(ws + NC * HY * HX);
-    float(*rt)[ST_TY][ST_TX] = reinterpret_cast<float(*)[ST_TY][ST_TX]>(ws + NC * (HY * HX + HY * ST_TX));
-    float(*W)[NW] = reinterpret_cast<float(*)[NW]>(ws + NC * (HY * HX + HY * ST_TX + ST_TY * ST_TX));
-    const Tab<float>& T = TabSel<float>::t(P);
-    const int tx = tid % ST_TX, ty = tid / ST_TX;
-    __syncthreads();  // the previous user of ws is done
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        W[cls][k] = class_weight<float, P, 0>(T, cls, k - P);
-    }
-    for (int i = tid; i < HY * HX; i += NT) {
-        const int r = i / HX, cc = i - r * HX;
-        int gx = gx0 - P + cc, gy = gy0 - P + r;
-        const bool in = wrap_node(m, gx, gy);
-        float s[NC];
-        float inv_mi = 0.f;
-        if (in) {
-            const NodeC<P> nc = node_c<P>(m, gx, gy);
-            gather_at<float, P, NC>(m, ER, nc, s);
-            inv_mi = PV<float>::inv_me(m) * inv_count<float>(nc.nxc * nc.nyc);
-        }
-        const int rr = r - P, ct = cc - P;
-        const bool tile = rr >= 0 && rr < ST_TY && ct >= 0 && ct < ST_TX;
-        // a node of this tile itself, not a wrapped copy of another tile's
-        const bool own = tile && gx0 + ct < m.nnx && gy0 + rr < m.nny;
-        const long long node = (long long)gy * m.nnx + gx;
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            xs[v][r][cc] = in ? s[v] * inv_mi : 0.f;
-            if (tile) {
-                rt[v][rr][ct] = in ? s[v] : 0.f;
-                if (in && own) rout[v * m.NN + node] = s[v];
-            }
-        }
-    }
-    __syncthreads();
-    const int gx = gx0 + tx;
-    const int clx = node_class<P>(gx, m.nnx, m.px);
-    for (int r = ty; r < HY; r += BYT) {
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            float sx = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) sx = fma_r(W[clx][k], xs[v][r][tx + k], sx);
-            t[v][r][tx] = sx;
-        }
-    }
-    __syncthreads();
-    const float h2 = PV<float>::h2(m);
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        const int r = ty + j * BYT, gy = gy0 + r;
-        if (gx >= m.nnx || gy >= m.nny) continue;
-        const int cly = node_class<P>(gy, m.nny, m.py);
-        const int cnt = (clx == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-        const float inv_mi = mul_r(PV<float>::inv_me(m), inv_count<float>(cnt));
-        const long long node = (long long)gy * m.nnx + gx;
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            float sy = 0.f;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) sy = fma_r(W[cly][k], t[v][r + k][tx], sy);
-            xout[v * m.NN + node] = sweep_value(xs[v][r + P][tx + P], rt[v][r][tx], sy, h2, inv_mi);
-        }
-    }
+template <class R, int P, int NV, bool SMALL>
+__global__ void __launch_bounds__(SMALL ? 64 : 256)
+    k_mass_sweep(MeshDev m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout) {
+    using TL = stage_tile_t<R, P, SMALL>;
+    pdl_begin();
+    __shared__ R ws[TL::sweep_ws];
+    mass_sweep_seg<R, P, NV, TL>(m, xin, b, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
 }
 
 }  // namespace cgl

@@ -88,27 +88,22 @@ DEV long long node_of(const MeshDev& m, int ex, int ey, int a, int b) {
     return (long long)gy * m.nnx + gx;
 }
 
-// the global node indices of element (ex, ey), degree P = m.p: the columns
-// and row offsets are formed once per element (only the last column and row
-// can wrap, in a periodic direction), so that each node index is one add;
-// the same indices as node_of
-template <int P>
-struct ElemNodes {
-    int gx[P + 1];
-    long long row[P + 1];
-    DEV ElemNodes(const MeshDev& m, int ex, int ey) {
+// the coefficients of element (ex, ey) of one nodal field: one pointer per
+// row, constant offsets along it, and the last column and row, the only ones
+// that can wrap (in a periodic direction), at offsets of their own
+template <class R, int P>
+DEV void load_comp(const R* __restrict__ u, const MeshDev& m, int ex, int ey, R (&V)[(P + 1) * (P + 1)]) {
+    constexpr int N1 = P + 1;
+    const R* __restrict__ r0 = u + ((long long)(ey * P) * m.nnx + ex * P);
+    const int dx = (m.px && ex == m.nx - 1) ? -ex * P : P;
+    const int ry = (m.py && ey == m.ny - 1) ? -ey * P : P;
 #pragma unroll
-        for (int a = 0; a <= P; ++a) gx[a] = ex * P + a;
-        if (m.px && gx[P] == m.nnx) gx[P] = 0;
+    for (int b = 0; b < N1; ++b) {
+        const R* __restrict__ r = r0 + (long long)(b < P ? b : ry) * m.nnx;
 #pragma unroll
-        for (int b = 0; b <= P; ++b) {
-            int gy = ey * P + b;
-            if (b == P && m.py && gy == m.nny) gy = 0;
-            row[b] = (long long)gy * m.nnx;
-        }
+        for (int a = 0; a < N1; ++a) V[b * N1 + a] = r[a < P ? a : dx];
     }
-    DEV long long operator()(int a, int b) const { return row[b] + gx[a]; }
-};
+}
 
 // face neighbour (0 W, 1 E, 2 S, 3 N) or -1 on a non-periodic boundary
 DEV int neighbour(const MeshDev& m, int ex, int ey, int dir) {
@@ -221,16 +216,8 @@ DEV bool node_of_thread(const MeshDev& m, int& gx, int& gy, long long& node) {
 template <class R, int P, int NC>
 DEV void load_block(const R* __restrict__ u, const MeshDev& m, int ex, int ey,
                     R (&U)[NC][Dim<P>::N2]) {
-    constexpr int N1 = P + 1;
-    const ElemNodes<P> en(m, ex, ey);
 #pragma unroll
-    for (int b = 0; b < N1; ++b)
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            const long long g = en(a, b);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) U[c][b * N1 + a] = u[c * m.NN + g];
-        }
+    for (int c = 0; c < NC; ++c) load_comp<R, P>(u + c * m.NN, m, ex, ey, U[c]);
 }
 
 // element mean of the coefficients as float64: plain sum for double data;
@@ -441,17 +428,6 @@ DEV double euler_alpha_of(const double* ub, const double* f, double m, double ep
     else return euler_alpha<double>(ub, f, m, eps);
 }
 
-template <class R, int P>
-DEV void load_comp(const R* __restrict__ u, const MeshDev& m, int ex, int ey, int c, R (&V)[Dim<P>::N2]) {
-    constexpr int N1 = P + 1;
-    const ElemNodes<P> en(m, ex, ey);
-    const R* __restrict__ uc = u + (long long)c * m.NN;
-#pragma unroll
-    for (int b = 0; b < N1; ++b)
-#pragma unroll
-        for (int a = 0; a < N1; ++a) V[b * N1 + a] = uc[en(a, b)];
-}
-
 // gamma_e of one component whose field is u (modal.cuh) from the element's own
 // block, the neighbours' blocks loaded and transformed by this thread
 template <class R, int P>
@@ -465,7 +441,7 @@ DEV R sensor_scalar(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u
         int jx, jy;
         neighbour_xy(m, ex, ey, d, jx, jy);
         R V[N2];
-        load_comp<R, P>(u, m, jx, jy, 0, V);
+        load_comp<R, P>(u, m, jx, jy, V);
         modal_block<R, P>(T, V, l);
     });
 }
@@ -1109,13 +1085,21 @@ DEV int halo_pos(int tx, int ty, int d) {
     return (ty + 1 + (d == 2 ? -1 : d == 3 ? 1 : 0)) * (K_TX + 2) + tx + 1 + (d == 0 ? -1 : d == 1 ? 1 : 0);
 }
 
+// The node speeds of nu_e are formed once per node of the tile (an element
+// has (p+1)^2 nodes but brings p^2 new ones) and pass through the same
+// shared memory.
 template <class R, int P, class Ph, int TY>
 __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const R* __restrict__ u,
                                                     double* __restrict__ gam_out, double* __restrict__ nu_out) {
-    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, HE = (K_TX + 2) * (TY + 2), NT = K_TX * TY;
+    constexpr int NC = Ph::NC, N2 = Dim<P>::N2, HE = (K_TX + 2) * (TY + 2), NT = K_TX * TY;
+    constexpr int NH = (HE + NT - 1) / NT;                        // halo positions per thread
+    constexpr int SX = K_TX * P + 1, SY = TY * P + 1, NS = SX * SY;  // the tile's nodes
     // four continued candidates in registers where they leave two blocks per SM
     constexpr bool KEEP = (N2 - 1) * sizeof(R) <= 128;
-    __shared__ R sM[N2 - 1][HE];
+    constexpr int WS = (N2 - 1) * HE > NS ? (N2 - 1) * HE : NS;
+    __shared__ R ws[WS];
+    R(*sM)[HE] = reinterpret_cast<R(*)[HE]>(ws);
+    R(*sS)[SX] = reinterpret_cast<R(*)[SX]>(ws);
     pdl_wait_then_trigger();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * K_TX + tx;
     const int ex0 = blockIdx.x * K_TX, ey0 = blockIdx.y * TY;
@@ -1124,21 +1108,24 @@ __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const
     const Tab<R>& T = tab_of<R>(m, P);
     R gam = R(1);
     if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-        int nb[4];
+        int nb[4], hx[NH], hy[NH];
+        bool hv[NH];
 #pragma unroll
         for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
+#pragma unroll
+        for (int j = 0; j < NH; ++j)
+            hv[j] = tid + j * NT < HE && halo_elem<TY>(m, ex0, ey0, tid + j * NT, hx[j], hy[j]);
 #pragma unroll 1
         for (int c = 0; c < NC; ++c) {
             if (c > 0) __syncthreads();  // the previous component is consumed
-#pragma unroll 1
-            for (int i = tid; i < HE; i += NT) {
-                int jx, jy;
-                if (!halo_elem<TY>(m, ex0, ey0, i, jx, jy)) continue;
+#pragma unroll
+            for (int j = 0; j < NH; ++j) {
+                if (!hv[j]) continue;
                 R V[N2], l[N2];
-                load_comp<R, P>(u, m, jx, jy, c, V);
+                load_comp<R, P>(u + c * m.NN, m, hx[j], hy[j], V);
                 modal_block<R, P>(T, V, l);
 #pragma unroll
-                for (int k = 1; k < N2; ++k) sM[k - 1][i] = l[k];
+                for (int k = 1; k < N2; ++k) sM[k - 1][tid + j * NT] = l[k];
             }
             __syncthreads();
             if (valid) {
@@ -1156,29 +1143,34 @@ __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const
                 gam = fmin(gam, g);
             }
         }
+        __syncthreads();  // the modes are consumed
     } else {
         gam = (pr.mode == MODE_HO) ? R(1) : R(0);
     }
-    if (!valid) return;
-    R lm = R(0);
-    const int gxe = (m.px && ex * P + P == m.nnx) ? 0 : ex * P + P;  // the last column may wrap
-#pragma unroll 1
-    for (int b = 0; b < N1; ++b) {
-        int gy = ey * P + b;
+    for (int i = tid; i < NS; i += NT) {
+        const int r = i / SX, q = i - r * SX;
+        int gx = ex0 * P + q, gy = ey0 * P + r;
+        if (m.px && gx == m.nnx) gx = 0;
         if (m.py && gy == m.nny) gy = 0;
-        const R* __restrict__ ur = u + (long long)gy * m.nnx;
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
+        if (gx < m.nnx && gy < m.nny) {
+            const R* __restrict__ un = u + ((long long)gy * m.nnx + gx);
             R ui[NC];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) ui[c] = ur[c * m.NN + (a < P ? ex * P + a : gxe)];
-            lm = fmax(lm, Ph::template node_speed<R>(ui, pr));
+            for (int c = 0; c < NC; ++c) ui[c] = un[c * m.NN];
+            ws[i] = Ph::template node_speed<R>(ui, pr);
         }
     }
+    __syncthreads();
+    if (!valid) return;
+    R lm = R(0);
+#pragma unroll
+    for (int b = 0; b <= P; ++b)
+#pragma unroll
+        for (int a = 0; a <= P; ++a) lm = fmax(lm, sS[ty * P + b][tx * P + a]);
     const int e = ey * m.nx + ex;
     gam_out[e] = (double)gam;
     if constexpr (sizeof(R) == 4) nu_out[e] = (double)(lm * (m.h_f * (0.5f / P)));
-    else nu_out[e] = lm * (m.h * (0.5 / m.p));
+    else nu_out[e] = lm * (m.h * (0.5 / P));
 }
 
 // global dt from the block minima folded into the bit pattern by k_pre
@@ -1319,407 +1311,21 @@ DEV R sweep_value(R x, R b, R s, R h2, R inv_mi) {
 // k is sum over the (at most two) elements containing i of Ax[a_e][k + a_e]
 // (a_e = local index of i in e); likewise along y.
 // ---------------------------------------------------------------------------
-// 1D weights of the assembled mass (WHICH 0: M[a][c]) or of the derivative on
-// the trial index (WHICH 1: C[c][a] = int B_c' B_a) for offsets -P..P. The
-// node's first containing element has local index a0 (0..P); a second one
-// (n == 2, a shared vertex) has local index 0. Built from compile-time table
-// entries by selects (no runtime-indexed arrays).
+// entries of the 1D tables: the assembled mass (WHICH 0: M[a][c]) or the
+// derivative on the trial index (WHICH 1: C[c][a] = int B_c' B_a)
 template <class R, int P, int WHICH>
 DEV R wtab(const Tab<R>& T, int a, int c) {
     return (WHICH == 0) ? T.M[a][c] : T.C[c][a];
 }
 
-template <class R, int P, int WHICH>
-DEV void weights_1d(const Tab<R>& T, int n, int a0, int /*a1*/, R (&w)[2 * P + 1]) {
-#pragma unroll
-    for (int k = 0; k < 2 * P + 1; ++k) {
-        const int off = k - P;
-        R s = R(0);
-#pragma unroll
-        for (int aa = 0; aa <= P; ++aa) {
-            const int cc = off + aa;
-            if (cc >= 0 && cc <= P) s = (a0 == aa) ? wtab<R, P, WHICH>(T, aa, cc) : s;
-        }
-        if (off >= 0 && off <= P) s += (n == 2) ? wtab<R, P, WHICH>(T, 0, off) : R(0);
-        w[k] = s;
-    }
-}
-
-// indices of the 2P+1 nodes at offsets -P..P around g along a direction of
-// n nodes (periodic wrap; clamped where only zero weights reach)
-template <int P>
-DEV void offsets_1d(int g, int n, int periodic, int (&idx)[2 * P + 1]) {
-#pragma unroll
-    for (int k = 0; k < 2 * P + 1; ++k) {
-        int x = g + k - P;
-        if (periodic) x = x < 0 ? x + n : (x >= n ? x - n : x);
-        else x = x < 0 ? 0 : (x >= n ? n - 1 : x);
-        idx[k] = x;
-    }
-}
-
-// g_h right-hand side b_i = sum_e int phi_i grad u_h (x: derivative weights
-// along x, mass along y; y: the reverse) and the lumped first iterate b / m_i;
-// b and g hold [x components (NC)][y components (NC)]
-template <class R, int P, int NC>
-DEV void grad_rhs_at(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout,
-                     int gx, int gy, long long node) {
-    const Tab<R>& T = tab_of<R>(m, P);
-    const NodeC<P> c = node_c<P>(m, gx, gy);
-    R wMx[2 * P + 1], wCx[2 * P + 1], wMy[2 * P + 1], wCy[2 * P + 1];
-    weights_1d<R, P, 0>(T, c.nxc, c.a0, c.a1, wMx);
-    weights_1d<R, P, 1>(T, c.nxc, c.a0, c.a1, wCx);
-    weights_1d<R, P, 0>(T, c.nyc, c.b0, c.b1, wMy);
-    weights_1d<R, P, 1>(T, c.nyc, c.b0, c.b1, wCy);
-    int cols[2 * P + 1], rows[2 * P + 1];
-    offsets_1d<P>(gx, m.nnx, m.px, cols);
-    offsets_1d<P>(gy, m.nny, m.py, rows);
-    R sx[NC], sy[NC];
-#pragma unroll
-    for (int v = 0; v < NC; ++v) sx[v] = sy[v] = R(0);
-#pragma unroll
-    for (int ky = 0; ky < 2 * P + 1; ++ky) {
-        const long long row = (long long)rows[ky] * m.nnx;
-        R tx[NC], ty[NC];
-#pragma unroll
-        for (int v = 0; v < NC; ++v) tx[v] = ty[v] = R(0);
-#pragma unroll
-        for (int kx = 0; kx < 2 * P + 1; ++kx) {
-            const long long idx = row + cols[kx];
-#pragma unroll
-            for (int v = 0; v < NC; ++v) {
-                const R x = u[v * m.NN + idx];
-                tx[v] = fma_r(wCx[kx], x, tx[v]);
-                ty[v] = fma_r(wMx[kx], x, ty[v]);
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < NC; ++v) {
-            sx[v] = fma_r(wMy[ky], tx[v], sx[v]);
-            sy[v] = fma_r(wCy[ky], ty[v], sy[v]);
-        }
-    }
-    const R h = PV<R>::h(m);
-    const R inv_mi = is_lgl<R>(m) ? R(inv_lumped_lgl<P>(m, c.nxc * c.nyc, c.a0, c.b0))
-                                  : mul_r(PV<R>::inv_me(m), inv_count<R>(c.nxc * c.nyc));
-#pragma unroll
-    for (int v = 0; v < NC; ++v) {
-        const R bx = mul_r(h, sx[v]), by = mul_r(h, sy[v]);
-        bout[v * m.NN + node] = bx;
-        bout[(NC + v) * m.NN + node] = by;
-        gout[v * m.NN + node] = mul_r(bx, inv_mi);
-        gout[(NC + v) * m.NN + node] = mul_r(by, inv_mi);
-    }
-}
-
-// one lumped-preconditioned Richardson sweep for NV fields,
-// x_out = x_in + (b - M_C x_in) / m_i, with M_C applied as a stencil
-template <class R, int P, int NV>
-DEV void mass_sweep_at(MeshDev m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout,
-                       int gx, int gy, long long node) {
-    const Tab<R>& T = tab_of<R>(m, P);
-    const NodeC<P> c = node_c<P>(m, gx, gy);
-    R wx[2 * P + 1], wy[2 * P + 1];
-    weights_1d<R, P, 0>(T, c.nxc, c.a0, c.a1, wx);
-    weights_1d<R, P, 0>(T, c.nyc, c.b0, c.b1, wy);
-    int cols[2 * P + 1], rows[2 * P + 1];
-    offsets_1d<P>(gx, m.nnx, m.px, cols);
-    offsets_1d<P>(gy, m.nny, m.py, rows);
-    R s[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) s[v] = R(0);
-#pragma unroll
-    for (int ky = 0; ky < 2 * P + 1; ++ky) {
-        const long long row = (long long)rows[ky] * m.nnx;
-        R t[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) t[v] = R(0);
-#pragma unroll
-        for (int kx = 0; kx < 2 * P + 1; ++kx) {
-            const long long idx = row + cols[kx];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) t[v] = fma_r(wx[kx], xin[v * m.NN + idx], t[v]);
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) s[v] = fma_r(wy[ky], t[v], s[v]);
-    }
-    const R h2 = PV<R>::h2(m);
-    const R inv_mi = is_lgl<R>(m) ? R(inv_lumped_lgl<P>(m, c.nxc * c.nyc, c.a0, c.b0))
-                                  : mul_r(PV<R>::inv_me(m), inv_count<R>(c.nxc * c.nyc));
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const long long k = v * m.NN + node;
-        xout[k] = sweep_value(xin[k], b[k], s[v], h2, inv_mi);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Tiled forms of the two stencils: a block of 32 x 8 threads owns a tile of
-// 32 x 16 nodes, stages one field of the tile plus a halo of p nodes in
-// shared memory (coalesced rows, periodic wrap, zeros outside a
-// non-periodic mesh, where every weight that reaches them is 0), applies
-// the 1D operator along x for all halo rows, then along y.  The weights of
-// a node depend only on its class along each direction (local index 1..p-1
-// inside an element, an interior vertex shared by two elements, or a
-// boundary vertex); the class tables are built per block from the element
-// tables with the same additions as weights_1d.  Same arithmetic, in the
-// same order with the same roundings, as grad_rhs_at / mass_sweep_at.
-// ---------------------------------------------------------------------------
-constexpr int ST_TX = 32, ST_TY = 16, ST_BY = 8;
-
-// class of node g along a direction of n nodes: 1..P-1 inside an element,
-// 0 vertex shared by two elements, P lower boundary vertex, P+1 upper one
-template <int P>
-DEV int node_class(int g, int n, int periodic) {
-    const int a = g % P;
-    if (a != 0) return a;
-    if (!periodic) {
-        if (g == 0) return P;
-        if (g == n - 1) return P + 1;
-    }
-    return 0;
-}
-
-// local index of a node of class cls in the first element containing it
-// (a shared vertex: p in the lower element; a low / high boundary vertex:
-// 0 / p; inside an element: cls)
-template <int P>
-DEV int class_index(int cls) {
-    return (cls == 0 || cls == P + 1) ? P : (cls == P ? 0 : cls);
-}
-
-// weight of offset off (-P..P) for a node of class cls (WHICH 0: mass,
-// 1: derivative on the trial index), as weights_1d computes it
-template <class R, int P, int WHICH>
-DEV R class_weight(const Tab<R>& T, int cls, int off) {
-    // first containing element and the node's local index in it
-    const int a0 = (cls == 0 || cls == P + 1) ? P : (cls == P ? 0 : cls);
-    const bool two = cls == 0;
-    R s = R(0);
-    const int cc = off + a0;
-    if (cc >= 0 && cc <= P) s = wtab<R, P, WHICH>(T, a0, cc);
-    if (two && off >= 0 && off <= P) s += wtab<R, P, WHICH>(T, 0, off);
-    return s;
-}
-
-// stage one field (rows gy0-P.., columns gx0-P..) of the tile in shared memory
-// a node index on a periodic direction of n nodes taken into [0, n) (the
-// fused stencils, halo 2p): one period covers every node of a tile and its
-// halo on meshes at least a tile wide; a narrower mesh (down to one element)
-// takes the remainder, so a staged halo value is always a node of the mesh
+// an index on a periodic direction of n taken into [0, n): one period covers
+// every node of a tile and its halo on meshes at least a tile wide; a
+// narrower mesh (down to one element) takes the remainder, so a staged halo
+// value is always a node of the mesh
 DEV int wrap_periodic(int g, int n) {
     g = g < 0 ? g + n : (g >= n ? g - n : g);
     if ((unsigned)g >= (unsigned)n) g = ((g % n) + n) % n;
     return g;
-}
-
-template <class R, int P, int BY, int TY = ST_TY>
-DEV void stage_tile(const MeshDev& m, const R* __restrict__ x, R (*xs)[ST_TX + 2 * P], int gx0, int gy0, int tid) {
-    constexpr int HX = ST_TX + 2 * P, HY = TY + 2 * P;
-    for (int i = tid; i < HX * HY; i += ST_TX * BY) {
-        const int r = i / HX, c = i - r * HX;
-        int gy = gy0 - P + r, gx = gx0 - P + c;
-        // one period on periodic directions: a halo of p never needs more on a
-        // mesh of at least one element (p nodes) per side; a position still
-        // outside after it (two periods away, on a mesh narrower than the
-        // tile) feeds no output of the tile and is not read
-        if (m.py) gy = gy < 0 ? gy + m.nny : (gy >= m.nny ? gy - m.nny : gy);
-        if (m.px) gx = gx < 0 ? gx + m.nnx : (gx >= m.nnx ? gx - m.nnx : gx);
-        const bool in = (unsigned)gy < (unsigned)m.nny && (unsigned)gx < (unsigned)m.nnx;
-        // through L2 (ld.global.cg): k_grad_rhs reads u without waiting for
-        // the kernel launched just before it
-        xs[r][c] = in ? __ldcg(&x[(long long)gy * m.nnx + gx]) : R(0);
-    }
-}
-
-// fields staged together: as many as fit in 32 KB of shared memory (a
-// divisor of NV), so one round of loads and barriers serves all of them
-template <class R, int P, int NV, int NT, int TY = ST_TY>
-struct StFields {
-    static constexpr int HX = ST_TX + 2 * P, HY = TY + 2 * P;
-    static constexpr int bytes(int f) { return f * (HY * HX + NT * HY * ST_TX) * (int)sizeof(R); }
-    static constexpr int value = (bytes(NV) <= 32768) ? NV
-                                 : (NV % 4 == 0 && bytes(4) <= 32768) ? 4
-                                 : (NV % 2 == 0 && bytes(2) <= 32768) ? 2 : 1;
-    // shared workspace in elements of R: staged fields, NT pass-1 arrays
-    // per field, NT class-weight tables
-    static constexpr int ws = value * (HY * HX + NT * HY * ST_TX) + NT * (P + 2) * (2 * P + 1);
-};
-
-// g_h right-hand side and lumped iterate on the 32 x 16 node tile at
-// (gx0, gy0) by a block of 32 x BY threads (thread (tx, ty)); ws: shared
-// workspace of StFields<R, P, NC, 2>::ws elements.  All threads of the block
-// call it together.
-template <class R, int P, int NC, int BY, int TY = ST_TY>
-DEV void grad_tile(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout,
-                   int gx0, int gy0, int tx, int ty, R* ws) {
-    constexpr int HX = ST_TX + 2 * P, HY = TY + 2 * P, NW = 2 * P + 1, NCL = P + 2, NJ = TY / BY;
-    constexpr int FB = StFields<R, P, NC, 2, TY>::value;
-    R(*xs)[HY][HX] = reinterpret_cast<R(*)[HY][HX]>(ws);
-    R(*tC)[HY][ST_TX] = reinterpret_cast<R(*)[HY][ST_TX]>(ws + FB * HY * HX);
-    R(*tM)[HY][ST_TX] = reinterpret_cast<R(*)[HY][ST_TX]>(ws + FB * HY * HX + FB * HY * ST_TX);
-    R(*WM)[NW] = reinterpret_cast<R(*)[NW]>(ws + FB * (HY * HX + 2 * HY * ST_TX));
-    R(*WC)[NW] = reinterpret_cast<R(*)[NW]>(ws + FB * (HY * HX + 2 * HY * ST_TX) + NCL * NW);
-    const Tab<R>& T = tab_of<R>(m, P);
-    const int tid = ty * ST_TX + tx;
-    __syncthreads();  // the workspace is free
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        WM[cls][k] = class_weight<R, P, 0>(T, cls, k - P);
-        WC[cls][k] = class_weight<R, P, 1>(T, cls, k - P);
-    }
-    const int gx = gx0 + tx;
-    const int clx = node_class<P>(gx, m.nnx, m.px);
-    const R h = PV<R>::h(m);
-    for (int v0 = 0; v0 < NC; v0 += FB) {
-        if (v0 > 0) __syncthreads();  // previous fields consumed
-#pragma unroll
-        for (int f = 0; f < FB; ++f) stage_tile<R, P, BY, TY>(m, u + (long long)(v0 + f) * m.NN, xs[f], gx0, gy0, tid);
-        __syncthreads();
-        R wcx[NW], wmx[NW];  // the column's x weights, for every row and field
-#pragma unroll
-        for (int k = 0; k < NW; ++k) {
-            wcx[k] = WC[clx][k];
-            wmx[k] = WM[clx][k];
-        }
-        // along x, every halo row: derivative (for b_x) and mass (for b_y)
-        for (int r = ty; r < HY; r += BY) {
-#pragma unroll
-            for (int f = 0; f < FB; ++f) {
-                R sc = R(0), sm = R(0);
-#pragma unroll
-                for (int k = 0; k < NW; ++k) {
-                    const R x = xs[f][r][tx + k];
-                    sc = fma_r(wcx[k], x, sc);
-                    sm = fma_r(wmx[k], x, sm);
-                }
-                tC[f][r][tx] = sc;
-                tM[f][r][tx] = sm;
-            }
-        }
-        __syncthreads();
-        // along y and the outputs
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int r = ty + j * BY, gy = gy0 + r;
-            if (gx >= m.nnx || gy >= m.nny) continue;
-            const int cly = node_class<P>(gy, m.nny, m.py);
-            const int cnt = (clx == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-            const R inv_mi = is_lgl<R>(m) ? R(inv_lumped_lgl<P>(m, cnt, class_index<P>(clx), class_index<P>(cly)))
-                                          : mul_r(PV<R>::inv_me(m), inv_count<R>(cnt));
-            const long long node = (long long)gy * m.nnx + gx;
-            R wmy[NW], wcy[NW];  // once for every field
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                wmy[k] = WM[cly][k];
-                wcy[k] = WC[cly][k];
-            }
-#pragma unroll
-            for (int f = 0; f < FB; ++f) {
-                const int v = v0 + f;
-                R sx = R(0), sy = R(0);
-#pragma unroll
-                for (int k = 0; k < NW; ++k) {
-                    sx = fma_r(wmy[k], tC[f][r + k][tx], sx);
-                    sy = fma_r(wcy[k], tM[f][r + k][tx], sy);
-                }
-                const R bx = mul_r(h, sx), by = mul_r(h, sy);
-                bout[v * m.NN + node] = bx;
-                bout[(NC + v) * m.NN + node] = by;
-                gout[v * m.NN + node] = mul_r(bx, inv_mi);
-                gout[(NC + v) * m.NN + node] = mul_r(by, inv_mi);
-            }
-        }
-    }
-}
-
-// one Richardson sweep for NV fields on the 32 x 16 node tile at (gx0, gy0);
-// ws: StFields<R, P, NV, 1>::ws elements of shared memory
-template <class R, int P, int NV, int BY, int TY = ST_TY>
-DEV void sweep_tile(const MeshDev& m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout,
-                    int gx0, int gy0, int tx, int ty, R* ws) {
-    constexpr int HX = ST_TX + 2 * P, HY = TY + 2 * P, NW = 2 * P + 1, NCL = P + 2, NJ = TY / BY;
-    constexpr int FB = StFields<R, P, NV, 1, TY>::value;
-    R(*xs)[HY][HX] = reinterpret_cast<R(*)[HY][HX]>(ws);
-    R(*t)[HY][ST_TX] = reinterpret_cast<R(*)[HY][ST_TX]>(ws + FB * HY * HX);
-    R(*W)[NW] = reinterpret_cast<R(*)[NW]>(ws + FB * (HY * HX + HY * ST_TX));
-    const Tab<R>& T = tab_of<R>(m, P);
-    const int tid = ty * ST_TX + tx;
-    __syncthreads();  // the workspace is free
-    if (tid < NCL * NW) {
-        const int cls = tid / NW, k = tid - cls * NW;
-        W[cls][k] = class_weight<R, P, 0>(T, cls, k - P);
-    }
-    const int gx = gx0 + tx;
-    const int clx = node_class<P>(gx, m.nnx, m.px);
-    const R h2 = PV<R>::h2(m);
-    for (int v0 = 0; v0 < NV; v0 += FB) {
-        // right-hand sides of this thread's nodes, loaded ahead of the barriers
-        R bv[FB][NJ];
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int gy = gy0 + ty + j * BY;
-            const bool in = gx < m.nnx && gy < m.nny;
-#pragma unroll
-            for (int f = 0; f < FB; ++f)
-                bv[f][j] = in ? b[(long long)(v0 + f) * m.NN + (long long)gy * m.nnx + gx] : R(0);
-        }
-        if (v0 > 0) __syncthreads();
-#pragma unroll
-        for (int f = 0; f < FB; ++f) stage_tile<R, P, BY, TY>(m, xin + (long long)(v0 + f) * m.NN, xs[f], gx0, gy0, tid);
-        __syncthreads();
-        for (int r = ty; r < HY; r += BY) {
-#pragma unroll
-            for (int f = 0; f < FB; ++f) {
-                R sx = R(0);
-#pragma unroll
-                for (int k = 0; k < NW; ++k) sx = fma_r(W[clx][k], xs[f][r][tx + k], sx);
-                t[f][r][tx] = sx;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int r = ty + j * BY, gy = gy0 + r;
-            if (gx >= m.nnx || gy >= m.nny) continue;
-            const int cly = node_class<P>(gy, m.nny, m.py);
-            const int cnt = (clx == 0 ? 2 : 1) * (cly == 0 ? 2 : 1);
-            const R inv_mi = is_lgl<R>(m) ? R(inv_lumped_lgl<P>(m, cnt, class_index<P>(clx), class_index<P>(cly)))
-                                          : mul_r(PV<R>::inv_me(m), inv_count<R>(cnt));
-#pragma unroll
-            for (int f = 0; f < FB; ++f) {
-                R sy = R(0);
-#pragma unroll
-                for (int k = 0; k < NW; ++k) sy = fma_r(W[cly][k], t[f][r + k][tx], sy);
-                const long long k = (long long)(v0 + f) * m.NN + (long long)gy * m.nnx + gx;
-                xout[k] = sweep_value(xs[f][r + P][tx + P], bv[f][j], sy, h2, inv_mi);
-            }
-        }
-    }
-}
-
-// needs only u, whose last writer completed before k_pre let this kernel
-// start (pdl_wait_then_trigger), so it runs beside k_pre and waits for it
-// only before exiting
-// TY: node rows per tile (8 on small meshes: shorter per-block chains in a
-// partial wave; 16 on large ones: less halo)
-template <class R, int P, int NC, int TY = ST_TY>
-__global__ void __launch_bounds__(ST_TX * ST_BY) k_grad_rhs(MeshDev m, const R* __restrict__ u,
-                                                            R* __restrict__ bout, R* __restrict__ gout) {
-    pdl_trigger();
-    __shared__ R ws[StFields<R, P, NC, 2, TY>::ws];
-    grad_tile<R, P, NC, ST_BY, TY>(m, u, bout, gout, blockIdx.x * ST_TX, blockIdx.y * TY, threadIdx.x, threadIdx.y,
-                                   ws);
-    pdl_wait();
-}
-
-template <class R, int P, int NV, int TY = ST_TY>
-__global__ void __launch_bounds__(ST_TX * ST_BY) k_mass_sweep(MeshDev m, const R* __restrict__ xin,
-                                                              const R* __restrict__ b, R* __restrict__ xout) {
-    pdl_begin();
-    __shared__ R ws[StFields<R, P, NV, 1, TY>::ws];
-    sweep_tile<R, P, NV, ST_BY, TY>(m, xin, b, xout, blockIdx.x * ST_TX, blockIdx.y * TY, threadIdx.x, threadIdx.y,
-                                    ws);
 }
 
 // runtime-degree candidate list (diagnostics only)
@@ -1956,18 +1562,11 @@ DEV void stab_part(const MeshDev& m, const R (&U)[Ph::NC][Dim<P>::N2], const R* 
     const R h = PV<R>::h(m);
     // stabilisation s = nu (K u - gamma (Gx gx + Gy gy))
     const R nue = R(nu[e]), ge = R(gam[e]);
-    const ElemNodes<P> en(m, ex, ey);
 #pragma unroll 1
     for (int c = 0; c < NC; ++c) {
         R GX[N2], GY[N2];
-#pragma unroll
-        for (int b = 0; b < N1; ++b)
-#pragma unroll
-            for (int a = 0; a < N1; ++a) {
-                const long long n = en(a, b);
-                GX[b * N1 + a] = g[(long long)c * m.NN + n];
-                GY[b * N1 + a] = g[(long long)(NC + c) * m.NN + n];
-            }
+        load_comp<R, P>(g + c * m.NN, m, ex, ey, GX);
+        load_comp<R, P>(g + (NC + c) * m.NN, m, ex, ey, GY);
         // x-direction products: D u, M u, C gx, M gy
         R Du[N1][N1], Mu[N1][N1], Cg[N1][N1], Mg[N1][N1];
 #pragma unroll
@@ -2426,15 +2025,10 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
     R F[NC][N2];
     // components unrolled for p >= 3 (registers); at p <= 2 the rolled loop
     // keeps occupancy higher (measured on the Euler workloads)
-    const ElemNodes<P> en(m, ex, ey);
 #pragma unroll (P >= 3 ? Ph::NC : 1)
     for (int c = 0; c < NC; ++c) {
         R UD[N2];
-#pragma unroll
-        for (int b = 0; b < N1; ++b)
-#pragma unroll
-            for (int a = 0; a < N1; ++a)
-                UD[b * N1 + a] = ud[(long long)c * m.NN + en(a, b)];
+        load_comp<R, P>(ud + c * m.NN, m, ex, ey, UD);
         R Y[N1][N1];
 #pragma unroll
         for (int d = 0; d < N1; ++d)

@@ -44,6 +44,22 @@ DEV double sub_r(double a, double b) { return __dsub_rn(a, b); }
 static __device__ __noinline__ float pow_rare(float x, float e) { return powf(x, e); }
 static __device__ __noinline__ double pow_rare(double x, double e) { return pow(x, e); }
 
+// 1 / x and sqrt(x) of a weight or norm: float by the hardware's approximations
+// (within one unit in the last place; 1/x of an infinite or zero norm and
+// sqrt(0) come out as in the exact operation), float64 as the operators
+DEV float recip(float x) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+DEV double recip(double x) { return 1.0 / x; }
+DEV float root(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+DEV double root(double x) { return sqrt(x); }
+
 // modal coefficients of one line
 template <class R, int P>
 DEV void modal_line(const Tab<R>& T, const R (&v)[P + 1], R (&l)[P + 1]) {
@@ -175,7 +191,7 @@ DEV R modal_sensor(const Tab<R>& T, int a2b, const ProbDev& pr, const R (&own)[(
     for (int d = 0; d < 4; ++d) ne += (nb[d] >= 0);
     const R sig0 = fmax(modal_norm<R, P>(own, a2b), R(0));
     R wt[5];
-    wt[0] = (R(1) - R(ne) * wl) / ((r2 ? sig0 : pow_rare(sig0, rh)) + eps);
+    wt[0] = (R(1) - R(ne) * wl) * recip((r2 ? sig0 : pow_rare(sig0, rh)) + eps);
     R W[KEEP ? 4 : 1][N2];
     each_dir([&](auto dir) {
         constexpr int d = decltype(dir)::value;
@@ -185,11 +201,11 @@ DEV R modal_sensor(const Tab<R>& T, int a2b, const ProbDev& pr, const R (&own)[(
             nbr(d, l);
             modal_continue<R, P, d>(T, l, W[KEEP ? d : 0]);
             const R sg = fmax(modal_norm<R, P>(W[KEEP ? d : 0], a2b), R(0));
-            wt[d + 1] = wl / ((r2 ? sg : pow_rare(sg, rh)) + eps);
+            wt[d + 1] = wl * recip((r2 ? sg : pow_rare(sg, rh)) + eps);
         }
     });
     const R tot = (((wt[0] + wt[1]) + wt[2]) + wt[3]) + wt[4];
-    const R rtot = R(1) / tot;  // one division for the four weights omega_l
+    const R rtot = recip(tot);
     R D[N2];
 #pragma unroll
     for (int i = 0; i < N2; ++i) D[i] = R(0);
@@ -206,9 +222,9 @@ DEV R modal_sensor(const Tab<R>& T, int a2b, const ProbDev& pr, const R (&own)[(
             for (int i = 1; i < N2; ++i) D[i] = fma_r(wd, sub_r(own[i], W[KEEP ? d : 0][i]), D[i]);
         }
     });
-    const R num = sqrt(fmax(modal_norm<R, P>(D, a2b), R(0)));
-    const R den = sqrt(sig0);
-    const R ratio = num / (den + geps);
+    const R num = root(fmax(modal_norm<R, P>(D, a2b), R(0)));
+    const R den = root(sig0);
+    const R ratio = num * recip(den + geps);
     return R(1) - (pr.q1 ? fmin(R(1), ratio) : pow_rare(fmin(R(1), ratio), PV<R>::q(pr)));
 }
 

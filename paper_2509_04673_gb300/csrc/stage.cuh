@@ -68,13 +68,10 @@ struct Prof {
 typedef cudaError_t (*StageFn)(const Bufs&, const MeshDev&, const ProbDev&, double a, double b,
                                bool first, bool dt_only, cudaStream_t st, Prof* prof);
 
-inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+// large stencil tiles below which the small ones are used
+constexpr int SMALL_TILES_BELOW = 304;
 
-// The fused first sweeps (fused.cuh) save the traffic of the lumped iterates
-// but lengthen each block's chain of dependent phases.  Measured on GB300,
-// they win from about 4M nodes (KPP 1024^2 Q2: -4 % per step, Euler blast
-// 2048^2) and lose below (KPP 256^2: +4 %; Euler 512^2 Q3: +1.5 %).
-inline bool fuse_sweeps(const MeshDev& m) { return m.NN >= (1LL << 22); }
+inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 // The split residual (k_res_w on the second stream, k_res_s) overlaps the
 // quadrature with k_pre and the g_h kernels but adds a kernel and the W^e
@@ -110,15 +107,17 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     constexpr int NC = Ph::NC;
     const dim3 be(64, 2), bn(128, 1);
     const dim3 ge(nblk(m.nx, 64), nblk(m.ny, 2)), gn(nblk(m.nnx, 128), m.nny);
-    const dim3 bt(ST_TX, ST_BY), gt(nblk(m.nnx, ST_TX), nblk(m.nny, ST_TY));  // tiled stencils
-    // small meshes: 32 x 8 node tiles for the unfused stencils (measured:
-    // KPP 256^2 Q2 -4.6 % per step; 8 rows lose 8-10 % from 2M nodes)
-    const bool small_tiles = m.NN < (1LL << 20);
-    const dim3 gt8(nblk(m.nnx, ST_TX), nblk(m.nny, 8));
-    auto* k_grad = small_tiles ? k_grad_rhs<R, P, NC, 8> : k_grad_rhs<R, P, NC, ST_TY>;
-    auto* k_sweep_g = small_tiles ? k_mass_sweep<R, P, 2 * NC, 8> : k_mass_sweep<R, P, 2 * NC, ST_TY>;
-    auto* k_sweep_u = small_tiles ? k_mass_sweep<R, P, NC, 8> : k_mass_sweep<R, P, NC, ST_TY>;
-    const dim3 gts = small_tiles ? gt8 : gt;
+    // the stencils' tiles: small ones where the large ones would leave SMs idle
+    using TL = stage_tile_t<R, P, false>;
+    using TS = stage_tile_t<R, P, true>;
+    const dim3 gl(nblk(m.nnx, TL::NX), nblk(m.nny, TL::NY));
+    const bool small_tiles = gl.x * gl.y < (unsigned)SMALL_TILES_BELOW;
+    const dim3 gt = small_tiles ? dim3(nblk(m.nnx, TS::NX), nblk(m.nny, TS::NY)) : gl, bt(small_tiles ? TS::NT : TL::NT);
+    auto* k_gradf = small_tiles ? k_grad_sweep<R, P, NC, true> : k_grad_sweep<R, P, NC, false>;
+    auto* k_grad = small_tiles ? k_grad_rhs<R, P, NC, true> : k_grad_rhs<R, P, NC, false>;
+    auto* k_udotf = small_tiles ? k_udot_sweep<R, P, NC, true> : k_udot_sweep<R, P, NC, false>;
+    auto* k_sweep_g = small_tiles ? k_mass_sweep<R, P, 2 * NC, true> : k_mass_sweep<R, P, 2 * NC, false>;
+    auto* k_sweep_u = small_tiles ? k_mass_sweep<R, P, NC, true> : k_mass_sweep<R, P, NC, false>;
     // the sensor's element tiles (k_sens): 8 rows of 32 in float, 4 in float64
     // (24 modes of 340 elements are 65 KB there)
     constexpr int STY = sizeof(R) == 4 ? 8 : 4;
@@ -222,27 +221,23 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         R* g = (R*)B.g;
         R* g2 = (R*)B.g2;
         R* bg = (R*)B.bg;
-        // FP32-mixed on large meshes: the right-hand side and the first sweep
-        // in one kernel
-        constexpr bool fuse = sizeof(R) == 4;
-        const bool fuse_here = fuse && fuse_sweeps(m) && !(pr.opts & OPT_UNFUSED_SWEEPS);
+        // the right-hand sides with their first sweeps in one kernel each
+        const bool fuse = !(pr.opts & OPT_UNFUSED_SWEEPS);
         int k0 = 0;
-        if (fuse_here && pr.k_g >= 1) {
-            if constexpr (fuse)
-                CGL_LAUNCH(prof, KID_GRADF, st,
-                           chk(launch(pdl, k_grad_sweep<P, NC>, gt, bt, st, m, (const float*)u,
-                                      pr.k_g > 1 ? (float*)bg : (float*)nullptr, (float*)g2)));
+        if (fuse && pr.k_g >= 1) {
+            CGL_LAUNCH(prof, KID_GRADF, st,
+                       chk(launch(pdl, k_gradf, gt, bt, st, m, (const R*)u, pr.k_g > 1 ? bg : (R*)nullptr, g2)));
             R* t = g;
             g = g2;
             g2 = t;
             k0 = 1;
         } else {
             CGL_LAUNCH(prof, KID_GRAD, st,
-                       chk(launch(pdl, k_grad, gts, bt, st, m, (const R*)u, bg, g)));
+                       chk(launch(pdl, k_grad, gt, bt, st, m, (const R*)u, bg, g)));
         }
         for (int k = k0; k < pr.k_g; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch(pdl, k_sweep_g, gts, bt, st, m, (const R*)g, (const R*)bg, g2)));
+                       chk(launch(pdl, k_sweep_g, gt, bt, st, m, (const R*)g, (const R*)bg, g2)));
             R* t = g;
             g = g2;
             g2 = t;
@@ -262,11 +257,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
                                   (const double*)B.gam, (const double*)B.nu, ER)));
         }
         int k1 = 0;
-        if (fuse_here && pr.k_u >= 1) {
-            if constexpr (fuse)
-                CGL_LAUNCH(prof, KID_UDOTF, st,
-                           chk(launch(pdl, k_udot_sweep<P, NC>, gt, bt, st, m, (const float*)ER, (float*)r,
-                                      (float*)ud2)));
+        if (fuse && pr.k_u >= 1) {
+            CGL_LAUNCH(prof, KID_UDOTF, st, chk(launch(pdl, k_udotf, gt, bt, st, m, (const R*)ER, r, ud2)));
             R* t = ud;
             ud = ud2;
             ud2 = t;
@@ -277,7 +269,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         }
         for (int k = k1; k < pr.k_u; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch(pdl, k_sweep_u, gts, bt, st, m, (const R*)ud, (const R*)r, ud2)));
+                       chk(launch(pdl, k_sweep_u, gt, bt, st, m, (const R*)ud, (const R*)r, ud2)));
             R* t = ud;
             ud = ud2;
             ud2 = t;
