@@ -1536,7 +1536,8 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
     if (!lo && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
         // the first sweep of each solve runs inside k_grad_sweep / k_udot_sweep
-        per_stage -= (S->prob.k_g >= 1) + (S->prob.k_u >= 1);
+        const bool small = S->prec == CGL_FP64 ? small_tiles_of<double>(S->mesh->m) : small_tiles_of<float>(S->mesh->m);
+        per_stage -= (S->prob.k_g >= 1 && fuse_grad_sweep(S->rsz, small)) + (S->prob.k_u >= 1);
     }
     if ((S->prob.options & CGL_OPT_AEC_Q1) && !lo) {
         // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_sens for systems, k_avg for mixed ones)

@@ -62,14 +62,23 @@ enum { PH_GRAD = 0, PH_SWEEP_G, PH_GATHER_R, PH_SWEEP_U, PH_FINAL, PH_GRADF, PH_
 
 constexpr int BT = 128;  // threads per block of the persistent grid
 
-// node tiles: the single-state stencils' large tiles, worked by NT threads
-template <int P, int NT>
-using BatchTile = SegTile<float, P, StageTile<float, P, false>::X, StageTile<float, P, false>::Y, NT>;
-static int tile_nx(int p) {
-    return p == 1 ? BatchTile<1, BT>::NX : p == 2 ? BatchTile<2, BT>::NX : p == 3 ? BatchTile<3, BT>::NX : BatchTile<4, BT>::NX;
-}
-static int tile_ny(int p) {
-    return p == 1 ? BatchTile<1, BT>::NY : p == 2 ? BatchTile<2, BT>::NY : p == 3 ? BatchTile<3, BT>::NY : BatchTile<4, BT>::NY;
+// node tiles of both forms: NX by NY nodes, each worked by NT threads; those
+// of the fused g_h phase are two elements smaller in each direction
+template <int P, int NT, bool HALO>
+struct BatchTileOf {
+    static constexpr int LX = P <= 2 ? 32 : 16, N = P == 3 ? (NT >= 192 ? 192 : 96) : NT;
+    using type = SegTile<float, P, LX, (P == 1 ? 16 : 8) / (N / (LX * P)), N, HALO>;
+};
+template <int P, int NT, bool HALO = false>
+using BatchTile = typename BatchTileOf<P, NT, HALO>::type;
+template <bool HALO>
+static void tile_dims(int p, int& nx, int& ny) {
+    switch (p) {
+        case 1: nx = BatchTile<1, BT, HALO>::NX, ny = BatchTile<1, BT, HALO>::NY; break;
+        case 2: nx = BatchTile<2, BT, HALO>::NX, ny = BatchTile<2, BT, HALO>::NY; break;
+        case 3: nx = BatchTile<3, BT, HALO>::NX, ny = BatchTile<3, BT, HALO>::NY; break;
+        default: nx = BatchTile<4, BT, HALO>::NX, ny = BatchTile<4, BT, HALO>::NY; break;
+    }
 }
 
 // shared workspace of the tiled stencils, the largest over the phases
@@ -77,7 +86,7 @@ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 template <int P>
 constexpr int ws_deg() {
     using TL = BatchTile<P, BT>;
-    return cmax(TL::grad_ws, cmax(TL::sweep_ws, TL::udot_ws(1)));
+    return cmax(cmax(BatchTile<P, BT, true>::grad_ws, TL::rhs_ws), cmax(TL::sweep_ws, TL::udot_ws(1)));
 }
 
 // bounded grid barrier: returns false if it gave up (or another block did)
@@ -177,10 +186,10 @@ DEV void node_phase_body(int phase, const InstDev& D, const MeshDev& m, int gx0,
         case PH_GRADF:
             // right-hand side and first sweep in one pass (k carries k_g: b is
             // kept only when more sweeps follow)
-            grad_sweep_seg<float, P, 1, TL>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tid, ws);
+            grad_sweep_seg<float, P, 1, BatchTile<P, NT, true>>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tid, ws);
             break;
         case PH_GATHERF: udot_sweep_seg<float, P, 1, TL>(m, D.ER, D.r, D.ud2, gx0, gy0, tid, ws); break;
-        case PH_GRAD: grad_sweep_seg<float, P, 1, TL, false>(m, D.u, D.bg, D.g, gx0, gy0, tid, ws); break;
+        case PH_GRAD: grad_rhs_seg<float, P, 1, TL>(m, D.u, D.bg, D.g, gx0, gy0, tid, ws); break;
         case PH_SWEEP_G:
             if (k & 1) mass_sweep_seg<float, P, 2, TL>(m, D.g2, D.bg, D.g, gx0, gy0, tid, ws);
             else mass_sweep_seg<float, P, 2, TL>(m, D.g, D.bg, D.g2, gx0, gy0, tid, ws);
@@ -251,7 +260,7 @@ constexpr int batch_min_blocks(int) { return 7; }
 template <int P>
 __global__ void __launch_bounds__(BT, batch_min_blocks(P))
     k_batch_stage(const InstDev* __restrict__ I, int ninst, const Tile* __restrict__ et, int net,
-                  const Tile* __restrict__ nt, int nnt, BatchSync* sync, float a, float b, int first,
+                  const Tile* __restrict__ nt, int nnt, const Tile* __restrict__ gt, int ngt, BatchSync* sync, float a, float b, int first,
                   int last, int kg, int ku, int mode_lo, long long limit) {
     __shared__ float ws[ws_deg<P>()];
     elem_loop<P>(PH_PRE, I, et, net, first != 0, kg, ku);
@@ -274,7 +283,7 @@ __global__ void __launch_bounds__(BT, batch_min_blocks(P))
         // arithmetic of the separate stencils, same bits): two phases and two
         // grid barriers fewer per stage
         if (kg >= 1) {
-            node_loop<P>(PH_GRADF, I, nt, nnt, a, b, kg, ws);
+            node_loop<P>(PH_GRADF, I, gt, ngt, a, b, kg, ws);
             if (!grid_sync(sync, limit)) return;
         } else {
             node_loop<P>(PH_GRAD, I, nt, nnt, a, b, 0, ws);
@@ -305,7 +314,7 @@ __global__ void __launch_bounds__(BT, batch_min_blocks(P))
     }
 }
 
-typedef void (*BatchKernel)(const InstDev*, int, const Tile*, int, const Tile*, int, BatchSync*, float, float, int,
+typedef void (*BatchKernel)(const InstDev*, int, const Tile*, int, const Tile*, int, const Tile*, int, BatchSync*, float, float, int,
                             int, int, int, int, long long);
 static BatchKernel batch_kernel(int p) {
     switch (p) {
@@ -363,9 +372,9 @@ __global__ void __launch_bounds__(BT) k_bph_elem(const InstDev* __restrict__ I, 
 
 // node tiles with 256 threads per block (2 rows per thread, as the
 // single-state stencils), the phase's code alone
-constexpr int BTN = 256;
+constexpr int btn(int p) { return p == 3 ? 192 : 256; }
 template <int P, int PHASE>
-__global__ void __launch_bounds__(BTN) k_bph_node(const InstDev* __restrict__ I, const Tile* __restrict__ nt,
+__global__ void __launch_bounds__(btn(P)) k_bph_node(const InstDev* __restrict__ I, const Tile* __restrict__ nt,
                                                   float a, float b, int k) {
     __shared__ float ws[ws_deg<P>()];
     __shared__ InstDev sD;
@@ -375,7 +384,7 @@ __global__ void __launch_bounds__(BTN) k_bph_node(const InstDev* __restrict__ I,
     // the mesh descriptor read from shared memory (a register copy measured
     // 3.70 -> 3.75 ms per step of the 256-instance batch)
     const MeshDev& m = sD.m;
-    node_phase_body<P, BTN>(PHASE, sD, m, T.begin, T.count, a, b, k, ws);
+    node_phase_body<P, btn(P)>(PHASE, sD, m, T.begin, T.count, a, b, k, ws);
 }
 
 // global dt of every instance of the group from its block minima (eq.
@@ -419,9 +428,9 @@ static void bph_elem(const InstDev* I, const Tile* et, const ElemRanges& er, int
 
 template <int P>
 static cudaError_t bph_stage(const InstDev* I, int ninst, const Tile* et, const ElemRanges& er, const Tile* nt,
-                             int nnt, float a, float b, int first, int last, int kg, int ku, int mode_lo,
+                             int nnt, const Tile* gt, int ngt, float a, float b, int first, int last, int kg, int ku, int mode_lo,
                              cudaStream_t st) {
-    const dim3 blk(BT), bn(BTN);
+    const dim3 blk(BT), bn(btn(P));
     const dim3 gi((ninst + BT - 1) / BT), gn(nnt);
     cudaError_t err = cudaSuccess;
     auto chk = [&](cudaError_t e) {
@@ -436,7 +445,7 @@ static cudaError_t bph_stage(const InstDev* I, int ninst, const Tile* et, const 
     bph_elem<P, PH_FACET>(I, et, er, 0, kg, ku, st, err);
     if (!mode_lo) {
         bph_elem<P, PH_RES_W>(I, et, er, 0, kg, ku, st, err);
-        if (kg >= 1) chk(launch(false, k_bph_node<P, PH_GRADF>, gn, bn, st, I, nt, a, b, kg));
+        if (kg >= 1) chk(launch(false, k_bph_node<P, PH_GRADF>, dim3(ngt), bn, st, I, gt, a, b, kg));
         else chk(launch(false, k_bph_node<P, PH_GRAD>, gn, bn, st, I, nt, a, b, 0));
         for (int k = (kg >= 1 ? 1 : 0); k < kg; ++k)
             chk(launch(false, k_bph_node<P, PH_SWEEP_G>, gn, bn, st, I, nt, a, b, k));
@@ -452,7 +461,7 @@ static cudaError_t bph_stage(const InstDev* I, int ninst, const Tile* et, const 
     return err;
 }
 
-typedef cudaError_t (*PhaseStage)(const InstDev*, int, const Tile*, const ElemRanges&, const Tile*, int, float, float,
+typedef cudaError_t (*PhaseStage)(const InstDev*, int, const Tile*, const ElemRanges&, const Tile*, int, const Tile*, int, float, float,
                                   int, int, int, int, int, cudaStream_t);
 static PhaseStage phase_stage(int p) {
     switch (p) {
@@ -476,8 +485,8 @@ struct DegreeGroup {
     int p;
     std::vector<int> members;  // indices into cgl_batch::states
     InstDev* d_inst;
-    Tile *d_et, *d_nt;
-    int net, nnt;
+    Tile *d_et, *d_nt, *d_gt;  // element tiles, node tiles, tiles of the fused g_h phase
+    int net, nnt, ngt;
     ElemRanges er;  // element tiles per flux (ordered by flux)
     BatchSync* d_sync;
     int grid;
@@ -508,7 +517,7 @@ static cgl_status bfail(cgl_status st, const char* msg, cudaError_t e = cudaSucc
 
 static cgl_status build_tiles(cgl_batch* B) {
     for (DegreeGroup& G : B->groups) {
-        std::vector<Tile> et, nt;
+        std::vector<Tile> et, nt, gt;
         const int T = std::max(1, std::min(BT, B->tile_elems[G.p]));
         for (int f = 0; f < 3; ++f) {
             G.er.eoff[f] = (int)et.size();
@@ -522,22 +531,32 @@ static cgl_status build_tiles(cgl_batch* B) {
         }
         for (int k = 0; k < (int)G.members.size(); ++k) {
             const MeshDev& m = B->states[G.members[k]]->mesh->m;
-            for (int gy0 = 0; gy0 < m.nny; gy0 += tile_ny(G.p))
-                for (int gx0 = 0; gx0 < m.nnx; gx0 += tile_nx(G.p)) nt.push_back(Tile{k, gx0, gy0, 0});
+            int tx, ty;
+            tile_dims<false>(G.p, tx, ty);
+            for (int gy0 = 0; gy0 < m.nny; gy0 += ty)
+                for (int gx0 = 0; gx0 < m.nnx; gx0 += tx) nt.push_back(Tile{k, gx0, gy0, 0});
+            tile_dims<true>(G.p, tx, ty);
+            for (int gy0 = 0; gy0 < m.nny; gy0 += ty)
+                for (int gx0 = 0; gx0 < m.nnx; gx0 += tx) gt.push_back(Tile{k, gx0, gy0, 0});
         }
         if (G.d_et) cudaFree(G.d_et);
         if (G.d_nt) cudaFree(G.d_nt);
-        G.d_et = G.d_nt = nullptr;
+        if (G.d_gt) cudaFree(G.d_gt);
+        G.d_et = G.d_nt = G.d_gt = nullptr;
         cudaError_t e = cudaMalloc(&G.d_et, et.size() * sizeof(Tile));
         if (e == cudaSuccess) e = cudaMalloc(&G.d_nt, nt.size() * sizeof(Tile));
+        if (e == cudaSuccess) e = cudaMalloc(&G.d_gt, gt.size() * sizeof(Tile));
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(G.d_et, et.data(), et.size() * sizeof(Tile), cudaMemcpyHostToDevice, B->st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(G.d_nt, nt.data(), nt.size() * sizeof(Tile), cudaMemcpyHostToDevice, B->st);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(G.d_gt, gt.data(), gt.size() * sizeof(Tile), cudaMemcpyHostToDevice, B->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(B->st);
         if (e != cudaSuccess) return bfail(CGL_ECUDA, "tile upload", e);
         G.net = (int)et.size();
         G.nnt = (int)nt.size();
+        G.ngt = (int)gt.size();
     }
     if (B->graph) {
         cudaGraphExecDestroy(B->graph);
@@ -548,7 +567,7 @@ static cgl_status build_tiles(cgl_batch* B) {
 
 static cudaError_t launch_stage(cgl_batch* B, DegreeGroup& G, float a, float b, int first, int last) {
     int ninst = (int)G.members.size();
-    void* args[] = {&G.d_inst, &ninst, &G.d_et, &G.net, &G.d_nt, &G.nnt, &G.d_sync, &a, &b,
+    void* args[] = {&G.d_inst, &ninst, &G.d_et, &G.net, &G.d_nt, &G.nnt, &G.d_gt, &G.ngt, &G.d_sync, &a, &b,
                     &first, &last, &B->kg, &B->ku, &B->mode_lo, &B->limit};
     return cudaLaunchCooperativeKernel((const void*)batch_kernel(G.p), dim3(G.grid), dim3(BT), args, 0, B->st);
 }
@@ -565,7 +584,7 @@ static cudaError_t enqueue_batch_step(cgl_batch* B) {
             if (e == cudaSuccess) e = cudaStreamWaitEvent(G.gst, B->ev_fork, 0);
             const int ninst = (int)G.members.size();
             for (int k = 0; k < 3 && e == cudaSuccess; ++k)
-                e = phase_stage(G.p)(G.d_inst, ninst, G.d_et, G.er, G.d_nt, G.nnt, sa[k], sb[k], k == 0, k == 2,
+                e = phase_stage(G.p)(G.d_inst, ninst, G.d_et, G.er, G.d_nt, G.nnt, G.d_gt, G.ngt, sa[k], sb[k], k == 0, k == 2,
                                      B->kg, B->ku, B->mode_lo, G.gst);
             if (e == cudaSuccess) e = cudaEventRecord(G.ev, G.gst);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(B->st, G.ev, 0);
@@ -621,6 +640,7 @@ extern "C" void cgl_batch_destroy(cgl_batch* B) {
         if (G.d_inst) cudaFree(G.d_inst);
         if (G.d_et) cudaFree(G.d_et);
         if (G.d_nt) cudaFree(G.d_nt);
+        if (G.d_gt) cudaFree(G.d_gt);
         if (G.d_sync) cudaFree(G.d_sync);
         if (G.gst) cudaStreamDestroy(G.gst);
         if (G.ev) cudaEventDestroy(G.ev);

@@ -21,7 +21,15 @@
 // Tiles start at vertices.  A field is staged by local index: plane a holds
 // the nodes of index a of every segment, so the segment reads of a warp along
 // x fall on consecutive words; planes are padded so that a warp running over
-// nodes (along y, and at the global stores) hits distinct banks as well.
+// nodes (along y, and at the global accesses) hits distinct banks as well.
+//
+// A tile (with the halo it works on) is LX segments wide, and so is the block:
+// in the x passes a thread keeps one segment and steps over rows, in the y passes and
+// at the global accesses one node column and steps over y segments.  Columns,
+// plane offsets, weights and masses are formed once per thread, and the loops
+// add constants (with the items of a pass numbered through, index arithmetic
+// was 40 % of k_grad_sweep's instructions, 64 of 161 warp instructions per
+// element of the Euler form at p = 2).
 //
 // The sums run over the offsets -p .. p in order with explicit rounding, so
 // the fused and the separate kernels, and every tile size, give the same bits.
@@ -42,15 +50,23 @@ DEV bool wrap_node(const MeshDev& m, int& gx, int& gy) {
     return in;
 }
 
-// a tile of TEX x TEY elements (NX x NY nodes) worked by NT threads
-template <class R, int P, int TEX_, int TEY_, int NT_>
+// A tile of TEX x TEY elements (NX x NY nodes) worked by NT threads: LX
+// segments wide in the x passes, RX rows of them per step; LY node columns
+// wide in the y passes, RY y segments per step, KY steps.  HALO: the passes
+// run on the tile and one element around it (the fused g_h kernel, whose
+// first iterate is needed there).
+template <class R, int P, int LX_, int KY_, int NT_, bool HALO_>
 struct SegTile {
-    static constexpr int TEX = TEX_, TEY = TEY_, NT = NT_;
+    static constexpr int LX = LX_, KY = KY_, NT = NT_, HALO = HALO_;
+    static constexpr int LY = LX * P, RX = NT / LX, RY = NT / LY;
+    static constexpr int TEX = HALO ? LX - 2 : LX, TEY = HALO ? RY * KY - 2 : RY * KY;
+    static_assert(NT % LX == 0 && NT % LY == 0 && TEY >= 1, "whole rows of threads");
     static constexpr int NX = TEX * P, NY = TEY * P;
-    // nodes and segments of the tile with one (1) and two (2) elements of halo
-    // on the low side and one, two vertices' reach on the high side
-    static constexpr int W1 = (TEX + 1) * P + 1, H1 = (TEY + 1) * P + 1, S1 = TEX + 2;
-    static constexpr int W2 = (TEX + 3) * P + 1, H2 = (TEY + 3) * P + 1, S2 = TEX + 4;
+    // nodes along x and y of the tile with one (1) and two (2) elements of halo
+    // (one less on the high side, where the last vertex suffices), segments
+    static constexpr int W1 = NX + P + 1, H1 = NY + P + 1, S1 = TEX + 2;
+    static constexpr int W2 = NX + 3 * P + 1, H2 = NY + 3 * P + 1, S2 = TEX + 4;
+    static constexpr int K1 = (H1 + RX - 1) / RX, K2 = (H2 + RX - 1) / RX;  // steps of the x passes
     // plane stride: n words or more, congruent to a p-th of the banks
     static constexpr int plane(int n) {
         constexpr int B = 128 / (int)sizeof(R), want = P == 1 ? 0 : (B + P - 1) / P;
@@ -58,18 +74,16 @@ struct SegTile {
         while (P > 1 && k % B != want % B) ++k;
         return k;
     }
-    static constexpr int PU = plane(H2 * S2);   // u on the two-element halo
-    static constexpr int PT = plane(H2 * S1);   // its x pass
-    static constexpr int PG = plane(H1 * S1);   // an iterate on the one-element halo
-    static constexpr int PS = plane(H1 * TEX);  // its x pass
-    static constexpr int PR = plane(NY * TEX);  // a field on the tile
-    static constexpr int NOWN = NX * TEY, NJ = (NOWN + NT - 1) / NT;  // (column, y segment) items
-    static constexpr int grad_a = P * PU > 2 * P * PG ? P * PU : 2 * P * PG;
-    static constexpr int grad_b = 2 * P * (PT > PS ? PT : PS);
-    static constexpr int grad_ws = grad_a + grad_b;
-    static constexpr int sweep_ws = P * (PG + PS);
+    static constexpr int PU = plane(H2 * S2);  // u on the two-element halo
+    static constexpr int PT = plane(H2 * S1);  // its x pass
+    static constexpr int PG = plane(H1 * S1);  // a field on the one-element halo, or its x pass
+    static constexpr int PR = plane(NY * S1);  // a field on the tile
+    // shared words of grad_sweep_seg, grad_rhs_seg, mass_sweep_seg
+    static constexpr int grad_ws = (P * PU > 2 * P * PG ? P * PU : 2 * P * PG) + 2 * P * PT;
+    static constexpr int rhs_ws = 3 * P * PG;
+    static constexpr int sweep_ws = 2 * P * PG;
     // fields of a udot sweep staged together: two where they take 32 KB at most
-    static constexpr int udot1 = P * (PG + PS + PR);
+    static constexpr int udot1 = P * (2 * PG + PR);
     static constexpr int udot_fields(int nc) { return (nc % 2 == 0 && 2 * udot1 * (int)sizeof(R) <= 32768) ? 2 : 1; }
     static constexpr int udot_ws(int nc) { return udot_fields(nc) * udot1; }
 };
@@ -105,17 +119,17 @@ DEV void seg_apply(const Tab<R>& T, const R (&x)[2 * P + 1], R w0, R (&out)[P]) 
     }
 }
 
-// a segment's values along x (planes of stride PL, at: its row and segment)
-// and along y (rows of stride S, at: its column, row the vertex's)
+// a segment's values along x (f: its vertex in plane 0, planes of stride PL)
+// and along y (f: its vertex, rows of stride S)
 template <class R, int P>
-DEV void seg_x(const R* f, int PL, int at, R (&x)[2 * P + 1]) {
+DEV void seg_x(const R* f, int PL, R (&x)[2 * P + 1]) {
 #pragma unroll
-    for (int k = 0; k <= 2 * P; ++k) x[k] = f[(k % P) * PL + at + k / P - 1];
+    for (int k = 0; k <= 2 * P; ++k) x[k] = f[(k % P) * PL + k / P - 1];
 }
 template <class R, int P>
-DEV void seg_y(const R* f, int S, int at, int row, R (&x)[2 * P + 1]) {
+DEV void seg_y(const R* f, int S, R (&x)[2 * P + 1]) {
 #pragma unroll
-    for (int k = 0; k <= 2 * P; ++k) x[k] = f[at + (row + k - P) * S];
+    for (int k = 0; k <= 2 * P; ++k) x[k] = f[(k - P) * S];
 }
 
 // 1 / m_i of node (gx, gy) with local indices a, b in its segments
@@ -129,238 +143,331 @@ DEV R seg_inv_mass(const MeshDev& m, int a, int kx, int b, int ky) {
     return mul_r(PV<R>::inv_me(m), inv_count<R>(cnt));
 }
 
+// what a thread keeps of its place in a tile: segment xs and first row xr of
+// the x passes, node column q (counted from one element below the tile), its
+// local index a and segment s, and first y segment yr of the y passes.  FULL:
+// the tile and its halo lie inside the mesh (all but the tiles at its edge),
+// so that no index wraps, every vertex is shared and no node is left out.
+template <class R, int P, class TL, bool FULL>
+struct SegThread {
+    int xr, xs, yr, q, a, s, gx, kx, xkind;
+    bool act, own_seg, own_x;
+    DEV SegThread(const MeshDev& m, int gx0, int tid) {
+        act = tid < TL::NT;  // a block may have more threads than the tile takes
+        xr = tid / TL::LX;
+        xs = tid - xr * TL::LX + (TL::HALO ? 0 : 1);
+        yr = tid / TL::LY;
+        q = tid - yr * TL::LY + (TL::HALO ? 0 : P);
+        yr += TL::HALO ? 0 : 1;
+        a = q % P;
+        s = q / P;
+        gx = gx0 - P + q;
+        kx = FULL ? 0 : vertex_kind(gx, m.nnx, m.px);
+        xkind = FULL ? 0 : vertex_kind(gx0 + (xs - 1) * P, m.nnx, m.px);
+        own_seg = act && (!TL::HALO || (xs >= 1 && xs <= TL::TEX));
+        own_x = act && (!TL::HALO || (q >= P && q < P + TL::NX)) && (FULL || gx < m.nnx);
+    }
+    DEV int ykind(const MeshDev& m, int gyv) const { return FULL ? 0 : vertex_kind(gyv, m.nny, m.py); }
+    DEV R inv_mass(const MeshDev& m, int b, int ky) const { return seg_inv_mass<R, P>(m, a, kx, b, ky); }
+};
+
+// Staging of a field on the tile and HALO elements around it (W nodes by H
+// rows, plane stride PL, row stride S): a thread takes one column and every
+// RY-th row, the few columns beyond the block's width go round the block.
+// load() reads into registers, so that it can run ahead of the barrier that
+// frees the planes, store() writes them.  Values outside a non-periodic mesh
+// are 0 (every weight that reaches them is 0).
+template <class R, int P, class TL, int HALO, int W, int H, int PL, int S, bool FULL>
+struct Stage {
+    static constexpr int K = (H + TL::RY - 1) / TL::RY;
+    static constexpr int XC = W > TL::LY ? W - TL::LY : 1, KE = W > TL::LY ? (XC * H + TL::NT - 1) / TL::NT : 0;
+    int q, r, gx, gxt, gyt;  // the thread's column and first row, its node column; the tile's first node
+    bool vx;
+    R v[K], e[KE > 0 ? KE : 1];
+
+    DEV Stage(const MeshDev& m, int gx0, int gy0, int tid) {
+        r = tid / TL::LY;
+        q = tid - r * TL::LY;
+        if (tid >= TL::NT) r = H;  // a thread beyond the tile's stages nothing
+        gxt = gx0 - HALO * P;
+        gyt = gy0 - HALO * P;
+        gx = gxt + q;
+        vx = q < W && inside(gx, m.nnx, m.px);
+    }
+    static DEV bool inside(int& g, int n, int periodic) {
+        if (FULL) return true;
+        if (periodic) g = wrap_periodic(g, n);
+        return g >= 0 && g < n;
+    }
+    // CG: through L2 (ld.global.cg), where the kernel launched just before may
+    // still run
+    template <bool CG>
+    static DEV R get(const R* __restrict__ p) {
+        if constexpr (CG) return __ldcg(p);
+        else return *p;
+    }
+    template <bool CG>
+    DEV void load(const MeshDev& m, const R* __restrict__ x, int tid) {
+        if constexpr (FULL) {
+            const R* __restrict__ p = x + ((long long)(gyt + r) * m.nnx + gx);
+            const long long step = (long long)TL::RY * m.nnx;
+#pragma unroll
+            for (int k = 0; k < K; ++k, p += step) v[k] = (r + k * TL::RY < H && vx) ? get<CG>(p) : R(0);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int row = r + k * TL::RY;
+                int gy = gyt + row;
+                v[k] = (row < H && vx && inside(gy, m.nny, m.py)) ? get<CG>(&x[(long long)gy * m.nnx + gx]) : R(0);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < KE; ++k) {
+            const int i = tid + k * TL::NT, row = tid < TL::NT ? i / XC : H;
+            int g = gxt + TL::LY + i - row * XC, gy = gyt + row;
+            e[k] = (row < H && inside(g, m.nnx, m.px) && inside(gy, m.nny, m.py)) ? get<CG>(&x[(long long)gy * m.nnx + g])
+                                                                                  : R(0);
+        }
+    }
+    DEV void store(R* f, int tid) const {
+        R* p = f + (q % P) * PL + q / P + r * S;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (q < W && r + k * TL::RY < H) p[k * TL::RY * S] = v[k];
+#pragma unroll
+        for (int k = 0; k < KE; ++k) {
+            const int i = tid + k * TL::NT, row = i / XC, c = TL::LY + i - row * XC;
+            if (tid < TL::NT && row < H) f[(c % P) * PL + row * S + c / P] = e[k];
+        }
+    }
+};
+
+// x pass with the mass operator over the rows of a field staged at X (planes
+// PG, rows of S1), into Y of the same shape: the thread's segment, its rows
+template <class R, int P, class TL>
+DEV void mass_x(const Tab<R>& T, const R* X, R* Y, int xs, int xr, R w0) {
+    X += xr * TL::S1 + xs;
+    Y += xr * TL::S1 + xs;
+#pragma unroll 2
+    for (int k = 0; k < TL::K1; ++k) {
+        if (k * TL::RX + xr < TL::H1) {
+            R x[2 * P + 1], o[P];
+            seg_x<R, P>(X + k * TL::RX * TL::S1, TL::PG, x);
+            seg_apply<R, P, 0>(T, x, w0, o);
+#pragma unroll
+            for (int a = 0; a < P; ++a) Y[a * TL::PG + k * TL::RX * TL::S1] = o[a];
+        }
+    }
+}
+
+// whether a tile with n elements of halo lies inside the mesh, away from its
+// ends
+template <int P, class TL, int N>
+DEV bool tile_full(const MeshDev& m, int gx0, int gy0) {
+    return gx0 >= N * P + 1 && gy0 >= N * P + 1 && gx0 + TL::NX + N * P < m.nnx && gy0 + TL::NY + N * P < m.nny;
+}
+
 // Right-hand side of the g_h projection, its lumped iterate and the first
 // sweep on the tile at (gx0, gy0), one component after the other: u on a
 // two-element halo (the next component's loads run under this one's passes),
 // x pass with the derivative and the mass operator, y pass to b and g0 on the
 // one-element halo, then the sweep's x and y passes.  A thread keeps b and g0
-// of its own nodes in registers from the first y pass to the second.  ws:
-// TL::grad_ws values.  All threads of the block call it together.
-// SWEEP false: b and g0 of the tile's nodes only.
-template <class R, int P, int NC, class TL, bool SWEEP = true>
-DEV void grad_sweep_seg(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
-                        int gy0, int tid, R* ws) {
-    constexpr int NT = TL::NT, NJ = TL::NJ, NX = TL::NX, TEX = TL::TEX, TEY = TL::TEY;
-    constexpr int NA = (TL::W2 * TL::H2 + NT - 1) / NT;
-    R* A = ws;                // u, then g0 (x and y parts)
-    R* B = ws + TL::grad_a;   // the x passes
+// of its own nodes in registers from the first y pass to the second.
+template <class R, int P, int NC, class TL, bool FULL>
+DEV void grad_sweep_body(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
+                         int gy0, int tid, R* ws) {
+    constexpr int TEY = TL::TEY, S1 = TL::S1, KY = TL::KY, RY = TL::RY, RX = TL::RX;
+    R* B = ws;                   // the x passes
+    R* A = ws + 2 * P * TL::PT;  // u, then g0 (x and y parts)
     const Tab<R>& T = tab_of<R>(m, P);
     const R h = PV<R>::h(m), h2 = PV<R>::h2(m);
-    // segments and rows that feed nodes of the mesh (ragged tiles stop there)
-    const int ns = min(TL::S1, (m.nnx - gx0 + P - 1) / P + 2), nr = min(TL::H2, m.nny - gy0 + 4 * P);
-    long long off[NA];
-    R next[NA];
-#pragma unroll
-    for (int j = 0; j < NA; ++j) {
-        const int i = tid + j * NT, r = i / TL::W2, q = i - r * TL::W2;
-        int gx = gx0 - 2 * P + q, gy = gy0 - 2 * P + r;
-        const bool in = r < nr && wrap_node(m, gx, gy);
-        off[j] = in ? (long long)gy * m.nnx + gx : -1;
-        // through L2 (ld.global.cg): this runs before the kernel launched just
-        // before it has completed
-        next[j] = in ? __ldcg(&u[off[j]]) : R(0);
-    }
+    const SegThread<R, P, TL, FULL> t(m, gx0, tid);
+    const R w0c = vertex_weight<R, P, 1>(T, t.xkind), w0m = vertex_weight<R, P, 0>(T, t.xkind);
+    const bool inx = FULL || m.px || (t.gx >= 0 && t.gx < m.nnx);
+    const bool feeds_x = t.act && t.q < TL::W1 && (FULL || t.gx < m.nnx + P);
+    const bool feeds_seg = t.act && (FULL || gx0 + (t.xs - 1) * P < m.nnx + P);
+    Stage<R, P, TL, 2, TL::W2, TL::H2, TL::PU, TL::S2, FULL> in(m, gx0, gy0, tid);
+    in.template load<true>(m, u, tid);
 #pragma unroll 1
     for (int c = 0; c < NC; ++c) {
-#pragma unroll
-        for (int j = 0; j < NA; ++j) {
-            const int i = tid + j * NT, r = i / TL::W2, q = i - r * TL::W2;
-            if (i < TL::W2 * TL::H2) A[(q % P) * TL::PU + r * TL::S2 + q / P] = next[j];
-        }
+        in.store(A, tid);
         __syncthreads();
-        if (c + 1 < NC) {
-            const R* __restrict__ uc = u + (c + 1) * m.NN;
+        if (c + 1 < NC) in.template load<true>(m, u + (c + 1) * m.NN, tid);
+        if (feeds_seg) {
+            const R* X = A + t.xr * TL::S2 + t.xs + 1;
+            R* Y = B + t.xr * S1 + t.xs;
+#pragma unroll 2
+            for (int k = 0; k < TL::K2; ++k) {
+                if (k * RX + t.xr < TL::H2) {
+                    R x[2 * P + 1], o[P];
+                    seg_x<R, P>(X + k * RX * TL::S2, TL::PU, x);
+                    seg_apply<R, P, 1>(T, x, w0c, o);
 #pragma unroll
-            for (int j = 0; j < NA; ++j)
-                if (off[j] >= 0) next[j] = __ldcg(&uc[off[j]]);
-        }
-        for (int i = tid; i < TL::H2 * TL::S1; i += NT) {
-            const int r = i / TL::S1, s = i - r * TL::S1;
-            if (s >= ns || r >= nr) continue;
-            if (!SWEEP && (s == 0 || s > TEX || r < P || r >= TL::H2 - P)) continue;  // feeds the halo only
-            R x[2 * P + 1], o[P];
-            seg_x<R, P>(A, TL::PU, r * TL::S2 + s + 1, x);
-            const int kind = vertex_kind(gx0 + (s - 1) * P, m.nnx, m.px);
-            seg_apply<R, P, 1>(T, x, vertex_weight<R, P, 1>(T, kind), o);
+                    for (int i = 0; i < P; ++i) Y[i * TL::PT + k * RX * S1] = o[i];
+                    seg_apply<R, P, 0>(T, x, w0m, o);
 #pragma unroll
-            for (int a = 0; a < P; ++a) B[a * TL::PT + i] = o[a];
-            seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, kind), o);
-#pragma unroll
-            for (int a = 0; a < P; ++a) B[(P + a) * TL::PT + i] = o[a];
-        }
-        __syncthreads();
-        // b and g0 = b / m_i (zero outside the mesh) on column q of the halo
-        // tile and the rows of y segment sy
-        R ob[NJ][2][P], og[NJ][2][P];
-        auto column = [&](int q, int sy, R(&bx)[P], R(&by)[P], R(&vx)[P], R(&vy)[P]) {
-            const int a = q % P, s = q / P;
-            const int gx = gx0 - P + q, gyv = gy0 + (sy - 1) * P;
-            const int kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
-            R t[2 * P + 1];
-            seg_y<R, P>(B + a * TL::PT, TL::S1, s, (sy + 1) * P, t);
-            seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), bx);
-            seg_y<R, P>(B + (P + a) * TL::PT, TL::S1, s, (sy + 1) * P, t);
-            seg_apply<R, P, 1>(T, t, vertex_weight<R, P, 1>(T, ky), by);
-            const bool inx = m.px || (gx >= 0 && gx < m.nnx);
-#pragma unroll
-            for (int b = 0; b < P; ++b) {
-                const int gy = gyv + b;
-                const bool in = inx && (m.py || (gy >= 0 && gy < m.nny));
-                const R inv = seg_inv_mass<R, P>(m, a, kx, b, ky);
-                bx[b] = mul_r(h, bx[b]);
-                by[b] = mul_r(h, by[b]);
-                vx[b] = in ? mul_r(bx[b], inv) : R(0);
-                vy[b] = in ? mul_r(by[b], inv) : R(0);
-                if (SWEEP && (sy <= TEY || b == 0)) {
-                    const int at = a * TL::PG + (sy * P + b) * TL::S1 + s;
-                    A[at] = vx[b];
-                    A[P * TL::PG + at] = vy[b];
+                    for (int i = 0; i < P; ++i) Y[(P + i) * TL::PT + k * RX * S1] = o[i];
                 }
             }
-        };
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
-            if (i < TL::NOWN && gx0 + q < m.nnx + P && gy0 + sy * P < m.nny + P)
-                column(q + P, sy + 1, ob[j][0], ob[j][1], og[j][0], og[j][1]);
         }
-        if constexpr (!SWEEP) {
+        __syncthreads();
+        R ob[KY][2][P], og[KY][2][P];  // b and g0 of the thread's nodes
+        if (feeds_x) {
+            const R* X = B + t.a * TL::PT + (t.yr + 1) * P * S1 + t.s;
+            R* Y = A + t.a * TL::PG + t.yr * P * S1 + t.s;
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
-                const int gx = gx0 + q, gyv = gy0 + sy * P;
-                if (i >= TL::NOWN || gx >= m.nnx || gyv >= m.nny) continue;
+            for (int k = 0; k < KY; ++k) {
+                const int sy = t.yr + k * RY;  // 0: the segment below the tile
+                const int gyv = gy0 + (sy - 1) * P, ky = t.ykind(m, gyv);
+                R x[2 * P + 1];
+                seg_y<R, P>(X + k * RY * P * S1, S1, x);
+                seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, ky), ob[k][0]);
+                seg_y<R, P>(X + P * TL::PT + k * RY * P * S1, S1, x);
+                seg_apply<R, P, 1>(T, x, vertex_weight<R, P, 1>(T, ky), ob[k][1]);
+#pragma unroll
+                for (int b = 0; b < P; ++b) {
+                    const bool in_mesh = FULL || (inx && (m.py || (gyv + b >= 0 && gyv + b < m.nny)));
+                    const R inv = t.inv_mass(m, b, ky);
+#pragma unroll
+                    for (int f = 0; f < 2; ++f) {
+                        ob[k][f][b] = mul_r(h, ob[k][f][b]);
+                        og[k][f][b] = in_mesh ? mul_r(ob[k][f][b], inv) : R(0);
+                        if (sy <= TEY || b == 0) Y[f * P * TL::PG + (k * RY * P + b) * S1] = og[k][f][b];
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        if (t.own_seg) {
+            mass_x<R, P, TL>(T, A, B, t.xs, t.xr, w0m);
+            mass_x<R, P, TL>(T, A + P * TL::PG, B + P * TL::PG, t.xs, t.xr, w0m);
+        }
+        __syncthreads();
+        if (t.own_x) {
+            const R* X = B + t.a * TL::PG + t.yr * P * S1 + t.s;
+#pragma unroll
+            for (int k = 0; k < KY; ++k) {
+                const int sy = t.yr + k * RY, gyv = gy0 + (sy - 1) * P, ky = t.ykind(m, gyv);
+                if (sy < 1 || sy > TEY || (!FULL && gyv >= m.nny)) continue;
 #pragma unroll
                 for (int f = 0; f < 2; ++f) {
-                    const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + gx;
+                    R x[2 * P + 1], o[P];
+                    seg_y<R, P>(X + f * P * TL::PG + k * RY * P * S1, S1, x);
+                    seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, ky), o);
+                    const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + t.gx;
 #pragma unroll
                     for (int b = 0; b < P; ++b)
-                        if (gyv + b < m.nny) {
-                            bout[node + (long long)b * m.nnx] = ob[j][f][b];
-                            gout[node + (long long)b * m.nnx] = og[j][f][b];
+                        if (FULL || gyv + b < m.nny) {
+                            const long long n = node + (long long)b * m.nnx;
+                            gout[n] = sweep_value(og[k][f][b], ob[k][f][b], o[b], h2, t.inv_mass(m, b, ky));
+                            if (bout) bout[n] = ob[k][f][b];
                         }
                 }
             }
-            continue;  // the next staging writes u, which no one reads any more
         }
-        // the halo: the rows below and above the tile, then its sides
-        constexpr int NROW = 2 * TL::W1, NEXT = NROW + (P + 1) * TEY;
-        for (int i = tid; i < NEXT; i += NT) {
-            int q, sy;
-            if (i < NROW) {
-                sy = i < TL::W1 ? 0 : TEY + 1;
-                q = i < TL::W1 ? i : i - TL::W1;
-            } else {
-                const int k = i - NROW, w = k % (P + 1);
-                sy = k / (P + 1) + 1;
-                q = w < P ? w : TL::W1 - 1;
+    }
+}
+
+// b and g0 alone, from u on a one-element halo
+template <class R, int P, int NC, class TL, bool FULL>
+DEV void grad_rhs_body(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
+                       int gy0, int tid, R* ws) {
+    constexpr int TEY = TL::TEY, S1 = TL::S1, RX = TL::RX, RY = TL::RY;
+    R* A = ws;
+    R* B = ws + P * TL::PG;
+    const Tab<R>& T = tab_of<R>(m, P);
+    const R h = PV<R>::h(m);
+    const SegThread<R, P, TL, FULL> t(m, gx0, tid);
+    const R w0c = vertex_weight<R, P, 1>(T, t.xkind), w0m = vertex_weight<R, P, 0>(T, t.xkind);
+    Stage<R, P, TL, 1, TL::W1, TL::H1, TL::PG, S1, FULL> in(m, gx0, gy0, tid);
+    in.template load<true>(m, u, tid);
+#pragma unroll 1
+    for (int c = 0; c < NC; ++c) {
+        in.store(A, tid);
+        __syncthreads();
+        if (c + 1 < NC) in.template load<true>(m, u + (c + 1) * m.NN, tid);
+        if (t.own_seg) {
+            const R* X = A + t.xr * S1 + t.xs;
+            R* Y = B + t.xr * S1 + t.xs;
+#pragma unroll 2
+            for (int k = 0; k < TL::K1; ++k) {
+                if (k * RX + t.xr < TL::H1) {
+                    R x[2 * P + 1], o[P];
+                    seg_x<R, P>(X + k * RX * S1, TL::PG, x);
+                    seg_apply<R, P, 1>(T, x, w0c, o);
+#pragma unroll
+                    for (int i = 0; i < P; ++i) Y[i * TL::PG + k * RX * S1] = o[i];
+                    seg_apply<R, P, 0>(T, x, w0m, o);
+#pragma unroll
+                    for (int i = 0; i < P; ++i) Y[(P + i) * TL::PG + k * RX * S1] = o[i];
+                }
             }
-            R b0[P], b1[P], v0[P], v1[P];
-            column(q, sy, b0, b1, v0, v1);
         }
         __syncthreads();
-        const int ns0 = ns - 2, nr1 = min(TL::H1, m.nny - gy0 + 2 * P);
-        for (int i = tid; i < 2 * TL::H1 * TEX; i += NT) {
-            const int f = i / (TL::H1 * TEX), k = i - f * (TL::H1 * TEX), r = k / TEX, s = k - r * TEX;
-            if (s >= ns0 || r >= nr1) continue;
-            R x[2 * P + 1], o[P];
-            seg_x<R, P>(A + f * P * TL::PG, TL::PG, r * TL::S1 + s + 1, x);
-            seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, vertex_kind(gx0 + s * P, m.nnx, m.px)), o);
+        if (t.own_x) {
+#pragma unroll 2
+            for (int k = 0; k < TL::KY; ++k) {
+                const int sy = t.yr + k * RY, gyv = gy0 + (sy - 1) * P, ky = t.ykind(m, gyv);
+                if (sy < 1 || sy > TEY || (!FULL && gyv >= m.nny)) continue;
+                const R* X = B + t.a * TL::PG + sy * P * S1 + t.s;
 #pragma unroll
-            for (int a = 0; a < P; ++a) B[(f * P + a) * TL::PS + k] = o[a];
-        }
-        __syncthreads();
+                for (int f = 0; f < 2; ++f) {
+                    R x[2 * P + 1], o[P];
+                    seg_y<R, P>(X + f * P * TL::PG, S1, x);
+                    if (f == 0) seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, ky), o);
+                    else seg_apply<R, P, 1>(T, x, vertex_weight<R, P, 1>(T, ky), o);
+                    const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + t.gx;
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-            const int i = tid + j * NT, sy = i / NX, q = i - sy * NX;
-            const int gx = gx0 + q, gyv = gy0 + sy * P;
-            if (i >= TL::NOWN || gx >= m.nnx || gyv >= m.nny) continue;
-            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
-#pragma unroll
-            for (int f = 0; f < 2; ++f) {
-                R t[2 * P + 1], o[P];
-                seg_y<R, P>(B + (f * P + a) * TL::PS, TEX, q / P, (sy + 1) * P, t);
-                seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
-                const long long node = (long long)(f * NC + c) * m.NN + (long long)gyv * m.nnx + gx;
-#pragma unroll
-                for (int b = 0; b < P; ++b)
-                    if (gyv + b < m.nny) {
-                        const long long k = node + (long long)b * m.nnx;
-                        gout[k] = sweep_value(og[j][f][b], ob[j][f][b], o[b], h2, seg_inv_mass<R, P>(m, a, kx, b, ky));
-                        if (bout) bout[k] = ob[j][f][b];
-                    }
+                    for (int b = 0; b < P; ++b)
+                        if (FULL || gyv + b < m.nny) {
+                            const long long n = node + (long long)b * m.nnx;
+                            const R v = mul_r(h, o[b]);
+                            bout[n] = v;
+                            gout[n] = mul_r(v, t.inv_mass(m, b, ky));
+                        }
+                }
             }
         }
     }
 }
 
-// x pass of a mass sweep for FB iterates staged at X (planes PG), into Y
-template <class R, int P, int FB, class TL>
-DEV void sweep_x(const MeshDev& m, const Tab<R>& T, const R* X, R* Y, int gx0, int gy0, int tid) {
-    constexpr int TEX = TL::TEX;
-    const int ns = (m.nnx - gx0 + P - 1) / P, nr = min(TL::H1, m.nny - gy0 + 2 * P);
-    for (int i = tid; i < FB * TL::H1 * TEX; i += TL::NT) {
-        const int f = i / (TL::H1 * TEX), k = i - f * (TL::H1 * TEX), r = k / TEX, s = k - r * TEX;
-        if (s >= ns || r >= nr) continue;
-        R x[2 * P + 1], o[P];
-        seg_x<R, P>(X + f * P * TL::PG, TL::PG, r * TL::S1 + s + 1, x);
-        seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, vertex_kind(gx0 + s * P, m.nnx, m.px)), o);
-#pragma unroll
-        for (int a = 0; a < P; ++a) Y[(f * P + a) * TL::PS + k] = o[a];
-    }
-}
-
-// one Richardson sweep for NV fields on the tile; ws: TL::sweep_ws values
-template <class R, int P, int NV, class TL>
-DEV void mass_sweep_seg(const MeshDev& m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout,
-                        int gx0, int gy0, int tid, R* ws) {
-    constexpr int NT = TL::NT, NX = TL::NX;
-    constexpr int NA = (TL::W1 * TL::H1 + NT - 1) / NT;
+// one Richardson sweep for NV fields on the tile
+template <class R, int P, int NV, class TL, bool FULL>
+DEV void mass_sweep_body(const MeshDev& m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout,
+                         int gx0, int gy0, int tid, R* ws) {
+    constexpr int TEY = TL::TEY, S1 = TL::S1, RY = TL::RY;
     R* A = ws;
     R* B = ws + P * TL::PG;
     const Tab<R>& T = tab_of<R>(m, P);
     const R h2 = PV<R>::h2(m);
-    long long off[NA];
-    R next[NA];
-#pragma unroll
-    for (int j = 0; j < NA; ++j) {
-        const int i = tid + j * NT, r = i / TL::W1, q = i - r * TL::W1;
-        int gx = gx0 - P + q, gy = gy0 - P + r;
-        const bool in = r < TL::H1 && wrap_node(m, gx, gy);
-        off[j] = in ? (long long)gy * m.nnx + gx : -1;
-        next[j] = in ? xin[off[j]] : R(0);
-    }
+    const SegThread<R, P, TL, FULL> t(m, gx0, tid);
+    const R w0 = vertex_weight<R, P, 0>(T, t.xkind);
+    Stage<R, P, TL, 1, TL::W1, TL::H1, TL::PG, S1, FULL> in(m, gx0, gy0, tid);
+    in.template load<false>(m, xin, tid);
 #pragma unroll 1
     for (int v = 0; v < NV; ++v) {
-#pragma unroll
-        for (int j = 0; j < NA; ++j) {
-            const int i = tid + j * NT, r = i / TL::W1, q = i - r * TL::W1;
-            if (i < TL::W1 * TL::H1) A[(q % P) * TL::PG + r * TL::S1 + q / P] = next[j];
-        }
+        in.store(A, tid);
         __syncthreads();
-        if (v + 1 < NV) {
-            const R* __restrict__ xv = xin + (v + 1) * m.NN;
-#pragma unroll
-            for (int j = 0; j < NA; ++j)
-                if (off[j] >= 0) next[j] = xv[off[j]];
-        }
-        sweep_x<R, P, 1, TL>(m, T, A, B, gx0, gy0, tid);
+        if (v + 1 < NV) in.template load<false>(m, xin + (v + 1) * m.NN, tid);
+        if (t.own_seg) mass_x<R, P, TL>(T, A, B, t.xs, t.xr, w0);
         __syncthreads();
-        for (int i = tid; i < TL::NOWN; i += NT) {
-            const int sy = i / NX, q = i - sy * NX, gx = gx0 + q, gyv = gy0 + sy * P;
-            if (gx >= m.nnx || gyv >= m.nny) continue;
-            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
-            R t[2 * P + 1], o[P];
-            seg_y<R, P>(B + a * TL::PS, TL::TEX, q / P, (sy + 1) * P, t);
-            seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
-            const long long node = v * m.NN + (long long)gyv * m.nnx + gx;
+        if (t.own_x) {
+#pragma unroll 2
+            for (int k = 0; k < TL::KY; ++k) {
+                const int sy = t.yr + k * RY, gyv = gy0 + (sy - 1) * P, ky = t.ykind(m, gyv);
+                if (sy < 1 || sy > TEY || (!FULL && gyv >= m.nny)) continue;
+                const int at = t.a * TL::PG + sy * P * S1 + t.s;
+                R x[2 * P + 1], o[P];
+                seg_y<R, P>(B + at, S1, x);
+                seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, ky), o);
+                const long long node = v * m.NN + (long long)gyv * m.nnx + t.gx;
 #pragma unroll
-            for (int c = 0; c < P; ++c)
-                if (gyv + c < m.nny) {
-                    const long long k = node + (long long)c * m.nnx;
-                    xout[k] = sweep_value(A[a * TL::PG + ((sy + 1) * P + c) * TL::S1 + q / P + 1], b[k], o[c], h2,
-                                          seg_inv_mass<R, P>(m, a, kx, c, ky));
-                }
+                for (int c = 0; c < P; ++c)
+                    if (FULL || gyv + c < m.nny) {
+                        const long long n = node + (long long)c * m.nnx;
+                        xout[n] = sweep_value(A[at + c * S1], b[n], o[c], h2, t.inv_mass(m, c, ky));
+                    }
+            }
         }
         if (v + 1 < NV) __syncthreads();  // the iterate is consumed
     }
@@ -372,152 +479,195 @@ DEV void mass_sweep_seg(const MeshDev& m, const R* __restrict__ xin, const R* __
 // value are consecutive in the element index, and no lane branches on its
 // node's position in the element.  r = sum over E_i (stored for further sweeps
 // and diagnostics), udot0 = r / m_i, udot1 = udot0 + (r - M_C udot0) / m_i.
-// ws: TL::udot_ws(NC) values.
-template <class R, int P, int NC, class TL>
-DEV void udot_sweep_seg(const MeshDev& m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout, int gx0,
-                        int gy0, int tid, R* ws) {
-    constexpr int NT = TL::NT, NX = TL::NX, TEX = TL::TEX, TEY = TL::TEY, N1 = P + 1;
-    constexpr int FB = TL::udot_fields(NC);
-    R* A = ws;                    // udot0 on the one-element halo
-    R* B = A + FB * P * TL::PG;   // its x pass
-    R* C = B + FB * P * TL::PS;   // r on the tile
+template <class R, int P, int NC, class TL, bool FULL>
+DEV void udot_sweep_body(const MeshDev& m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout,
+                         int gx0, int gy0, int tid, R* ws) {
+    constexpr int TEX = TL::TEX, TEY = TL::TEY, S1 = TL::S1, RY = TL::RY, N1 = P + 1;
+    constexpr int FB = TL::udot_fields(NC), NI = S1 * (TEY + 2);
+    R* A = ws;                   // udot0 on the one-element halo
+    R* B = A + FB * P * TL::PG;  // its x pass
+    R* C = B + FB * P * TL::PG;  // r on the tile
     const Tab<R>& T = tab_of<R>(m, P);
     const R h2 = PV<R>::h2(m);
-    const int ex0 = gx0 / P, ey0 = gy0 / P;
-    const long long E = m.E;
+    const int E = m.E, nx = m.nx;
+    const SegThread<R, P, TL, FULL> t(m, gx0, tid);
+    const R w0 = vertex_weight<R, P, 0>(T, t.xkind);
 #pragma unroll 1
     for (int v0 = 0; v0 < NC; v0 += FB) {
         if (v0 > 0) __syncthreads();  // the previous fields are consumed
-        for (int i = tid; i < (TEX + 2) * (TEY + 2); i += NT) {
-            const int sy = i / (TEX + 2), sx = i - sy * (TEX + 2);
+#pragma unroll 1
+        for (int it = tid; it < NI && t.act; it += TL::NT) {
+            const int sy = it / S1, xs = it - sy * S1;
             // the elements before (l) and after (h) the vertex along x and y;
             // hx, hy false: the segment has its vertex only (or lies outside)
-            int xl = ex0 + sx - 2, xh = xl + 1, yl = ey0 + sy - 2, yh = yl + 1;
-            if (xl > m.nx || yl > m.ny) continue;  // feeds no node of the mesh
-            if (m.px) xl = wrap_periodic(xl, m.nx), xh = wrap_periodic(xh, m.nx);
-            if (m.py) yl = wrap_periodic(yl, m.ny), yh = wrap_periodic(yh, m.ny);
-            const bool lx = xl >= 0 && xl < m.nx, hx = xh >= 0 && xh < m.nx;
-            const bool ly = yl >= 0 && yl < m.ny, hy = yh >= 0 && yh < m.ny;
-            const int kx = m.px ? 0 : (!lx ? 1 : !hx ? 2 : 0), ky = m.py ? 0 : (!ly ? 1 : !hy ? 2 : 0);
-            const bool tile = sx >= 1 && sx <= TEX && sy >= 1 && sy <= TEY;
-            const long long ell = (long long)yl * m.nx + xl, ehl = (long long)yl * m.nx + xh;
-            const long long elh = (long long)yh * m.nx + xl, ehh = (long long)yh * m.nx + xh;
+            int xl = gx0 / P + xs - 2, xh = xl + 1, yl = gy0 / P + sy - 2, yh = yl + 1;
+            if (!FULL) {
+                if (xl > nx || yl > m.ny) continue;  // feeds no node of the mesh
+                if (m.px) xl = wrap_periodic(xl, nx), xh = wrap_periodic(xh, nx);
+                if (m.py) yl = wrap_periodic(yl, m.ny), yh = wrap_periodic(yh, m.ny);
+            }
+            const bool lx = FULL || (xl >= 0 && xl < nx), hx = FULL || (xh >= 0 && xh < nx);
+            const bool ly = FULL || (yl >= 0 && yl < m.ny), hy = FULL || (yh >= 0 && yh < m.ny);
+            const int xkind = m.px || FULL ? 0 : (!lx ? 1 : !hx ? 2 : 0);
+            const int ykind = m.py || FULL ? 0 : (!ly ? 1 : !hy ? 2 : 0);
+            const bool tile = xs >= 1 && xs <= TEX && sy >= 1 && sy <= TEY;
+            const int ell = yl * nx + xl, ehl = yl * nx + xh, elh = yh * nx + xl, ehh = yh * nx + xh;
 #pragma unroll
             for (int f = 0; f < FB; ++f) {
-                const R* __restrict__ Ev = ER + (v0 + f) * E;
-                auto val = [&](bool in, long long e, int a, int b) {
-                    return in ? Ev[(long long)((b * N1 + a) * NC) * E + e] : R(0);
+                auto val = [&](bool in, int e, int i, int j) {
+                    return in ? (ER + (long long)((j * N1 + i) * NC + v0 + f) * E)[e] : R(0);
                 };
 #pragma unroll
-                for (int b = 0; b < P; ++b)
+                for (int j = 0; j < P; ++j)
 #pragma unroll
-                    for (int a = 0; a < P; ++a) {
+                    for (int i = 0; i < P; ++i) {
                         // past the last vertex of the halo
-                        if ((a > 0 && sx == TEX + 1) || (b > 0 && sy == TEY + 1)) continue;
-                        R s;
+                        if ((i > 0 && xs == TEX + 1) || (j > 0 && sy == TEY + 1)) continue;
+                        R sum;
                         bool in;
-                        if (a == 0 && b == 0) {
-                            s = ((val(lx && ly, ell, P, P) + val(hx && ly, ehl, 0, P)) + val(lx && hy, elh, P, 0)) +
-                                val(hx && hy, ehh, 0, 0);
+                        if (i == 0 && j == 0) {
+                            sum = ((val(lx && ly, ell, P, P) + val(hx && ly, ehl, 0, P)) + val(lx && hy, elh, P, 0)) +
+                                  val(hx && hy, ehh, 0, 0);
                             in = (lx || hx) && (ly || hy);
-                        } else if (b == 0) {
-                            s = val(hx && ly, ehl, a, P) + val(hx && hy, ehh, a, 0);
+                        } else if (j == 0) {
+                            sum = val(hx && ly, ehl, i, P) + val(hx && hy, ehh, i, 0);
                             in = hx && (ly || hy);
-                        } else if (a == 0) {
-                            s = val(lx && hy, elh, P, b) + val(hx && hy, ehh, 0, b);
+                        } else if (i == 0) {
+                            sum = val(lx && hy, elh, P, j) + val(hx && hy, ehh, 0, j);
                             in = (lx || hx) && hy;
                         } else {
-                            s = val(hx && hy, ehh, a, b);
+                            sum = val(hx && hy, ehh, i, j);
                             in = hx && hy;
                         }
-                        const int q = sx, row = sy * P + b;
-                        A[(f * P + a) * TL::PG + row * TL::S1 + q] =
-                            in ? mul_r(s, seg_inv_mass<R, P>(m, a, kx, b, ky)) : R(0);
-                        if (tile) C[(f * P + a) * TL::PR + (row - P) * TEX + q - 1] = s;
+                        const int row = sy * P + j;
+                        A[(f * P + i) * TL::PG + row * S1 + xs] =
+                            in ? mul_r(sum, seg_inv_mass<R, P>(m, i, xkind, j, ykind)) : R(0);
+                        if (tile) C[(f * P + i) * TL::PR + (row - P) * S1 + xs] = sum;
                     }
             }
         }
         __syncthreads();
-        sweep_x<R, P, FB, TL>(m, T, A, B, gx0, gy0, tid);
+        if (t.own_seg) {
+#pragma unroll
+            for (int f = 0; f < FB; ++f) mass_x<R, P, TL>(T, A + f * P * TL::PG, B + f * P * TL::PG, t.xs, t.xr, w0);
+        }
         __syncthreads();
-        for (int i = tid; i < TL::NOWN; i += NT) {
-            const int sy = i / NX, q = i - sy * NX, gx = gx0 + q, gyv = gy0 + sy * P;
-            if (gx >= m.nnx || gyv >= m.nny) continue;
-            const int a = q % P, kx = vertex_kind(gx, m.nnx, m.px), ky = vertex_kind(gyv, m.nny, m.py);
+        if (t.own_x) {
+#pragma unroll 2
+            for (int k = 0; k < TL::KY; ++k) {
+                const int sy = t.yr + k * RY, gyv = gy0 + (sy - 1) * P, ky = t.ykind(m, gyv);
+                if (sy < 1 || sy > TEY || (!FULL && gyv >= m.nny)) continue;
 #pragma unroll
-            for (int f = 0; f < FB; ++f) {
-                R t[2 * P + 1], o[P];
-                seg_y<R, P>(B + (f * P + a) * TL::PS, TEX, q / P, (sy + 1) * P, t);
-                seg_apply<R, P, 0>(T, t, vertex_weight<R, P, 0>(T, ky), o);
-                const long long node = (v0 + f) * m.NN + (long long)gyv * m.nnx + gx;
+                for (int f = 0; f < FB; ++f) {
+                    const int at = (f * P + t.a) * TL::PG + sy * P * S1 + t.s;
+                    R x[2 * P + 1], o[P];
+                    seg_y<R, P>(B + at, S1, x);
+                    seg_apply<R, P, 0>(T, x, vertex_weight<R, P, 0>(T, ky), o);
+                    const long long node = (v0 + f) * m.NN + (long long)gyv * m.nnx + t.gx;
 #pragma unroll
-                for (int c = 0; c < P; ++c)
-                    if (gyv + c < m.nny) {
-                        const long long k = node + (long long)c * m.nnx;
-                        const R r = C[(f * P + a) * TL::PR + (sy * P + c) * TEX + q / P];
-                        rout[k] = r;
-                        xout[k] = sweep_value(A[(f * P + a) * TL::PG + ((sy + 1) * P + c) * TL::S1 + q / P + 1], r, o[c],
-                                              h2, seg_inv_mass<R, P>(m, a, kx, c, ky));
-                    }
+                    for (int c = 0; c < P; ++c)
+                        if (FULL || gyv + c < m.nny) {
+                            const long long n = node + (long long)c * m.nnx;
+                            const R r = C[(f * P + t.a) * TL::PR + ((sy - 1) * P + c) * S1 + t.s];
+                            rout[n] = r;
+                            xout[n] = sweep_value(A[at + c * S1], r, o[c], h2, t.inv_mass(m, c, ky));
+                        }
+                }
             }
         }
     }
 }
 
-// The tiles of the single-state kernels.  Large: about 1024 nodes and 256
-// threads (float64 with fewer rows at p >= 3, where 48 KB of shared memory
-// ends); small: 4 x 4 elements (8 x 8 at p = 1) and 64 threads, for meshes
-// whose large tiles leave SMs idle.
-template <class R, int P, bool SMALL>
+// The same on any tile: inside the mesh or at its edge.  ws: TL::grad_ws,
+// rhs_ws, sweep_ws or udot_ws(NC) values.  All threads of the block call them
+// together.
+template <class R, int P, int NC, class TL>
+DEV void grad_sweep_seg(const MeshDev& m, const R* u, R* bout, R* gout, int gx0, int gy0, int tid, R* ws) {
+    if (tile_full<P, TL, 2>(m, gx0, gy0)) grad_sweep_body<R, P, NC, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
+    else grad_sweep_body<R, P, NC, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
+}
+template <class R, int P, int NC, class TL>
+DEV void grad_rhs_seg(const MeshDev& m, const R* u, R* bout, R* gout, int gx0, int gy0, int tid, R* ws) {
+    if (tile_full<P, TL, 1>(m, gx0, gy0)) grad_rhs_body<R, P, NC, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
+    else grad_rhs_body<R, P, NC, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
+}
+template <class R, int P, int NV, class TL>
+DEV void mass_sweep_seg(const MeshDev& m, const R* xin, const R* b, R* xout, int gx0, int gy0, int tid, R* ws) {
+    if (tile_full<P, TL, 1>(m, gx0, gy0)) mass_sweep_body<R, P, NV, TL, true>(m, xin, b, xout, gx0, gy0, tid, ws);
+    else mass_sweep_body<R, P, NV, TL, false>(m, xin, b, xout, gx0, gy0, tid, ws);
+}
+template <class R, int P, int NC, class TL>
+DEV void udot_sweep_seg(const MeshDev& m, const R* ER, R* rout, R* xout, int gx0, int gy0, int tid, R* ws) {
+    if (tile_full<P, TL, 2>(m, gx0, gy0)) udot_sweep_body<R, P, NC, TL, true>(m, ER, rout, xout, gx0, gy0, tid, ws);
+    else udot_sweep_body<R, P, NC, TL, false>(m, ER, rout, xout, gx0, gy0, tid, ws);
+}
+
+// The tiles of the single-state kernels (HALO: of the fused g_h kernel, by two
+// elements smaller in each direction).  Large: 32 (p <= 2) or 16 elements wide
+// and 16 or 8 high, in float64 16 by 16 (p = 3) and 16 by 12 (p = 4), where the
+// float64 pipe pays for every operation on the halo.  Small, for meshes whose
+// large tiles leave SMs idle: in float 16 (p = 1: 32) by 8 or 6; in float64,
+// where a block's work is long against a launch, 8 by 4 to 8.
+template <class R, int P, bool SMALL, bool HALO>
 struct StageTile {
     static constexpr bool F = sizeof(R) == 4;
-    static constexpr int X = SMALL ? (P == 1 ? 8 : 4) : (P == 1 ? 32 : P == 2 ? 16 : P == 3 ? 12 : 8);
-    static constexpr int Y = SMALL ? (P == 1 ? 8 : 4) : (P <= 2 ? 16 : P == 3 ? (F ? 12 : 7) : (F ? 8 : 6));
-    using type = SegTile<R, P, X, Y, SMALL ? 64 : 256>;
+    static constexpr int LX = SMALL ? (F ? (P == 1 ? 32 : 16) : 8) : (P <= 2 ? 32 : 16);
+    static constexpr int NT = SMALL ? (F ? (P == 3 ? 96 : 128) : (P == 3 ? 72 : 64)) : (P == 3 ? 192 : 256);
+    static constexpr int RY = NT / (LX * P);
+    static constexpr int ROWS = SMALL ? (RY >= 8 ? 8 : RY == 4 ? (F ? 8 : 4) : 6)
+                                      : (P <= 2 ? 16 : F ? 8 : P == 3 ? 16 : 12);  // y segments
+    using type = SegTile<R, P, LX, ROWS / RY, NT, HALO>;
 };
-template <class R, int P, bool SMALL>
-using stage_tile_t = typename StageTile<R, P, SMALL>::type;
+template <class R, int P, bool SMALL, bool HALO = false>
+using stage_tile_t = typename StageTile<R, P, SMALL, HALO>::type;
+
+// dynamic shared memory as an array of R (more than 48 KB in float64)
+template <class R>
+DEV R* dyn_shared() {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    return reinterpret_cast<R*>(dyn_smem);
+}
 
 template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 64 : 256, SMALL ? 1 : (sizeof(R) == 4 ? 3 : 2))
+__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT, SMALL ? 1 : (P == 3 ? 4 : 3))
     k_grad_sweep(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
-    using TL = stage_tile_t<R, P, SMALL>;
+    using TL = stage_tile_t<R, P, SMALL, true>;
     // like k_grad_rhs: runs beside k_pre, waits for it before exiting
     pdl_trigger();
-    __shared__ R ws[TL::grad_ws];
-    grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
+    grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                                 dyn_shared<R>());
     pdl_wait();
 }
 
 template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 64 : 256)
+__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
     k_grad_rhs(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
     using TL = stage_tile_t<R, P, SMALL>;
     // needs only u, whose last writer completed before k_pre let this kernel
     // start (pdl_wait_then_trigger), so it runs beside k_pre and waits for it
     // only before exiting
     pdl_trigger();
-    __shared__ R ws[TL::grad_ws];
-    grad_sweep_seg<R, P, NC, TL, false>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
+    grad_rhs_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                               dyn_shared<R>());
     pdl_wait();
 }
 
 template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 64 : 256)
+__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
     k_udot_sweep(MeshDev m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout) {
     using TL = stage_tile_t<R, P, SMALL>;
     pdl_begin();
-    __shared__ R ws[TL::udot_ws(NC)];
-    udot_sweep_seg<R, P, NC, TL>(m, ER, rout, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
+    udot_sweep_seg<R, P, NC, TL>(m, ER, rout, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                                 dyn_shared<R>());
 }
 
 template <class R, int P, int NV, bool SMALL>
-__global__ void __launch_bounds__(SMALL ? 64 : 256)
+__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
     k_mass_sweep(MeshDev m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout) {
     using TL = stage_tile_t<R, P, SMALL>;
     pdl_begin();
-    __shared__ R ws[TL::sweep_ws];
-    mass_sweep_seg<R, P, NV, TL>(m, xin, b, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x, ws);
+    mass_sweep_seg<R, P, NV, TL>(m, xin, b, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                                 dyn_shared<R>());
 }
 
 }  // namespace cgl

@@ -68,10 +68,26 @@ struct Prof {
 typedef cudaError_t (*StageFn)(const Bufs&, const MeshDev&, const ProbDev&, double a, double b,
                                bool first, bool dt_only, cudaStream_t st, Prof* prof);
 
-// large stencil tiles below which the small ones are used
-constexpr int SMALL_TILES_BELOW = 304;
-
 inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+
+// small stencil tiles where the large ones (nx by ny nodes) make fewer blocks
+// than this
+constexpr long long SMALL_TILES_BELOW = 304;
+inline bool use_small_tiles(const MeshDev& m, int nx, int ny) {
+    return (long long)nblk(m.nnx, nx) * nblk(m.nny, ny) < SMALL_TILES_BELOW;
+}
+// the g_h right-hand side and the first sweep in one kernel (rsz: bytes per value)
+inline bool fuse_grad_sweep(size_t rsz, bool small_tiles) { return rsz == 4 || small_tiles; }
+// the same for a state's mesh and precision
+template <class R>
+inline bool small_tiles_of(const MeshDev& m) {
+    switch (m.p) {
+        case 1: return use_small_tiles(m, stage_tile_t<R, 1, false>::NX, stage_tile_t<R, 1, false>::NY);
+        case 2: return use_small_tiles(m, stage_tile_t<R, 2, false>::NX, stage_tile_t<R, 2, false>::NY);
+        case 3: return use_small_tiles(m, stage_tile_t<R, 3, false>::NX, stage_tile_t<R, 3, false>::NY);
+        default: return use_small_tiles(m, stage_tile_t<R, 4, false>::NX, stage_tile_t<R, 4, false>::NY);
+    }
+}
 
 // The split residual (k_res_w on the second stream, k_res_s) overlaps the
 // quadrature with k_pre and the g_h kernels but adds a kernel and the W^e
@@ -99,6 +115,27 @@ inline cudaError_t launch(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, 
     return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// the same with dynamic shared memory (opted in above the default 48 KB)
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_shared(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, int smem, cudaStream_t st,
+                                 Args... args) {
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
+}
+
 template <class R, int P, class Ph>
 cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, double a, double b,
                       bool first, bool dt_only, cudaStream_t st, Prof* prof) {
@@ -110,10 +147,17 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     // the stencils' tiles: small ones where the large ones would leave SMs idle
     using TL = stage_tile_t<R, P, false>;
     using TS = stage_tile_t<R, P, true>;
+    const bool small_tiles = use_small_tiles(m, TL::NX, TL::NY);
     const dim3 gl(nblk(m.nnx, TL::NX), nblk(m.nny, TL::NY));
-    const bool small_tiles = gl.x * gl.y < (unsigned)SMALL_TILES_BELOW;
     const dim3 gt = small_tiles ? dim3(nblk(m.nnx, TS::NX), nblk(m.nny, TS::NY)) : gl, bt(small_tiles ? TS::NT : TL::NT);
-    auto* k_gradf = small_tiles ? k_grad_sweep<R, P, NC, true> : k_grad_sweep<R, P, NC, false>;
+    // the fused g_h kernel's tiles leave room for their halo
+    using HL = stage_tile_t<R, P, false, true>;
+    using HS = stage_tile_t<R, P, true, true>;
+    const dim3 gth = small_tiles ? dim3(nblk(m.nnx, HS::NX), nblk(m.nny, HS::NY)) : dim3(nblk(m.nnx, HL::NX), nblk(m.nny, HL::NY));
+    const int ws = sizeof(R), ws_grad = ws * (small_tiles ? HS::grad_ws : HL::grad_ws);
+    const int ws_rhs = ws * (small_tiles ? TS::rhs_ws : TL::rhs_ws);
+    const int ws_udot = ws * (small_tiles ? TS::udot_ws(NC) : TL::udot_ws(NC));
+    const int ws_sweep = ws * (small_tiles ? TS::sweep_ws : TL::sweep_ws);
     auto* k_grad = small_tiles ? k_grad_rhs<R, P, NC, true> : k_grad_rhs<R, P, NC, false>;
     auto* k_udotf = small_tiles ? k_udot_sweep<R, P, NC, true> : k_udot_sweep<R, P, NC, false>;
     auto* k_sweep_g = small_tiles ? k_mass_sweep<R, P, 2 * NC, true> : k_mass_sweep<R, P, 2 * NC, false>;
@@ -221,23 +265,29 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         R* g = (R*)B.g;
         R* g2 = (R*)B.g2;
         R* bg = (R*)B.bg;
-        // the right-hand sides with their first sweeps in one kernel each
-        const bool fuse = !(pr.opts & OPT_UNFUSED_SWEEPS);
+        // the right-hand sides with their first sweeps in one kernel each; the
+        // float64 form on large tiles keeps the g_h pair apart (the sweep's
+        // halo costs it a fifth of the float64 operations of both, their
+        // traffic less)
+        const bool fuse = !(pr.opts & OPT_UNFUSED_SWEEPS), fuse_g = fuse && fuse_grad_sweep(sizeof(R), small_tiles);
         int k0 = 0;
-        if (fuse && pr.k_g >= 1) {
+        if (fuse_g && pr.k_g >= 1) {
+            auto* k_gradf = k_grad_sweep<R, P, NC, true>;
+            if constexpr (sizeof(R) == 4)
+                if (!small_tiles) k_gradf = k_grad_sweep<R, P, NC, false>;
             CGL_LAUNCH(prof, KID_GRADF, st,
-                       chk(launch(pdl, k_gradf, gt, bt, st, m, (const R*)u, pr.k_g > 1 ? bg : (R*)nullptr, g2)));
+                       chk(launch_shared(pdl, k_gradf, gth, bt, ws_grad, st, m, (const R*)u, pr.k_g > 1 ? bg : (R*)nullptr, g2)));
             R* t = g;
             g = g2;
             g2 = t;
             k0 = 1;
         } else {
             CGL_LAUNCH(prof, KID_GRAD, st,
-                       chk(launch(pdl, k_grad, gt, bt, st, m, (const R*)u, bg, g)));
+                       chk(launch_shared(pdl, k_grad, gt, bt, ws_rhs, st, m, (const R*)u, bg, g)));
         }
         for (int k = k0; k < pr.k_g; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch(pdl, k_sweep_g, gt, bt, st, m, (const R*)g, (const R*)bg, g2)));
+                       chk(launch_shared(pdl, k_sweep_g, gt, bt, ws_sweep, st, m, (const R*)g, (const R*)bg, g2)));
             R* t = g;
             g = g2;
             g2 = t;
@@ -258,7 +308,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         }
         int k1 = 0;
         if (fuse && pr.k_u >= 1) {
-            CGL_LAUNCH(prof, KID_UDOTF, st, chk(launch(pdl, k_udotf, gt, bt, st, m, (const R*)ER, r, ud2)));
+            CGL_LAUNCH(prof, KID_UDOTF, st, chk(launch_shared(pdl, k_udotf, gt, bt, ws_udot, st, m, (const R*)ER, r, ud2)));
             R* t = ud;
             ud = ud2;
             ud2 = t;
@@ -269,7 +319,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         }
         for (int k = k1; k < pr.k_u; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch(pdl, k_sweep_u, gt, bt, st, m, (const R*)ud, (const R*)r, ud2)));
+                       chk(launch_shared(pdl, k_sweep_u, gt, bt, ws_sweep, st, m, (const R*)ud, (const R*)r, ud2)));
             R* t = ud;
             ud = ud2;
             ud2 = t;
