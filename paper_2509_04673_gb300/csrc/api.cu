@@ -373,6 +373,30 @@ static void build_modal_tables(int p, Tab<double>& T, double* m2) {
         }
 }
 
+// weighted quadrature tables and the derivative of the basis in itself: phi_k'
+// = sum_i dn[i][k] phi_i.  Bernstein: the degree-(p-1) differences p (u_{i+1}
+// - u_i) raised to degree p, i (u_i - u_{i-1}) + (p - i) (u_{i+1} - u_i);
+// Lagrange: dn[i][k] = l_k'(x_i)
+static void build_point_tables(int p, bool lgl, Tab<double>& T) {
+    const int n = p + 1, nq = p + 2;
+    for (int q = 0; q < nq; ++q)
+        for (int a = 0; a < n; ++a) {
+            T.wB[q][a] = T.wq[q] * T.Bq[q][a];
+            T.wdB[q][a] = T.wq[q] * T.dBq[q][a];
+        }
+    for (int k = 0; k < n; ++k) {
+        double c[N1MAX], d[N1MAX];
+        if (lgl) {
+            lagrange_coeffs(p, T.xn, k, c);
+            poly_deriv(p, c, 1, d);
+        }
+        for (int i = 0; i < n; ++i) {
+            if (lgl) T.dn[i][k] = poly_eval(p, d, T.xn[i]);
+            else T.dn[i][k] = (k == i) ? 2.0 * i - p : (k == i - 1) ? -(double)i : (k == i + 1) ? (double)(p - i) : 0.0;
+        }
+    }
+}
+
 static void semi_norm_blocks(int p, std::vector<std::vector<double>>& S) {
     // S[k][a*(p+1)+b] = int B_a^(k) B_b^(k), with
     // B_a^(k) = p!/(p-k)! sum_j (-1)^(k-j) C(k,j) B^{p-k}_{a-j}
@@ -441,6 +465,7 @@ static void build_tables(HostTables& H) {
                                     S[k1][a * n + c] * S[k2][b * n + d];
             }
         build_modal_tables(p, T, H.m2d + off);
+        build_point_tables(p, false, T);
         // float copies
         Tab<float>& F = H.tf[p];
         const double* src = (const double*)&T;
@@ -451,6 +476,7 @@ static void build_tables(HostTables& H) {
     for (int p = 1; p <= PMAX; ++p) {
         build_lgl_tables(p, H.td[PMAX + 1 + p], H.a2d + A2_TOTAL + A2_OFF[p]);
         build_modal_tables(p, H.td[PMAX + 1 + p], H.m2d + A2_TOTAL + A2_OFF[p]);
+        build_point_tables(p, true, H.td[PMAX + 1 + p]);
     }
 }
 
@@ -756,7 +782,7 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
         {&B.bg, 2 * nc * NN * r},     {&B.r, nc * NN * r},         {&B.ud, nc * NN * r},
         {&B.EV, 16},                  {&B.ER, E * N2 * nc * r},    {&B.EW, E * N2 * nc * r},     {(void**)&B.q, 2 * E * r},
         {(void**)&B.ue, nc * E * 8},  {(void**)&B.cf, (1 + nc) * E * 4},  {(void**)&B.avg, 2 * nc * E * 4},
-        {(void**)&B.fht, nc * E * 4},
+        {&B.fht, nc * E * r},
         {(void**)&B.cq, (precision == CGL_FP32_MIXED && nc > 1) ? (2 * nc + 5) * E * 4 : 16},
         {(void**)&B.dte, 3 * E * 8},  {(void**)&B.fl, 4 * nc * E * r},      {(void**)&B.ubl, nc * E * 8}, {(void**)&B.gam, E * 8},
         {(void**)&B.nu, E * 8},       {(void**)&B.ube, nc * E * 8}, {(void**)&B.beta, E * 8},
@@ -1532,7 +1558,7 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     int64_t per_stage = 1 + 2 + (lo ? 0 : 3 + (S->prob.k_g + S->prob.k_u));
     if (S->nc > 1) per_stage += 1;                                // k_sens
     if (S->prec == CGL_FP32_MIXED && S->nc > 1) per_stage += 1;  // k_avg
-    if (S->prec == CGL_FP32_MIXED) per_stage += 1;                // k_facet
+    if (S->prec == CGL_FP32_MIXED || S->nc > 1) per_stage += 1;  // k_facet
     if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
     if (!lo && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
         // the first sweep of each solve runs inside k_grad_sweep / k_udot_sweep

@@ -150,6 +150,9 @@ struct Tab {
     // mode j > k of the lower neighbour in the continued mode k
     T mf[N1MAX][2];
     T mc[N1MAX][N1MAX];
+    T wB[NQMAX][N1MAX];    // wq B_a(x_q)
+    T wdB[NQMAX][N1MAX];   // wq B_a'(x_q)
+    T dn[N1MAX][N1MAX];    // [i][k]: coefficients i of phi_k' in the basis itself
 };
 
 // semi-norm matrices (n2 x n2 for p = 1..4) packed at offsets; on the device
@@ -195,9 +198,53 @@ DEV int a2_base(const MeshDev& m) {
     return is_lgl<R>(m) ? A2_TOTAL : 0;
 }
 
+// 1 / x of a density: the hardware's approximation (about 23 bits, 20 of a
+// float64) refined by Newton-Raphson, one step in float, one third-order step
+// in float64, to within a unit in the last place; unlike the IEEE division it
+// has no slow path, and in float64 it takes 3 instructions of GB300's narrow
+// pipe instead of about 10
+DEV float rcp_nr(float x) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_rn(r, __fmaf_rn(-x, r, 1.f), r);
+}
+DEV double rcp_nr(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+// a double that is 0 or infinite (integer tests: a float64 comparison runs on
+// the float64 pipe too)
+DEV bool is_zero_or_inf(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return hi == 0x7ff00000u || (hi | (unsigned)__double2loint(x)) == 0u;
+}
+DEV bool is_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
+DEV bool is_finite(float x) { return isfinite(x); }
+
+// sqrt of a squared speed or norm, x >= 0: in float the hardware's
+// approximation (within a unit in the last place, no slow path); in float64
+// the reciprocal square root's approximation y (20 bits) refined by one
+// third-order Newton-Raphson step: with d = 1 - x y^2, sqrt(x) = x y (1 + d/2
+// + 3 d^2/8 + O(d^3)), 5 float64 instructions
+DEV float root(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+DEV double root(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = __dmul_rn(x, y), d = __fma_rn(-t, y, 1.0);
+    const double s = __fma_rn(__dmul_rn(t, d), __fma_rn(0.375, d, 0.5), t);
+    return is_zero_or_inf(x) ? x : s;
+}
+
 // ---------------------------------------------------------------------------
 // physics policies. Each provides, for value type T:
-//   NC, flux(u, fx, fy), max_speed(uL, uR, nx, ny), node_speed(u)
+//   NC, flux(u, fx, fy), normal(u, axis, f) (f_x or f_y alone),
+//   max_speed(uL, uR, nx, ny), node_speed(u)
 // Speeds: Sec. 2.2 defers them to the literature; the readings are
 // advection |v.n|; Burgers max(|uL|,|uR|)|nx+ny|; KPP 1 (|f'(u).n| <= 1);
 // Euler the two-rarefaction upper bound of Guermond & Popov (2016).
@@ -209,6 +256,9 @@ struct PhysAdv {
     template <class T> static DEV void flux(const T* u, T* fx, T* fy, const ProbDev& pr) {
         fx[0] = PV<T>::vx(pr) * u[0];
         fy[0] = PV<T>::vy(pr) * u[0];
+    }
+    template <class T> static DEV void normal(const T* u, int axis, T* f, const ProbDev& pr) {
+        f[0] = (axis == 0 ? PV<T>::vx(pr) : PV<T>::vy(pr)) * u[0];
     }
     template <class T> static DEV T max_speed(const T*, const T*, T nx, T ny, const ProbDev& pr) {
         return fabs(PV<T>::vx(pr) * nx + PV<T>::vy(pr) * ny);
@@ -226,6 +276,7 @@ struct PhysBurgers {
         fx[0] = f;
         fy[0] = f;
     }
+    template <class T> static DEV void normal(const T* u, int, T* f, const ProbDev&) { f[0] = T(0.5) * u[0] * u[0]; }
     template <class T> static DEV T max_speed(const T* uL, const T* uR, T nx, T ny, const ProbDev&) {
         return fmax(fabs(uL[0]), fabs(uR[0])) * fabs(nx + ny);
     }
@@ -293,8 +344,16 @@ struct PhysKPP {
         if constexpr (sizeof(T) == 4) {
             kpp_sincos(u[0], fx[0], fy[0]);
         } else {
-            fx[0] = sin(u[0]);
-            fy[0] = cos(u[0]);
+            sincos(u[0], fx, fy);  // one argument reduction
+        }
+    }
+    template <class T> static DEV void normal(const T* u, int axis, T* f, const ProbDev&) {
+        if constexpr (sizeof(T) == 4) {
+            float s, c;
+            kpp_sincos(u[0], s, c);
+            f[0] = axis == 0 ? s : c;
+        } else {
+            f[0] = axis == 0 ? sin(u[0]) : cos(u[0]);
         }
     }
     template <class T> static DEV T max_speed(const T*, const T*, T, T, const ProbDev&) { return T(1); }
@@ -310,20 +369,10 @@ struct PhysEuler {
     template <class T> static DEV void flux(const T* u, T* fx, T* fy, const ProbDev& pr) {
         const T g = PV<T>::gam(pr);
         T rho = u[0], mx = u[1], my = u[2], E = u[3];
-        T vx, vy, p;
-        if constexpr (sizeof(T) == 4) {
-            // float: one correctly rounded reciprocal of rho instead of three
-            // divisions (the flux is evaluated at every quadrature point and
-            // face node of the float kernels)
-            const T r = __frcp_rn(rho);
-            vx = mx * r;
-            vy = my * r;
-            p = (g - T(1)) * (E - T(0.5) * (mx * vx + my * vy));
-        } else {
-            vx = mx / rho;
-            vy = my / rho;
-            p = (g - T(1)) * (E - T(0.5) * (mx * mx + my * my) / rho);
-        }
+        // one reciprocal of rho (the flux is evaluated at every quadrature
+        // point and face node)
+        const T r = rcp_nr(rho), vx = mx * r, vy = my * r;
+        const T p = (g - T(1)) * (E - T(0.5) * (mx * vx + my * vy));
         fx[0] = mx;
         fx[1] = mx * vx + p;
         fx[2] = my * vx;
@@ -332,6 +381,16 @@ struct PhysEuler {
         fy[1] = mx * vy;
         fy[2] = my * vy + p;
         fy[3] = (E + p) * vy;
+    }
+    template <class T> static DEV void normal(const T* u, int axis, T* f, const ProbDev& pr) {
+        const T g = PV<T>::gam(pr);
+        const T r = rcp_nr(u[0]), vx = u[1] * r, vy = u[2] * r;
+        const T p = (g - T(1)) * (u[3] - T(0.5) * (u[1] * vx + u[2] * vy));
+        const T v = axis == 0 ? vx : vy;
+        f[0] = axis == 0 ? u[1] : u[2];
+        f[1] = axis == 0 ? u[1] * vx + p : u[1] * vy;
+        f[2] = axis == 0 ? u[2] * vx : u[2] * vy + p;
+        f[3] = (u[3] + p) * v;
     }
     template <class T> static DEV T max_speed(const T* uL, const T* uR, T nx, T ny, const ProbDev& pr) {
         const T g = PV<T>::gam(pr);
@@ -381,16 +440,9 @@ struct PhysEuler {
     }
     template <class T> static DEV T node_speed(const T* u, const ProbDev& pr) {
         const T g = PV<T>::gam(pr);
-        if constexpr (sizeof(T) == 4) {
-            // float: one reciprocal of rho (nu_e takes the largest node speed)
-            const T r = __frcp_rn(u[0]);
-            const T vx = u[1] * r, vy = u[2] * r;
-            const T p = (g - T(1)) * (u[3] - T(0.5) * (u[1] * vx + u[2] * vy));
-            return sqrt(vx * vx + vy * vy) + sqrt(fmax(T(0), g * p * r));
-        } else {
-            T c = sqrt(fmax(T(0), g * pressure(u, g) / u[0]));
-            return hypot(u[1], u[2]) / u[0] + c;
-        }
+        const T r = rcp_nr(u[0]), vx = u[1] * r, vy = u[2] * r;
+        const T p = (g - T(1)) * (u[3] - T(0.5) * (u[1] * vx + u[2] * vy));
+        return root(vx * vx + vy * vy) + root(fmax(T(0), g * p * r));
     }
 };
 

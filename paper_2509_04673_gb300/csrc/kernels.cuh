@@ -944,8 +944,11 @@ DEV double pre_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, 
                 // (s/4)(umin - ubar^{e,L}) <= 0
                 q_out[e] = fmax(0.0, (0.25 * s) * (pr.umax - bl));
                 q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
+            } else {
+                cf_out[(1 + c) * m.E + e] = (float)bl;  // for the certificate of the facet limiter
             }
         }
+        if (NC > 1) cf_out[e] = (float)s;
         if constexpr (NC == 1) {  // systems: k_sens
             double gam;
             if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
@@ -1383,14 +1386,13 @@ DEV NodeCands node_cands(const MeshDev& m, int gx, int gy) {
 // boundary-face part of the weak form of element (ex, ey) on face d: the
 // (p+2)-point quadrature of phi_i F(u_h, u_hat; n), u_hat of the side at
 // each Gauss point, or of phi_i f(u_h).n on a side that is OUTFLOW
-// everywhere; scaled by h; Uf and term are [NC][p+1]
+// everywhere; per unit of h; Uf and term are [NC][p+1]
 template <class R, int P, class Ph>
 __device__ __noinline__ void boundary_face_term(const MeshDev& m, const ProbDev& pr, int d, int ex, int ey,
                                                 const R* Uf, R* term) {
     constexpr int NC = Ph::NC, N1 = P + 1, NQ = Dim<P>::NQ;
     const Tab<R>& T = tab_of<R>(m, P);
     const Tab<double>& Td = tab_of<double>(m, P);
-    const R h = PV<R>::h(m);
     const R nxo = (d == 0) ? R(-1) : (d == 1) ? R(1) : R(0);
     const R nyo = (d == 2) ? R(-1) : (d == 3) ? R(1) : R(0);
     const bool plain = side_plain(pr, d);
@@ -1433,191 +1435,206 @@ __device__ __noinline__ void boundary_face_term(const MeshDev& m, const ProbDev&
 #pragma unroll
         for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int b = 0; b < N1; ++b) acc[c][b] += (F[c] * T.wq[r]) * T.Bq[r][b];
+            for (int b = 0; b < N1; ++b) acc[c][b] += F[c] * T.wB[r][b];
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
-        for (int b = 0; b < N1; ++b) term[c * N1 + b] = acc[c][b] * h;
+        for (int b = 0; b < N1; ++b) term[c * N1 + b] = acc[c][b];
 }
 
-// Galerkin part W^e of the element residual: volume and face terms of the
-// weak form (needs only u)
+// local node k of face d (W, E, S, N)
+template <int P>
+DEV constexpr int face_node(int d, int k) {
+    return d == 0 ? k * (P + 1) : d == 1 ? k * (P + 1) + P : d == 2 ? k : P * (P + 1) + k;
+}
+
+// volume integral of one component from its fluxes at the quadrature points
+// of row q2 (fx(q1), fy(q1)), added to W (per unit of h): the weights are
+// folded into the tables
+template <class R, int P, class FX, class FY>
+DEV void volume_row(const Tab<R>& T, int q2, const FX& fx, const FY& fy, R (&W)[Dim<P>::N2]) {
+    constexpr int N1 = P + 1, NQ = P + 2;
+    R Tx[N1], Ty[N1];
+#pragma unroll
+    for (int a = 0; a < N1; ++a) Tx[a] = Ty[a] = R(0);
+#pragma unroll
+    for (int q1 = 0; q1 < NQ; ++q1) {
+        const R x = fx(q1), y = fy(q1);
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+            Tx[a] += T.wdB[q1][a] * x;
+            Ty[a] += T.wB[q1][a] * y;
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < N1; ++b)
+#pragma unroll
+        for (int a = 0; a < N1; ++a) W[b * N1 + a] += T.wB[q2][b] * Tx[a] + T.wdB[q2][b] * Ty[a];
+}
+
+// Galerkin part W^e of the element residual of a scalar: volume and face terms
+// of the weak form (needs only u)
 template <class R, int P, class Ph>
-DEV void w_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Dim<P>::N2], int ex, int ey,
-                R (&W)[Ph::NC][Dim<P>::N2]) {
-    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, NQ = Dim<P>::NQ;
+DEV void w_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Dim<P>::N2], int ex, int ey, R (&W)[Dim<P>::N2]) {
+    constexpr int N1 = P + 1, N2 = Dim<P>::N2, NQ = Dim<P>::NQ;
+    static_assert(Ph::NC == 1, "systems: k_res_sys");
     const Tab<R>& T = tab_of<R>(m, P);
-    const R h = PV<R>::h(m);
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int i = 0; i < N2; ++i) W[c][i] = R(0);
+    for (int i = 0; i < N2; ++i) W[i] = R(0);
     // volume term: interpolate along x first
-    R X[NC][N1][NQ];
+    R X[N1][NQ];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int d = 0; d < N1; ++d)
-#pragma unroll
-            for (int q1 = 0; q1 < NQ; ++q1) {
-                R s = R(0);
-#pragma unroll
-                for (int a = 0; a < N1; ++a) s += T.Bq[q1][a] * U[c][d * N1 + a];
-                X[c][d][q1] = s;
-            }
-#pragma unroll 1
-    for (int q2 = 0; q2 < NQ; ++q2) {
-        R Tx[NC][N1], Ty[NC][N1];
-#pragma unroll
-        for (int c = 0; c < NC; ++c)
-#pragma unroll
-            for (int a = 0; a < N1; ++a) Tx[c][a] = Ty[c][a] = R(0);
+    for (int d = 0; d < N1; ++d)
 #pragma unroll
         for (int q1 = 0; q1 < NQ; ++q1) {
-            R uq[NC], fx[NC], fy[NC];
+            R s = R(0);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                R s = R(0);
-#pragma unroll
-                for (int d = 0; d < N1; ++d) s += T.Bq[q2][d] * X[c][d][q1];
-                uq[c] = s;
-            }
-            Ph::template flux<R>(uq, fx, fy, pr);
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-#pragma unroll
-                for (int a = 0; a < N1; ++a) {
-                    Tx[c][a] += T.wq[q1] * T.dBq[q1][a] * fx[c];
-                    Ty[c][a] += T.wq[q1] * T.Bq[q1][a] * fy[c];
-                }
+            for (int a = 0; a < N1; ++a) s += T.Bq[q1][a] * U[d * N1 + a];
+            X[d][q1] = s;
         }
-        const R hw = h * T.wq[q2];
+#pragma unroll 1
+    for (int q2 = 0; q2 < NQ; ++q2) {
+        R fx[NQ], fy[NQ];
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+        for (int q1 = 0; q1 < NQ; ++q1) {
+            R s = R(0);
 #pragma unroll
-            for (int b = 0; b < N1; ++b)
-#pragma unroll
-                for (int a = 0; a < N1; ++a)
-                    W[c][b * N1 + a] += hw * (T.Bq[q2][b] * Tx[c][a] + T.dBq[q2][b] * Ty[c][a]);
+            for (int d = 0; d < N1; ++d) s += T.Bq[q2][d] * X[d][q1];
+            Ph::template flux<R>(&s, &fx[q1], &fy[q1], pr);
+        }
+        volume_row<R, P>(T, q2, [&](int q) { return fx[q]; }, [&](int q) { return fy[q]; }, W);
     }
     // face terms
-    int nb[4];
-#pragma unroll
-    for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
-        const R nxo = (d == 0) ? R(-1) : (d == 1) ? R(1) : R(0);
-        const R nyo = (d == 2) ? R(-1) : (d == 3) ? R(1) : R(0);
-        R Uf[NC][N1];
+        R Uf[N1], term[N1];
 #pragma unroll
-        for (int k = 0; k < N1; ++k) {
-            int li = (d == 0) ? k * N1 : (d == 1) ? k * N1 + P : (d == 2) ? k : P * N1 + k;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) Uf[c][k] = U[c][li];
-        }
-        R term[NC][N1];
-        if (nb[d] >= 0) {
-            R fn[NC][N1];
+        for (int k = 0; k < N1; ++k) Uf[k] = U[face_node<P>(d, k)];
+        if (neighbour(m, ex, ey, d) >= 0) {
+            R fn[N1];
 #pragma unroll
             for (int k = 0; k < N1; ++k) {
-                R uk[NC], fx[NC], fy[NC];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) uk[c] = Uf[c][k];
-                Ph::template flux<R>(uk, fx, fy, pr);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) fn[c][k] = fx[c] * nxo + fy[c] * nyo;
+                Ph::template normal<R>(&Uf[k], d >> 1, &fn[k], pr);
+                if ((d & 1) == 0) fn[k] = -fn[k];
             }
 #pragma unroll
-            for (int c = 0; c < NC; ++c)
+            for (int b = 0; b < N1; ++b) {
+                R s = R(0);
 #pragma unroll
-                for (int b = 0; b < N1; ++b) {
-                    R s = R(0);
-#pragma unroll
-                    for (int k = 0; k < N1; ++k) s += fn[c][k] * T.M[b][k];
-                    term[c][b] = h * s;
-                }
+                for (int k = 0; k < N1; ++k) s += fn[k] * T.M[b][k];
+                term[b] = s;
+            }
         } else {
             // a face on the domain boundary: out of line, so the common
             // interior path stays compact in the instruction cache
-            boundary_face_term<R, P, Ph>(m, pr, d, ex, ey, &Uf[0][0], &term[0][0]);
+            boundary_face_term<R, P, Ph>(m, pr, d, ex, ey, Uf, term);
         }
 #pragma unroll
-        for (int k = 0; k < N1; ++k) {
-            int li = (d == 0) ? k * N1 : (d == 1) ? k * N1 + P : (d == 2) ? k : P * N1 + k;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) W[c][li] -= term[c][k];
-        }
+        for (int k = 0; k < N1; ++k) W[face_node<P>(d, k)] -= term[k];
     }
-}
-
-// stabilisation s^e = nu_e (K u - gamma_e G g_h) and the residual
-// R^e = W^e - s^e into ER
-template <class R, int P, class Ph>
-DEV void stab_part(const MeshDev& m, const R (&U)[Ph::NC][Dim<P>::N2], const R* __restrict__ g,
-                   const double* __restrict__ gam, const double* __restrict__ nu, const R (&W)[Ph::NC][Dim<P>::N2],
-                   R* __restrict__ ER, int ex, int ey, int e) {
-    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2;
-    const Tab<R>& T = tab_of<R>(m, P);
     const R h = PV<R>::h(m);
-    // stabilisation s = nu (K u - gamma (Gx gx + Gy gy))
-    const R nue = R(nu[e]), ge = R(gam[e]);
-#pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
-        R GX[N2], GY[N2];
-        load_comp<R, P>(g + c * m.NN, m, ex, ey, GX);
-        load_comp<R, P>(g + (NC + c) * m.NN, m, ex, ey, GY);
-        // x-direction products: D u, M u, C gx, M gy
-        R Du[N1][N1], Mu[N1][N1], Cg[N1][N1], Mg[N1][N1];
 #pragma unroll
-        for (int d = 0; d < N1; ++d)
+    for (int i = 0; i < N2; ++i) W[i] = mul_r(W[i], h);
+}
+
+// coefficients of h u_h' along a line
+template <class R, int P>
+DEV void deriv_line(const MeshDev& m, const Tab<R>& T, const R (&u)[P + 1], R (&d)[P + 1]) {
+    if (is_lgl<R>(m)) {
 #pragma unroll
-            for (int a = 0; a < N1; ++a) {
-                R s1 = R(0), s2 = R(0), s3 = R(0), s4 = R(0);
+        for (int i = 0; i <= P; ++i) {
+            R s = R(0);
 #pragma unroll
-                for (int k = 0; k < N1; ++k) {
-                    s1 += T.D[a][k] * U[c][d * N1 + k];
-                    s2 += T.M[a][k] * U[c][d * N1 + k];
-                    s3 += T.C[a][k] * GX[d * N1 + k];
-                    s4 += T.M[a][k] * GY[d * N1 + k];
-                }
-                Du[d][a] = s1;
-                Mu[d][a] = s2;
-                Cg[d][a] = s3;
-                Mg[d][a] = s4;
+            for (int k = 0; k <= P; ++k) s += T.dn[i][k] * u[k];
+            d[i] = s;
+        }
+        return;
+    }
+    // Bernstein: differences raised to degree p
+    R D[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) D[i] = u[i + 1] - u[i];
+#pragma unroll
+    for (int i = 0; i <= P; ++i)
+        d[i] = i == 0 ? R(P) * D[0] : i == P ? R(P) * D[P - 1] : R(i) * D[i - 1] + R(P - i) * D[i];
+}
+
+// stabilisation s^e = nu_e int grad phi_i . (grad u_h - gamma_e g_h) of one
+// component.  The integrand's coefficients w_d = h d_d u_h - gamma_e h g_d are
+// formed first (u_h' in the basis itself), so that one application of the
+// tensor operators C (x) M and M (x) C serves both terms: at p = 2 144
+// multiply-adds instead of the 234 of separate stiffness and gradient terms.
+template <class R, int P>
+DEV void stab_comp(const MeshDev& m, const Tab<R>& T, const R (&U)[Dim<P>::N2], const R (&GX)[Dim<P>::N2],
+                   const R (&GY)[Dim<P>::N2], R gh, R nue, R (&s)[Dim<P>::N2]) {
+    constexpr int N1 = P + 1;
+    R Z[N1][N1];
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+        // w along the direction's lines, then C along it
+#pragma unroll
+        for (int t = 0; t < N1; ++t) {
+            R l[N1], d[N1];
+#pragma unroll
+            for (int k = 0; k < N1; ++k) l[k] = U[dir == 0 ? t * N1 + k : k * N1 + t];
+            deriv_line<R, P>(m, T, l, d);
+#pragma unroll
+            for (int k = 0; k < N1; ++k) {
+                const int i = dir == 0 ? t * N1 + k : k * N1 + t;
+                d[k] -= gh * (dir == 0 ? GX[i] : GY[i]);
             }
 #pragma unroll
-        for (int b = 0; b < N1; ++b)
+            for (int a = 0; a < N1; ++a) {
+                R z = R(0);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) z += T.C[a][k] * d[k];
+                Z[t][a] = z;  // line t, index a along the direction
+            }
+        }
+        // M across the lines
+#pragma unroll
+        for (int t = 0; t < N1; ++t)
 #pragma unroll
             for (int a = 0; a < N1; ++a) {
-                R ku = R(0), gg = R(0);
+                R z = R(0);
 #pragma unroll
-                for (int d = 0; d < N1; ++d) {
-                    ku += T.M[b][d] * Du[d][a] + T.D[b][d] * Mu[d][a];
-                    gg += T.M[b][d] * Cg[d][a] + T.C[b][d] * Mg[d][a];
-                }
-                R s = nue * (ku - ge * (h * gg));
-                ER[ev_at(m.E, e, b * N1 + a, c, NC)] = W[c][b * N1 + a] - s;
+                for (int k = 0; k < N1; ++k) z += T.M[t][k] * Z[k][a];
+                const int i = dir == 0 ? t * N1 + a : a * N1 + t;
+                s[i] = dir == 0 ? z : mul_r(nue, add_r(s[i], z));
             }
     }
 }
 
-// Euler at p = 2: 3 blocks of 128 per SM (170-register cap; measured faster)
+// stabilisation and the residual R^e = W^e - s^e of a scalar into ER (W^e and
+// s^e rounded on their own, so that the residual in one kernel and in two
+// gives the same bits)
+template <class R, int P>
+DEV void stab_part(const MeshDev& m, const R (&U)[Dim<P>::N2], const R* __restrict__ g,
+                   const double* __restrict__ gam, const double* __restrict__ nu, const R (&W)[Dim<P>::N2],
+                   R* __restrict__ ER, int ex, int ey, int e) {
+    constexpr int N2 = Dim<P>::N2;
+    R GX[N2], GY[N2], s[N2];
+    load_comp<R, P>(g, m, ex, ey, GX);
+    load_comp<R, P>(g + m.NN, m, ex, ey, GY);
+    stab_comp<R, P>(m, tab_of<R>(m, P), U, GX, GY, R(gam[e]) * PV<R>::h(m), R(nu[e]), s);
+#pragma unroll
+    for (int i = 0; i < N2; ++i) ER[ev_at(m.E, e, i, 0, 1)] = sub_r(W[i], s[i]);
+}
 
 template <class R, int P, class Ph>
 DEV void res_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, const R* __restrict__ g,
                          const double* __restrict__ gam, const double* __restrict__ nu,
                          R* __restrict__ ER, int ex, int ey, int e) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    R U[NC][N2];
-    load_block<R, P, NC>(u, m, ex, ey, U);
-    R W[NC][N2];
+    constexpr int N2 = Dim<P>::N2;
+    R U[N2], W[N2];
+    load_comp<R, P>(u, m, ex, ey, U);
     w_part<R, P, Ph>(m, pr, U, ex, ey, W);
-    stab_part<R, P, Ph>(m, U, g, gam, nu, W, ER, ex, ey, e);
+    stab_part<R, P>(m, U, g, gam, nu, W, ER, ex, ey, e);
 }
 
 template <class R, int P, class Ph>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_RES)) k_res_ev(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ g,
+__global__ void __launch_bounds__(128) k_res_ev(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ g,
                          const double* __restrict__ gam, const double* __restrict__ nu,
                          R* __restrict__ ER) {
     pdl_begin();
@@ -1626,6 +1643,140 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_RES)
     res_at<R, P, Ph>(m, pr, u, g, gam, nu, ER, ex, ey, e);
 }
 
+// The residual of systems with one thread per element and component: a block
+// holds 32 elements of a row, a warp each component.  The threads interpolate
+// and integrate their own component; only the fluxes couple the components,
+// so the states at the quadrature points and the face nodes pass through
+// shared memory, where the block's warps share the points and leave the
+// fluxes in the states' place.  One thread per element held 4 (p+1)^2
+// coefficients and residuals at 128 registers with the rest in local memory
+// and 16 warps per SM.
+template <class R, int P, int NC>
+struct ResSys {
+    static constexpr int NQ = P + 2, QP = NQ * NQ, PTS = QP + 4 * P, TX = 32;  // quadrature points, then face nodes
+    static constexpr int points = PTS * 2 * NC * TX;    // [point][f_x, f_y][component][element]
+    static constexpr int faces = 4 * NC * (P + 1) * TX;  // boundary terms [face][component][node][element]
+    static constexpr int ws = points + faces;
+};
+// slot of node k of face d among the 4 p face nodes: the rows below and above,
+// then the sides between
+template <int P>
+DEV constexpr int face_slot(int d, int k) {
+    return d == 2 ? k
+                  : d == 3 ? P + 1 + k
+                           : k == 0 ? (d == 0 ? 0 : P)
+                                    : k == P ? P + 1 + (d == 0 ? 0 : P) : 2 * (P + 1) + 2 * (k - 1) + d;
+}
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 6 : P == 3 ? 4 : 3) : (P <= 2 ? 3 : 2))
+    k_res_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ g, const double* __restrict__ gam,
+              const double* __restrict__ nu, R* __restrict__ ER) {
+    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, NQ = Dim<P>::NQ, TX = 32, NF = 2 * NC;
+    using WS = ResSys<R, P, NC>;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    R(*sF)[NF][TX] = reinterpret_cast<R(*)[NF][TX]>(dyn_smem);
+    R(*sB)[NC * N1][TX] = reinterpret_cast<R(*)[NC * N1][TX]>(reinterpret_cast<R*>(dyn_smem) + WS::points);
+    pdl_begin();
+    const int tx = threadIdx.x, c = threadIdx.y;
+    const int ex = min(blockIdx.x * TX + tx, m.nx - 1), ey = blockIdx.y;  // a lane past the row repeats its last element
+    const int e = ey * m.nx + ex;
+    const Tab<R>& T = tab_of<R>(m, P);
+    R W[N2], s[N2];
+    {
+        R U[N2];
+        load_comp<R, P>(u + c * m.NN, m, ex, ey, U);
+        R X[N1][NQ];
+#pragma unroll
+        for (int d = 0; d < N1; ++d)
+#pragma unroll
+            for (int q1 = 0; q1 < NQ; ++q1) {
+                R v = R(0);
+#pragma unroll
+                for (int a = 0; a < N1; ++a) v += T.Bq[q1][a] * U[d * N1 + a];
+                X[d][q1] = v;
+            }
+#pragma unroll
+        for (int q2 = 0; q2 < NQ; ++q2)
+#pragma unroll
+            for (int q1 = 0; q1 < NQ; ++q1) {
+                R v = R(0);
+#pragma unroll
+                for (int d = 0; d < N1; ++d) v += T.Bq[q2][d] * X[d][q1];
+                sF[q2 * NQ + q1][c][tx] = v;
+            }
+#pragma unroll
+        for (int d = 0; d < 4; ++d)
+#pragma unroll
+            for (int k = 0; k < N1; ++k)
+                if (d >= 2 || (k > 0 && k < P)) sF[WS::QP + face_slot<P>(d, k)][c][tx] = U[face_node<P>(d, k)];
+        // the component's stabilisation needs no other
+        R GX[N2], GY[N2];
+        load_comp<R, P>(g + c * m.NN, m, ex, ey, GX);
+        load_comp<R, P>(g + (NC + c) * m.NN, m, ex, ey, GY);
+        stab_comp<R, P>(m, T, U, GX, GY, R(gam[e]) * PV<R>::h(m), R(nu[e]), s);
+    }
+    // terms on the domain boundary: warp c takes face c, all components
+    if (neighbour(m, ex, ey, c) < 0) {
+        R Uf[NC][N1], term[NC][N1];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const R* __restrict__ uk = u + k * m.NN;
+#pragma unroll
+            for (int j = 0; j < N1; ++j)
+                Uf[k][j] = uk[node_of(m, ex, ey, c == 0 ? 0 : c == 1 ? P : j, c == 2 ? 0 : c == 3 ? P : j)];
+        }
+        boundary_face_term<R, P, Ph>(m, pr, c, ex, ey, &Uf[0][0], &term[0][0]);
+#pragma unroll
+        for (int k = 0; k < NC; ++k)
+#pragma unroll
+            for (int j = 0; j < N1; ++j) sB[c][k * N1 + j][tx] = term[k][j];
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int pt = c; pt < WS::PTS; pt += NC) {
+        R uq[NC], fx[NC], fy[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) uq[k] = sF[pt][k][tx];
+        Ph::template flux<R>(uq, fx, fy, pr);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            sF[pt][k][tx] = fx[k];
+            sF[pt][NC + k][tx] = fy[k];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N2; ++i) W[i] = R(0);
+#pragma unroll
+    for (int q2 = 0; q2 < NQ; ++q2)
+        volume_row<R, P>(T, q2, [&](int q) { return sF[q2 * NQ + q][c][tx]; },
+                         [&](int q) { return sF[q2 * NQ + q][NC + c][tx]; }, W);
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        if (neighbour(m, ex, ey, d) >= 0) {
+            R fn[N1];
+#pragma unroll
+            for (int k = 0; k < N1; ++k) fn[k] = sF[WS::QP + face_slot<P>(d, k)][(d >> 1) * NC + c][tx];
+#pragma unroll
+            for (int b = 0; b < N1; ++b) {
+                R t = R(0);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) t += fn[k] * T.M[b][k];
+                W[face_node<P>(d, b)] += (d & 1) ? -t : t;
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < N1; ++b) W[face_node<P>(d, b)] -= sB[d][c * N1 + b][tx];
+        }
+    }
+    const R h = PV<R>::h(m);
+    if (blockIdx.x * TX + tx < m.nx) {
+        R* __restrict__ out = ER + ((long long)c * m.E + e);
+        const long long step = (long long)NC * m.E;
+#pragma unroll
+        for (int i = 0; i < N2; ++i, out += step) *out = h * W[i] - s[i];
+    }
+}
 
 // ---------------------------------------------------------------------------
 // k_update_ev: facet fluxes and flux limiter, ubar^e, f_i^e, beta_e and the
@@ -1748,7 +1899,7 @@ template <class R, int P, class Ph>
 DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Dim<P>::N2], const int (&nb)[4],
                     const double (&uec)[Ph::NC], const double (&ublc)[Ph::NC], double rs,
                     const double* __restrict__ dte_a, const double* __restrict__ ubl,
-                    const R* __restrict__ qcap, const R* __restrict__ fl_in, const float* __restrict__ cf, int e,
+                    const R* __restrict__ qcap, const R* __restrict__ fl_in, const float* cf, int e,
                     double (&ubec)[Ph::NC], R (&fh)[Ph::NC], double& rs_out,
                     unsigned long long* __restrict__ cnt) {
     constexpr int NC = Ph::NC, N1 = P + 1;
@@ -1788,24 +1939,24 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
 #pragma unroll
                 for (int k = 0; k < N1; ++k) {
                     const int li = (d == 0) ? k * N1 : (d == 1) ? k * N1 + P : (d == 2) ? k : P * N1 + k;
-                    R uk[NC], fx[NC], fy[NC];
+                    R uk[NC], fn[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) uk[c] = U[c][li];
-                    Ph::template flux<R>(uk, fx, fy, pr);
+                    Ph::template normal<R>(uk, d >> 1, fn, pr);
                     if (is_lgl<R>(m)) {
                         // LGL: the face mean weights node k by w_k
                         const R wk = R(c_tabd[PMAX + 1 + P].wl[k]);
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) acc[c] += wk * (fx[c] * cnx + fy[c] * cny);
+                        for (int c = 0; c < NC; ++c) acc[c] += wk * fn[c];
                     } else {
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) acc[c] += fx[c] * cnx + fy[c] * cny;
+                        for (int c = 0; c < NC; ++c) acc[c] += fn[c];
                     }
                 }
             }
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                const R a = is_lgl<R>(m) ? acc[c] : acc[c] / R(N1);
+                const R a = is_lgl<R>(m) ? acc[c] : mul_r(acc[c], R(1.0 / N1));
                 FHr[d][c] = fixed_b ? sg * a : a;
                 if constexpr (!mixed_sys) FH[d][c] = (double)FHr[d][c];
             }
@@ -1877,35 +2028,39 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                 double fA[NC];
 #pragma unroll
                 for (int c = 0; c < NC; ++c) fA[c] = (double)FLr[d][c] - (double)FHr[d][c];
-                if constexpr (sizeof(R) == 4) {
-                    // float32 certificate first: where both cells certainly
-                    // give alpha = 1 the float64 formula is skipped (same result)
-                    if (!(pr.opts & OPT_FP64_LIMITER)) {
-                        float fAf[NC], fAm[NC], ub[NC];
+                // float32 certificate first: where both cells certainly give
+                // alpha = 1 the float64 formula is skipped (same result; in
+                // the float64 form too, where it is 100 float64 instructions
+                // a facet against 4 conversions)
+                if (!(pr.opts & OPT_FP64_LIMITER)) {
+                    float fAf[NC], fAm[NC], ub[NC];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        fAf[c] = sizeof(R) == 4 ? __fsub_rn((float)FLr[d][c], (float)FHr[d][c]) : (float)fA[c];
+                        fAm[c] = -fAf[c];
+                    }
+                    bool one = true;
+                    if (Lc >= 0) {
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Lc];
+                        one = euler_alpha_is_one(ub, fAf, 0.25f * cf[Lc], pr.ome_f);
+                    }
+                    if (one && Rc >= 0) {
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Rc];
+                        one = euler_alpha_is_one(ub, fAm, 0.25f * cf[Rc], pr.ome_f);
+                    }
+                    if (one) {
 #pragma unroll
                         for (int c = 0; c < NC; ++c) {
-                            fAf[c] = __fsub_rn(FLr[d][c], FHr[d][c]);
-                            fAm[c] = -fAf[c];
-                        }
-                        bool one = true;
-                        if (Lc >= 0) {
-#pragma unroll
-                            for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Lc];
-                            one = euler_alpha_is_one(ub, fAf, 0.25f * cf[Lc], pr.ome_f);
-                        }
-                        if (one && Rc >= 0) {
-#pragma unroll
-                            for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Rc];
-                            one = euler_alpha_is_one(ub, fAm, 0.25f * cf[Rc], pr.ome_f);
-                        }
-                        if (one) {
-#pragma unroll
-                            for (int c = 0; c < NC; ++c) {
+                            if constexpr (mixed_sys) {
                                 TH[d][c] = FLr[d][c];
                                 TL[d][c] = -FHr[d][c];
+                            } else {
+                                FB[d][c] = fA[c];
                             }
-                            continue;
                         }
+                        continue;
                     }
                 }
                 double alpha = 1.0;
@@ -2354,25 +2509,25 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_UPD)
 }
 
 
-// FP32-mixed: the update in two kernels.  k_facet needs only u and the
-// outputs of k_pre, so it runs on a second stream beside the g_h and udot
-// kernels; k_update_el then reads its ubar^e and facet terms.  Together they
-// compute what k_update_ev computes, in the same arithmetic.  The bodies are
-// device functions of one element, also run by the batched stage.
-template <int P, class Ph>
-DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
+// The update in two kernels (FP32-mixed, and systems in both forms).  k_facet
+// needs only u and the outputs of k_pre, so in the FP32-mixed form it runs on
+// a second stream beside the g_h and udot kernels; k_update_el and k_upd_sys
+// then read its ubar^e and facet terms.  The scalar bodies are device
+// functions of one element, also run by the batched stage.
+template <class R, int P, class Ph>
+DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
                      const double* __restrict__ ue, double* dte_a, const double* __restrict__ ubl,
-                     const float* __restrict__ qcap, const float* __restrict__ fl_in, float* cf,
-                     double* __restrict__ ube_out, float* __restrict__ fht, unsigned long long* __restrict__ cnt,
+                     const R* __restrict__ qcap, const R* __restrict__ fl_in, float* cf,
+                     double* __restrict__ ube_out, R* __restrict__ fht, unsigned long long* __restrict__ cnt,
                      int ex, int ey, int e) {
     constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
     int nb[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-    float U[NC][N2];
-    load_block<float, P, NC>(u, m, ex, ey, U);
+    R U[NC][N2];
+    load_block<R, P, NC>(u, m, ex, ey, U);
     double uec[NC], ublc[NC], ubec[NC];
-    float fh[NC];
+    R fh[NC];
     const bool need_ue = pr.fl == FL_NONE;  // u^e enters ubar^e only without the flux limiter
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -2381,7 +2536,7 @@ DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const float* __restric
     }
     const double rs = dte_a[m.E + e];
     double rs2;
-    facet_part<float, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
+    facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         ube_out[c * m.E + e] = ubec[c];
@@ -2423,17 +2578,17 @@ DEV void update_el_at(const MeshDev& m, const ProbDev& pr, const float* __restri
                                e);
 }
 
-template <int P, class Ph>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_FACET)) k_facet(MeshDev m, ProbDev pr, const float* __restrict__ u,
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_FACET)) k_facet(MeshDev m, ProbDev pr, const R* __restrict__ u,
                                                const double* __restrict__ ue, double* dte_a,
-                                               const double* __restrict__ ubl, const float* __restrict__ qcap,
-                                               const float* __restrict__ fl_in, float* cf,
-                                               double* __restrict__ ube_out, float* __restrict__ fht,
+                                               const double* __restrict__ ubl, const R* __restrict__ qcap,
+                                               const R* __restrict__ fl_in, float* cf,
+                                               double* __restrict__ ube_out, R* __restrict__ fht,
                                                unsigned long long* __restrict__ cnt) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    facet_el_at<P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
+    facet_el_at<R, P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
 }
 
 template <int P, class Ph>
@@ -2449,6 +2604,145 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_UPD))
     update_el_at<P, Ph>(m, pr, u, ud, ER, cf, avg, ube, fht, dtp, EW, beta_out, cnt, ex, ey, e);
 }
 
+// The element part of the update of systems (f_i^e, the slope limiter beta_e,
+// the SSP increments) with one thread per element and component, as k_res_sys:
+// the contributions f_i^e pass through shared memory for the positivity
+// factors, which couple the components, the block's warps sharing the nodes.
+// One thread per element waited on its 27 loads a component one component
+// after the other, at 128 registers and 16 warps per SM.
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P == 3 ? 5 : 4) : (P <= 2 ? 4 : P == 3 ? 3 : 2))
+    k_upd_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ ud, const double* __restrict__ ue,
+              const double* __restrict__ dte_a, const R* __restrict__ ER, const float* __restrict__ cf,
+              const float* __restrict__ avg, const double* __restrict__ ube, const R* __restrict__ fht,
+              const double* __restrict__ dtp, R* __restrict__ EW, double* __restrict__ beta_out,
+              unsigned long long* __restrict__ cnt) {
+    constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, TX = 32;
+    __shared__ R sF[N2][NC][TX];
+    __shared__ double sU[NC][TX], sB[NC][TX];
+    pdl_begin();
+    const int tx = threadIdx.x, c = threadIdx.y;
+    const bool valid = blockIdx.x * TX + tx < m.nx;
+    const int ex = valid ? blockIdx.x * TX + tx : m.nx - 1, ey = blockIdx.y;  // a lane past the row repeats its last element
+    const int e = ey * m.nx + ex;
+    const Tab<R>& T = tab_of<R>(m, P);
+    // theta = dt / dt_e and dt_e; FP32-mixed: in float from the float speed sum
+    R thR, dteR;
+    if constexpr (sizeof(R) == 4) {
+        const float s = cf[e];
+        thR = __fmul_rn((float)*dtp, __fmul_rn(s, m.inv_h_f));
+        dteR = __fmul_rn(m.h_f, __frcp_rn(s));
+    } else {
+        thR = *dtp * dte_a[2 * m.E + e];
+        dteR = dte_a[e];
+    }
+    if (valid && c == 0 && thR > R(1)) atomicAdd(&cnt[CNT_CFL], 1ull);
+    const double ubd = ube[c * m.E + e];
+    R ubh, ubo;
+    split<R>(ubd, ubh, ubo);
+    R U[N2], F[N2];
+    load_comp<R, P>(u + c * m.NN, m, ex, ey, U);
+    if (pr.mode == MODE_LO) {
+        if (!valid) return;
+#pragma unroll
+        for (int i = 0; i < N2; ++i) EW[ev_at(m.E, e, i, c, NC)] = thR * ((ubh - U[i]) + ubo);
+        if (c == 0) beta_out[e] = 0.0;
+        return;
+    }
+    // f_i^e, eq. (aec) with eq. (aecb) folded into the residual
+    const R meR = PV<R>::me(m), h2 = PV<R>::h2(m), inv_meR = PV<R>::inv_me(m);
+    const bool lgl = is_lgl<R>(m);
+    const Tab<double>& TL = c_tabd[PMAX + 1 + P];
+    {
+        R UD[N2];
+        load_comp<R, P>(ud + c * m.NN, m, ex, ey, UD);
+        const R* __restrict__ r = ER + ((long long)c * m.E + e);
+#pragma unroll
+        for (int i = 0; i < N2; ++i) F[i] = r[(long long)(i * NC) * m.E];
+        R ueh, uel;
+        if constexpr (sizeof(R) == 4) {
+            ueh = avg[(2 * c) * m.E + e];
+            uel = avg[(2 * c + 1) * m.E + e];
+        } else {
+            split<R>(ue[c * m.E + e], ueh, uel);
+        }
+        const R fh = fht[c * m.E + e];
+        R Y[N1][N1];
+#pragma unroll
+        for (int d = 0; d < N1; ++d)
+#pragma unroll
+            for (int a = 0; a < N1; ++a) {
+                R s = R(0);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) s += T.M[a][k] * UD[d * N1 + k];
+                Y[d][a] = s;
+            }
+#pragma unroll
+        for (int b = 0; b < N1; ++b)
+#pragma unroll
+            for (int a = 0; a < N1; ++a) {
+                R s = R(0);
+#pragma unroll
+                for (int d = 0; d < N1; ++d) s += T.M[b][d] * Y[d][a];
+                const int i = b * N1 + a;
+                const R dev = (U[i] - ueh) - uel;
+                if (lgl) {
+                    const R w2 = R(TL.wl[a] * TL.wl[b]);
+                    const R mi = h2 * w2;
+                    F[i] = mi * dev + dteR * (((F[i] + fh * w2) - h2 * s) + mi * UD[i]);
+                } else {
+                    F[i] = meR * dev + dteR * (((F[i] + fh) - h2 * s) + meR * UD[i]);
+                }
+            }
+    }
+    R beta = R(1);
+    if (pr.mode == MODE_WENO_L) {
+#pragma unroll
+        for (int i = 0; i < N2; ++i) sF[i][c][tx] = F[i];
+        sU[c][tx] = ubd;
+        __syncthreads();
+        double ub[NC], b = 1.0;
+        float ubf[NC];
+        const bool cert = !(pr.opts & OPT_FP64_LIMITER);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            ub[k] = sU[k][tx];
+            ubf[k] = (float)ub[k];
+        }
+#pragma unroll 1
+        for (int i = c; i < N2; i += NC) {
+            // float32 certificate first; the float64 formula only where it
+            // cannot show alpha_i = 1 (min(b, 1) = b: same result)
+            if (cert) {
+                float ff[NC];
+#pragma unroll
+                for (int k = 0; k < NC; ++k) ff[k] = (float)sF[i][k][tx];
+                float mi = m.me_f;
+                if (lgl) mi = (float)(m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]));
+                if (euler_alpha_is_one(ubf, ff, mi, pr.ome_f)) continue;
+            }
+            double f[NC];
+#pragma unroll
+            for (int k = 0; k < NC; ++k) f[k] = (double)sF[i][k][tx];
+            const double mi = lgl ? m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]) : m.me;
+            b = fmin(b, euler_alpha_rare(ub, f, mi, pr.pos_eps));
+        }
+        sB[c][tx] = b;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NC; ++k) b = fmin(b, sB[k][tx]);
+        beta = R(b);
+    }
+    if (!valid) return;
+    if (c == 0) beta_out[e] = (double)beta;
+    R* __restrict__ out = EW + ((long long)c * m.E + e);
+#pragma unroll
+    for (int i = 0; i < N2; ++i) {
+        const R inv_mi = lgl ? R(m.inv_h2 * (TL.iwl[i % N1] * TL.iwl[i / N1])) : inv_meR;
+        out[(long long)(i * NC) * m.E] = thR * (((ubh - U[i]) + ubo) + (beta * F[i]) * inv_mi);
+    }
+}
+
 // FP32-mixed: the residual in two kernels.  k_res_w (the Galerkin part W^e,
 // needs only u) runs on the second stream from the start of the stage,
 // beside k_pre and the g_h kernels; k_res_s adds the stabilisation, which
@@ -2457,28 +2751,24 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_UPD))
 template <int P, class Ph>
 DEV void res_w_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u, float* __restrict__ WV, int ex,
                   int ey, int e) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    float U[NC][N2], W[NC][N2];
-    load_block<float, P, NC>(u, m, ex, ey, U);
+    constexpr int N2 = Dim<P>::N2;
+    float U[N2], W[N2];
+    load_comp<float, P>(u, m, ex, ey, U);
     w_part<float, P, Ph>(m, pr, U, ex, ey, W);
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int i = 0; i < N2; ++i) WV[ev_at(m.E, e, i, c, NC)] = W[c][i];
+    for (int i = 0; i < N2; ++i) WV[ev_at(m.E, e, i, 0, 1)] = W[i];
 }
 
-template <int P, class Ph>
+template <int P>
 DEV void res_s_at(const MeshDev& m, const float* __restrict__ u, const float* __restrict__ g,
                   const double* __restrict__ gam, const double* __restrict__ nu, const float* __restrict__ WV,
                   float* __restrict__ ER, int ex, int ey, int e) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    float U[NC][N2], W[NC][N2];
-    load_block<float, P, NC>(u, m, ex, ey, U);
+    constexpr int N2 = Dim<P>::N2;
+    float U[N2], W[N2];
+    load_comp<float, P>(u, m, ex, ey, U);
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int i = 0; i < N2; ++i) W[c][i] = WV[ev_at(m.E, e, i, c, NC)];
-    stab_part<float, P, Ph>(m, U, g, gam, nu, W, ER, ex, ey, e);
+    for (int i = 0; i < N2; ++i) W[i] = WV[ev_at(m.E, e, i, 0, 1)];
+    stab_part<float, P>(m, U, g, gam, nu, W, ER, ex, ey, e);
 }
 
 template <int P, class Ph>
@@ -2490,14 +2780,14 @@ __global__ void __launch_bounds__(128) k_res_w(MeshDev m, ProbDev pr, const floa
     res_w_at<P, Ph>(m, pr, u, WV, ex, ey, e);
 }
 
-template <int P, class Ph>
+template <int P>
 __global__ void __launch_bounds__(128) k_res_s(MeshDev m, const float* __restrict__ u, const float* __restrict__ g,
                                                const double* __restrict__ gam, const double* __restrict__ nu,
                                                const float* __restrict__ WV, float* __restrict__ ER) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    res_s_at<P, Ph>(m, u, g, gam, nu, WV, ER, ex, ey, e);
+    res_s_at<P>(m, u, g, gam, nu, WV, ER, ex, ey, e);
 }
 
 // ---------------------------------------------------------------------------
@@ -2514,7 +2804,6 @@ __global__ void __launch_bounds__(128) k_res_s(MeshDev m, const float* __restric
 // 3.1 2^-24 A, A = |rho E| + kin, so t > 2^-21 A certifies it; A is kept in
 // [2^-100, 2^100] (no underflow or overflow in the products).  Otherwise
 // (near-vacuum or near-zero pressure states, NaN) the float64 check decides.
-// Float64 states never take this path.
 template <class R>
 DEV bool euler_positive_certified(const R* u) {
     if constexpr (sizeof(R) == 4) {
@@ -2525,7 +2814,14 @@ DEV bool euler_positive_certified(const R* u) {
         const float A = __fadd_rn(fabsf(__fmul_rn(rho, E)), kin);
         return t > 0x1p-21f * A && A > 0x1p-100f && A < 0x1p100f;
     } else {
-        return false;
+        // the same in float64: t differs from the exact value by at most about
+        // 3.1 2^-53 (rho E + kin), and kin < rho E where t > 0, so t > 2^-40 rho
+        // E certifies it; integer tests of the high words (rho and the
+        // difference positive and finite, rho E away from under- and overflow)
+        const double A = __dmul_rn(u[0], u[3]);
+        const double t = __fma_rn(u[0], u[3], -(0.5 * __fma_rn(u[1], u[1], __dmul_rn(u[2], u[2]))));
+        const int hr = __double2hiint(u[0]), ha = __double2hiint(A), hd = __double2hiint(__fma_rn(-0x1p-40, A, t));
+        return hr > 0 && hr < 0x7ff00000 && ha > (123 << 20) && ha < (1923 << 20) && hd > 0 && hd < 0x7ff00000;
     }
 }
 
@@ -2549,7 +2845,7 @@ DEV void final_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ EW,
             out[c] = b * ufe;
             un[c * m.NN + node] = uold;  // first stage: keep u^n for the later stages
         }
-        bad |= !isfinite(out[c]);
+        bad |= !is_finite(out[c]);
     }
     if (bad) atomicAdd(&cnt[CNT_NONFINITE], 1ull);
     if (NC == 1) {

@@ -44,21 +44,15 @@ DEV double sub_r(double a, double b) { return __dsub_rn(a, b); }
 static __device__ __noinline__ float pow_rare(float x, float e) { return powf(x, e); }
 static __device__ __noinline__ double pow_rare(double x, double e) { return pow(x, e); }
 
-// 1 / x and sqrt(x) of a weight or norm: float by the hardware's approximations
-// (within one unit in the last place; 1/x of an infinite or zero norm and
-// sqrt(0) come out as in the exact operation), float64 as the operators
+// 1 / x of a weight: float by the hardware's approximation (within one unit in
+// the last place), float64 by rcp_nr; an infinite norm gives 0, as the exact
+// operation does (x > 0 otherwise)
 DEV float recip(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-DEV double recip(double x) { return 1.0 / x; }
-DEV float root(float x) {
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-DEV double root(double x) { return sqrt(x); }
+DEV double recip(double x) { return is_zero_or_inf(x) ? 0.0 : rcp_nr(x); }
 
 // modal coefficients of one line
 template <class R, int P>

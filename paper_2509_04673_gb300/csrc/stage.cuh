@@ -24,7 +24,7 @@ struct Bufs {
     float* cf;    // float copies for the Euler limiter certificate [1+NC][E]: s, ubar^{e,L}
     float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_pre for scalars)
     float* cq;    // FP32-mixed systems: flux of the mean and speed parts per cell [2NC + 5][E] (k_avg)
-    float* fht;   // facet terms of f_i^e [NC][E] (FP32-mixed, k_facet -> k_update_el)
+    void* fht;    // facet terms of f_i^e [NC][E]  (R) (k_facet -> k_update_el, k_upd_sys)
     cudaStream_t st2;            // second stream of a stage (k_facet)
     cudaEvent_t ev_fork0, ev_fork, ev_w, ev_join;
     double *ue, *dte, *ubl, *gam, *nu, *ube, *beta;
@@ -185,7 +185,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     if (split_res && !dt_only && pr.mode != MODE_LO) {
         chk(cudaEventRecord(B.ev_fork0, st));
         chk(cudaStreamWaitEvent(s2, B.ev_fork0, 0));
-        if constexpr (split)
+        if constexpr (split && NC == 1)
             CGL_LAUNCH(prof, KID_RESW, s2,
                        chk(launch(false, k_res_w<P, Ph>, ge, be, s2, m, pr, (const float*)u, (float*)B.EW)));
         chk(cudaEventRecord(B.ev_w, s2));
@@ -228,9 +228,9 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
                 chk(cudaEventRecord(B.ev_w, s2));
             }
             CGL_LAUNCH(prof, KID_FACET, s2,
-                       chk(launch(false, k_facet<P, Ph>, ge, be, s2, m, pr, (const float*)u, (const double*)B.ue,
+                       chk(launch(false, k_facet<float, P, Ph>, ge, be, s2, m, pr, (const float*)u, (const double*)B.ue,
                                   B.dte, (const double*)B.ubl, (const float*)B.q, (const float*)B.fl, B.cf, B.ube,
-                                  B.fht, B.cnt)));
+                                  (float*)B.fht, B.cnt)));
             chk(cudaEventRecord(B.ev_join, s2));
         }
     }
@@ -240,6 +240,12 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         if (!split || q1)
             CGL_LAUNCH(prof, KID_SENS, st,
                        chk(launch(pdl, k_sens<R, P, Ph, STY>, gs, bs, st, m, pr, (const R*)u, B.gam, B.nu)));
+        if constexpr (!split_update)
+            if (!q1)
+                CGL_LAUNCH(prof, KID_FACET, st,
+                           chk(launch(pdl, k_facet<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const double*)B.ue,
+                                      B.dte, (const double*)B.ubl, (const R*)B.q, (const R*)B.fl, B.cf, B.ube,
+                                      (R*)B.fht, B.cnt)));
     }
     if (q1) {
         CGL_LAUNCH(prof, KID_Q1F, st,
@@ -295,13 +301,19 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         R* ER = (R*)B.ER;
         R* r = (R*)B.r;
         R* ud2 = (R*)B.ud2;
-        if (split_res) {
-            chk(cudaStreamWaitEvent(st, B.ev_w, 0));
-            CGL_LAUNCH(prof, KID_RES, st,
-                       chk(launch(pdl, k_res_s<P, Ph>, ge, be, st, m, (const float*)u, (const float*)g,
-                                  (const double*)B.gam, (const double*)B.nu, (const float*)B.EW, (float*)ER)));
-        } else {
+        if constexpr (NC > 1) {
             if constexpr (use_avg) chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e, nu_e of k_sens
+            const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
+            CGL_LAUNCH(prof, KID_RES, st,
+                       chk(launch_shared(pdl, k_res_sys<R, P, Ph>, grs, brs, (int)sizeof(R) * ResSys<R, P, NC>::ws, st, m,
+                                         pr, (const R*)u, (const R*)g, (const double*)B.gam, (const double*)B.nu, ER)));
+        } else if (split_res) {
+            chk(cudaStreamWaitEvent(st, B.ev_w, 0));
+            if constexpr (split)
+                CGL_LAUNCH(prof, KID_RES, st,
+                           chk(launch(pdl, k_res_s<P>, ge, be, st, m, (const float*)u, (const float*)g,
+                                      (const double*)B.gam, (const double*)B.nu, (const float*)B.EW, (float*)ER)));
+        } else {
             CGL_LAUNCH(prof, KID_RES, st,
                        chk(launch(pdl, k_res_ev<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)g,
                                   (const double*)B.gam, (const double*)B.nu, ER)));
@@ -325,8 +337,15 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
             ud2 = t;
         }
     }
-    if constexpr (split_update) {
-        chk(cudaStreamWaitEvent(st, B.ev_join, 0));
+    if constexpr (split_update) chk(cudaStreamWaitEvent(st, B.ev_join, 0));
+    if constexpr (NC > 1) {
+        const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
+        CGL_LAUNCH(prof, KID_UPDATE, st,
+                   chk(launch(pdl, k_upd_sys<R, P, Ph>, grs, brs, st, m, pr, (const R*)u, (const R*)ud,
+                              (const double*)B.ue, (const double*)B.dte, (const R*)B.ER, (const float*)B.cf,
+                              (const float*)B.avg, (const double*)B.ube, (const R*)B.fht, (const double*)B.dt,
+                              (R*)B.EW, B.beta, B.cnt)));
+    } else if constexpr (split_update) {
         CGL_LAUNCH(prof, KID_UPDATE, st,
                    chk(launch(pdl, k_update_el<P, Ph>, ge, be, st, m, pr, (const float*)u, (const float*)ud,
                               (const double*)B.ue, (const double*)B.dte, (const float*)B.ER, (const float*)B.cf,
