@@ -783,7 +783,7 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
         {&B.EV, 16},                  {&B.ER, E * N2 * nc * r},    {&B.EW, E * N2 * nc * r},     {(void**)&B.q, 2 * E * r},
         {(void**)&B.ue, nc * E * 8},  {(void**)&B.cf, (1 + nc) * E * 4},  {(void**)&B.avg, 2 * nc * E * 4},
         {&B.fht, nc * E * r},
-        {(void**)&B.cq, (precision == CGL_FP32_MIXED && nc > 1) ? (2 * nc + 5) * E * 4 : 16},
+        {&B.cq, nc > 1 ? (2 * nc + PhysEuler::NPART) * E * r : 16},
         {(void**)&B.dte, 3 * E * 8},  {(void**)&B.fl, 4 * nc * E * r},      {(void**)&B.ubl, nc * E * 8}, {(void**)&B.gam, E * 8},
         {(void**)&B.nu, E * 8},       {(void**)&B.ube, nc * E * 8}, {(void**)&B.beta, E * 8},
         {(void**)&B.cnt, CNT_N * 8},  {(void**)&B.dtbits, 8},      {(void**)&B.dt, 8},
@@ -1556,8 +1556,7 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
     const int lo = S->prob.mode == CGL_MODE_LO;
     int64_t per_stage = 1 + 2 + (lo ? 0 : 3 + (S->prob.k_g + S->prob.k_u));
-    if (S->nc > 1) per_stage += 1;                                // k_sens
-    if (S->prec == CGL_FP32_MIXED && S->nc > 1) per_stage += 1;  // k_avg
+    if (S->nc > 1) per_stage += 2;                                // k_avg, k_sens
     if (S->prec == CGL_FP32_MIXED || S->nc > 1) per_stage += 1;  // k_facet
     if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
     if (!lo && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
@@ -1566,8 +1565,8 @@ extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
         per_stage -= (S->prob.k_g >= 1 && fuse_grad_sweep(S->rsz, small)) + (S->prob.k_u >= 1);
     }
     if ((S->prob.options & CGL_OPT_AEC_Q1) && !lo) {
-        // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_sens for systems, k_avg for mixed ones)
-        per_stage = 5 + (S->nc > 1) + (S->prec == CGL_FP32_MIXED && S->nc > 1);
+        // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_avg, k_sens for systems)
+        per_stage = 5 + (S->nc > 1 ? 2 : 0);
     }
     *kernels = 3 * per_stage + 1;  // + dt finalisation; the time advance rides in the last k_final
     return CGL_OK;

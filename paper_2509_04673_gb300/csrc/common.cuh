@@ -223,6 +223,38 @@ DEV bool is_zero_or_inf(double x) {
 DEV bool is_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
 DEV bool is_finite(float x) { return isfinite(x); }
 
+// Conversions between float and float64 in integer arithmetic: the hardware's
+// run on the float64 pipe, 16 clocks a warp there, where they were half of the
+// float64 instructions of the FP32-mixed kernels.  widen is exact; narrow cuts
+// to 24 bits (exact for a widened float); split_ff gives a float pair hi + lo
+// that holds the leading 47 bits.  Zeros take the same path; subnormal,
+// infinite and out-of-range values the hardware's.
+DEV double widen(float f) {
+    const unsigned b = (unsigned)__float_as_int(f), e = b & 0x7f800000u;
+    if ((e == 0 && (b << 1) != 0) || e == 0x7f800000u) return (double)f;
+    const unsigned hi = (b & 0x80000000u) | (e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+DEV float narrow(double d) {
+    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x0fe00000u) return (a | l) == 0u ? __int_as_float((int)h) : __double2float_rz(d);
+    return __int_as_float((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
+}
+DEV void split_ff(double d, float& hi, float& lo) {
+    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
+    // 2^-74 <= |d| < 2^127, so that the unit of the low part is normal
+    if (a - 0x3b500000u >= 0x0c900000u) {
+        const bool zero = (a | l) == 0u;
+        hi = zero ? 0.f : __double2float_rz(d);
+        lo = zero ? 0.f : __double2float_rn(d - (double)hi);
+        return;
+    }
+    hi = __int_as_float((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
+    // the 29 bits left, in units of 2^(exponent - 52)
+    const float s = __int_as_float((int)((h & 0x80000000u) | (((a >> 20) - 896u - 52u) << 23)));
+    lo = __fmul_rn((float)(l & 0x1fffffffu), s);
+}
+
 // sqrt of a squared speed or norm, x >= 0: in float the hardware's
 // approximation (within a unit in the last place, no slow path); in float64
 // the reciprocal square root's approximation y (20 bits) refined by one
@@ -252,7 +284,6 @@ DEV double root(double x) {
 
 struct PhysAdv {
     static constexpr int NC = 1;
-    static constexpr int NPART_OR_1 = 1;
     template <class T> static DEV void flux(const T* u, T* fx, T* fy, const ProbDev& pr) {
         fx[0] = PV<T>::vx(pr) * u[0];
         fy[0] = PV<T>::vy(pr) * u[0];
@@ -270,7 +301,6 @@ struct PhysAdv {
 
 struct PhysBurgers {
     static constexpr int NC = 1;
-    static constexpr int NPART_OR_1 = 1;
     template <class T> static DEV void flux(const T* u, T* fx, T* fy, const ProbDev&) {
         T f = T(0.5) * u[0] * u[0];
         fx[0] = f;
@@ -339,7 +369,6 @@ HDEV void kpp_sincos(float x, float& s, float& c) {
 
 struct PhysKPP {
     static constexpr int NC = 1;
-    static constexpr int NPART_OR_1 = 1;
     template <class T> static DEV void flux(const T* u, T* fx, T* fy, const ProbDev&) {
         if constexpr (sizeof(T) == 4) {
             kpp_sincos(u[0], fx[0], fy[0]);
@@ -362,7 +391,7 @@ struct PhysKPP {
 
 struct PhysEuler {
     static constexpr int NC = 4;
-    static constexpr int NPART_OR_1 = 5;  // speed parts per cell (speed_parts)
+    static constexpr int NPART = 6;  // speed parts per cell (speed_parts)
     template <class T> static DEV T pressure(const T* u, T g) {
         return (g - T(1)) * (u[3] - T(0.5) * (u[1] * u[1] + u[2] * u[2]) / u[0]);
     }
@@ -409,34 +438,31 @@ struct PhysEuler {
         T lam3 = vR + aR * sqrt(T(1) + cg * fmax(T(0), (ptr - pR) / pR));
         return fmax(fabs(lam1), fabs(lam3));
     }
-    // max_speed split into its per-cell and per-facet parts (float, interior
-    // facets with normal +x or +y): the cell part holds v_x, v_y, p, the
-    // sound speed a = sqrt(g p / rho) and p^(-(g-1)/(2g)), formed with the
-    // operations max_speed applies to each state; the facet part completes
+    // max_speed split into its per-cell and per-facet parts (interior facets
+    // with normal +x or +y): the cell part holds v_x, v_y, p, the sound speed
+    // a = sqrt(g p / rho), p^(-(g-1)/(2g)) and 1/p; the facet part completes
     // the two-rarefaction bound from the parts of the left and right cells
     // along axis 0 (x) or 1 (y)
-    static DEV void speed_parts(const float* u, float g, float* q) {
-        const float rho = u[0];
-        q[0] = (u[1] * 1.f + u[2] * 0.f) / rho;
-        q[1] = (u[1] * 0.f + u[2] * 1.f) / rho;
-        const float p = pressure(u, g);
+    template <class T> static DEV void speed_parts(const T* u, T g, T* q) {
+        const T r = rcp_nr(u[0]);
+        q[0] = u[1] * r;
+        q[1] = u[2] * r;
+        const T p = (g - T(1)) * (u[3] - T(0.5) * (u[1] * q[0] + u[2] * q[1]));
         q[2] = p;
-        q[3] = sqrt(g * p / rho);
-        const float expo = (g - 1.f) / (2.f * g);
-        q[4] = pow(p, -expo);
+        q[3] = root(g * p * r);
+        q[4] = pow(p, -(g - T(1)) / (T(2) * g));
+        q[5] = rcp_nr(p);
     }
-    static DEV float facet_speed_parts(const float* L, const float* R, int axis, float g) {
-        const float vL = L[axis], vR = R[axis];
-        const float pL = L[2], pR = R[2], aL = L[3], aR = R[3];
-        const float expo = (g - 1.f) / (2.f * g);
-        const float num = aL + aR - 0.5f * (g - 1.f) * (vR - vL);
-        const float den = aL * L[4] + aR * R[4];
-        const float base = num > 0.f ? fmaxf(num, 0.f) / den : 0.f;
-        const float ptr = pow(base, 1.f / expo);
-        const float cg = (g + 1.f) / (2.f * g);
-        const float lam1 = vL - aL * sqrt(1.f + cg * fmaxf(0.f, (ptr - pL) / pL));
-        const float lam3 = vR + aR * sqrt(1.f + cg * fmaxf(0.f, (ptr - pR) / pR));
-        return fmaxf(fabsf(lam1), fabsf(lam3));
+    // vL .. iL: v along the axis, p, a, p^(-..), 1/p of the left cell
+    template <class T>
+    static DEV T facet_speed_parts(T vL, T pL, T aL, T wL, T iL, T vR, T pR, T aR, T wR, T iR, T g) {
+        const T num = aL + aR - T(0.5) * (g - T(1)) * (vR - vL);
+        const T base = num > T(0) ? num * rcp_nr(aL * wL + aR * wR) : T(0);
+        const T ptr = pow(base, (T(2) * g) / (g - T(1)));
+        const T cg = (g + T(1)) / (T(2) * g);
+        const T lam1 = vL - aL * root(T(1) + cg * fmax(T(0), (ptr - pL) * iL));
+        const T lam3 = vR + aR * root(T(1) + cg * fmax(T(0), (ptr - pR) * iR));
+        return fmax(fabs(lam1), fabs(lam3));
     }
     template <class T> static DEV T node_speed(const T* u, const ProbDev& pr) {
         const T g = PV<T>::gam(pr);
@@ -505,8 +531,8 @@ HDEV T euler_alpha(const T* ub, const T* f, T m, T eps) {
 // (ub, f) and 1 in (f, m), so the inputs are first scaled by exact powers of
 // two to rho, m in [1, 2); this changes neither sign.  Each T is then
 // evaluated in float together with A, the same expression with every
-// monomial in absolute value.  With n operations and k rounded inputs
-// (n + k < 40) the float error is below (n + k) 2^-24 A and the float64 one
+// monomial in absolute value.  With n operations and k inputs off by 2^-23
+// (n + 2k < 60) the float error is below (n + 2k) 2^-24 A and the float64 one
 // below (n + k) 2^-53 A.  Scaled values are required to be at most 2^40, so
 // an underflowed input or product (error <= 2^-150) is amplified to at most
 // 2^-109 and all of them together stay below 2^-100.  So T > 2^-16 A +

@@ -671,84 +671,101 @@ __device__ __noinline__ CompVec<float, Ph::NC + 1> boundary_facet_lo(const MeshD
 
 // SUB: pseudo time steps from the subcell bound of Lemma 1 (a separate
 // instantiation, so that the default kernels carry none of its code).
-// LO (systems): the low-order part only: the element's own float-float mean
-// comes from k_avg like its neighbours' (the same ff_mean of the same block,
-// hence the same bits), no coefficient block is loaded, and gamma_e, nu_e
-// are left to k_sens
-template <int P, class Ph, bool SUB = false, bool LO = false>
+// What follows the four facets of an element in the FP32-mixed form: dt_e,
+// ubar^{e,L}, the flux-limiter capacities (scalars) or the float copies for
+// the limiter's certificate (systems), from the canonical facet fluxes F, the
+// speeds lam and the float-float mean
+template <int P, class Ph, bool SUB>
+DEV double lo_outputs_mixed(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u, const float (&lam)[4],
+                            const float (&F)[4][Ph::NC], const float (&uh)[Ph::NC], const float (&ul)[Ph::NC],
+                            double* __restrict__ ue_out, double* __restrict__ dte_out, double* __restrict__ ubl_out,
+                            float* __restrict__ q_out, float* __restrict__ fl_out, float* __restrict__ cf_out,
+                            float* __restrict__ avg, int ex, int ey, int e) {
+    constexpr int NC = Ph::NC;
+    float sf = __fadd_rn(__fadd_rn(__fadd_rn(lam[0], lam[1]), lam[2]), lam[3]);
+    sf = fmaxf(sf, pr.lambda_floor_f);
+    // dt_e / h = 1 / s: float reciprocal refined by one float64 Newton step
+    // (relative error ~2^-46, far inside the 2^-20 inflation of the speeds;
+    // GB300's float64 divide is a long sequence on its narrow float64 pipe)
+    double s, rs;
+    if constexpr (SUB) {
+        // Lemma 1 bound; the float speed sum is rounded up (a float dt_e no
+        // larger than the bound)
+        rs = subcell_dt<float, P, Ph>(u, m, pr, ex, ey) * m.inv_h;
+        s = 1.0 / rs;
+        sf = __double2float_ru(s);
+    } else {
+        s = widen(sf);
+        const double r0 = widen(__frcp_rn(sf));
+        rs = fma(r0, fma(-s, r0, 1.0), r0);
+    }
+    const double dte = m.h * rs;
+    dte_out[e] = dte;
+    dte_out[m.E + e] = rs;
+    dte_out[2 * m.E + e] = s * m.inv_h;
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = F[d][c];
+    const float s4 = 0.25f * sf;  // |K| / (|dK| dt_e), exact
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        // facet flux sum (F_E - F_W) + F_N - F_S as a float-float pair, widened once
+        float osh, osl;
+        ff_sum4(F[1][c], F[0][c], F[3][c], F[2][c], osh, osl);
+        const double ued = widen(uh[c]) + widen(ul[c]);
+        ue_out[c * m.E + e] = ued;
+        const double bl = ued - rs * (widen(osh) + widen(osl));
+        ubl_out[c * m.E + e] = bl;
+        if (NC == 1) {
+            // capacities (s/4)(umax - bl) >= 0 and (s/4)(umin - bl) <= 0: bound
+            // gaps in float64, both factors and the product rounded toward zero
+            // (smaller magnitudes stay admissible)
+            q_out[e] = __fmul_rz(s4, fmaxf(0.f, narrow(pr.umax - bl)));
+            q_out[m.E + e] = __fmul_rz(s4, fminf(0.f, narrow(pr.umin - bl)));
+            // the float-float mean, for the element contributions of k_update_ev
+            avg[e] = uh[0];
+            avg[m.E + e] = ul[0];
+        } else {
+            // float copies for the certificate of the facet limiter (euler_alpha_is_one)
+            cf_out[(1 + c) * m.E + e] = narrow(bl);
+        }
+    }
+    cf_out[e] = sf;  // the float speed sum (dt_e in float for k_update_ev)
+    return dte;
+}
+
+// FP32-mixed scalars, the whole of k_pre for one element (the batched stage
+// and k_pre)
+template <int P, class Ph, bool SUB = false>
 DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
                         double* __restrict__ ue_out, double* __restrict__ dte_out,
                         double* __restrict__ ubl_out, double* __restrict__ gam_out,
                         double* __restrict__ nu_out, float* __restrict__ q_out,
-                        float* __restrict__ fl_out, float* __restrict__ EV, float* __restrict__ cf_out,
-                        float* __restrict__ avg, int ex, int ey, int e, const float* __restrict__ cq = nullptr) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    static_assert(!LO || NC > 1, "the low-order-only form reads the means of k_avg (systems)");
+                        float* __restrict__ fl_out, float* __restrict__ cf_out,
+                        float* __restrict__ avg, int ex, int ey, int e) {
+    constexpr int NC = 1, N2 = Dim<P>::N2;
+    static_assert(Ph::NC == 1, "systems: k_lo_sys");
     int nb[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-    float U[LO ? 1 : NC][LO ? 1 : N2];
-    if constexpr (!LO) load_block<float, P, NC>(u, m, ex, ey, U);
-    float uh[NC], ul[NC], fxs[NC], fys[NC];
-    double ued[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        if constexpr (LO) {
-            uh[c] = avg[(2 * c) * m.E + e];
-            ul[c] = avg[(2 * c + 1) * m.E + e];
-        } else {
-            ff_mean<N2>(U[c], uh[c], ul[c]);
-        }
-        ued[c] = (double)uh[c] + (double)ul[c];
-        ue_out[c * m.E + e] = ued[c];
-    }
-    // LO: the fluxes of the means and the speed parts were formed by k_avg
-    constexpr int NQP = LO ? Ph::NPART_OR_1 : 1;
-    float qs[NQP], qn[4][NQP];
-    if constexpr (LO) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            fxs[c] = cq[c * m.E + e];
-            fys[c] = cq[(NC + c) * m.E + e];
-        }
-#pragma unroll
-        for (int k = 0; k < NQP; ++k) qs[k] = cq[(2 * NC + k) * m.E + e];
-    } else {
-        Ph::template flux<float>(uh, fxs, fys, pr);
-    }
-    // neighbours: means, fluxes (and, for scalars, the blocks for the sensor)
+    float U[N2], uh[NC], ul[NC], fxs[NC], fys[NC];
+    load_comp<float, P>(u, m, ex, ey, U);
+    ff_mean<N2>(U, uh[0], ul[0]);
+    Ph::template flux<float>(uh, fxs, fys, pr);
+    // neighbours: means and fluxes
     float oh[4][NC], ol[4][NC], ofx[4][NC], ofy[4][NC];
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
         if (nb[d] >= 0) {
-            if constexpr (NC > 1) {
-                // systems: the neighbours' float-float means from k_avg
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    oh[d][c] = avg[(2 * c) * m.E + nb[d]];
-                    ol[d][c] = avg[(2 * c + 1) * m.E + nb[d]];
-                }
-                if constexpr (LO) {
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        ofx[d][c] = cq[c * m.E + nb[d]];
-                        ofy[d][c] = cq[(NC + c) * m.E + nb[d]];
-                    }
-#pragma unroll
-                    for (int k = 0; k < NQP; ++k) qn[d][k] = cq[(2 * NC + k) * m.E + nb[d]];
-                }
-            } else {
-                int jx, jy;
-                neighbour_xy(m, ex, ey, d, jx, jy);
-                float B[NC][N2];
-                load_block<float, P, NC>(u, m, jx, jy, B);
-#pragma unroll
-                for (int c = 0; c < NC; ++c) ff_mean<N2>(B[c], oh[d][c], ol[d][c]);
-            }
-            if constexpr (!LO) Ph::template flux<float>(oh[d], ofx[d], ofy[d], pr);
+            int jx, jy;
+            neighbour_xy(m, ex, ey, d, jx, jy);
+            float B[N2];
+            load_comp<float, P>(u, m, jx, jy, B);
+            ff_mean<N2>(B, oh[d][0], ol[d][0]);
+            Ph::template flux<float>(oh[d], ofx[d], ofy[d], pr);
         } else {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) oh[d][c] = ol[d][c] = ofx[d][c] = ofy[d][c] = 0.f;
+            oh[d][0] = ol[d][0] = ofx[d][0] = ofy[d][0] = 0.f;
         }
     }
     // canonical facet fluxes F(u^L, u^R; n), n = +x (W, E) or +y (S, N)
@@ -766,248 +783,171 @@ DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __rest
             const float* Rl = self_is_L ? ol[d] : ul;
             const float* fL = xf ? (self_is_L ? fxs : ofx[d]) : (self_is_L ? fys : ofy[d]);
             const float* fR = xf ? (self_is_L ? ofx[d] : fxs) : (self_is_L ? ofy[d] : fys);
-            float ls;
-            if constexpr (LO) {
-                const float* qL = self_is_L ? qs : qn[d];
-                const float* qR = self_is_L ? qn[d] : qs;
-                ls = Ph::facet_speed_parts(qL, qR, xf ? 0 : 1, PV<float>::gam(pr));
-            } else {
-                ls = Ph::template max_speed<float>(Lh, Rh, cnx, cny, pr);
-            }
-            const float l = __fmul_rn(ls, inflate);
+            const float l = __fmul_rn(Ph::template max_speed<float>(Lh, Rh, cnx, cny, pr), inflate);
             lam[d] = l;
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-                F[d][c] = llf_value(fL[c], fR[c], l, ff_diff(Rh[c], Rl[c], Lh[c], Ll[c]));
+            F[d][0] = llf_value(fL[0], fR[0], l, ff_diff(Rh[0], Rl[0], Lh[0], Ll[0]));
         } else {
             // boundary facet: out of line (rare; keeps the hot code small)
             CompVec<float, NC> vh, vl, vf;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                vh.v[c] = uh[c];
-                vl.v[c] = ul[c];
-                vf.v[c] = xf ? fxs[c] : fys[c];
-            }
+            vh.v[0] = uh[0];
+            vl.v[0] = ul[0];
+            vf.v[0] = xf ? fxs[0] : fys[0];
             const CompVec<float, NC + 1> o =
                 boundary_facet_lo<Ph>(m, pr, d, ex, ey, self_is_L ? 1.f : -1.f, vh, vl, vf);
             lam[d] = o.v[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) F[d][c] = o.v[c];
+            F[d][0] = o.v[0];
         }
     }
-    float sf = __fadd_rn(__fadd_rn(__fadd_rn(lam[0], lam[1]), lam[2]), lam[3]);
-    sf = fmaxf(sf, pr.lambda_floor_f);
-    // dt_e / h = 1 / s: float reciprocal refined by one float64 Newton step
-    // (relative error ~2^-46, far inside the 2^-20 inflation of the speeds;
-    // GB300's float64 divide is a long sequence on its narrow float64 pipe)
-    double s, rs;
-    if constexpr (SUB) {
-        // Lemma 1 bound; the float speed sum is rounded up (a float dt_e no
-        // larger than the bound)
-        rs = subcell_dt<float, P, Ph>(u, m, pr, ex, ey) * m.inv_h;
-        s = 1.0 / rs;
-        sf = __double2float_ru(s);
-    } else {
-        s = (double)sf;
-        const double r0 = (double)__frcp_rn(sf);
-        rs = fma(r0, fma(-s, r0, 1.0), r0);
-    }
-    const double dte = m.h * rs;
-    dte_out[e] = dte;
-    dte_out[m.E + e] = rs;
-    dte_out[2 * m.E + e] = s * m.inv_h;
-#pragma unroll
-    for (int d = 0; d < 4; ++d)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = F[d][c];
-    const float s4 = 0.25f * sf;  // |K| / (|dK| dt_e), exact
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        // facet flux sum (F_E - F_W) + F_N - F_S as a float-float pair, widened once
-        float osh, osl;
-        ff_sum4(F[1][c], F[0][c], F[3][c], F[2][c], osh, osl);
-        const double os = (double)osh + (double)osl;
-        const double bl = ued[c] - rs * os;
-        ubl_out[c * m.E + e] = bl;
-        if (NC == 1) {
-            // capacities (s/4)(umax - bl) >= 0 and (s/4)(umin - bl) <= 0: bound
-            // gaps in float64, both factors and the product rounded toward zero
-            // (smaller magnitudes stay admissible)
-            q_out[e] = __fmul_rz(s4, fmaxf(0.f, __double2float_rz(pr.umax - bl)));
-            q_out[m.E + e] = __fmul_rz(s4, fminf(0.f, __double2float_rz(pr.umin - bl)));
-            // the float-float mean, for the element contributions of k_update_ev
-            avg[e] = uh[0];
-            avg[m.E + e] = ul[0];
-        } else {
-            // float copies for the certificate of the facet limiter (euler_alpha_is_one)
-            cf_out[(1 + c) * m.E + e] = (float)bl;
-        }
-    }
-    cf_out[e] = sf;  // the float speed sum (dt_e in float for k_update_ev)
-    if constexpr (LO) {
-        return dte;
-    } else {
+    const double dte = lo_outputs_mixed<P, Ph, SUB>(m, pr, u, lam, F, uh, ul, ue_out, dte_out, ubl_out, q_out, fl_out,
+                                                    cf_out, avg, ex, ey, e);
     float gam;
     if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-        gam = sensor_scalar<float, P>(m, pr, u, U[0], nb, ex, ey);
+        gam = sensor_scalar<float, P>(m, pr, u, U, nb, ex, ey);
     } else {
         gam = (pr.mode == MODE_HO) ? 1.f : 0.f;
     }
-    gam_out[e] = (double)gam;
+    gam_out[e] = widen(gam);
     float lm = 0.f;
 #pragma unroll
-    for (int i = 0; i < N2; ++i) {
-        float ui[NC];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ui[c] = U[c][i];
-        lm = fmaxf(lm, Ph::template node_speed<float>(ui, pr));
-    }
-    nu_out[e] = (double)(lm * (m.h_f * (0.5f / P)));
-    if (EV) grad_vectors<float, P, NC>(m, U, m.h_f, m.E, e, EV);
+    for (int i = 0; i < N2; ++i) lm = fmaxf(lm, Ph::template node_speed<float>(&U[i], pr));
+    nu_out[e] = widen(lm * (m.h_f * (0.5f / P)));
     return dte;
+}
+
+// the same in float64: dt_e, ubar^{e,L} and the capacities or certificate
+// copies from the facets
+template <int P, class Ph, bool SUB>
+DEV double lo_outputs_fp64(const MeshDev& m, const ProbDev& pr, const double* __restrict__ u, const double (&lam)[4],
+                           const double (&FL)[4][Ph::NC], const double (&us)[Ph::NC], double* __restrict__ dte_out,
+                           double* __restrict__ ubl_out, double* __restrict__ q_out, double* __restrict__ fl_out,
+                           float* __restrict__ cf_out, int ex, int ey, int e) {
+    constexpr int NC = Ph::NC;
+    double s = ((lam[0] + lam[1]) + lam[2]) + lam[3];
+    s = fmax(s, pr.lambda_floor);
+    // dt_e = |K| / (|S| sum lambda) = h / s; dt_e / h = 1 / s
+    double rs = 1.0 / s;
+    if constexpr (SUB) {
+        // Lemma 1 bound instead (the unlimited-flux variant)
+        rs = subcell_dt<double, P, Ph>(u, m, pr, ex, ey) * m.inv_h;
+        s = 1.0 / rs;
     }
+    const double dte = m.h * rs;
+    dte_out[e] = dte;
+    dte_out[m.E + e] = rs;              // dt_e / h
+    dte_out[2 * m.E + e] = s * m.inv_h; // 1 / dt_e
+#pragma unroll
+    for (int d = 0; d < 4; ++d)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = FL[d][c];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const double os = ((FL[1][c] - FL[0][c]) + FL[3][c]) - FL[2][c];
+        const double bl = us[c] - rs * os;
+        ubl_out[c * m.E + e] = bl;
+        if (NC == 1) {
+            // admissible antidiffusive capacities of eq. (fAlim):
+            // (|K|/|dK|)(umax - ubar^{e,L})/dt_e = (s/4)(umax - ubar^{e,L}) >= 0, and
+            // (s/4)(umin - ubar^{e,L}) <= 0
+            q_out[e] = fmax(0.0, (0.25 * s) * (pr.umax - bl));
+            q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
+        } else {
+            cf_out[(1 + c) * m.E + e] = narrow(bl);  // for the certificate of the facet limiter
+        }
+    }
+    if (NC > 1) cf_out[e] = narrow(s);
+    return dte;
 }
 
 template <class R, int P, class Ph, bool SUB = false>
 DEV double pre_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, double* __restrict__ ue_out,
                   double* __restrict__ dte_out, double* __restrict__ ubl_out,
                   double* __restrict__ gam_out, double* __restrict__ nu_out,
-                  R* __restrict__ q_out, R* __restrict__ fl_out, R* __restrict__ EV,
+                  R* __restrict__ q_out, R* __restrict__ fl_out,
                   float* __restrict__ cf_out, float* __restrict__ avg, int ex, int ey, int e) {
+    static_assert(Ph::NC == 1, "systems: k_lo_sys and k_sens");
     if constexpr (sizeof(R) == 4) {
-        return pre_at_mixed<P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, EV,
-                                        cf_out, avg, ex, ey, e);
+        return pre_at_mixed<P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, cf_out, avg,
+                                        ex, ey, e);
     } else {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    double dte;
-    {
+        constexpr int N2 = Dim<P>::N2;
         int nb[4];
 #pragma unroll
         for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-        R U[NC][N2];
-        load_block<R, P, NC>(u, m, ex, ey, U);
-        double us[NC], fxs[NC], fys[NC];
-        {
-            R aR[NC], fxR[NC], fyR[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                us[c] = cell_mean<R, P>(m, U[c]);
-                aR[c] = R(us[c]);
-                ue_out[c * m.E + e] = us[c];
-            }
-            Ph::template flux<R>(aR, fxR, fyR, pr);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                fxs[c] = (double)fxR[c];
-                fys[c] = (double)fyR[c];
-            }
-        }
-        double uo[4][NC], fxo[4][NC], fyo[4][NC];
+        R U[N2];
+        load_comp<R, P>(u, m, ex, ey, U);
+        double us[1], fxs[1], fys[1];
+        us[0] = cell_mean<R, P>(m, U);
+        ue_out[e] = us[0];
+        Ph::template flux<R>(us, fxs, fys, pr);
+        double uo[4][1], fxo[4][1], fyo[4][1];
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
+            uo[d][0] = fxo[d][0] = fyo[d][0] = 0.0;
             if (nb[d] >= 0) {
                 int jx, jy;
                 neighbour_xy(m, ex, ey, d, jx, jy);
                 cell_state<R, P, Ph>(u, m, pr, jx, jy, uo[d], fxo[d], fyo[d]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < NC; ++c) uo[d][c] = fxo[d][c] = fyo[d][c] = 0.0;
             }
         }
-        double lam[4], FL[4][NC];
+        double lam[4], FL[4][1];
         lo_facets<Ph, R>(m, pr, nb, ex, ey, us, fxs, fys, uo, fxo, fyo, lam, FL);
-        double s = ((lam[0] + lam[1]) + lam[2]) + lam[3];
-        s = fmax(s, pr.lambda_floor);
-        // dt_e = |K| / (|S| sum lambda) = h / s; dt_e / h = 1 / s
-        double rs = 1.0 / s;
-        if constexpr (SUB) {
-            // Lemma 1 bound instead (the unlimited-flux variant)
-            rs = subcell_dt<R, P, Ph>(u, m, pr, ex, ey) * m.inv_h;
-            s = 1.0 / rs;
+        const double dte = lo_outputs_fp64<P, Ph, SUB>(m, pr, u, lam, FL, us, dte_out, ubl_out, q_out, fl_out, cf_out, ex,
+                                                       ey, e);
+        double gam;
+        if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
+            gam = sensor_scalar<R, P>(m, pr, u, U, nb, ex, ey);
+        } else {
+            gam = (pr.mode == MODE_HO) ? 1.0 : 0.0;
         }
-        dte = m.h * rs;
-        dte_out[e] = dte;
-        dte_out[m.E + e] = rs;              // dt_e / h
-        dte_out[2 * m.E + e] = s * m.inv_h; // 1 / dt_e
+        gam_out[e] = gam;
+        R lm = R(0);
 #pragma unroll
-        for (int d = 0; d < 4; ++d)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = FL[d][c];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            double os = ((FL[1][c] - FL[0][c]) + FL[3][c]) - FL[2][c];
-            double bl = us[c] - rs * os;
-            ubl_out[c * m.E + e] = bl;
-            if (NC == 1) {
-                // admissible antidiffusive capacities of eq. (fAlim):
-                // (|K|/|dK|)(umax - ubar^{e,L})/dt_e = (s/4)(umax - ubar^{e,L}) >= 0, and
-                // (s/4)(umin - ubar^{e,L}) <= 0
-                q_out[e] = fmax(0.0, (0.25 * s) * (pr.umax - bl));
-                q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
-            } else {
-                cf_out[(1 + c) * m.E + e] = (float)bl;  // for the certificate of the facet limiter
-            }
-        }
-        if (NC > 1) cf_out[e] = (float)s;
-        if constexpr (NC == 1) {  // systems: k_sens
-            double gam;
-            if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-                gam = sensor_scalar<R, P>(m, pr, u, U[0], nb, ex, ey);
-            } else {
-                gam = (pr.mode == MODE_HO) ? 1.0 : 0.0;
-            }
-            gam_out[e] = gam;
-            R lm = R(0);
-#pragma unroll
-            for (int i = 0; i < N2; ++i) {
-                R ui[NC];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) ui[c] = U[c][i];
-                lm = fmax(lm, Ph::template node_speed<R>(ui, pr));
-            }
-            nu_out[e] = (double)lm * (m.h * (0.5 / m.p));
-        }
-        if (EV) grad_vectors<R, P, NC>(m, U, PV<R>::h(m), m.E, e, EV);
-    }
-    return dte;
+        for (int i = 0; i < N2; ++i) lm = fmax(lm, Ph::template node_speed<R>(&U[i], pr));
+        nu_out[e] = lm * (m.h * (0.5 / P));
+        return dte;
     }
 }
 
-// k_avg (FP32-mixed systems): float-float cell means of every element, read
-// by k_pre_lo for the element and its four face neighbours instead of their
-// coefficient blocks; avg[(2c) E + e] = high part, avg[(2c+1) E + e] = low
-// part of component c.  Beside them the quantities of the mean's state that
+// k_avg (systems): cell means of every element, read by k_lo_sys for the facets
+// of the cell instead of its coefficient block: float-float in the FP32-mixed
+// form (avg[(2c) E + e] high, avg[(2c+1) E + e] low part of component c), u^e
+// itself in float64.  Beside them the quantities of the mean's state that
 // every facet of the cell needs, formed once per cell: cq[c E + e] = f_x(u^e)
 // and cq[(NC + c) E + e] = f_y(u^e) (the flux of the high parts), then the
 // speed parts of the two-rarefaction bound.
-template <int P, class Ph>
-__global__ void k_avg(MeshDev m, ProbDev pr, const float* __restrict__ u, float* __restrict__ avg,
-                      float* __restrict__ cq) {
+template <class R, int P, class Ph>
+__global__ void k_avg(MeshDev m, ProbDev pr, const R* __restrict__ u, float* __restrict__ avg, double* __restrict__ ue_out,
+                      R* __restrict__ cq) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
     constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    float U[NC][N2];
-    load_block<float, P, NC>(u, m, ex, ey, U);
-    float uh[NC];
+    R uh[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        float hi, lo;
-        ff_mean<N2>(U[c], hi, lo);
-        avg[(2 * c) * m.E + e] = hi;
-        avg[(2 * c + 1) * m.E + e] = lo;
-        uh[c] = hi;
+        R U[N2];
+        load_comp<R, P>(u + c * m.NN, m, ex, ey, U);
+        if constexpr (sizeof(R) == 4) {
+            float hi, lo;
+            ff_mean<N2>(U, hi, lo);
+            avg[(2 * c) * m.E + e] = hi;
+            avg[(2 * c + 1) * m.E + e] = lo;
+            uh[c] = hi;
+        } else {
+            uh[c] = cell_mean<R, P>(m, U);
+            ue_out[c * m.E + e] = uh[c];
+        }
     }
-    float fx[NC], fy[NC], q[Ph::NPART_OR_1];
-    Ph::template flux<float>(uh, fx, fy, pr);
-    Ph::speed_parts(uh, PV<float>::gam(pr), q);
+    R fx[NC], fy[NC], q[Ph::NPART];
+    Ph::template flux<R>(uh, fx, fy, pr);
+    Ph::speed_parts(uh, PV<R>::gam(pr), q);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         cq[c * m.E + e] = fx[c];
         cq[(NC + c) * m.E + e] = fy[c];
     }
 #pragma unroll
-    for (int k = 0; k < Ph::NPART_OR_1; ++k) cq[(2 * NC + k) * m.E + e] = q[k];
+    for (int k = 0; k < Ph::NPART; ++k) cq[(2 * NC + k) * m.E + e] = q[k];
 }
 
 // Resident blocks of 128 threads per SM requested from the compiler for the
@@ -1033,32 +973,189 @@ template <class R, int P, class Ph, bool SUB = false>
 __global__ void k_pre(MeshDev m, ProbDev pr, const R* __restrict__ u, double* __restrict__ ue_out,
                       double* __restrict__ dte_out, double* __restrict__ ubl_out,
                       double* __restrict__ gam_out, double* __restrict__ nu_out,
-                      R* __restrict__ q_out, R* __restrict__ fl_out, R* __restrict__ EV,
+                      R* __restrict__ q_out, R* __restrict__ fl_out,
                       float* __restrict__ cf_out, float* __restrict__ avg,
                       unsigned long long* __restrict__ dtbits) {
     pdl_wait_then_trigger();
     int ex, ey, e;
     double dte = __longlong_as_double(0x7ff0000000000000LL);
     if (elem_of_thread(m, ex, ey, e))
-        dte = pre_at<R, P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, EV, cf_out,
+        dte = pre_at<R, P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, cf_out,
                                     avg, ex, ey, e);
     if (dtbits) block_min_to(dte, dtbits);
 }
 
-// FP32-mixed systems: the low-order part of k_pre (cell states from k_avg,
-// facet speeds and f^L, dt_e, ubar^{e,L}, the float copies for the facet
+// The facets of a tile of TX x TY elements (systems): the TX + 1 by TY
+// vertical ones, then the TX by TY + 1 horizontal ones.  A block evaluates
+// each once, where one thread per element evaluated its four (every interior
+// facet twice), and the elements take them from shared memory.
+constexpr int F_TX = 32, F_TY = 4;
+struct FacetItem {
+    int axis, slot;        // x (0) or y (1); position among the facets of its axis
+    int eL, eR;            // cells left and right (below and above), -1 outside the domain
+    int ex, ey, d;         // a cell of the facet and its side there (the one inside on the boundary)
+};
+// item i of the tile at (ex0, ey0): false where no element of the tile has it
+DEV bool facet_item(const MeshDev& m, int ex0, int ey0, int i, FacetItem& f) {
+    constexpr int NV = (F_TX + 1) * F_TY;
+    f.axis = i < NV ? 0 : 1;
+    const int k = f.axis == 0 ? i : i - NV, w = f.axis == 0 ? F_TX + 1 : F_TX;
+    const int r = k / w, c = k - r * w;
+    f.slot = k;
+    // the cell right of (above) the facet, and the one left of (below) it
+    const int xR = ex0 + c, yR = ey0 + r, xL = f.axis == 0 ? xR - 1 : xR, yL = f.axis == 0 ? yR : yR - 1;
+    const bool inR = xR < m.nx && yR < m.ny, inL = xL >= 0 && yL >= 0 && xL < m.nx && yL < m.ny;
+    // a cell of the tile itself: the right one unless it is the far end's
+    const bool tR = f.axis == 0 ? c < F_TX : r < F_TY, tL = f.axis == 0 ? c > 0 : r > 0;
+    if (!((tR && inR) || (tL && inL))) return false;
+    if (inR) {
+        f.eR = yR * m.nx + xR;
+        f.ex = xR, f.ey = yR, f.d = f.axis == 0 ? 0 : 2;
+        f.eL = neighbour(m, xR, yR, f.d);
+    } else {
+        f.eL = yL * m.nx + xL;
+        f.ex = xL, f.ey = yL, f.d = f.axis == 0 ? 1 : 3;
+        f.eR = neighbour(m, xL, yL, f.d);
+    }
+    return true;
+}
+// slots of the element (tx, ty)'s facets W, E (x) and S, N (y)
+DEV int facet_of(int tx, int ty, int d) { return d < 2 ? ty * (F_TX + 1) + tx + d : (ty + d - 2) * F_TX + tx; }
+constexpr int F_NV = (F_TX + 1) * F_TY, F_NH = F_TX * (F_TY + 1);
+
+// low-order quantities of a boundary facet in float64, as boundary_facet_lo
+template <class Ph>
+__device__ __noinline__ CompVec<double, Ph::NC + 1> boundary_facet_lo64(const MeshDev& m, const ProbDev& pr, int d,
+                                                                       int ex, int ey, CompVec<double, Ph::NC> us,
+                                                                       CompVec<double, Ph::NC> fn) {
+    constexpr int NC = Ph::NC;
+    const bool xf = d < 2;
+    const double sg = (d & 1) ? 1.0 : -1.0, nx = xf ? sg : 0.0, ny = xf ? 0.0 : sg;
+    // external state u_hat at the facet midpoint from the cell average
+    const int slot = side_split(pr, d) ? side_slot(pr, d, side_mid_pos(m, d, ex, ey)) : 0;
+    double ux[NC], fx[NC];
+    ext_state<double, NC>(pr, d, slot, us.v, ux);
+    if (pr.side[d].kind[slot] != BC_OUTFLOW) {
+        Ph::template normal<double>(ux, xf ? 0 : 1, fx, pr);
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) fx[c] = fn.v[c];
+    }
+    const double l = Ph::template max_speed<double>(us.v, ux, nx, ny, pr);
+    CompVec<double, NC + 1> out;
+    out.v[NC] = l;
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        out.v[c] = sg * (0.5 * (sg * fn.v[c] + sg * fx[c]) - 0.5 * l * (ux[c] - us.v[c]));
+    return out;
+}
+
+// systems: the low-order part of the stage from the cell states of k_avg
+// (facet speeds and f^L, dt_e, ubar^{e,L}, the float copies for the facet
 // limiter's certificate); gamma_e and nu_e come from k_sens
-template <int P, class Ph, bool SUB = false>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_PRE_LO)) k_pre_lo(MeshDev m, ProbDev pr, const float* __restrict__ u, double* __restrict__ ue_out,
-                         double* __restrict__ dte_out, double* __restrict__ ubl_out,
-                         float* __restrict__ fl_out, float* __restrict__ cf_out, float* __restrict__ avg,
-                         const float* __restrict__ cq, unsigned long long* __restrict__ dtbits) {
+template <class R, int P, class Ph, bool SUB = false>
+__global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 3)
+    k_lo_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, double* __restrict__ ue_io, double* __restrict__ dte_out,
+             double* __restrict__ ubl_out, R* __restrict__ fl_out, float* __restrict__ cf_out,
+             const float* __restrict__ avg, const R* __restrict__ cq, unsigned long long* __restrict__ dtbits) {
+    constexpr int NC = Ph::NC, NT = F_TX * F_TY;
+    __shared__ R sV[NC + 1][F_NV], sH[NC + 1][F_NH];
     pdl_wait_then_trigger();
-    int ex, ey, e;
+    const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * F_TX, ey0 = blockIdx.y * F_TY;
+    const int E = m.E;
+    const R g = PV<R>::gam(pr);
+#pragma unroll 1
+    for (int i = ty * F_TX + tx; i < F_NV + F_NH; i += NT) {
+        FacetItem f;
+        if (!facet_item(m, ex0, ey0, i, f)) continue;
+        R F[NC], lam;
+        const R* __restrict__ fa = cq + (long long)(f.axis * NC) * E;  // the means' fluxes along the facet's axis
+        if (f.eL >= 0 && f.eR >= 0) {
+            const R* __restrict__ q = cq + (long long)(2 * NC) * E;
+            const R* __restrict__ qv = q + (long long)f.axis * E;
+            const R l = Ph::facet_speed_parts(qv[f.eL], q[2 * E + f.eL], q[3 * E + f.eL], q[4 * E + f.eL], q[5 * E + f.eL],
+                                              qv[f.eR], q[2 * E + f.eR], q[3 * E + f.eR], q[4 * E + f.eR], q[5 * E + f.eR],
+                                              g);
+            if constexpr (sizeof(R) == 4) {
+                lam = __fmul_rn(l, 1.0f + 0x1p-20f);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const float* __restrict__ ah = avg + (long long)(2 * c) * E;
+                    F[c] = llf_value(fa[c * E + f.eL], fa[c * E + f.eR], lam,
+                                     ff_diff(ah[f.eR], ah[E + f.eR], ah[f.eL], ah[E + f.eL]));
+                }
+            } else {
+                lam = l;
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+                    F[c] = 0.5 * (fa[c * E + f.eL] + fa[c * E + f.eR]) -
+                           0.5 * l * (ue_io[c * E + f.eR] - ue_io[c * E + f.eL]);
+            }
+        } else {
+            // a facet on the domain boundary: out of line (rare)
+            const int e = f.ey * m.nx + f.ex;
+            if constexpr (sizeof(R) == 4) {
+                CompVec<float, NC> vh, vl, vf;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    vh.v[c] = avg[(long long)(2 * c) * E + e];
+                    vl.v[c] = avg[(long long)(2 * c + 1) * E + e];
+                    vf.v[c] = fa[c * E + e];
+                }
+                const CompVec<float, NC + 1> o =
+                    boundary_facet_lo<Ph>(m, pr, f.d, f.ex, f.ey, (f.d & 1) ? 1.f : -1.f, vh, vl, vf);
+                lam = o.v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) F[c] = o.v[c];
+            } else {
+                CompVec<double, NC> us, vf;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    us.v[c] = ue_io[c * E + e];
+                    vf.v[c] = fa[c * E + e];
+                }
+                const CompVec<double, NC + 1> o = boundary_facet_lo64<Ph>(m, pr, f.d, f.ex, f.ey, us, vf);
+                lam = o.v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) F[c] = o.v[c];
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (f.axis == 0) sV[c][f.slot] = F[c];
+            else sH[c][f.slot] = F[c];
+        }
+        if (f.axis == 0) sV[NC][f.slot] = lam;
+        else sH[NC][f.slot] = lam;
+    }
+    __syncthreads();
+    const int ex = ex0 + tx, ey = ey0 + ty, e = ey * m.nx + ex;
     double dte = __longlong_as_double(0x7ff0000000000000LL);
-    if (elem_of_thread(m, ex, ey, e))
-        dte = pre_at_mixed<P, Ph, SUB, true>(m, pr, u, ue_out, dte_out, ubl_out, nullptr, nullptr, nullptr, fl_out,
-                                             nullptr, cf_out, avg, ex, ey, e, cq);
+    if (ex < m.nx && ey < m.ny) {
+        R lam[4], F[4][NC];
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            const int s = facet_of(tx, ty, d);
+            lam[d] = d < 2 ? sV[NC][s] : sH[NC][s];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) F[d][c] = d < 2 ? sV[c][s] : sH[c][s];
+        }
+        R us[NC];
+        if constexpr (sizeof(R) == 4) {
+            float ul[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                us[c] = avg[(long long)(2 * c) * E + e];
+                ul[c] = avg[(long long)(2 * c + 1) * E + e];
+            }
+            dte = lo_outputs_mixed<P, Ph, SUB>(m, pr, u, lam, F, us, ul, ue_io, dte_out, ubl_out, nullptr, fl_out, cf_out,
+                                               nullptr, ex, ey, e);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) us[c] = ue_io[c * E + e];
+            dte = lo_outputs_fp64<P, Ph, SUB>(m, pr, u, lam, F, us, dte_out, ubl_out, nullptr, fl_out, cf_out, ex, ey, e);
+        }
+    }
     if (dtbits) block_min_to(dte, dtbits);
 }
 
@@ -1171,8 +1268,9 @@ __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const
 #pragma unroll
         for (int a = 0; a <= P; ++a) lm = fmax(lm, sS[ty * P + b][tx * P + a]);
     const int e = ey * m.nx + ex;
-    gam_out[e] = (double)gam;
-    if constexpr (sizeof(R) == 4) nu_out[e] = (double)(lm * (m.h_f * (0.5f / P)));
+    if constexpr (sizeof(R) == 4) gam_out[e] = widen(gam);
+    else gam_out[e] = gam;
+    if constexpr (sizeof(R) == 4) nu_out[e] = widen(lm * (m.h_f * (0.5f / P)));
     else nu_out[e] = lm * (m.h * (0.5 / P));
 }
 
@@ -1538,6 +1636,13 @@ DEV void w_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Dim<P>::N2], i
     for (int i = 0; i < N2; ++i) W[i] = mul_r(W[i], h);
 }
 
+// a per-element float64 scalar in the bulk precision (gamma_e, nu_e)
+template <class R>
+DEV R bulk(double v) {
+    if constexpr (sizeof(R) == 4) return narrow(v);
+    else return v;
+}
+
 // coefficients of h u_h' along a line
 template <class R, int P>
 DEV void deriv_line(const MeshDev& m, const Tab<R>& T, const R (&u)[P + 1], R (&d)[P + 1]) {
@@ -1617,7 +1722,7 @@ DEV void stab_part(const MeshDev& m, const R (&U)[Dim<P>::N2], const R* __restri
     R GX[N2], GY[N2], s[N2];
     load_comp<R, P>(g, m, ex, ey, GX);
     load_comp<R, P>(g + m.NN, m, ex, ey, GY);
-    stab_comp<R, P>(m, tab_of<R>(m, P), U, GX, GY, R(gam[e]) * PV<R>::h(m), R(nu[e]), s);
+    stab_comp<R, P>(m, tab_of<R>(m, P), U, GX, GY, bulk<R>(gam[e]) * PV<R>::h(m), bulk<R>(nu[e]), s);
 #pragma unroll
     for (int i = 0; i < N2; ++i) ER[ev_at(m.E, e, i, 0, 1)] = sub_r(W[i], s[i]);
 }
@@ -1713,7 +1818,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 6 : P 
         R GX[N2], GY[N2];
         load_comp<R, P>(g + c * m.NN, m, ex, ey, GX);
         load_comp<R, P>(g + (NC + c) * m.NN, m, ex, ey, GY);
-        stab_comp<R, P>(m, T, U, GX, GY, R(gam[e]) * PV<R>::h(m), R(nu[e]), s);
+        stab_comp<R, P>(m, T, U, GX, GY, bulk<R>(gam[e]) * PV<R>::h(m), bulk<R>(nu[e]), s);
     }
     // terms on the domain boundary: warp c takes face c, all components
     if (neighbour(m, ex, ey, c) < 0) {
@@ -1892,6 +1997,17 @@ __device__ __noinline__ CompVec<double, Ph::NC + 1> reduce_pseudo_step(const Pro
     return out;
 }
 
+// a pseudo time step decreased by the remark after eq. (dtmaxcell): the float
+// speed sum that the element part reads is rounded up (its float dt_e never
+// exceeds the reduced one)
+DEV void store_reduced_step(const MeshDev& m, double* dte_a, float* cf, double rs2, int e) {
+    const double dte2 = m.h * rs2;
+    dte_a[e] = dte2;
+    dte_a[m.E + e] = rs2;
+    dte_a[2 * m.E + e] = 1.0 / dte2;
+    cf[e] = __double2float_ru(1.0 / rs2);
+}
+
 // facet part of the element update: canonical f^H, the flux limiter and
 // ubar^e (eqs. (hoflux), (fAlim)/(uelim), Appendix A), and the facet term
 // (h/(p+1)^2) sum_d +-f^H_d of the element contributions f_i^e (eq. (aec))
@@ -1974,7 +2090,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
             if constexpr (mixed_sys) {
                 float osh, osl;
                 ff_sum4(FHr[1][c], FHr[0][c], FHr[3][c], FHr[2][c], osh, osl);
-                os = (double)osh + (double)osl;
+                os = widen(osh) + widen(osl);
             } else {
                 os = ((FH[1][c] - FH[0][c]) + FH[3][c]) - FH[2][c];
             }
@@ -2023,7 +2139,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     fminv = fmax(fminv, -qcap[Rc]);
                 }
                 FBr[d] = (fA >= R(0)) ? fmin(fA, fmaxv) : fmax(fA, fminv);
-                FB[d][0] = (double)FBr[d];
+                if constexpr (sizeof(R) == 8) FB[d][0] = FBr[d];
             } else {
                 double fA[NC];
 #pragma unroll
@@ -2036,7 +2152,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     float fAf[NC], fAm[NC], ub[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
-                        fAf[c] = sizeof(R) == 4 ? __fsub_rn((float)FLr[d][c], (float)FHr[d][c]) : (float)fA[c];
+                        fAf[c] = sizeof(R) == 4 ? __fsub_rn((float)FLr[d][c], (float)FHr[d][c]) : narrow(fA[c]);
                         fAm[c] = -fAf[c];
                     }
                     bool one = true;
@@ -2106,7 +2222,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                 // float limited fluxes summed as a float-float pair, widened once
                 float osh, osl;
                 ff_sum4(FBr[1], FBr[0], FBr[3], FBr[2], osh, osl);
-                os = (double)osh + (double)osl;
+                os = widen(osh) + widen(osl);
             } else if constexpr (mixed_sys) {
                 // (fbar_E - fbar_W) + fbar_N - fbar_S from the eight float terms,
                 // compensated, widened once
@@ -2114,7 +2230,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                                     TH[3][c], TL[3][c], -TH[2][c], -TL[2][c]};
                 float osh, osl;
                 ff_sum<8>(t, osh, osl);
-                os = (double)osh + (double)osl;
+                os = widen(osh) + widen(osl);
             } else {
                 os = ((FB[1][c] - FB[0][c]) + FB[3][c]) - FB[2][c];
             }
@@ -2280,7 +2396,8 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
             beta = R(b);
         }
     }
-    beta_out[e] = (double)beta;
+    if constexpr (sizeof(R) == 4) beta_out[e] = widen(beta);
+    else beta_out[e] = beta;
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
@@ -2509,49 +2626,33 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_UPD)
 }
 
 
-// The update in two kernels (FP32-mixed, and systems in both forms).  k_facet
-// needs only u and the outputs of k_pre, so in the FP32-mixed form it runs on
-// a second stream beside the g_h and udot kernels; k_update_el and k_upd_sys
-// then read its ubar^e and facet terms.  The scalar bodies are device
-// functions of one element, also run by the batched stage.
-template <class R, int P, class Ph>
-DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
+// FP32-mixed scalars: the update in two kernels.  k_facet needs only u and the
+// outputs of k_pre, so it runs on a second stream beside the g_h and udot
+// kernels; k_update_el then reads its ubar^e and facet terms.  Together they
+// compute what k_update_ev computes, in the same arithmetic.  The bodies are
+// device functions of one element, also run by the batched stage.
+template <int P, class Ph>
+DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
                      const double* __restrict__ ue, double* dte_a, const double* __restrict__ ubl,
-                     const R* __restrict__ qcap, const R* __restrict__ fl_in, float* cf,
-                     double* __restrict__ ube_out, R* __restrict__ fht, unsigned long long* __restrict__ cnt,
+                     const float* __restrict__ qcap, const float* __restrict__ fl_in, float* cf,
+                     double* __restrict__ ube_out, float* __restrict__ fht, unsigned long long* __restrict__ cnt,
                      int ex, int ey, int e) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
+    constexpr int N2 = Dim<P>::N2;
     int nb[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-    R U[NC][N2];
-    load_block<R, P, NC>(u, m, ex, ey, U);
-    double uec[NC], ublc[NC], ubec[NC];
-    R fh[NC];
-    const bool need_ue = pr.fl == FL_NONE;  // u^e enters ubar^e only without the flux limiter
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        uec[c] = need_ue ? ue[c * m.E + e] : 0.0;
-        ublc[c] = ubl[c * m.E + e];
-    }
+    float U[1][N2];
+    load_block<float, P, 1>(u, m, ex, ey, U);
+    double uec[1], ublc[1], ubec[1];
+    float fh[1];
+    uec[0] = pr.fl == FL_NONE ? ue[e] : 0.0;  // u^e enters ubar^e only without the flux limiter
+    ublc[0] = ubl[e];
     const double rs = dte_a[m.E + e];
     double rs2;
-    facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        ube_out[c * m.E + e] = ubec[c];
-        fht[c * m.E + e] = fh[c];
-    }
-    if (rs2 != rs) {
-        // a pseudo time step decreased by the remark after eq. (dtmaxcell):
-        // the float speed sum that k_update_el reads is rounded up (its float
-        // dt_e never exceeds the reduced one)
-        const double dte2 = m.h * rs2;
-        dte_a[e] = dte2;
-        dte_a[m.E + e] = rs2;
-        dte_a[2 * m.E + e] = 1.0 / dte2;
-        cf[e] = __double2float_ru(1.0 / rs2);
-    }
+    facet_part<float, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
+    ube_out[e] = ubec[0];
+    fht[e] = fh[0];
+    if (rs2 != rs) store_reduced_step(m, dte_a, cf, rs2, e);
 }
 
 template <int P, class Ph>
@@ -2578,17 +2679,17 @@ DEV void update_el_at(const MeshDev& m, const ProbDev& pr, const float* __restri
                                e);
 }
 
-template <class R, int P, class Ph>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_FACET)) k_facet(MeshDev m, ProbDev pr, const R* __restrict__ u,
+template <int P, class Ph>
+__global__ void __launch_bounds__(128) k_facet(MeshDev m, ProbDev pr, const float* __restrict__ u,
                                                const double* __restrict__ ue, double* dte_a,
-                                               const double* __restrict__ ubl, const R* __restrict__ qcap,
-                                               const R* __restrict__ fl_in, float* cf,
-                                               double* __restrict__ ube_out, R* __restrict__ fht,
+                                               const double* __restrict__ ubl, const float* __restrict__ qcap,
+                                               const float* __restrict__ fl_in, float* cf,
+                                               double* __restrict__ ube_out, float* __restrict__ fht,
                                                unsigned long long* __restrict__ cnt) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    facet_el_at<R, P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
+    facet_el_at<P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
 }
 
 template <int P, class Ph>
@@ -2602,6 +2703,223 @@ __global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_UPD))
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
     update_el_at<P, Ph>(m, pr, u, ud, ER, cf, avg, ube, fht, dtp, EW, beta_out, cnt, ex, ey, e);
+}
+
+// The facet part of the update of systems: f^H (eq. (hoflux)), the facet
+// limiter of Appendix A, ubar^e (eqs. (uebar), (uelim), (uebar2)) and the
+// facet terms of f_i^e.  As in k_lo_sys each facet of a tile is evaluated once
+// (f^H from its p + 1 nodes, the positivity factors of its two cells) and the
+// elements take its terms from shared memory.  A limited facet enters ubar^e
+// as two terms T0 + T1: (f^L, -f^H) where alpha = 1 (certified in float, or
+// computed as 1 in float64: the same terms either way, so the certificate
+// changes no bit), else alpha f^A, split into two floats in the FP32-mixed
+// form; the eight float terms are summed as a compensated pair.
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 4)
+    k_facet_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, const double* __restrict__ ue, double* dte_a,
+                const double* __restrict__ ubl, const R* __restrict__ fl_in, float* cf, double* __restrict__ ube_out,
+                R* __restrict__ fht, unsigned long long* __restrict__ cnt) {
+    constexpr int NC = Ph::NC, N1 = P + 1, NT = F_TX * F_TY, NFC = F_NV + F_NH;
+    constexpr int NTERM = sizeof(R) == 4 ? 3 : 2;  // f^H, and T0, T1 (float64: their sum)
+    __shared__ R sT[NTERM][NC][NFC];
+    pdl_begin();
+    const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * F_TX, ey0 = blockIdx.y * F_TY;
+    const int E = m.E;
+    const bool need_fh = !(pr.mode == MODE_LO && pr.fl == FL_LOW);
+    if (need_fh) {
+#pragma unroll 1
+        for (int i = ty * F_TX + tx; i < NFC; i += NT) {
+            FacetItem f;
+            if (!facet_item(m, ex0, ey0, i, f)) continue;
+            // the face's coefficients
+            R Uf[NC * N1];
+            {
+                const int gx0 = f.ex * P + (f.d == 1 ? P : 0), gy0 = f.ey * P + (f.d == 3 ? P : 0);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) {
+                    int gx = gx0 + (f.axis == 0 ? 0 : k), gy = gy0 + (f.axis == 0 ? k : 0);
+                    if (m.px && gx == m.nnx) gx = 0;
+                    if (m.py && gy == m.nny) gy = 0;
+                    const R* __restrict__ un = u + ((long long)gy * m.nnx + gx);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) Uf[c * N1 + k] = un[c * m.NN];
+                }
+            }
+            const bool bnd = f.eL < 0 || f.eR < 0;
+            R FH[NC];
+            if (bnd && !side_plain(pr, f.d)) {
+                // boundary data u_hat: out of line (rare)
+                const R sg = (f.d & 1) ? R(1) : R(-1);
+                const CompVec<R, NC> fs = bnd_face_llf_sum<R, P, Ph>(m, pr, f.d, f.ey * m.nx + f.ex, f.axis == 0 ? sg : R(0),
+                                                                     f.axis == 0 ? R(0) : sg, Uf);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) FH[c] = sg * (is_lgl<R>(m) ? fs.v[c] : mul_r(fs.v[c], R(1.0 / N1)));
+            } else {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) FH[c] = R(0);
+#pragma unroll
+                for (int k = 0; k < N1; ++k) {
+                    R uk[NC], fn[NC];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) uk[c] = Uf[c * N1 + k];
+                    Ph::template normal<R>(uk, f.axis, fn, pr);
+                    const R wk = is_lgl<R>(m) ? R(c_tabd[PMAX + 1 + P].wl[k]) : R(1);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) FH[c] += is_lgl<R>(m) ? wk * fn[c] : fn[c];
+                }
+                if (!is_lgl<R>(m)) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) FH[c] = mul_r(FH[c], R(1.0 / N1));
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) sT[0][c][i] = FH[c];
+            if (pr.fl != FL_LIMITED) continue;
+            R FL[NC], T0[NC], T1[NC];
+            const long long lo = ((long long)(f.ey * m.nx + f.ex) * 4 + f.d) * NC;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                FL[c] = fl_in[lo + c];
+                T0[c] = FL[c];
+                T1[c] = -FH[c];
+            }
+            // float32 certificate first: where both cells certainly give alpha
+            // = 1 the float64 formula is skipped (same result; in the float64
+            // form it is some 100 float64 instructions a facet)
+            bool one = !(pr.opts & OPT_FP64_LIMITER);
+            if (one) {
+                float fA[NC], ub[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+                    fA[c] = sizeof(R) == 4 ? __fsub_rn((float)FL[c], (float)FH[c]) : narrow((double)FL[c] - (double)FH[c]);
+                if (f.eL >= 0) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * E + f.eL];
+                    one = euler_alpha_is_one(ub, fA, 0.25f * cf[f.eL], pr.ome_f);
+                }
+                if (one && f.eR >= 0) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        ub[c] = cf[(1 + c) * E + f.eR];
+                        fA[c] = -fA[c];
+                    }
+                    one = euler_alpha_is_one(ub, fA, 0.25f * cf[f.eR], pr.ome_f);
+                }
+            }
+            if (!one) {
+                double alpha = 1.0, fA[NC], ub[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) fA[c] = (double)FL[c] - (double)FH[c];
+                if (f.eL >= 0) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) ub[c] = ubl[c * E + f.eL];
+                    alpha = fmin(alpha, euler_alpha_rare(ub, fA, (0.25 * m.h) * dte_a[2 * E + f.eL], pr.pos_eps));
+                }
+                if (f.eR >= 0) {
+                    double fm[NC];
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        ub[c] = ubl[c * E + f.eR];
+                        fm[c] = -fA[c];
+                    }
+                    alpha = fmin(alpha, euler_alpha_rare(ub, fm, (0.25 * m.h) * dte_a[2 * E + f.eR], pr.pos_eps));
+                }
+                if (alpha != 1.0) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const double v = alpha * fA[c];
+                        if constexpr (sizeof(R) == 4) {
+                            T0[c] = __double2float_rn(v);
+                            T1[c] = __double2float_rn(v - (double)T0[c]);
+                        } else {
+                            T0[c] = v;
+                            T1[c] = 0.0;
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                if constexpr (sizeof(R) == 4) {
+                    sT[1][c][i] = T0[c];
+                    sT[2][c][i] = T1[c];
+                } else {
+                    sT[1][c][i] = T0[c] + T1[c];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const int ex = ex0 + tx, ey = ey0 + ty, e = ey * m.nx + ex;
+    if (ex >= m.nx || ey >= m.ny) return;
+    int at[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) at[d] = facet_of(tx, ty, d) + (d < 2 ? 0 : F_NV);
+    const double rs = dte_a[E + e];
+    double rs2 = rs, ub[NC];
+    R fh[NC];
+    // (m_i^e / |K_e|) |S| times the outward sum of f^H, the facet term of eq.
+    // (aecb): h / (p+1)^2 for every node (Bernstein); on an LGL mesh h,
+    // weighted by w_a w_b per node in k_upd_sys
+    const R hw = (sizeof(R) == 4) ? R(m.h_over_n2_f) : (is_lgl<R>(m) ? R(m.h) : R(m.h_over_n2));
+    // outward sum (E - W) + N - S of a facet term, in float as a pair
+    auto outward = [&](int k, int c) {
+        const R w = sT[k][c][at[0]], ea = sT[k][c][at[1]], so = sT[k][c][at[2]], no = sT[k][c][at[3]];
+        if constexpr (sizeof(R) == 4) {
+            float hi, lo;
+            ff_sum4(ea, w, no, so, hi, lo);
+            return widen(hi) + widen(lo);
+        } else {
+            return ((ea - w) + no) - so;
+        }
+    };
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        fh[c] = need_fh ? hw * (((sT[0][c][at[1]] - sT[0][c][at[0]]) + sT[0][c][at[3]]) - sT[0][c][at[2]]) : R(0);
+    if (pr.fl == FL_LOW) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ub[c] = ubl[c * E + e];
+    } else if (pr.fl == FL_NONE) {
+        double uec[NC], osv[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            uec[c] = ue[c * E + e];
+            osv[c] = outward(0, c);
+            ub[c] = uec[c] - rs * osv[c];
+        }
+        // eq. (uebar) with the macrocell dt_e need not stay in G: count such
+        // averages, and with the option decrease dt_e as the remark after
+        // eq. (dtmaxcell) says (out of line: rare)
+        if (!average_in_G<Ph>(pr, ub)) {
+            const CompVec<double, NC + 1> red = reduce_pseudo_step<Ph>(pr, uec, osv, rs, cnt);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ub[c] = red.v[c];
+            rs2 = red.v[NC];
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            double os;
+            if constexpr (sizeof(R) == 4) {
+                // (fbar_E - fbar_W) + fbar_N - fbar_S from the eight float
+                // terms, compensated, widened once
+                const float t[8] = {sT[1][c][at[1]], sT[2][c][at[1]], -sT[1][c][at[0]], -sT[2][c][at[0]],
+                                    sT[1][c][at[3]], sT[2][c][at[3]], -sT[1][c][at[2]], -sT[2][c][at[2]]};
+                float hi, lo;
+                ff_sum<8>(t, hi, lo);
+                os = widen(hi) + widen(lo);
+            } else {
+                os = outward(1, c);
+            }
+            ub[c] = ubl[c * E + e] + rs * os;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        ube_out[c * E + e] = ub[c];
+        fht[c * E + e] = fh[c];
+    }
+    if (rs2 != rs) store_reduced_step(m, dte_a, cf, rs2, e);
 }
 
 // The element part of the update of systems (f_i^e, the slope limiter beta_e,
@@ -2619,7 +2937,8 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
               unsigned long long* __restrict__ cnt) {
     constexpr int NC = Ph::NC, N1 = P + 1, N2 = Dim<P>::N2, TX = 32;
     __shared__ R sF[N2][NC][TX];
-    __shared__ double sU[NC][TX], sB[NC][TX];
+    __shared__ R sB[NC][TX];
+    __shared__ float sU[NC][TX];
     pdl_begin();
     const int tx = threadIdx.x, c = threadIdx.y;
     const bool valid = blockIdx.x * TX + tx < m.nx;
@@ -2630,7 +2949,9 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
     R thR, dteR;
     if constexpr (sizeof(R) == 4) {
         const float s = cf[e];
-        thR = __fmul_rn((float)*dtp, __fmul_rn(s, m.inv_h_f));
+        float dth, dtl;
+        split_ff(*dtp, dth, dtl);
+        thR = __fmul_rn(__fadd_rn(dth, dtl), __fmul_rn(s, m.inv_h_f));
         dteR = __fmul_rn(m.h_f, __frcp_rn(s));
     } else {
         thR = *dtp * dte_a[2 * m.E + e];
@@ -2639,7 +2960,8 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
     if (valid && c == 0 && thR > R(1)) atomicAdd(&cnt[CNT_CFL], 1ull);
     const double ubd = ube[c * m.E + e];
     R ubh, ubo;
-    split<R>(ubd, ubh, ubo);
+    if constexpr (sizeof(R) == 4) split_ff(ubd, ubh, ubo);
+    else split<R>(ubd, ubh, ubo);
     R U[N2], F[N2];
     load_comp<R, P>(u + c * m.NN, m, ex, ey, U);
     if (pr.mode == MODE_LO) {
@@ -2699,16 +3021,12 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
     if (pr.mode == MODE_WENO_L) {
 #pragma unroll
         for (int i = 0; i < N2; ++i) sF[i][c][tx] = F[i];
-        sU[c][tx] = ubd;
+        sU[c][tx] = narrow(ubd);
         __syncthreads();
-        double ub[NC], b = 1.0;
         float ubf[NC];
         const bool cert = !(pr.opts & OPT_FP64_LIMITER);
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            ub[k] = sU[k][tx];
-            ubf[k] = (float)ub[k];
-        }
+        for (int k = 0; k < NC; ++k) ubf[k] = sU[k][tx];
 #pragma unroll 1
         for (int i = c; i < N2; i += NC) {
             // float32 certificate first; the float64 formula only where it
@@ -2716,25 +3034,30 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
             if (cert) {
                 float ff[NC];
 #pragma unroll
-                for (int k = 0; k < NC; ++k) ff[k] = (float)sF[i][k][tx];
+                for (int k = 0; k < NC; ++k) ff[k] = sizeof(R) == 4 ? (float)sF[i][k][tx] : narrow((double)sF[i][k][tx]);
                 float mi = m.me_f;
                 if (lgl) mi = (float)(m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]));
                 if (euler_alpha_is_one(ubf, ff, mi, pr.ome_f)) continue;
             }
-            double f[NC];
+            double f[NC], ub[NC];
 #pragma unroll
-            for (int k = 0; k < NC; ++k) f[k] = (double)sF[i][k][tx];
+            for (int k = 0; k < NC; ++k) {
+                f[k] = (double)sF[i][k][tx];
+                ub[k] = ube[k * m.E + e];
+            }
             const double mi = lgl ? m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]) : m.me;
-            b = fmin(b, euler_alpha_rare(ub, f, mi, pr.pos_eps));
+            beta = fmin(beta, R(euler_alpha_rare(ub, f, mi, pr.pos_eps)));  // rounding keeps the order
         }
-        sB[c][tx] = b;
+        sB[c][tx] = beta;
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < NC; ++k) b = fmin(b, sB[k][tx]);
-        beta = R(b);
+        for (int k = 0; k < NC; ++k) beta = fmin(beta, sB[k][tx]);
     }
     if (!valid) return;
-    if (c == 0) beta_out[e] = (double)beta;
+    if (c == 0) {
+        if constexpr (sizeof(R) == 4) beta_out[e] = widen(beta);
+        else beta_out[e] = beta;
+    }
     R* __restrict__ out = EW + ((long long)c * m.E + e);
 #pragma unroll
     for (int i = 0; i < N2; ++i) {

@@ -23,7 +23,7 @@ struct Bufs {
     void* fl;     // low-order facet fluxes [E][4][NC]         (R)
     float* cf;    // float copies for the Euler limiter certificate [1+NC][E]: s, ubar^{e,L}
     float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_pre for scalars)
-    float* cq;    // FP32-mixed systems: flux of the mean and speed parts per cell [2NC + 5][E] (k_avg)
+    void* cq;     // systems: flux of the mean and speed parts per cell [2NC + 6][E]  (R) (k_avg)
     void* fht;    // facet terms of f_i^e [NC][E]  (R) (k_facet -> k_update_el, k_upd_sys)
     cudaStream_t st2;            // second stream of a stage (k_facet)
     cudaEvent_t ev_fork0, ev_fork, ev_w, ev_join;
@@ -166,6 +166,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     // (24 modes of 340 elements are 65 KB there)
     constexpr int STY = sizeof(R) == 4 ? 8 : 4;
     const dim3 bs(K_TX, STY), gs(nblk(m.nx, K_TX), nblk(m.ny, STY));
+    // the facet tiles of systems (k_lo_sys, k_facet_sys)
+    const dim3 bf(F_TX, F_TY), gf(nblk(m.nx, F_TX), nblk(m.ny, F_TY));
     // per-launch timing records events between kernels: plain launches then
     const bool pdl = prof == nullptr;
     cudaError_t err = cudaSuccess;
@@ -191,20 +193,18 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         chk(cudaEventRecord(B.ev_w, s2));
     }
     constexpr bool use_avg = sizeof(R) == 4 && NC > 1;
-    if constexpr (use_avg)
-        CGL_LAUNCH(prof, KID_AVG, st, chk(launch(pdl, k_avg<P, Ph>, ge, be, st, m, pr, (const float*)u, B.avg, B.cq)));
-    if constexpr (use_avg) {
-        // mixed systems: the low-order part here, the sensor in k_sens below
-        auto* kpre = (pr.opts & OPT_SUBCELL_DT) ? k_pre_lo<P, Ph, true> : k_pre_lo<P, Ph, false>;
+    if constexpr (NC > 1) {
+        // the low-order part here, the sensor in k_sens below
+        CGL_LAUNCH(prof, KID_AVG, st, chk(launch(pdl, k_avg<R, P, Ph>, ge, be, st, m, pr, (const R*)u, B.avg, B.ue, (R*)B.cq)));
+        auto* klo = (pr.opts & OPT_SUBCELL_DT) ? k_lo_sys<R, P, Ph, true> : k_lo_sys<R, P, Ph, false>;
         CGL_LAUNCH(prof, KID_PRE, st,
-                   chk(launch(pdl, kpre, ge, be, st, m, pr, (const float*)u, B.ue, B.dte, B.ubl, (float*)B.fl, B.cf,
-                              B.avg, (const float*)B.cq, first ? B.dtbits : nullptr)));
+                   chk(launch(pdl, klo, gf, bf, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.fl, B.cf,
+                              (const float*)B.avg, (const R*)B.cq, first ? B.dtbits : nullptr)));
     } else {
         auto* kpre = (pr.opts & OPT_SUBCELL_DT) ? k_pre<R, P, Ph, true> : k_pre<R, P, Ph, false>;
         CGL_LAUNCH(prof, KID_PRE, st,
                    chk(launch(pdl, kpre, ge, be, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, B.gam, B.nu,
-                              (R*)B.q, (R*)B.fl, (R*)nullptr, B.cf, B.avg,
-                              first ? B.dtbits : nullptr)));
+                              (R*)B.q, (R*)B.fl, B.cf, B.avg, first ? B.dtbits : nullptr)));
     }
     if (first)
         CGL_LAUNCH(prof, KID_DT, st,
@@ -227,10 +227,15 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
                            chk(launch(false, k_sens<float, P, Ph, STY>, gs, bs, s2, m, pr, (const float*)u, B.gam, B.nu)));
                 chk(cudaEventRecord(B.ev_w, s2));
             }
-            CGL_LAUNCH(prof, KID_FACET, s2,
-                       chk(launch(false, k_facet<float, P, Ph>, ge, be, s2, m, pr, (const float*)u, (const double*)B.ue,
-                                  B.dte, (const double*)B.ubl, (const float*)B.q, (const float*)B.fl, B.cf, B.ube,
-                                  (float*)B.fht, B.cnt)));
+            if constexpr (NC > 1)
+                CGL_LAUNCH(prof, KID_FACET, s2,
+                           chk(launch(false, k_facet_sys<R, P, Ph>, gf, bf, s2, m, pr, (const R*)u, (const double*)B.ue,
+                                      B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
+            else
+                CGL_LAUNCH(prof, KID_FACET, s2,
+                           chk(launch(false, k_facet<P, Ph>, ge, be, s2, m, pr, (const float*)u, (const double*)B.ue,
+                                      B.dte, (const double*)B.ubl, (const float*)B.q, (const float*)B.fl, B.cf, B.ube,
+                                      (float*)B.fht, B.cnt)));
             chk(cudaEventRecord(B.ev_join, s2));
         }
     }
@@ -243,9 +248,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         if constexpr (!split_update)
             if (!q1)
                 CGL_LAUNCH(prof, KID_FACET, st,
-                           chk(launch(pdl, k_facet<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const double*)B.ue,
-                                      B.dte, (const double*)B.ubl, (const R*)B.q, (const R*)B.fl, B.cf, B.ube,
-                                      (R*)B.fht, B.cnt)));
+                           chk(launch(pdl, k_facet_sys<R, P, Ph>, gf, bf, st, m, pr, (const R*)u, (const double*)B.ue,
+                                      B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
     }
     if (q1) {
         CGL_LAUNCH(prof, KID_Q1F, st,
