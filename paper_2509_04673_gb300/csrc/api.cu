@@ -1554,19 +1554,19 @@ extern "C" cgl_status cgl_profile(cgl_state* S, int32_t nsteps, int32_t nk, doub
 extern "C" cgl_status cgl_launches_per_step(cgl_state* S, int64_t* kernels) {
     if (!S || !kernels) return fail(CGL_EINVAL, "null argument");
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
-    const int lo = S->prob.mode == CGL_MODE_LO;
-    int64_t per_stage = 1 + 2 + (lo ? 0 : 3 + (S->prob.k_g + S->prob.k_u));
-    if (S->nc > 1) per_stage += 2;                                // k_avg, k_sens
-    if (S->prec == CGL_FP32_MIXED || S->nc > 1) per_stage += 1;  // k_facet
-    if (S->prec == CGL_FP32_MIXED && !lo && split_residual(S->mesh->m, S->nc)) per_stage += 1;  // k_res_w beside k_res_s
-    if (!lo && !(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
-        // the first sweep of each solve runs inside k_grad_sweep / k_udot_sweep
-        const bool small = S->prec == CGL_FP64 ? small_tiles_of<double>(S->mesh->m) : small_tiles_of<float>(S->mesh->m);
-        per_stage -= (S->prob.k_g >= 1 && fuse_grad_sweep(S->rsz, small)) + (S->prob.k_u >= 1);
-    }
+    const bool lo = S->prob.mode == CGL_MODE_LO, sys = S->nc > 1;
+    // k_lo, k_sens, k_facet, k_update_el, k_final (+ k_avg for systems)
+    int64_t per_stage = 5 + sys;
     if ((S->prob.options & CGL_OPT_AEC_Q1) && !lo) {
-        // k_pre, k_q1_facet, k_udl, k_q1_update, k_final (+ k_avg, k_sens for systems)
-        per_stage = 5 + (S->nc > 1 ? 2 : 0);
+        per_stage += 1;  // k_q1_facet, k_udl, k_q1_update in place of k_facet, k_update_el
+    } else if (!lo) {
+        // k_res_sys or k_res_w and k_res_s, the two right-hand sides, the sweeps
+        per_stage += (sys ? 1 : 2) + 2 + S->prob.k_g + S->prob.k_u;
+        if (!(S->prob.options & CGL_OPT_UNFUSED_SWEEPS)) {
+            // the first sweep of each solve runs inside k_grad_sweep / k_udot_sweep
+            const int size = S->prec == CGL_FP64 ? tile_size_of<double>(S->mesh->m) : tile_size_of<float>(S->mesh->m);
+            per_stage -= (S->prob.k_g >= 1 && fuse_grad_sweep(S->rsz, size)) + (S->prob.k_u >= 1);
+        }
     }
     *kernels = 3 * per_stage + 1;  // + dt finalisation; the time advance rides in the last k_final
     return CGL_OK;

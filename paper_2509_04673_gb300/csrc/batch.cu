@@ -133,7 +133,7 @@ DEV void elem_phase(int phase, const InstDev& D, int ex, int ey, int e, double& 
                                         int ku) {
     switch (phase) {
         case PH_PRE:
-            dte = pre_at<float, P, Ph>(D.m, D.pr, D.u, D.ue, D.dte, D.ubl, D.gam, D.nu, D.q, D.fl, D.cf,
+            dte = pre_at_mixed<P, Ph>(D.m, D.pr, D.u, D.ue, D.dte, D.ubl, D.gam, D.nu, D.q, D.fl, D.cf,
                                        D.avg, ex, ey, e);
             break;
         case PH_RES:
@@ -149,16 +149,16 @@ DEV void elem_phase(int phase, const InstDev& D, int ex, int ey, int e, double& 
 template <int P, int PHASE, class Ph>
 DEV void elem_phase_ct(const InstDev& D, const MeshDev& m, int ex, int ey, int e, double& dte, int kg, int ku) {
     if constexpr (PHASE == PH_FACET)
-        facet_el_at<P, Ph>(m, D.pr, D.u, D.ue, D.dte, D.ubl, D.q, D.fl, D.cf, D.ube, D.fht, D.cnt, ex, ey, e);
+        facet_el_at<float, P, Ph>(m, D.pr, D.u, D.ue, D.dte, D.ubl, D.q, D.fl, D.cf, D.ube, D.fht, D.cnt, ex, ey, e);
     else if constexpr (PHASE == PH_UPDATE_EL)
-        update_el_at<P, Ph>(m, D.pr, D.u, ud_final(D, ku), D.ER, D.cf, D.avg, D.ube, D.fht, D.dt, D.EW, D.beta,
+        update_el_at<float, P, Ph>(m, D.pr, D.u, ud_final(D, ku), D.ue, D.dte, D.ER, D.cf, D.avg, D.ube, D.fht, D.dt, D.EW, D.beta,
                             D.cnt, ex, ey, e);
     else if constexpr (PHASE == PH_RES_W)
-        res_w_at<P, Ph>(m, D.pr, D.u, D.EW, ex, ey, e);  // W^e in the increment buffer until PH_UPDATE_EL
+        res_w_at<float, P, Ph>(m, D.pr, D.u, D.EW, ex, ey, e);  // W^e in the increment buffer until PH_UPDATE_EL
     else if constexpr (PHASE == PH_RES_S)
-        res_s_at<P>(m, D.u, g_final(D, kg), D.gam, D.nu, D.EW, D.ER, ex, ey, e);
+        res_s_at<float, P>(m, D.u, g_final(D, kg), D.gam, D.nu, D.EW, D.ER, ex, ey, e);
     else if constexpr (PHASE == PH_PRE)
-        dte = pre_at<float, P, Ph>(m, D.pr, D.u, D.ue, D.dte, D.ubl, D.gam, D.nu, D.q, D.fl, D.cf, D.avg, ex,
+        dte = pre_at_mixed<P, Ph>(m, D.pr, D.u, D.ue, D.dte, D.ubl, D.gam, D.nu, D.q, D.fl, D.cf, D.avg, ex,
                                    ey, e);
     else
         elem_phase<P, Ph>(PHASE, D, ex, ey, e, dte, kg, ku);

@@ -603,23 +603,25 @@ DEV void udot_sweep_seg(const MeshDev& m, const R* ER, R* rout, R* xout, int gx0
 }
 
 // The tiles of the single-state kernels (HALO: of the fused g_h kernel, by two
-// elements smaller in each direction).  Large: 32 (p <= 2) or 16 elements wide
-// and 16 or 8 high, in float64 16 by 16 (p = 3) and 16 by 12 (p = 4), where the
-// float64 pipe pays for every operation on the halo.  Small, for meshes whose
-// large tiles leave SMs idle: in float 16 (p = 1: 32) by 8 or 6; in float64,
-// where a block's work is long against a launch, 8 by 4 to 8.
-template <class R, int P, bool SMALL, bool HALO>
+// elements smaller in each direction).  SIZE 0, large: 32 (p <= 2) or 16
+// elements wide and 16 or 8 high, in float64 16 by 16 (p = 3) and 16 by 12 (p =
+// 4), where the float64 pipe pays for every operation on the halo.  1, for
+// meshes whose large tiles leave SMs idle: 16 (p = 1: 32) by 8 or 6.  2, for
+// tiny meshes in float64, where a block's work is long against a launch: 8 by
+// 4 to 8.
+template <class R, int P, int SIZE, bool HALO>
 struct StageTile {
     static constexpr bool F = sizeof(R) == 4;
-    static constexpr int LX = SMALL ? (F ? (P == 1 ? 32 : 16) : 8) : (P <= 2 ? 32 : 16);
-    static constexpr int NT = SMALL ? (F ? (P == 3 ? 96 : 128) : (P == 3 ? 72 : 64)) : (P == 3 ? 192 : 256);
+    static constexpr int LX = SIZE == 2 ? 8 : SIZE == 1 ? (P == 1 ? 32 : 16) : (P <= 2 ? 32 : 16);
+    static constexpr int NT = SIZE == 2 ? (P == 3 ? 72 : 64) : SIZE == 1 ? (P == 3 ? 96 : 128) : (P == 3 ? 192 : 256);
     static constexpr int RY = NT / (LX * P);
-    static constexpr int ROWS = SMALL ? (RY >= 8 ? 8 : RY == 4 ? (F ? 8 : 4) : 6)
-                                      : (P <= 2 ? 16 : F ? 8 : P == 3 ? 16 : 12);  // y segments
+    static constexpr int ROWS = SIZE == 2 ? (RY >= 8 ? 8 : RY == 4 ? 4 : 6)
+                                : SIZE == 1 ? (RY == 4 ? 8 : 6)
+                                            : (P <= 2 ? 16 : F ? 8 : P == 3 ? 16 : 12);  // y segments
     using type = SegTile<R, P, LX, ROWS / RY, NT, HALO>;
 };
-template <class R, int P, bool SMALL, bool HALO = false>
-using stage_tile_t = typename StageTile<R, P, SMALL, HALO>::type;
+template <class R, int P, int SIZE, bool HALO = false>
+using stage_tile_t = typename StageTile<R, P, SIZE, HALO>::type;
 
 // dynamic shared memory as an array of R (more than 48 KB in float64)
 template <class R>
@@ -628,10 +630,10 @@ DEV R* dyn_shared() {
     return reinterpret_cast<R*>(dyn_smem);
 }
 
-template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT, SMALL ? 1 : (P == 3 ? 4 : 3))
+template <class R, int P, int NC, int SIZE>
+__global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT, SIZE ? 1 : (P == 3 ? 4 : 3))
     k_grad_sweep(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
-    using TL = stage_tile_t<R, P, SMALL, true>;
+    using TL = stage_tile_t<R, P, SIZE, true>;
     // like k_grad_rhs: runs beside k_pre, waits for it before exiting
     pdl_trigger();
     grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
@@ -639,10 +641,10 @@ __global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT, SMALL ? 1 : (P 
     pdl_wait();
 }
 
-template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
+template <class R, int P, int NC, int SIZE>
+__global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_grad_rhs(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
-    using TL = stage_tile_t<R, P, SMALL>;
+    using TL = stage_tile_t<R, P, SIZE>;
     // needs only u, whose last writer completed before k_pre let this kernel
     // start (pdl_wait_then_trigger), so it runs beside k_pre and waits for it
     // only before exiting
@@ -652,19 +654,19 @@ __global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
     pdl_wait();
 }
 
-template <class R, int P, int NC, bool SMALL>
-__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
+template <class R, int P, int NC, int SIZE>
+__global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_udot_sweep(MeshDev m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout) {
-    using TL = stage_tile_t<R, P, SMALL>;
+    using TL = stage_tile_t<R, P, SIZE>;
     pdl_begin();
     udot_sweep_seg<R, P, NC, TL>(m, ER, rout, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
                                  dyn_shared<R>());
 }
 
-template <class R, int P, int NV, bool SMALL>
-__global__ void __launch_bounds__(stage_tile_t<R, P, SMALL>::NT)
+template <class R, int P, int NV, int SIZE>
+__global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_mass_sweep(MeshDev m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout) {
-    using TL = stage_tile_t<R, P, SMALL>;
+    using TL = stage_tile_t<R, P, SIZE>;
     pdl_begin();
     mass_sweep_seg<R, P, NV, TL>(m, xin, b, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
                                  dyn_shared<R>());

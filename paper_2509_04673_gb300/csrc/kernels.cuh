@@ -390,28 +390,6 @@ DEV void lo_facets(const MeshDev& m, const ProbDev& pr, const int (&nb)[4], int 
     }
 }
 
-// cell average u^e (float64) and f(u^e) (evaluated in the bulk precision R,
-// widened) of the block of element (jx, jy)
-template <class R, int P, class Ph>
-DEV void cell_state(const R* __restrict__ u, const MeshDev& m, const ProbDev& pr, int jx, int jy,
-                    double (&avg)[Ph::NC], double (&fx)[Ph::NC], double (&fy)[Ph::NC]) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    R U[NC][N2];
-    load_block<R, P, NC>(u, m, jx, jy, U);
-    R aR[NC], fxR[NC], fyR[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        avg[c] = cell_mean<R, P>(m, U[c]);
-        aR[c] = R(avg[c]);
-    }
-    Ph::template flux<R>(aR, fxR, fyR, pr);
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        fx[c] = (double)fxR[c];
-        fy[c] = (double)fyR[c];
-    }
-}
-
 // the float64 Appendix-A factor where the float32 certificate of the
 // FP32-mixed form could not show alpha = 1 (rare): out of line, so that the
 // unrolled node loop of the slope limiter carries a call per node instead of
@@ -735,9 +713,9 @@ DEV double lo_outputs_mixed(const MeshDev& m, const ProbDev& pr, const float* __
     return dte;
 }
 
-// FP32-mixed scalars, the whole of k_pre for one element (the batched stage
-// and k_pre)
-template <int P, class Ph, bool SUB = false>
+// FP32-mixed scalars, the arithmetic of k_lo and k_sens for one element (the
+// batched stage)
+template <int P, class Ph>
 DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
                         double* __restrict__ ue_out, double* __restrict__ dte_out,
                         double* __restrict__ ubl_out, double* __restrict__ gam_out,
@@ -798,8 +776,8 @@ DEV double pre_at_mixed(const MeshDev& m, const ProbDev& pr, const float* __rest
             F[d][0] = o.v[0];
         }
     }
-    const double dte = lo_outputs_mixed<P, Ph, SUB>(m, pr, u, lam, F, uh, ul, ue_out, dte_out, ubl_out, q_out, fl_out,
-                                                    cf_out, avg, ex, ey, e);
+    const double dte = lo_outputs_mixed<P, Ph, false>(m, pr, u, lam, F, uh, ul, ue_out, dte_out, ubl_out, q_out, fl_out,
+                                                      cf_out, avg, ex, ey, e);
     float gam;
     if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
         gam = sensor_scalar<float, P>(m, pr, u, U, nb, ex, ey);
@@ -858,56 +836,6 @@ DEV double lo_outputs_fp64(const MeshDev& m, const ProbDev& pr, const double* __
     return dte;
 }
 
-template <class R, int P, class Ph, bool SUB = false>
-DEV double pre_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, double* __restrict__ ue_out,
-                  double* __restrict__ dte_out, double* __restrict__ ubl_out,
-                  double* __restrict__ gam_out, double* __restrict__ nu_out,
-                  R* __restrict__ q_out, R* __restrict__ fl_out,
-                  float* __restrict__ cf_out, float* __restrict__ avg, int ex, int ey, int e) {
-    static_assert(Ph::NC == 1, "systems: k_lo_sys and k_sens");
-    if constexpr (sizeof(R) == 4) {
-        return pre_at_mixed<P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, cf_out, avg,
-                                        ex, ey, e);
-    } else {
-        constexpr int N2 = Dim<P>::N2;
-        int nb[4];
-#pragma unroll
-        for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-        R U[N2];
-        load_comp<R, P>(u, m, ex, ey, U);
-        double us[1], fxs[1], fys[1];
-        us[0] = cell_mean<R, P>(m, U);
-        ue_out[e] = us[0];
-        Ph::template flux<R>(us, fxs, fys, pr);
-        double uo[4][1], fxo[4][1], fyo[4][1];
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            uo[d][0] = fxo[d][0] = fyo[d][0] = 0.0;
-            if (nb[d] >= 0) {
-                int jx, jy;
-                neighbour_xy(m, ex, ey, d, jx, jy);
-                cell_state<R, P, Ph>(u, m, pr, jx, jy, uo[d], fxo[d], fyo[d]);
-            }
-        }
-        double lam[4], FL[4][1];
-        lo_facets<Ph, R>(m, pr, nb, ex, ey, us, fxs, fys, uo, fxo, fyo, lam, FL);
-        const double dte = lo_outputs_fp64<P, Ph, SUB>(m, pr, u, lam, FL, us, dte_out, ubl_out, q_out, fl_out, cf_out, ex,
-                                                       ey, e);
-        double gam;
-        if (pr.mode == MODE_WENO || pr.mode == MODE_WENO_L) {
-            gam = sensor_scalar<R, P>(m, pr, u, U, nb, ex, ey);
-        } else {
-            gam = (pr.mode == MODE_HO) ? 1.0 : 0.0;
-        }
-        gam_out[e] = gam;
-        R lm = R(0);
-#pragma unroll
-        for (int i = 0; i < N2; ++i) lm = fmax(lm, Ph::template node_speed<R>(&U[i], pr));
-        nu_out[e] = lm * (m.h * (0.5 / P));
-        return dte;
-    }
-}
-
 // k_avg (systems): cell means of every element, read by k_lo_sys for the facets
 // of the cell instead of its coefficient block: float-float in the FP32-mixed
 // form (avg[(2c) E + e] high, avg[(2c+1) E + e] low part of component c), u^e
@@ -950,38 +878,107 @@ __global__ void k_avg(MeshDev m, ProbDev pr, const R* __restrict__ u, float* __r
     for (int k = 0; k < Ph::NPART; ++k) cq[(2 * NC + k) * m.E + e] = q[k];
 }
 
-// Resident blocks of 128 threads per SM requested from the compiler for the
-// one-thread-per-element kernels (a register cap of 65536 / (128 n)),
-// chosen by measurement on GB300 (time per launch against the uncapped
-// form): FP32-mixed Euler at p = 2 (blast 2048^2 Q2) k_pre_lo 5 (-13 %),
-// k_facet 7 (-25 %), k_res_ev and k_update_el 4 (-8 %, -13 %); at p = 3
-// (quadrants 512^2 Q3) k_pre_lo 5 (-9 %), k_facet 6 (-17 %), the residual
-// and the update uncapped (3 blocks: +18 %, +7 %); the FP64 Euler p = 2
-// residual and update 3; every other instantiation 1 (the compiler's choice).
-enum { EK_PRE_LO = 0, EK_FACET, EK_RES, EK_UPD };
-template <int P, int NC, int RSZ>
-constexpr int elem_blocks(int k) {
-    if (NC > 1 && P == 2) {
-        if (RSZ == 8) return (k == EK_RES || k == EK_UPD) ? 3 : 1;
-        return k == EK_PRE_LO ? 5 : k == EK_FACET ? 7 : 4;
-    }
-    if (NC > 1 && P == 3 && RSZ == 4) return k == EK_PRE_LO ? 5 : k == EK_FACET ? 6 : 1;
-    return 1;
+// element of position i of a tile's halo rows (tiles of K_TX x TY elements, one
+// element of halo): false where it does not exist or no element of the tile
+// reads it (wrapped once on periodic directions)
+constexpr int K_TX = 32;
+template <int TY>
+DEV bool halo_elem(const MeshDev& m, int ex0, int ey0, int i, int& jx, int& jy) {
+    constexpr int HX = K_TX + 2;
+    const int hy = i / HX, hx = i - hy * HX;
+    jx = ex0 + hx - 1;
+    jy = ey0 + hy - 1;
+    if ((hx == 0 || hx == HX - 1) && (hy == 0 || hy == TY + 1)) return false;
+    if (jx > m.nx || jy > m.ny) return false;
+    if (m.px) jx = jx < 0 ? m.nx - 1 : (jx == m.nx ? 0 : jx);
+    if (m.py) jy = jy < 0 ? m.ny - 1 : (jy == m.ny ? 0 : jy);
+    return jx >= 0 && jx < m.nx && jy >= 0 && jy < m.ny;
+}
+// halo position of the face neighbour d of the tile element (tx, ty) (-1: its own)
+DEV int halo_pos(int tx, int ty, int d) {
+    return (ty + 1 + (d == 2 ? -1 : d == 3 ? 1 : 0)) * (K_TX + 2) + tx + 1 + (d == 0 ? -1 : d == 1 ? 1 : 0);
 }
 
-template <class R, int P, class Ph, bool SUB = false>
-__global__ void k_pre(MeshDev m, ProbDev pr, const R* __restrict__ u, double* __restrict__ ue_out,
-                      double* __restrict__ dte_out, double* __restrict__ ubl_out,
-                      double* __restrict__ gam_out, double* __restrict__ nu_out,
-                      R* __restrict__ q_out, R* __restrict__ fl_out,
-                      float* __restrict__ cf_out, float* __restrict__ avg,
-                      unsigned long long* __restrict__ dtbits) {
+// scalars: the low-order part of the stage (cell means, facet speeds and f^L,
+// dt_e, ubar^{e,L}, the flux-limiter capacities); gamma_e and nu_e come from
+// k_sens, which runs beside it.  The means and their fluxes of a tile of 32 x
+// TY elements and its halo are formed once in shared memory, instead of five
+// times per element.  The arithmetic of pre_at.
+template <class R, int P, class Ph, int TY, bool SUB = false>
+__global__ void __launch_bounds__(K_TX * TY) k_lo(MeshDev m, ProbDev pr, const R* __restrict__ u,
+                                                  double* __restrict__ ue_out, double* __restrict__ dte_out,
+                                                  double* __restrict__ ubl_out, R* __restrict__ q_out,
+                                                  R* __restrict__ fl_out, float* __restrict__ cf_out,
+                                                  float* __restrict__ avg, unsigned long long* __restrict__ dtbits) {
+    constexpr int N2 = Dim<P>::N2, HE = (K_TX + 2) * (TY + 2), NT = K_TX * TY;
+    __shared__ R sA[HE], sL[sizeof(R) == 4 ? HE : 1], sX[HE], sY[HE];  // mean (high, low part), its fluxes
     pdl_wait_then_trigger();
-    int ex, ey, e;
+    const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * K_TX, ey0 = blockIdx.y * TY;
+    for (int i = ty * K_TX + tx; i < HE; i += NT) {
+        int jx, jy;
+        if (!halo_elem<TY>(m, ex0, ey0, i, jx, jy)) continue;
+        R B[N2], a[1], fx[1], fy[1];
+        load_comp<R, P>(u, m, jx, jy, B);
+        if constexpr (sizeof(R) == 4) ff_mean<N2>(B, a[0], sL[i]);
+        else a[0] = cell_mean<R, P>(m, B);
+        Ph::template flux<R>(a, fx, fy, pr);
+        sA[i] = a[0];
+        sX[i] = fx[0];
+        sY[i] = fy[0];
+    }
+    __syncthreads();
+    const int ex = ex0 + tx, ey = ey0 + ty, e = ey * m.nx + ex;
     double dte = __longlong_as_double(0x7ff0000000000000LL);
-    if (elem_of_thread(m, ex, ey, e))
-        dte = pre_at<R, P, Ph, SUB>(m, pr, u, ue_out, dte_out, ubl_out, gam_out, nu_out, q_out, fl_out, cf_out,
-                                    avg, ex, ey, e);
+    if (ex < m.nx && ey < m.ny) {
+        int nb[4];
+#pragma unroll
+        for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
+        const int own = halo_pos(tx, ty, -1);
+        R us[1] = {sA[own]}, lam[4], F[4][1];
+        const R fxs[1] = {sX[own]}, fys[1] = {sY[own]};
+        if constexpr (sizeof(R) == 4) {
+            const float ul[1] = {sL[own]};
+            const float inflate = 1.0f + 0x1p-20f;
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+                const bool xf = d < 2, self_is_L = (d == 1 || d == 3);
+                if (nb[d] >= 0) {
+                    const int j = halo_pos(tx, ty, d);
+                    const float oh = sA[j], ol = sL[j], of = xf ? sX[j] : sY[j], sf = xf ? fxs[0] : fys[0];
+                    const float Lh = self_is_L ? us[0] : oh, Rh = self_is_L ? oh : us[0];
+                    const float Ll = self_is_L ? ul[0] : ol, Rl = self_is_L ? ol : ul[0];
+                    const float l = __fmul_rn(
+                        Ph::template max_speed<float>(&Lh, &Rh, xf ? 1.f : 0.f, xf ? 0.f : 1.f, pr), inflate);
+                    lam[d] = l;
+                    F[d][0] = llf_value(self_is_L ? sf : of, self_is_L ? of : sf, l, ff_diff(Rh, Rl, Lh, Ll));
+                } else {
+                    // boundary facet: out of line (rare; keeps the hot code small)
+                    CompVec<float, 1> vh, vl, vf;
+                    vh.v[0] = us[0];
+                    vl.v[0] = ul[0];
+                    vf.v[0] = xf ? fxs[0] : fys[0];
+                    const CompVec<float, 2> o =
+                        boundary_facet_lo<Ph>(m, pr, d, ex, ey, self_is_L ? 1.f : -1.f, vh, vl, vf);
+                    lam[d] = o.v[1];
+                    F[d][0] = o.v[0];
+                }
+            }
+            dte = lo_outputs_mixed<P, Ph, SUB>(m, pr, u, lam, F, us, ul, ue_out, dte_out, ubl_out, q_out, fl_out, cf_out,
+                                               avg, ex, ey, e);
+        } else {
+            ue_out[e] = us[0];
+            double uo[4][1], fxo[4][1], fyo[4][1];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+                const int j = halo_pos(tx, ty, d);
+                uo[d][0] = nb[d] >= 0 ? sA[j] : 0.0;
+                fxo[d][0] = nb[d] >= 0 ? sX[j] : 0.0;
+                fyo[d][0] = nb[d] >= 0 ? sY[j] : 0.0;
+            }
+            lo_facets<Ph, R>(m, pr, nb, ex, ey, us, fxs, fys, uo, fxo, fyo, lam, F);
+            dte = lo_outputs_fp64<P, Ph, SUB>(m, pr, u, lam, F, us, dte_out, ubl_out, q_out, fl_out, cf_out, ex, ey, e);
+        }
+    }
     if (dtbits) block_min_to(dte, dtbits);
 }
 
@@ -1159,32 +1156,12 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 3)
     if (dtbits) block_min_to(dte, dtbits);
 }
 
-// systems: the WENO sensor gamma_e (eqs. (WENO:alpha), (WENO:norm)) and nu_e
-// (eq. (stab:WENO)).  A block of K_TX x TY threads holds a tile of K_TX x TY
+// the WENO sensor gamma_e (eqs. (WENO:alpha), (WENO:norm)) and nu_e (eq.
+// (stab:WENO)).  A block of K_TX x TY threads holds a tile of K_TX x TY
 // elements; component by component it puts the modal coefficients of the tile
 // and its one-element halo in shared memory (modal.cuh), so that each block of
 // coefficients is loaded and transformed 1.3 to 1.6 times instead of five,
 // and one thread per element evaluates the sensor from them.
-constexpr int K_TX = 32;
-// element of position i of a tile's halo rows: false where it does not exist
-// or no sensor of the tile reads it (wrapped once on periodic directions)
-template <int TY>
-DEV bool halo_elem(const MeshDev& m, int ex0, int ey0, int i, int& jx, int& jy) {
-    constexpr int HX = K_TX + 2;
-    const int hy = i / HX, hx = i - hy * HX;
-    jx = ex0 + hx - 1;
-    jy = ey0 + hy - 1;
-    if ((hx == 0 || hx == HX - 1) && (hy == 0 || hy == TY + 1)) return false;
-    if (jx > m.nx || jy > m.ny) return false;
-    if (m.px) jx = jx < 0 ? m.nx - 1 : (jx == m.nx ? 0 : jx);
-    if (m.py) jy = jy < 0 ? m.ny - 1 : (jy == m.ny ? 0 : jy);
-    return jx >= 0 && jx < m.nx && jy >= 0 && jy < m.ny;
-}
-// halo position of the face neighbour d of the tile element (tx, ty)
-DEV int halo_pos(int tx, int ty, int d) {
-    return (ty + 1 + (d == 2 ? -1 : d == 3 ? 1 : 0)) * (K_TX + 2) + tx + 1 + (d == 0 ? -1 : d == 1 ? 1 : 0);
-}
-
 // The node speeds of nu_e are formed once per node of the tile (an element
 // has (p+1)^2 nodes but brings p^2 new ones) and pass through the same
 // shared memory.
@@ -1736,16 +1713,6 @@ DEV void res_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, co
     load_comp<R, P>(u, m, ex, ey, U);
     w_part<R, P, Ph>(m, pr, U, ex, ey, W);
     stab_part<R, P>(m, U, g, gam, nu, W, ER, ex, ey, e);
-}
-
-template <class R, int P, class Ph>
-__global__ void __launch_bounds__(128) k_res_ev(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ g,
-                         const double* __restrict__ gam, const double* __restrict__ nu,
-                         R* __restrict__ ER) {
-    pdl_begin();
-    int ex, ey, e;
-    if (!elem_of_thread(m, ex, ey, e)) return;
-    res_at<R, P, Ph>(m, pr, u, g, gam, nu, ER, ex, ey, e);
 }
 
 // The residual of systems with one thread per element and component: a block
@@ -2355,20 +2322,28 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
                 gm = R(me * (pr.umin - ubec[0]));
             }
             R b = R(1);
+            if (!lgl) {
+                // the gaps are the same for every node and the quotients
+                // monotone: the smallest comes from the extreme contributions
+                R hi = R(0), lo = R(0);
 #pragma unroll
-            for (int i = 0; i < N2; ++i) {
-                R f = F[0][i];
-                R gpi = gp, gmi = gm;
-                if (lgl) {
+                for (int i = 0; i < N2; ++i) {
+                    hi = fmax(hi, F[0][i]);
+                    lo = fmin(lo, F[0][i]);
+                }
+                if (hi > R(0)) b = fmin(b, gp / hi);
+                if (lo < R(0)) b = fmin(b, gm / lo);
+            } else {
+#pragma unroll
+                for (int i = 0; i < N2; ++i) {
+                    const R f = F[0][i];
                     // m_i^e of this node (the gaps scale with it)
                     const double mi = m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]);
-                    gpi = R(mi * (pr.umax - ubec[0]));
-                    gmi = R(mi * (pr.umin - ubec[0]));
+                    R bi = R(1);
+                    if (f > R(0)) bi = fmin(R(1), R(mi * (pr.umax - ubec[0])) / f);
+                    else if (f < R(0)) bi = fmin(R(1), R(mi * (pr.umin - ubec[0])) / f);
+                    b = fmin(b, bi);
                 }
-                R bi = R(1);
-                if (f > R(0)) bi = fmin(R(1), gpi / f);
-                else if (f < R(0)) bi = fmin(R(1), gmi / f);
-                b = fmin(b, bi);
             }
             beta = fmin(fmax(b, R(0)), R(1));
         } else {
@@ -2607,102 +2582,82 @@ __global__ void __launch_bounds__(128) k_q1_update(MeshDev m, ProbDev pr, const 
                                  beta_out, cnt, ex, ey, e, gam[e]);
 }
 
-// Euler at p = 2: 3 blocks of 128 per SM (a 170-register cap, no spills)
-// instead of the 2 that the uncapped allocation leaves (measured faster)
-template <class R, int P, class Ph>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, sizeof(R)>(EK_UPD)) k_update_ev(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ ud,
-                            const double* __restrict__ ue, double* dte_a, const double* __restrict__ ubl,
-                            const R* __restrict__ qcap, const R* __restrict__ fl_in,
-                            const R* __restrict__ ER, const float* __restrict__ cf,
-                            const float* __restrict__ avg,
-                            const double* __restrict__ dtp, R* __restrict__ EW,
-                            double* __restrict__ ube_out, double* __restrict__ beta_out,
-                            unsigned long long* __restrict__ cnt) {
-    pdl_begin();
-    int ex, ey, e;
-    if (!elem_of_thread(m, ex, ey, e)) return;
-    update_at<R, P, Ph>(m, pr, u, ud, ue, dte_a, ubl, qcap, fl_in, ER, cf, avg, dtp, EW, ube_out, beta_out, cnt, ex,
-                        ey, e);
-}
-
-
-// FP32-mixed scalars: the update in two kernels.  k_facet needs only u and the
-// outputs of k_pre, so it runs on a second stream beside the g_h and udot
-// kernels; k_update_el then reads its ubar^e and facet terms.  Together they
-// compute what k_update_ev computes, in the same arithmetic.  The bodies are
+// Scalars: the update in two kernels.  k_facet needs only u and the outputs of
+// k_lo, so it runs on a second stream beside the g_h and udot kernels;
+// k_update_el then reads its ubar^e and facet terms.  The bodies are
 // device functions of one element, also run by the batched stage.
-template <int P, class Ph>
-DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
+template <class R, int P, class Ph>
+DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
                      const double* __restrict__ ue, double* dte_a, const double* __restrict__ ubl,
-                     const float* __restrict__ qcap, const float* __restrict__ fl_in, float* cf,
-                     double* __restrict__ ube_out, float* __restrict__ fht, unsigned long long* __restrict__ cnt,
+                     const R* __restrict__ qcap, const R* __restrict__ fl_in, float* cf,
+                     double* __restrict__ ube_out, R* __restrict__ fht, unsigned long long* __restrict__ cnt,
                      int ex, int ey, int e) {
     constexpr int N2 = Dim<P>::N2;
     int nb[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
-    float U[1][N2];
-    load_block<float, P, 1>(u, m, ex, ey, U);
+    R U[1][N2];
+    load_block<R, P, 1>(u, m, ex, ey, U);
     double uec[1], ublc[1], ubec[1];
-    float fh[1];
+    R fh[1];
     uec[0] = pr.fl == FL_NONE ? ue[e] : 0.0;  // u^e enters ubar^e only without the flux limiter
     ublc[0] = ubl[e];
     const double rs = dte_a[m.E + e];
     double rs2;
-    facet_part<float, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
+    facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
     ube_out[e] = ubec[0];
     fht[e] = fh[0];
     if (rs2 != rs) store_reduced_step(m, dte_a, cf, rs2, e);
 }
 
-template <int P, class Ph>
-DEV void update_el_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u,
-                      const float* __restrict__ ud, const float* __restrict__ ER, const float* __restrict__ cf,
+template <class R, int P, class Ph>
+DEV void update_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
+                      const R* __restrict__ ud, const double* __restrict__ ue, const double* __restrict__ dte_a,
+                      const R* __restrict__ ER, const float* __restrict__ cf,
                       const float* __restrict__ avg, const double* __restrict__ ube,
-                      const float* __restrict__ fht, const double* __restrict__ dtp, float* __restrict__ EW,
+                      const R* __restrict__ fht, const double* __restrict__ dtp, R* __restrict__ EW,
                       double* __restrict__ beta_out, unsigned long long* __restrict__ cnt, int ex, int ey, int e) {
-    constexpr int NC = Ph::NC, N2 = Dim<P>::N2;
-    float U[NC][N2];
-    load_block<float, P, NC>(u, m, ex, ey, U);
+    constexpr int N2 = Dim<P>::N2;
+    R U[1][N2];
+    load_block<R, P, 1>(u, m, ex, ey, U);
+    const double ubec[1] = {ube[e]};
+    const R fh[1] = {fht[e]};
     // the float path of element_part takes dt_e and theta from the float
-    // speed sum and the mean from the float-float pair: u^e, dt_e and 1/dt_e
-    // in float64 are not read
-    double uec[NC], ubec[NC];
-    float fh[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        uec[c] = 0.0;
-        ubec[c] = ube[c * m.E + e];
-        fh[c] = fht[c * m.E + e];
+    // speed sum and the mean from the float-float pair
+    if constexpr (sizeof(R) == 4) {
+        const double uec[1] = {0.0};
+        element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, 0.0, 0.0, ubec, fh, EW, beta_out, cnt, ex, ey, e);
+    } else {
+        const double uec[1] = {ue[e]};
+        element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, dte_a[e], dte_a[2 * m.E + e], ubec, fh, EW, beta_out,
+                               cnt, ex, ey, e);
     }
-    element_part<float, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, 0.0, 0.0, ubec, fh, EW, beta_out, cnt, ex, ey,
-                               e);
 }
 
-template <int P, class Ph>
-__global__ void __launch_bounds__(128) k_facet(MeshDev m, ProbDev pr, const float* __restrict__ u,
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(128) k_facet(MeshDev m, ProbDev pr, const R* __restrict__ u,
                                                const double* __restrict__ ue, double* dte_a,
-                                               const double* __restrict__ ubl, const float* __restrict__ qcap,
-                                               const float* __restrict__ fl_in, float* cf,
-                                               double* __restrict__ ube_out, float* __restrict__ fht,
+                                               const double* __restrict__ ubl, const R* __restrict__ qcap,
+                                               const R* __restrict__ fl_in, float* cf,
+                                               double* __restrict__ ube_out, R* __restrict__ fht,
                                                unsigned long long* __restrict__ cnt) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    facet_el_at<P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
+    facet_el_at<R, P, Ph>(m, pr, u, ue, dte_a, ubl, qcap, fl_in, cf, ube_out, fht, cnt, ex, ey, e);
 }
 
-template <int P, class Ph>
-__global__ void __launch_bounds__(128, elem_blocks<P, Ph::NC, 4>(EK_UPD))
-    k_update_el(MeshDev m, ProbDev pr, const float* __restrict__ u, const float* __restrict__ ud,
-                const double* __restrict__ ue, const double* __restrict__ dte_a, const float* __restrict__ ER,
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(128)
+    k_update_el(MeshDev m, ProbDev pr, const R* __restrict__ u, const R* __restrict__ ud,
+                const double* __restrict__ ue, const double* __restrict__ dte_a, const R* __restrict__ ER,
                 const float* __restrict__ cf, const float* __restrict__ avg, const double* __restrict__ ube,
-                const float* __restrict__ fht, const double* __restrict__ dtp, float* __restrict__ EW,
+                const R* __restrict__ fht, const double* __restrict__ dtp, R* __restrict__ EW,
                 double* __restrict__ beta_out, unsigned long long* __restrict__ cnt) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    update_el_at<P, Ph>(m, pr, u, ud, ER, cf, avg, ube, fht, dtp, EW, beta_out, cnt, ex, ey, e);
+    update_el_at<R, P, Ph>(m, pr, u, ud, ue, dte_a, ER, cf, avg, ube, fht, dtp, EW, beta_out, cnt, ex, ey, e);
 }
 
 // The facet part of the update of systems: f^H (eq. (hoflux)), the facet
@@ -3066,51 +3021,50 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
     }
 }
 
-// FP32-mixed: the residual in two kernels.  k_res_w (the Galerkin part W^e,
-// needs only u) runs on the second stream from the start of the stage,
-// beside k_pre and the g_h kernels; k_res_s adds the stabilisation, which
-// needs g_h, gamma_e and nu_e.  W^e passes through the increment buffer,
-// which is free until k_update_el.  Same device functions as k_res_ev.
-template <int P, class Ph>
-DEV void res_w_at(const MeshDev& m, const ProbDev& pr, const float* __restrict__ u, float* __restrict__ WV, int ex,
-                  int ey, int e) {
+// Scalars: the residual in two kernels.  k_res_w (the Galerkin part W^e, needs
+// only u) runs on the second stream from the start of the stage, beside k_lo
+// and the g_h kernels; k_res_s adds the stabilisation, which needs g_h,
+// gamma_e and nu_e.  W^e passes through the increment buffer, which is free
+// until k_update_el.
+template <class R, int P, class Ph>
+DEV void res_w_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u, R* __restrict__ WV, int ex, int ey,
+                  int e) {
     constexpr int N2 = Dim<P>::N2;
-    float U[N2], W[N2];
-    load_comp<float, P>(u, m, ex, ey, U);
-    w_part<float, P, Ph>(m, pr, U, ex, ey, W);
+    R U[N2], W[N2];
+    load_comp<R, P>(u, m, ex, ey, U);
+    w_part<R, P, Ph>(m, pr, U, ex, ey, W);
 #pragma unroll
     for (int i = 0; i < N2; ++i) WV[ev_at(m.E, e, i, 0, 1)] = W[i];
 }
 
-template <int P>
-DEV void res_s_at(const MeshDev& m, const float* __restrict__ u, const float* __restrict__ g,
-                  const double* __restrict__ gam, const double* __restrict__ nu, const float* __restrict__ WV,
-                  float* __restrict__ ER, int ex, int ey, int e) {
+template <class R, int P>
+DEV void res_s_at(const MeshDev& m, const R* __restrict__ u, const R* __restrict__ g,
+                  const double* __restrict__ gam, const double* __restrict__ nu, const R* __restrict__ WV,
+                  R* __restrict__ ER, int ex, int ey, int e) {
     constexpr int N2 = Dim<P>::N2;
-    float U[N2], W[N2];
-    load_comp<float, P>(u, m, ex, ey, U);
+    R U[N2], W[N2];
+    load_comp<R, P>(u, m, ex, ey, U);
 #pragma unroll
     for (int i = 0; i < N2; ++i) W[i] = WV[ev_at(m.E, e, i, 0, 1)];
-    stab_part<float, P>(m, U, g, gam, nu, W, ER, ex, ey, e);
+    stab_part<R, P>(m, U, g, gam, nu, W, ER, ex, ey, e);
 }
 
-template <int P, class Ph>
-__global__ void __launch_bounds__(128) k_res_w(MeshDev m, ProbDev pr, const float* __restrict__ u,
-                                               float* __restrict__ WV) {
+template <class R, int P, class Ph>
+__global__ void __launch_bounds__(128) k_res_w(MeshDev m, ProbDev pr, const R* __restrict__ u, R* __restrict__ WV) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    res_w_at<P, Ph>(m, pr, u, WV, ex, ey, e);
+    res_w_at<R, P, Ph>(m, pr, u, WV, ex, ey, e);
 }
 
-template <int P>
-__global__ void __launch_bounds__(128) k_res_s(MeshDev m, const float* __restrict__ u, const float* __restrict__ g,
+template <class R, int P>
+__global__ void __launch_bounds__(128) k_res_s(MeshDev m, const R* __restrict__ u, const R* __restrict__ g,
                                                const double* __restrict__ gam, const double* __restrict__ nu,
-                                               const float* __restrict__ WV, float* __restrict__ ER) {
+                                               const R* __restrict__ WV, R* __restrict__ ER) {
     pdl_begin();
     int ex, ey, e;
     if (!elem_of_thread(m, ex, ey, e)) return;
-    res_s_at<P>(m, u, g, gam, nu, WV, ER, ex, ey, e);
+    res_s_at<R, P>(m, u, g, gam, nu, WV, ER, ex, ey, e);
 }
 
 // ---------------------------------------------------------------------------

@@ -2,6 +2,8 @@
 // the paper: element loop, udot solve, facet loop, element loop, SSP update).
 #pragma once
 
+#include <utility>
+
 #include "fused.cuh"
 
 namespace cgl {
@@ -70,32 +72,31 @@ typedef cudaError_t (*StageFn)(const Bufs&, const MeshDev&, const ProbDev&, doub
 
 inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// small stencil tiles where the large ones (nx by ny nodes) make fewer blocks
-// than this
-constexpr long long SMALL_TILES_BELOW = 304;
-inline bool use_small_tiles(const MeshDev& m, int nx, int ny) {
-    return (long long)nblk(m.nnx, nx) * nblk(m.nny, ny) < SMALL_TILES_BELOW;
+// Size of the stencils' tiles (StageTile): large ones unless they make fewer
+// than two blocks per SM, tiny ones (float64) where the small ones make fewer
+// than one
+template <class R, int P>
+inline int tile_size(const MeshDev& m) {
+    using TL = stage_tile_t<R, P, 0>;
+    using TS = stage_tile_t<R, P, 1>;
+    if ((long long)nblk(m.nnx, TL::NX) * nblk(m.nny, TL::NY) >= 304) return 0;
+    if (sizeof(R) == 4) return 1;
+    return (long long)nblk(m.nnx, TS::NX) * nblk(m.nny, TS::NY) >= 152 ? 1 : 2;
 }
-// the g_h right-hand side and the first sweep in one kernel (rsz: bytes per value)
-inline bool fuse_grad_sweep(size_t rsz, bool small_tiles) { return rsz == 4 || small_tiles; }
-// the same for a state's mesh and precision
 template <class R>
-inline bool small_tiles_of(const MeshDev& m) {
+inline int tile_size_of(const MeshDev& m) {
     switch (m.p) {
-        case 1: return use_small_tiles(m, stage_tile_t<R, 1, false>::NX, stage_tile_t<R, 1, false>::NY);
-        case 2: return use_small_tiles(m, stage_tile_t<R, 2, false>::NX, stage_tile_t<R, 2, false>::NY);
-        case 3: return use_small_tiles(m, stage_tile_t<R, 3, false>::NX, stage_tile_t<R, 3, false>::NY);
-        default: return use_small_tiles(m, stage_tile_t<R, 4, false>::NX, stage_tile_t<R, 4, false>::NY);
+        case 1: return tile_size<R, 1>(m);
+        case 2: return tile_size<R, 2>(m);
+        case 3: return tile_size<R, 3>(m);
+        default: return tile_size<R, 4>(m);
     }
 }
-
-// The split residual (k_res_w on the second stream, k_res_s) overlaps the
-// quadrature with k_pre and the g_h kernels but adds a kernel and the W^e
-// traffic: measured, it wins on KPP 1024^2 (-4 % per step) and loses
-// slightly at 256^2 (+0.7 %); for systems (four components: a W^e of four
-// element vectors) the single k_res_ev is faster (Euler blast 2048^2 Q2:
-// 17.0 against 17.8 ms per step).
-inline bool split_residual(const MeshDev& m, int nc) { return nc == 1 && m.NN >= (1LL << 20); }
+// The g_h right-hand side and the first sweep in one kernel: always in float;
+// in float64 (rsz: bytes per value) only on tiny meshes, elsewhere the sweep's
+// halo costs a fifth of the float64 operations of both kernels and their
+// traffic less.
+inline bool fuse_grad_sweep(size_t rsz, int size) { return rsz == 4 || size == 2; }
 
 // Launch with programmatic stream serialisation (pdl): the kernel may be
 // scheduled while the previous kernel of the stream drains and waits for it
@@ -136,38 +137,69 @@ inline cudaError_t launch_shared(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 
     return cudaLaunchKernelEx(&cfg, k, static_cast<KArgs>(args)...);
 }
 
+// the stencil kernels of a tile size
+template <class R, int P, int NC>
+struct Stencils {
+    void (*grad)(MeshDev, const R*, R*, R*);
+    void (*grad_sweep)(MeshDev, const R*, R*, R*);
+    void (*udot)(MeshDev, const R*, R*, R*);
+    void (*sweep_g)(MeshDev, const R*, const R*, R*);
+    void (*sweep_u)(MeshDev, const R*, const R*, R*);
+    dim3 grid, grid_halo, block;
+    int ws_grad, ws_rhs, ws_udot, ws_sweep;
+};
+template <class R, int P, int NC, int SIZE>
+Stencils<R, P, NC> stencils_of(const MeshDev& m) {
+    using T = stage_tile_t<R, P, SIZE>;
+    using H = stage_tile_t<R, P, SIZE, true>;
+    Stencils<R, P, NC> s;
+    s.grad = k_grad_rhs<R, P, NC, SIZE>;
+    s.grad_sweep = nullptr;
+    if constexpr (sizeof(R) == 4 || SIZE == 2) s.grad_sweep = k_grad_sweep<R, P, NC, SIZE>;
+    s.udot = k_udot_sweep<R, P, NC, SIZE>;
+    s.sweep_g = k_mass_sweep<R, P, 2 * NC, SIZE>;
+    s.sweep_u = k_mass_sweep<R, P, NC, SIZE>;
+    s.grid = dim3(nblk(m.nnx, T::NX), nblk(m.nny, T::NY));
+    s.grid_halo = dim3(nblk(m.nnx, H::NX), nblk(m.nny, H::NY));
+    s.block = dim3(T::NT);
+    s.ws_grad = (int)sizeof(R) * H::grad_ws;
+    s.ws_rhs = (int)sizeof(R) * T::rhs_ws;
+    s.ws_udot = (int)sizeof(R) * T::udot_ws(NC);
+    s.ws_sweep = (int)sizeof(R) * T::sweep_ws;
+    return s;
+}
+
+// Two streams: the second (s2) carries, from the start of the stage, what needs
+// only u, the Galerkin part of a scalar's residual and the sensor, then the
+// facet part of the update, which needs the low-order part; the main stream the
+// low-order part, the g_h solve, the residual, the udot solve, the element part
+// and the node gather.  In float64 on large meshes both fill the same pipe,
+// and the second stream fills the tails of the first.
 template <class R, int P, class Ph>
 cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, double a, double b,
                       bool first, bool dt_only, cudaStream_t st, Prof* prof) {
     ProbDev pr = pr_in;
     if (dt_only) pr.mode = MODE_HO;  // no sensor needed for dt_e
     constexpr int NC = Ph::NC;
-    const dim3 be(64, 2), bn(128, 1);
-    const dim3 ge(nblk(m.nx, 64), nblk(m.ny, 2)), gn(nblk(m.nnx, 128), m.nny);
-    // the stencils' tiles: small ones where the large ones would leave SMs idle
-    using TL = stage_tile_t<R, P, false>;
-    using TS = stage_tile_t<R, P, true>;
-    const bool small_tiles = use_small_tiles(m, TL::NX, TL::NY);
-    const dim3 gl(nblk(m.nnx, TL::NX), nblk(m.nny, TL::NY));
-    const dim3 gt = small_tiles ? dim3(nblk(m.nnx, TS::NX), nblk(m.nny, TS::NY)) : gl, bt(small_tiles ? TS::NT : TL::NT);
-    // the fused g_h kernel's tiles leave room for their halo
-    using HL = stage_tile_t<R, P, false, true>;
-    using HS = stage_tile_t<R, P, true, true>;
-    const dim3 gth = small_tiles ? dim3(nblk(m.nnx, HS::NX), nblk(m.nny, HS::NY)) : dim3(nblk(m.nnx, HL::NX), nblk(m.nny, HL::NY));
-    const int ws = sizeof(R), ws_grad = ws * (small_tiles ? HS::grad_ws : HL::grad_ws);
-    const int ws_rhs = ws * (small_tiles ? TS::rhs_ws : TL::rhs_ws);
-    const int ws_udot = ws * (small_tiles ? TS::udot_ws(NC) : TL::udot_ws(NC));
-    const int ws_sweep = ws * (small_tiles ? TS::sweep_ws : TL::sweep_ws);
-    auto* k_grad = small_tiles ? k_grad_rhs<R, P, NC, true> : k_grad_rhs<R, P, NC, false>;
-    auto* k_udotf = small_tiles ? k_udot_sweep<R, P, NC, true> : k_udot_sweep<R, P, NC, false>;
-    auto* k_sweep_g = small_tiles ? k_mass_sweep<R, P, 2 * NC, true> : k_mass_sweep<R, P, 2 * NC, false>;
-    auto* k_sweep_u = small_tiles ? k_mass_sweep<R, P, NC, true> : k_mass_sweep<R, P, NC, false>;
-    // the sensor's element tiles (k_sens): 8 rows of 32 in float, 4 in float64
-    // (24 modes of 340 elements are 65 KB there)
-    constexpr int STY = sizeof(R) == 4 ? 8 : 4;
-    const dim3 bs(K_TX, STY), gs(nblk(m.nx, K_TX), nblk(m.ny, STY));
-    // the facet tiles of systems (k_lo_sys, k_facet_sys)
+    constexpr bool F32 = sizeof(R) == 4;
+    // element blocks: fewer threads on small meshes, for an even spread over
+    // the SMs (KPP 256^2: 3.4 blocks of 64 x 2 per SM)
+    const int bex = m.E < (1 << 18) ? 32 : 64, bey = !F32 && m.E < (1 << 14) ? 1 : 2;
+    const dim3 be(bex, bey), bn(128, 1);
+    const dim3 ge(nblk(m.nx, bex), nblk(m.ny, bey)), gn(nblk(m.nnx, 128), m.nny);
+    const int size = tile_size<R, P>(m);
+    Stencils<R, P, NC> S = size == 0 ? stencils_of<R, P, NC, 0>(m) : stencils_of<R, P, NC, 1>(m);
+    if constexpr (!F32)
+        if (size == 2) S = stencils_of<R, P, NC, 2>(m);
+    // the element tiles of k_sens and k_lo: 32 by 8 in float, by 4 in float64
+    // (24 modes of 340 elements are 65 KB there); lower ones on small meshes
+    constexpr int STY = F32 ? 8 : 4, STS = F32 ? 4 : 1;
+    const bool low = (long long)nblk(m.nx, K_TX) * nblk(m.ny, STY) < 304;
+    const dim3 bs(K_TX, low ? STS : STY), gs(nblk(m.nx, K_TX), nblk(m.ny, low ? STS : STY));
+    // the facet tiles of systems (k_lo_sys, k_facet_sys) and the rows of
+    // k_res_sys and k_upd_sys
     const dim3 bf(F_TX, F_TY), gf(nblk(m.nx, F_TX), nblk(m.ny, F_TY));
+    const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
     // per-launch timing records events between kernels: plain launches then
     const bool pdl = prof == nullptr;
     cudaError_t err = cudaSuccess;
@@ -175,82 +207,42 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         if (e != cudaSuccess && err == cudaSuccess) err = e;
     };
     R* u = (R*)B.u;
-    // FP32-mixed: the second stream starts with the Galerkin part of the
-    // residual, which needs only u
-    constexpr bool split = sizeof(R) == 4;
     // the Q1 variant of eq. (aecQ1) needs neither g_h, nor the residual, nor udot
-    const bool q1 = (pr.opts & OPT_AEC_Q1) != 0 && pr.mode != MODE_LO;
-    const bool split_res = split && split_residual(m, NC) && !q1;
+    const bool lo = pr.mode == MODE_LO, q1 = (pr.opts & OPT_AEC_Q1) != 0 && !lo;
     // per-launch timing serialises the stage on one stream, so that each
     // kernel's events bracket its own run and no overlap with the other stream
     const cudaStream_t s2 = prof ? st : B.st2;
-    if (split_res && !dt_only && pr.mode != MODE_LO) {
+    if (!dt_only) {
         chk(cudaEventRecord(B.ev_fork0, st));
         chk(cudaStreamWaitEvent(s2, B.ev_fork0, 0));
-        if constexpr (split && NC == 1)
-            CGL_LAUNCH(prof, KID_RESW, s2,
-                       chk(launch(false, k_res_w<P, Ph>, ge, be, s2, m, pr, (const float*)u, (float*)B.EW)));
+        if constexpr (NC == 1) {
+            if (!q1 && !lo)
+                CGL_LAUNCH(prof, KID_RESW, s2,
+                           chk(launch(false, k_res_w<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, (R*)B.EW)));
+        }
+        auto* ksens = low ? k_sens<R, P, Ph, STS> : k_sens<R, P, Ph, STY>;
+        CGL_LAUNCH(prof, KID_SENS, s2, chk(launch(false, ksens, gs, bs, s2, m, pr, (const R*)u, B.gam, B.nu)));
         chk(cudaEventRecord(B.ev_w, s2));
     }
-    constexpr bool use_avg = sizeof(R) == 4 && NC > 1;
     if constexpr (NC > 1) {
-        // the low-order part here, the sensor in k_sens below
         CGL_LAUNCH(prof, KID_AVG, st, chk(launch(pdl, k_avg<R, P, Ph>, ge, be, st, m, pr, (const R*)u, B.avg, B.ue, (R*)B.cq)));
         auto* klo = (pr.opts & OPT_SUBCELL_DT) ? k_lo_sys<R, P, Ph, true> : k_lo_sys<R, P, Ph, false>;
         CGL_LAUNCH(prof, KID_PRE, st,
                    chk(launch(pdl, klo, gf, bf, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.fl, B.cf,
                               (const float*)B.avg, (const R*)B.cq, first ? B.dtbits : nullptr)));
     } else {
-        auto* kpre = (pr.opts & OPT_SUBCELL_DT) ? k_pre<R, P, Ph, true> : k_pre<R, P, Ph, false>;
+        const bool sub = (pr.opts & OPT_SUBCELL_DT) != 0;
+        auto* klo = low ? (sub ? k_lo<R, P, Ph, STS, true> : k_lo<R, P, Ph, STS, false>)
+                        : (sub ? k_lo<R, P, Ph, STY, true> : k_lo<R, P, Ph, STY, false>);
         CGL_LAUNCH(prof, KID_PRE, st,
-                   chk(launch(pdl, kpre, ge, be, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, B.gam, B.nu,
-                              (R*)B.q, (R*)B.fl, B.cf, B.avg, first ? B.dtbits : nullptr)));
+                   chk(launch(pdl, klo, gs, bs, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.q, (R*)B.fl, B.cf, B.avg,
+                              first ? B.dtbits : nullptr)));
     }
     if (first)
         CGL_LAUNCH(prof, KID_DT, st,
                    chk(launch(pdl, k_dt_final, dim3(1), dim3(1), st, B.dtbits, pr.cfl, (const double*)B.t,
                               (const double*)B.t_end, B.dt)));
     if (dt_only) return err != cudaSuccess ? err : cudaGetLastError();
-    // FP32-mixed: the facet part of the update (for systems after the sensor)
-    // on the second stream, beside the g_h and udot kernels
-    constexpr bool split_update = sizeof(R) == 4;
-    if constexpr (split_update) {
-        if (!q1) {
-            chk(cudaEventRecord(B.ev_fork, st));
-            chk(cudaStreamWaitEvent(s2, B.ev_fork, 0));
-            if constexpr (use_avg) {
-                // systems: the sensor first on the second stream, beside the
-                // g_h kernels of the main stream (k_sens is arithmetic-bound,
-                // the fused g_h sweep shared-memory-bound; measured: quadrants
-                // 512^2 Q3 2.368 -> 2.312 ms per step, blast 2048^2 -0.3 %)
-                CGL_LAUNCH(prof, KID_SENS, s2,
-                           chk(launch(false, k_sens<float, P, Ph, STY>, gs, bs, s2, m, pr, (const float*)u, B.gam, B.nu)));
-                chk(cudaEventRecord(B.ev_w, s2));
-            }
-            if constexpr (NC > 1)
-                CGL_LAUNCH(prof, KID_FACET, s2,
-                           chk(launch(false, k_facet_sys<R, P, Ph>, gf, bf, s2, m, pr, (const R*)u, (const double*)B.ue,
-                                      B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
-            else
-                CGL_LAUNCH(prof, KID_FACET, s2,
-                           chk(launch(false, k_facet<P, Ph>, ge, be, s2, m, pr, (const float*)u, (const double*)B.ue,
-                                      B.dte, (const double*)B.ubl, (const float*)B.q, (const float*)B.fl, B.cf, B.ube,
-                                      (float*)B.fht, B.cnt)));
-            chk(cudaEventRecord(B.ev_join, s2));
-        }
-    }
-    if constexpr (NC > 1) {
-        // the FP64 form, and eq. (aecQ1), which scales its contributions by
-        // gamma_e: the sensor on the main stream
-        if (!split || q1)
-            CGL_LAUNCH(prof, KID_SENS, st,
-                       chk(launch(pdl, k_sens<R, P, Ph, STY>, gs, bs, st, m, pr, (const R*)u, B.gam, B.nu)));
-        if constexpr (!split_update)
-            if (!q1)
-                CGL_LAUNCH(prof, KID_FACET, st,
-                           chk(launch(pdl, k_facet_sys<R, P, Ph>, gf, bf, st, m, pr, (const R*)u, (const double*)B.ue,
-                                      B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
-    }
     if (q1) {
         CGL_LAUNCH(prof, KID_Q1F, st,
                    chk(launch(pdl, k_q1_facet<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const double*)B.ue,
@@ -259,6 +251,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         CGL_LAUNCH(prof, KID_UDL, st,
                    chk(launch(pdl, k_udl<R, P, NC>, gn, bn, st, m, (const R*)u, (const double*)B.ube,
                               (const double*)B.dte, (R*)B.ud)));
+        chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e scales the contributions
         CGL_LAUNCH(prof, KID_UPDATE, st,
                    chk(launch(pdl, k_q1_update<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)B.ud,
                               (const double*)B.ue, (const double*)B.dte, (const R*)B.ER, (const float*)B.cf,
@@ -269,65 +262,59 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
                               B.cnt, pr.last_stage ? B.t : (double*)nullptr, (const double*)B.dt)));
         return err != cudaSuccess ? err : cudaGetLastError();
     }
+    // the facet part of the update
+    chk(cudaEventRecord(B.ev_fork, st));
+    chk(cudaStreamWaitEvent(s2, B.ev_fork, 0));
+    if constexpr (NC > 1)
+        CGL_LAUNCH(prof, KID_FACET, s2,
+                   chk(launch(false, k_facet_sys<R, P, Ph>, gf, bf, s2, m, pr, (const R*)u, (const double*)B.ue,
+                              B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
+    else
+        CGL_LAUNCH(prof, KID_FACET, s2,
+                   chk(launch(false, k_facet<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, (const double*)B.ue, B.dte,
+                              (const double*)B.ubl, (const R*)B.q, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
+    chk(cudaEventRecord(B.ev_join, s2));
     R* ud = (R*)B.ud;
-    if (pr.mode != MODE_LO) {
-        // g_h: stencil right-hand side and lumped iterate, then k_g sweeps (ping-pong)
+    if (!lo) {
+        // g_h: right-hand side, lumped iterate and k_g sweeps (ping-pong), the
+        // first sweep fused with the right-hand side where fuse_grad_sweep says
         R* g = (R*)B.g;
         R* g2 = (R*)B.g2;
         R* bg = (R*)B.bg;
-        // the right-hand sides with their first sweeps in one kernel each; the
-        // float64 form on large tiles keeps the g_h pair apart (the sweep's
-        // halo costs it a fifth of the float64 operations of both, their
-        // traffic less)
-        const bool fuse = !(pr.opts & OPT_UNFUSED_SWEEPS), fuse_g = fuse && fuse_grad_sweep(sizeof(R), small_tiles);
+        const bool fuse = !(pr.opts & OPT_UNFUSED_SWEEPS), fuse_g = fuse && fuse_grad_sweep(sizeof(R), size);
         int k0 = 0;
         if (fuse_g && pr.k_g >= 1) {
-            auto* k_gradf = k_grad_sweep<R, P, NC, true>;
-            if constexpr (sizeof(R) == 4)
-                if (!small_tiles) k_gradf = k_grad_sweep<R, P, NC, false>;
             CGL_LAUNCH(prof, KID_GRADF, st,
-                       chk(launch_shared(pdl, k_gradf, gth, bt, ws_grad, st, m, (const R*)u, pr.k_g > 1 ? bg : (R*)nullptr, g2)));
-            R* t = g;
-            g = g2;
-            g2 = t;
+                       chk(launch_shared(pdl, S.grad_sweep, S.grid_halo, S.block, S.ws_grad, st, m, (const R*)u,
+                                         pr.k_g > 1 ? bg : (R*)nullptr, g2)));
+            std::swap(g, g2);
             k0 = 1;
         } else {
             CGL_LAUNCH(prof, KID_GRAD, st,
-                       chk(launch_shared(pdl, k_grad, gt, bt, ws_rhs, st, m, (const R*)u, bg, g)));
+                       chk(launch_shared(pdl, S.grad, S.grid, S.block, S.ws_rhs, st, m, (const R*)u, bg, g)));
         }
         for (int k = k0; k < pr.k_g; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch_shared(pdl, k_sweep_g, gt, bt, ws_sweep, st, m, (const R*)g, (const R*)bg, g2)));
-            R* t = g;
-            g = g2;
-            g2 = t;
+                       chk(launch_shared(pdl, S.sweep_g, S.grid, S.block, S.ws_sweep, st, m, (const R*)g, (const R*)bg, g2)));
+            std::swap(g, g2);
         }
         R* ER = (R*)B.ER;
         R* r = (R*)B.r;
         R* ud2 = (R*)B.ud2;
-        if constexpr (NC > 1) {
-            if constexpr (use_avg) chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e, nu_e of k_sens
-            const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
+        chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e, nu_e, the Galerkin part
+        if constexpr (NC > 1)
             CGL_LAUNCH(prof, KID_RES, st,
                        chk(launch_shared(pdl, k_res_sys<R, P, Ph>, grs, brs, (int)sizeof(R) * ResSys<R, P, NC>::ws, st, m,
                                          pr, (const R*)u, (const R*)g, (const double*)B.gam, (const double*)B.nu, ER)));
-        } else if (split_res) {
-            chk(cudaStreamWaitEvent(st, B.ev_w, 0));
-            if constexpr (split)
-                CGL_LAUNCH(prof, KID_RES, st,
-                           chk(launch(pdl, k_res_s<P>, ge, be, st, m, (const float*)u, (const float*)g,
-                                      (const double*)B.gam, (const double*)B.nu, (const float*)B.EW, (float*)ER)));
-        } else {
+        else
             CGL_LAUNCH(prof, KID_RES, st,
-                       chk(launch(pdl, k_res_ev<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)g,
-                                  (const double*)B.gam, (const double*)B.nu, ER)));
-        }
+                       chk(launch(pdl, k_res_s<R, P>, ge, be, st, m, (const R*)u, (const R*)g, (const double*)B.gam,
+                                  (const double*)B.nu, (const R*)B.EW, ER)));
         int k1 = 0;
         if (fuse && pr.k_u >= 1) {
-            CGL_LAUNCH(prof, KID_UDOTF, st, chk(launch_shared(pdl, k_udotf, gt, bt, ws_udot, st, m, (const R*)ER, r, ud2)));
-            R* t = ud;
-            ud = ud2;
-            ud2 = t;
+            CGL_LAUNCH(prof, KID_UDOTF, st,
+                       chk(launch_shared(pdl, S.udot, S.grid, S.block, S.ws_udot, st, m, (const R*)ER, r, ud2)));
+            std::swap(ud, ud2);
             k1 = 1;
         } else {
             CGL_LAUNCH(prof, KID_GATHER, st,
@@ -335,33 +322,23 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         }
         for (int k = k1; k < pr.k_u; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch_shared(pdl, k_sweep_u, gt, bt, ws_sweep, st, m, (const R*)ud, (const R*)r, ud2)));
-            R* t = ud;
-            ud = ud2;
-            ud2 = t;
+                       chk(launch_shared(pdl, S.sweep_u, S.grid, S.block, S.ws_sweep, st, m, (const R*)ud, (const R*)r, ud2)));
+            std::swap(ud, ud2);
         }
     }
-    if constexpr (split_update) chk(cudaStreamWaitEvent(st, B.ev_join, 0));
-    if constexpr (NC > 1) {
-        const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
+    chk(cudaStreamWaitEvent(st, B.ev_join, 0));
+    if constexpr (NC > 1)
         CGL_LAUNCH(prof, KID_UPDATE, st,
                    chk(launch(pdl, k_upd_sys<R, P, Ph>, grs, brs, st, m, pr, (const R*)u, (const R*)ud,
                               (const double*)B.ue, (const double*)B.dte, (const R*)B.ER, (const float*)B.cf,
                               (const float*)B.avg, (const double*)B.ube, (const R*)B.fht, (const double*)B.dt,
                               (R*)B.EW, B.beta, B.cnt)));
-    } else if constexpr (split_update) {
+    else
         CGL_LAUNCH(prof, KID_UPDATE, st,
-                   chk(launch(pdl, k_update_el<P, Ph>, ge, be, st, m, pr, (const float*)u, (const float*)ud,
-                              (const double*)B.ue, (const double*)B.dte, (const float*)B.ER, (const float*)B.cf,
-                              (const float*)B.avg, (const double*)B.ube, (const float*)B.fht,
-                              (const double*)B.dt, (float*)B.EW, B.beta, B.cnt)));
-    } else
-    CGL_LAUNCH(prof, KID_UPDATE, st,
-               chk(launch(pdl, k_update_ev<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)ud,
-                          (const double*)B.ue, B.dte, (const double*)B.ubl, (const R*)B.q,
-                          (const R*)B.fl, (const R*)B.ER, (const float*)B.cf, (const float*)B.avg,
-                          (const double*)B.dt, (R*)B.EW,
-                          B.ube, B.beta, B.cnt)));
+                   chk(launch(pdl, k_update_el<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)ud,
+                              (const double*)B.ue, (const double*)B.dte, (const R*)B.ER, (const float*)B.cf,
+                              (const float*)B.avg, (const double*)B.ube, (const R*)B.fht, (const double*)B.dt,
+                              (R*)B.EW, B.beta, B.cnt)));
     CGL_LAUNCH(prof, KID_FINAL, st,
                chk(launch(pdl, k_final<R, P, NC>, gn, bn, st, m, pr, (const R*)B.EW, (R*)B.un, u, R(a), R(b),
                           B.cnt, pr.last_stage ? B.t : (double*)nullptr, (const double*)B.dt)));
