@@ -697,11 +697,12 @@ extern "C" void cgl_state_destroy(cgl_state* S) {
     }
     if (S->cst_in) cudaStreamDestroy(S->cst_in);
     if (S->cst_out) cudaStreamDestroy(S->cst_out);
-    if (S->B.ev_fork) cudaEventDestroy(S->B.ev_fork);
+    if (S->B.ev_s) cudaEventDestroy(S->B.ev_s);
     if (S->B.ev_join) cudaEventDestroy(S->B.ev_join);
     if (S->B.ev_fork0) cudaEventDestroy(S->B.ev_fork0);
     if (S->B.ev_w) cudaEventDestroy(S->B.ev_w);
-    if (S->B.st2) cudaStreamDestroy(S->B.st2);
+    for (cudaStream_t s : {S->B.st2, S->B.st3, S->B.st4})
+        if (s) cudaStreamDestroy(s);
     if (S->own_stream && S->st) cudaStreamDestroy(S->st);
     delete S;
 }
@@ -796,10 +797,12 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
             return rc;
         }
     }
-    // second stream and fork/join events of a stage (k_facet beside the g_h and udot kernels)
+    // the side streams of a stage and their fork/join events (run_stage)
     {
         cudaError_t e1 = cudaStreamCreateWithFlags(&B.st2, cudaStreamNonBlocking);
-        cudaError_t e2 = e1 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_fork, cudaEventDisableTiming) : e1;
+        if (e1 == cudaSuccess) e1 = cudaStreamCreateWithFlags(&B.st3, cudaStreamNonBlocking);
+        if (e1 == cudaSuccess) e1 = cudaStreamCreateWithFlags(&B.st4, cudaStreamNonBlocking);
+        cudaError_t e2 = e1 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_s, cudaEventDisableTiming) : e1;
         if (e2 == cudaSuccess) e2 = cudaEventCreateWithFlags(&B.ev_fork0, cudaEventDisableTiming);
         if (e2 == cudaSuccess) e2 = cudaEventCreateWithFlags(&B.ev_w, cudaEventDisableTiming);
         cudaError_t e3 = e2 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_join, cudaEventDisableTiming) : e2;

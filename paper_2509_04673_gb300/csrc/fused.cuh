@@ -634,24 +634,18 @@ template <class R, int P, int NC, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT, SIZE ? 1 : (P == 3 ? 4 : 3))
     k_grad_sweep(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
     using TL = stage_tile_t<R, P, SIZE, true>;
-    // like k_grad_rhs: runs beside k_pre, waits for it before exiting
-    pdl_trigger();
+    pdl_begin();
     grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
                                  dyn_shared<R>());
-    pdl_wait();
 }
 
 template <class R, int P, int NC, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_grad_rhs(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
     using TL = stage_tile_t<R, P, SIZE>;
-    // needs only u, whose last writer completed before k_pre let this kernel
-    // start (pdl_wait_then_trigger), so it runs beside k_pre and waits for it
-    // only before exiting
-    pdl_trigger();
+    pdl_begin();
     grad_rhs_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
                                dyn_shared<R>());
-    pdl_wait();
 }
 
 template <class R, int P, int NC, int SIZE>

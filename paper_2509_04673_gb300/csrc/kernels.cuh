@@ -53,17 +53,12 @@ DEV void pdl_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// k_pre waits first and lets the next kernel be scheduled only then: when
-// k_grad_rhs / k_grad_sweep (which need only u) start, the kernel that last
-// wrote u has completed, so they can run beside k_pre.
+// the batched kernels, whose phases run on one stream: the next is scheduled
+// only once this one's predecessor has completed
 DEV void pdl_wait_then_trigger() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-DEV void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// the gradient kernels wait for k_pre only before they exit, so that they
-// complete after it and later kernels may rely on both
-DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 
 template <int P>
@@ -912,7 +907,7 @@ __global__ void __launch_bounds__(K_TX * TY) k_lo(MeshDev m, ProbDev pr, const R
                                                   float* __restrict__ avg, unsigned long long* __restrict__ dtbits) {
     constexpr int N2 = Dim<P>::N2, HE = (K_TX + 2) * (TY + 2), NT = K_TX * TY;
     __shared__ R sA[HE], sL[sizeof(R) == 4 ? HE : 1], sX[HE], sY[HE];  // mean (high, low part), its fluxes
-    pdl_wait_then_trigger();
+    pdl_begin();
     const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * K_TX, ey0 = blockIdx.y * TY;
     for (int i = ty * K_TX + tx; i < HE; i += NT) {
         int jx, jy;
@@ -1057,7 +1052,7 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 3)
              const float* __restrict__ avg, const R* __restrict__ cq, unsigned long long* __restrict__ dtbits) {
     constexpr int NC = Ph::NC, NT = F_TX * F_TY;
     __shared__ R sV[NC + 1][F_NV], sH[NC + 1][F_NH];
-    pdl_wait_then_trigger();
+    pdl_begin();
     const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * F_TX, ey0 = blockIdx.y * F_TY;
     const int E = m.E;
     const R g = PV<R>::gam(pr);
@@ -1177,7 +1172,7 @@ __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const
     __shared__ R ws[WS];
     R(*sM)[HE] = reinterpret_cast<R(*)[HE]>(ws);
     R(*sS)[SX] = reinterpret_cast<R(*)[SX]>(ws);
-    pdl_wait_then_trigger();
+    pdl_begin();
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * K_TX + tx;
     const int ex0 = blockIdx.x * K_TX, ey0 = blockIdx.y * TY;
     const int ex = ex0 + tx, ey = ey0 + ty;

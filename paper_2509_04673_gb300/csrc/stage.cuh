@@ -27,8 +27,8 @@ struct Bufs {
     float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_pre for scalars)
     void* cq;     // systems: flux of the mean and speed parts per cell [2NC + 6][E]  (R) (k_avg)
     void* fht;    // facet terms of f_i^e [NC][E]  (R) (k_facet -> k_update_el, k_upd_sys)
-    cudaStream_t st2;            // second stream of a stage (k_facet)
-    cudaEvent_t ev_fork0, ev_fork, ev_w, ev_join;
+    cudaStream_t st2, st3, st4;            // second stream of a stage (k_facet)
+    cudaEvent_t ev_fork0, ev_s, ev_w, ev_join;
     double *ue, *dte, *ubl, *gam, *nu, *ube, *beta;
     unsigned long long* cnt;     // CNT_N counters
     unsigned long long* dtbits;  // min dt_e as bits
@@ -73,13 +73,15 @@ typedef cudaError_t (*StageFn)(const Bufs&, const MeshDev&, const ProbDev&, doub
 inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 // Size of the stencils' tiles (StageTile): large ones unless they make fewer
-// than two blocks per SM, tiny ones (float64) where the small ones make fewer
-// than one
+// than four (p <= 2) or two blocks per SM, tiny ones (float64) where the small
+// ones make fewer than one.  Euler 768 x 192 Q2 FP32-mixed, 325 large tiles: 569
+// us/step with them, 557 with small ones; Burgers 301 x 199 Q4, 475 large
+// tiles: 259 and 273.
 template <class R, int P>
 inline int tile_size(const MeshDev& m) {
     using TL = stage_tile_t<R, P, 0>;
     using TS = stage_tile_t<R, P, 1>;
-    if ((long long)nblk(m.nnx, TL::NX) * nblk(m.nny, TL::NY) >= 304) return 0;
+    if ((long long)nblk(m.nnx, TL::NX) * nblk(m.nny, TL::NY) >= (P <= 2 ? 608 : 304)) return 0;
     if (sizeof(R) == 4) return 1;
     return (long long)nblk(m.nnx, TS::NX) * nblk(m.nny, TS::NY) >= 152 ? 1 : 2;
 }
@@ -169,12 +171,17 @@ Stencils<R, P, NC> stencils_of(const MeshDev& m) {
     return s;
 }
 
-// Two streams: the second (s2) carries, from the start of the stage, what needs
-// only u, the Galerkin part of a scalar's residual and the sensor, then the
-// facet part of the update, which needs the low-order part; the main stream the
-// low-order part, the g_h solve, the residual, the udot solve, the element part
-// and the node gather.  In float64 on large meshes both fill the same pipe,
-// and the second stream fills the tails of the first.
+// Four streams, from the start of the stage: the main one carries the g_h
+// solve, the residual, the udot solve, the element part of the update and the
+// node gather; what needs only u runs beside it, the low-order part, dt and the
+// facet part of the update (s2), the sensor (s3) and a scalar's Galerkin part
+// of the residual (s4).  On small meshes a stage is as long as its longest
+// chain of launches: KPP 256^2 Q2 FP32-mixed 125 us/step with the low-order
+// part on the main stream and the rest on one other, 121 with four; advection
+// 32^2 Q2 float64 186 and 168; KPP 256^2 Q2 LGL float64, whose streams fill the
+// float64 pipe, 1296 and 1246.  On large meshes the order changes nothing.
+// The streams are the state's own, and each is joined to the main stream
+// before the last kernel of the stage.
 template <class R, int P, class Ph>
 cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, double a, double b,
                       bool first, bool dt_only, cudaStream_t st, Prof* prof) {
@@ -182,9 +189,11 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     if (dt_only) pr.mode = MODE_HO;  // no sensor needed for dt_e
     constexpr int NC = Ph::NC;
     constexpr bool F32 = sizeof(R) == 4;
-    // element blocks: fewer threads on small meshes, for an even spread over
-    // the SMs (KPP 256^2: 3.4 blocks of 64 x 2 per SM)
-    const int bex = m.E < (1 << 18) ? 32 : 64, bey = !F32 && m.E < (1 << 14) ? 1 : 2;
+    // element blocks: 64 threads on middle meshes, for an even spread over the
+    // SMs (KPP 256^2: 6.7 blocks of 32 x 2 per SM); full blocks on tiny ones,
+    // where the time is fetching instructions, once per SM (advection 32^2
+    // float64: the step 6 % shorter with blocks of 128 than with 32)
+    const int bex = m.E < (1 << 18) ? 32 : 64, bey = m.E < (1 << 14) ? 4 : 2;
     const dim3 be(bex, bey), bn(128, 1);
     const dim3 ge(nblk(m.nx, bex), nblk(m.ny, bey)), gn(nblk(m.nnx, 128), m.nny);
     const int size = tile_size<R, P>(m);
@@ -210,37 +219,49 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     // the Q1 variant of eq. (aecQ1) needs neither g_h, nor the residual, nor udot
     const bool lo = pr.mode == MODE_LO, q1 = (pr.opts & OPT_AEC_Q1) != 0 && !lo;
     // per-launch timing serialises the stage on one stream, so that each
-    // kernel's events bracket its own run and no overlap with the other stream
-    const cudaStream_t s2 = prof ? st : B.st2;
-    if (!dt_only) {
-        chk(cudaEventRecord(B.ev_fork0, st));
-        chk(cudaStreamWaitEvent(s2, B.ev_fork0, 0));
-        if constexpr (NC == 1) {
-            if (!q1 && !lo)
-                CGL_LAUNCH(prof, KID_RESW, s2,
-                           chk(launch(false, k_res_w<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, (R*)B.EW)));
+    // kernel's events bracket its own run and no overlap with the other streams
+    const cudaStream_t s2 = prof || dt_only || q1 ? st : B.st2, s3 = prof ? st : B.st3, s4 = prof ? st : B.st4;
+    auto fork = [&](cudaStream_t s) {
+        if (s != st) chk(cudaStreamWaitEvent(s, B.ev_fork0, 0));
+    };
+    auto join = [&](cudaEvent_t e, cudaStream_t s) {
+        if (s != st) {
+            chk(cudaEventRecord(e, s));
+            chk(cudaStreamWaitEvent(st, e, 0));
         }
+    };
+    chk(cudaEventRecord(B.ev_fork0, st));
+    fork(s2);
+    if (!dt_only) {
+        fork(s3);
         auto* ksens = low ? k_sens<R, P, Ph, STS> : k_sens<R, P, Ph, STY>;
-        CGL_LAUNCH(prof, KID_SENS, s2, chk(launch(false, ksens, gs, bs, s2, m, pr, (const R*)u, B.gam, B.nu)));
-        chk(cudaEventRecord(B.ev_w, s2));
+        if constexpr (NC == 1) {
+            if (!q1 && !lo) {
+                fork(s4);
+                CGL_LAUNCH(prof, KID_RESW, s4,
+                           chk(launch(false, k_res_w<R, P, Ph>, ge, be, s4, m, pr, (const R*)u, (R*)B.EW)));
+            }
+        }
+        CGL_LAUNCH(prof, KID_SENS, s3, chk(launch(false, ksens, gs, bs, s3, m, pr, (const R*)u, B.gam, B.nu)));
     }
+    const bool pdl2 = pdl && s2 == st;
     if constexpr (NC > 1) {
-        CGL_LAUNCH(prof, KID_AVG, st, chk(launch(pdl, k_avg<R, P, Ph>, ge, be, st, m, pr, (const R*)u, B.avg, B.ue, (R*)B.cq)));
+        CGL_LAUNCH(prof, KID_AVG, s2, chk(launch(pdl2, k_avg<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, B.avg, B.ue, (R*)B.cq)));
         auto* klo = (pr.opts & OPT_SUBCELL_DT) ? k_lo_sys<R, P, Ph, true> : k_lo_sys<R, P, Ph, false>;
-        CGL_LAUNCH(prof, KID_PRE, st,
-                   chk(launch(pdl, klo, gf, bf, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.fl, B.cf,
+        CGL_LAUNCH(prof, KID_PRE, s2,
+                   chk(launch(pdl, klo, gf, bf, s2, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.fl, B.cf,
                               (const float*)B.avg, (const R*)B.cq, first ? B.dtbits : nullptr)));
     } else {
         const bool sub = (pr.opts & OPT_SUBCELL_DT) != 0;
         auto* klo = low ? (sub ? k_lo<R, P, Ph, STS, true> : k_lo<R, P, Ph, STS, false>)
                         : (sub ? k_lo<R, P, Ph, STY, true> : k_lo<R, P, Ph, STY, false>);
-        CGL_LAUNCH(prof, KID_PRE, st,
-                   chk(launch(pdl, klo, gs, bs, st, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.q, (R*)B.fl, B.cf, B.avg,
+        CGL_LAUNCH(prof, KID_PRE, s2,
+                   chk(launch(pdl2, klo, gs, bs, s2, m, pr, (const R*)u, B.ue, B.dte, B.ubl, (R*)B.q, (R*)B.fl, B.cf, B.avg,
                               first ? B.dtbits : nullptr)));
     }
     if (first)
-        CGL_LAUNCH(prof, KID_DT, st,
-                   chk(launch(pdl, k_dt_final, dim3(1), dim3(1), st, B.dtbits, pr.cfl, (const double*)B.t,
+        CGL_LAUNCH(prof, KID_DT, s2,
+                   chk(launch(pdl, k_dt_final, dim3(1), dim3(1), s2, B.dtbits, pr.cfl, (const double*)B.t,
                               (const double*)B.t_end, B.dt)));
     if (dt_only) return err != cudaSuccess ? err : cudaGetLastError();
     if (q1) {
@@ -251,7 +272,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         CGL_LAUNCH(prof, KID_UDL, st,
                    chk(launch(pdl, k_udl<R, P, NC>, gn, bn, st, m, (const R*)u, (const double*)B.ube,
                               (const double*)B.dte, (R*)B.ud)));
-        chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e scales the contributions
+        join(B.ev_s, s3);  // gamma_e scales the contributions
         CGL_LAUNCH(prof, KID_UPDATE, st,
                    chk(launch(pdl, k_q1_update<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const R*)B.ud,
                               (const double*)B.ue, (const double*)B.dte, (const R*)B.ER, (const float*)B.cf,
@@ -263,17 +284,14 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         return err != cudaSuccess ? err : cudaGetLastError();
     }
     // the facet part of the update
-    chk(cudaEventRecord(B.ev_fork, st));
-    chk(cudaStreamWaitEvent(s2, B.ev_fork, 0));
     if constexpr (NC > 1)
         CGL_LAUNCH(prof, KID_FACET, s2,
-                   chk(launch(false, k_facet_sys<R, P, Ph>, gf, bf, s2, m, pr, (const R*)u, (const double*)B.ue,
+                   chk(launch(pdl, k_facet_sys<R, P, Ph>, gf, bf, s2, m, pr, (const R*)u, (const double*)B.ue,
                               B.dte, (const double*)B.ubl, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
     else
         CGL_LAUNCH(prof, KID_FACET, s2,
-                   chk(launch(false, k_facet<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, (const double*)B.ue, B.dte,
+                   chk(launch(pdl, k_facet<R, P, Ph>, ge, be, s2, m, pr, (const R*)u, (const double*)B.ue, B.dte,
                               (const double*)B.ubl, (const R*)B.q, (const R*)B.fl, B.cf, B.ube, (R*)B.fht, B.cnt)));
-    chk(cudaEventRecord(B.ev_join, s2));
     R* ud = (R*)B.ud;
     if (!lo) {
         // g_h: right-hand side, lumped iterate and k_g sweeps (ping-pong), the
@@ -301,7 +319,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         R* ER = (R*)B.ER;
         R* r = (R*)B.r;
         R* ud2 = (R*)B.ud2;
-        chk(cudaStreamWaitEvent(st, B.ev_w, 0));  // gamma_e, nu_e, the Galerkin part
+        join(B.ev_s, s3);  // gamma_e and nu_e
+        if (NC == 1) join(B.ev_w, s4);  // the Galerkin part
         if constexpr (NC > 1)
             CGL_LAUNCH(prof, KID_RES, st,
                        chk(launch_shared(pdl, k_res_sys<R, P, Ph>, grs, brs, (int)sizeof(R) * ResSys<R, P, NC>::ws, st, m,
@@ -326,7 +345,8 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
             std::swap(ud, ud2);
         }
     }
-    chk(cudaStreamWaitEvent(st, B.ev_join, 0));
+    if (lo) join(B.ev_s, s3);
+    join(B.ev_join, s2);
     if constexpr (NC > 1)
         CGL_LAUNCH(prof, KID_UPDATE, st,
                    chk(launch(pdl, k_upd_sys<R, P, Ph>, grs, brs, st, m, pr, (const R*)u, (const R*)ud,
