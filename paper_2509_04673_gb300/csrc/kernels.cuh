@@ -491,6 +491,35 @@ DEV float llf_value(float nL, float nR, float lam, float jump) {
     return __fmaf_rn(__fmul_rn(-0.5f, lam), jump, __fmul_rn(0.5f, __fadd_rn(nL, nR)));
 }
 
+// the NC values of facet i of an array [4E][NC] of facet values (the four
+// components of a system in 16-byte accesses: one by one they are stores of 4
+// bytes at a stride of 64)
+template <class R, int NC>
+DEV void store_facet(R* __restrict__ f, long long i, const R (&v)[NC]) {
+    if constexpr (NC == 4 && sizeof(R) == 4) {
+        reinterpret_cast<float4*>(f)[i] = make_float4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (NC == 4) {
+        reinterpret_cast<double2*>(f)[2 * i] = make_double2(v[0], v[1]);
+        reinterpret_cast<double2*>(f)[2 * i + 1] = make_double2(v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) f[i * NC + c] = v[c];
+    }
+}
+template <class R, int NC>
+DEV void load_facet(const R* __restrict__ f, long long i, R (&v)[NC]) {
+    if constexpr (NC == 4 && sizeof(R) == 4) {
+        const float4 a = reinterpret_cast<const float4*>(f)[i];
+        v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    } else if constexpr (NC == 4) {
+        const double2 a = reinterpret_cast<const double2*>(f)[2 * i], b = reinterpret_cast<const double2*>(f)[2 * i + 1];
+        v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = f[i * NC + c];
+    }
+}
+
 // ---------------------------------------------------------------------------
 // k_pre: dt_e, ubar^{e,L}, gamma_e, nu_e
 // ---------------------------------------------------------------------------
@@ -678,8 +707,7 @@ DEV double lo_outputs_mixed(const MeshDev& m, const ProbDev& pr, const float* __
     dte_out[2 * m.E + e] = s * m.inv_h;
 #pragma unroll
     for (int d = 0; d < 4; ++d)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = F[d][c];
+store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
     const float s4 = 0.25f * sf;  // |K| / (|dK| dt_e), exact
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -810,8 +838,7 @@ DEV double lo_outputs_fp64(const MeshDev& m, const ProbDev& pr, const double* __
     dte_out[2 * m.E + e] = s * m.inv_h; // 1 / dt_e
 #pragma unroll
     for (int d = 0; d < 4; ++d)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fl_out[((long long)e * 4 + d) * NC + c] = FL[d][c];
+store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const double os = ((FL[1][c] - FL[0][c]) + FL[3][c]) - FL[2][c];
@@ -977,43 +1004,55 @@ __global__ void __launch_bounds__(K_TX * TY) k_lo(MeshDev m, ProbDev pr, const R
     if (dtbits) block_min_to(dte, dtbits);
 }
 
-// The facets of a tile of TX x TY elements (systems): the TX + 1 by TY
-// vertical ones, then the TX by TY + 1 horizontal ones.  A block evaluates
-// each once, where one thread per element evaluated its four (every interior
-// facet twice), and the elements take them from shared memory.
+// The facets of a tile of F_TX x F_TY elements (systems).  A block of F_TX x
+// (F_TY + 1) threads evaluates each once, where one thread per element
+// evaluated its four (every interior facet twice), and the elements take them
+// from shared memory.  Two rounds: the vertical facets, a row of threads the
+// facets left of a row of elements (aligned, as all arrays of elements are),
+// the last row the far ends; then the F_TY + 1 rows of horizontal ones.
+// Bound by latency (six blocks of loads per facet and few instructions): four
+// rows of threads taking the 292 facets in turn left a third round of 36 and
+// split addresses, 489 us for k_lo_sys and 407 for k_facet_sys on 2048^2
+// elements of degree 2 (FP32-mixed); five rows, and f^L in 16-byte accesses,
+// 319 and 348.
 constexpr int F_TX = 32, F_TY = 4;
 struct FacetItem {
-    int axis, slot;        // x (0) or y (1); position among the facets of its axis
+    int axis, slot;        // x (0) or y (1); position in the tile's facets (facet_of)
     int eL, eR;            // cells left and right (below and above), -1 outside the domain
     int ex, ey, d;         // a cell of the facet and its side there (the one inside on the boundary)
 };
-// item i of the tile at (ex0, ey0): false where no element of the tile has it
-DEV bool facet_item(const MeshDev& m, int ex0, int ey0, int i, FacetItem& f) {
-    constexpr int NV = (F_TX + 1) * F_TY;
-    f.axis = i < NV ? 0 : 1;
-    const int k = f.axis == 0 ? i : i - NV, w = f.axis == 0 ? F_TX + 1 : F_TX;
-    const int r = k / w, c = k - r * w;
-    f.slot = k;
+// the facet of thread (tx, ty) in the round of an axis: false where it has none
+DEV bool facet_item(const MeshDev& m, int ex0, int ey0, int axis, FacetItem& f) {
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    int c = tx, r = ty;
+    if (axis == 0 && ty == F_TY) {
+        c = F_TX, r = tx;
+        if (r >= F_TY) return false;
+    }
+    f.axis = axis;
+    f.slot = axis == 0 ? r * (F_TX + 1) + c : (F_TX + 1) * F_TY + r * F_TX + c;
     // the cell right of (above) the facet, and the one left of (below) it
-    const int xR = ex0 + c, yR = ey0 + r, xL = f.axis == 0 ? xR - 1 : xR, yL = f.axis == 0 ? yR : yR - 1;
+    const int xR = ex0 + c, yR = ey0 + r, xL = axis == 0 ? xR - 1 : xR, yL = axis == 0 ? yR : yR - 1;
     const bool inR = xR < m.nx && yR < m.ny, inL = xL >= 0 && yL >= 0 && xL < m.nx && yL < m.ny;
     // a cell of the tile itself: the right one unless it is the far end's
-    const bool tR = f.axis == 0 ? c < F_TX : r < F_TY, tL = f.axis == 0 ? c > 0 : r > 0;
+    const bool tR = axis == 0 ? c < F_TX : r < F_TY, tL = axis == 0 ? c > 0 : r > 0;
     if (!((tR && inR) || (tL && inL))) return false;
     if (inR) {
         f.eR = yR * m.nx + xR;
-        f.ex = xR, f.ey = yR, f.d = f.axis == 0 ? 0 : 2;
+        f.ex = xR, f.ey = yR, f.d = axis == 0 ? 0 : 2;
         f.eL = neighbour(m, xR, yR, f.d);
     } else {
         f.eL = yL * m.nx + xL;
-        f.ex = xL, f.ey = yL, f.d = f.axis == 0 ? 1 : 3;
+        f.ex = xL, f.ey = yL, f.d = axis == 0 ? 1 : 3;
         f.eR = neighbour(m, xL, yL, f.d);
     }
     return true;
 }
 // slots of the element (tx, ty)'s facets W, E (x) and S, N (y)
-DEV int facet_of(int tx, int ty, int d) { return d < 2 ? ty * (F_TX + 1) + tx + d : (ty + d - 2) * F_TX + tx; }
-constexpr int F_NV = (F_TX + 1) * F_TY, F_NH = F_TX * (F_TY + 1);
+DEV int facet_of(int tx, int ty, int d) {
+    return d < 2 ? ty * (F_TX + 1) + tx + d : (F_TX + 1) * F_TY + (ty + d - 2) * F_TX + tx;
+}
+constexpr int F_NT = F_TX * (F_TY + 1), F_N = (F_TX + 1) * F_TY + F_TX * (F_TY + 1);
 
 // low-order quantities of a boundary facet in float64, as boundary_facet_lo
 template <class Ph>
@@ -1046,20 +1085,20 @@ __device__ __noinline__ CompVec<double, Ph::NC + 1> boundary_facet_lo64(const Me
 // (facet speeds and f^L, dt_e, ubar^{e,L}, the float copies for the facet
 // limiter's certificate); gamma_e and nu_e come from k_sens
 template <class R, int P, class Ph, bool SUB = false>
-__global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 3)
+__global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? (SUB ? 5 : 6) : (SUB ? 2 : 3))
     k_lo_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, double* __restrict__ ue_io, double* __restrict__ dte_out,
              double* __restrict__ ubl_out, R* __restrict__ fl_out, float* __restrict__ cf_out,
              const float* __restrict__ avg, const R* __restrict__ cq, unsigned long long* __restrict__ dtbits) {
-    constexpr int NC = Ph::NC, NT = F_TX * F_TY;
-    __shared__ R sV[NC + 1][F_NV], sH[NC + 1][F_NH];
+    constexpr int NC = Ph::NC;
+    __shared__ R sF[NC + 1][F_N];  // f^L, speed
     pdl_begin();
     const int tx = threadIdx.x, ty = threadIdx.y, ex0 = blockIdx.x * F_TX, ey0 = blockIdx.y * F_TY;
     const int E = m.E;
     const R g = PV<R>::gam(pr);
 #pragma unroll 1
-    for (int i = ty * F_TX + tx; i < F_NV + F_NH; i += NT) {
+    for (int axis = 0; axis < 2; ++axis) {
         FacetItem f;
-        if (!facet_item(m, ex0, ey0, i, f)) continue;
+        if (!facet_item(m, ex0, ey0, axis, f)) continue;
         R F[NC], lam;
         const R* __restrict__ fa = cq + (long long)(f.axis * NC) * E;  // the means' fluxes along the facet's axis
         if (f.eL >= 0 && f.eR >= 0) {
@@ -1113,24 +1152,20 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 3)
             }
         }
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            if (f.axis == 0) sV[c][f.slot] = F[c];
-            else sH[c][f.slot] = F[c];
-        }
-        if (f.axis == 0) sV[NC][f.slot] = lam;
-        else sH[NC][f.slot] = lam;
+        for (int c = 0; c < NC; ++c) sF[c][f.slot] = F[c];
+        sF[NC][f.slot] = lam;
     }
     __syncthreads();
     const int ex = ex0 + tx, ey = ey0 + ty, e = ey * m.nx + ex;
     double dte = __longlong_as_double(0x7ff0000000000000LL);
-    if (ex < m.nx && ey < m.ny) {
+    if (ty < F_TY && ex < m.nx && ey < m.ny) {
         R lam[4], F[4][NC];
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
             const int s = facet_of(tx, ty, d);
-            lam[d] = d < 2 ? sV[NC][s] : sH[NC][s];
+            lam[d] = sF[NC][s];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) F[d][c] = d < 2 ? sV[c][s] : sH[c][s];
+            for (int c = 0; c < NC; ++c) F[d][c] = sF[c][s];
         }
         R us[NC];
         if constexpr (sizeof(R) == 4) {
@@ -2665,11 +2700,11 @@ __global__ void __launch_bounds__(128)
 // changes no bit), else alpha f^A, split into two floats in the FP32-mixed
 // form; the eight float terms are summed as a compensated pair.
 template <class R, int P, class Ph>
-__global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 4)
+__global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
     k_facet_sys(MeshDev m, ProbDev pr, const R* __restrict__ u, const double* __restrict__ ue, double* dte_a,
                 const double* __restrict__ ubl, const R* __restrict__ fl_in, float* cf, double* __restrict__ ube_out,
                 R* __restrict__ fht, unsigned long long* __restrict__ cnt) {
-    constexpr int NC = Ph::NC, N1 = P + 1, NT = F_TX * F_TY, NFC = F_NV + F_NH;
+    constexpr int NC = Ph::NC, N1 = P + 1, NFC = F_N;
     constexpr int NTERM = sizeof(R) == 4 ? 3 : 2;  // f^H, and T0, T1 (float64: their sum)
     __shared__ R sT[NTERM][NC][NFC];
     pdl_begin();
@@ -2678,9 +2713,10 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 4)
     const bool need_fh = !(pr.mode == MODE_LO && pr.fl == FL_LOW);
     if (need_fh) {
 #pragma unroll 1
-        for (int i = ty * F_TX + tx; i < NFC; i += NT) {
+        for (int axis = 0; axis < 2; ++axis) {
             FacetItem f;
-            if (!facet_item(m, ex0, ey0, i, f)) continue;
+            if (!facet_item(m, ex0, ey0, axis, f)) continue;
+            const int i = f.slot;
             // the face's coefficients
             R Uf[NC * N1];
             {
@@ -2726,10 +2762,9 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 4)
             for (int c = 0; c < NC; ++c) sT[0][c][i] = FH[c];
             if (pr.fl != FL_LIMITED) continue;
             R FL[NC], T0[NC], T1[NC];
-            const long long lo = ((long long)(f.ey * m.nx + f.ex) * 4 + f.d) * NC;
+            load_facet<R, NC>(fl_in, (long long)(f.ey * m.nx + f.ex) * 4 + f.d, FL);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                FL[c] = fl_in[lo + c];
                 T0[c] = FL[c];
                 T1[c] = -FH[c];
             }
@@ -2801,10 +2836,10 @@ __global__ void __launch_bounds__(F_TX * F_TY, sizeof(R) == 4 ? 6 : 4)
     }
     __syncthreads();
     const int ex = ex0 + tx, ey = ey0 + ty, e = ey * m.nx + ex;
-    if (ex >= m.nx || ey >= m.ny) return;
+    if (ty >= F_TY || ex >= m.nx || ey >= m.ny) return;
     int at[4];
 #pragma unroll
-    for (int d = 0; d < 4; ++d) at[d] = facet_of(tx, ty, d) + (d < 2 ? 0 : F_NV);
+    for (int d = 0; d < 4; ++d) at[d] = facet_of(tx, ty, d);
     const double rs = dte_a[E + e];
     double rs2 = rs, ub[NC];
     R fh[NC];

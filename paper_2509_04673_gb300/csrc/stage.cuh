@@ -207,7 +207,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     const dim3 bs(K_TX, low ? STS : STY), gs(nblk(m.nx, K_TX), nblk(m.ny, low ? STS : STY));
     // the facet tiles of systems (k_lo_sys, k_facet_sys) and the rows of
     // k_res_sys and k_upd_sys
-    const dim3 bf(F_TX, F_TY), gf(nblk(m.nx, F_TX), nblk(m.ny, F_TY));
+    const dim3 bf(F_TX, F_TY + 1), gf(nblk(m.nx, F_TX), nblk(m.ny, F_TY));
     const dim3 grs(nblk(m.nx, 32), m.ny), brs(32, NC);
     // per-launch timing records events between kernels: plain launches then
     const bool pdl = prof == nullptr;
