@@ -801,10 +801,10 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
     {
         cudaError_t e1 = cudaStreamCreateWithFlags(&B.st2, cudaStreamNonBlocking);
         if (e1 == cudaSuccess) e1 = cudaStreamCreateWithFlags(&B.st3, cudaStreamNonBlocking);
-        if (e1 == cudaSuccess) e1 = cudaStreamCreateWithFlags(&B.st4, cudaStreamNonBlocking);
+        if (e1 == cudaSuccess && nc == 1) e1 = cudaStreamCreateWithFlags(&B.st4, cudaStreamNonBlocking);
         cudaError_t e2 = e1 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_s, cudaEventDisableTiming) : e1;
         if (e2 == cudaSuccess) e2 = cudaEventCreateWithFlags(&B.ev_fork0, cudaEventDisableTiming);
-        if (e2 == cudaSuccess) e2 = cudaEventCreateWithFlags(&B.ev_w, cudaEventDisableTiming);
+        if (e2 == cudaSuccess && nc == 1) e2 = cudaEventCreateWithFlags(&B.ev_w, cudaEventDisableTiming);
         cudaError_t e3 = e2 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_join, cudaEventDisableTiming) : e2;
         if (e3 != cudaSuccess) {
             cgl_state_destroy(S);
@@ -1431,6 +1431,20 @@ static cgl_status build_graph(cgl_state* S) {
     return CGL_OK;
 }
 
+// One step: the step graph, or, for the first step of a problem, plain launches
+// behind which the graph is captured while they run (the capture costs about
+// as much as a step of 256^2 elements: a new state's first step of KPP 256^2 Q2
+// took 307 us with the graph built first, 274 us so).  The launches and the graph follow one another on S->st, to
+// which the side streams are joined.
+static cgl_status run_step(cgl_state* S) {
+    if (S->step_graph) {
+        CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
+        return CGL_OK;
+    }
+    CUDA_TRY(enqueue_step(S));
+    return build_graph(S);
+}
+
 extern "C" cgl_status cgl_step(cgl_state* S, int32_t nsteps, double t_end, cgl_step_info* info) {
     if (!S) return fail(CGL_EINVAL, "null state");
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
@@ -1440,8 +1454,6 @@ extern "C" cgl_status cgl_step(cgl_state* S, int32_t nsteps, double t_end, cgl_s
     CUDA_TRY(cudaMemcpyAsync(c0, S->B.cnt, sizeof(c0), cudaMemcpyDeviceToHost, S->st));
     CUDA_TRY(cudaMemcpyAsync(S->B.t_end, &t_end, 8, cudaMemcpyHostToDevice, S->st));
     CUDA_TRY(cudaStreamSynchronize(S->st));
-    cgl_status rc = build_graph(S);
-    if (rc) return rc;
     long long taken = 0;
     const bool finite_end = std::isfinite(t_end);
     for (int s = 0; s < nsteps; ++s) {
@@ -1451,7 +1463,7 @@ extern "C" cgl_status cgl_step(cgl_state* S, int32_t nsteps, double t_end, cgl_s
             CUDA_TRY(cudaStreamSynchronize(S->st));
             if (t >= t_end) break;
         }
-        CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
+        if (cgl_status rc = run_step(S)) return rc;
         ++taken;
     }
     return read_info(S, info, taken, c0);
@@ -1488,6 +1500,8 @@ extern "C" cgl_status cgl_time_step(cgl_state* S, double* dt) {
 // per-kernel timing
 // ---------------------------------------------------------------------------
 static_assert(KID_COUNT <= 32, "cgl_profile reports at most 32 kernel identifiers");
+// (k_pre: k_lo and k_lo_sys; k_res_ev: k_res_s and k_res_sys; k_update_ev:
+// k_update_el, k_upd_sys and k_q1_update; k_facet: also k_facet_sys)
 static const char* const KNAMES[KID_COUNT] = {
     "k_avg", "k_pre", "k_dt", "k_grad_rhs", "k_gather_init", "k_grad_sweep", "k_mass_sweep",
     "k_res_ev", "k_update_ev", "k_final", "k_t_advance", "k_udot_sweep", "k_facet", "k_res_w", "k_q1_facet", "k_udl",
@@ -1579,9 +1593,8 @@ extern "C" cgl_status cgl_step_async(cgl_state* S, int32_t nsteps) {
     if (!S) return fail(CGL_EINVAL, "null state");
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
     if (nsteps < 0) return fail(CGL_EINVAL, "nsteps < 0");
-    cgl_status rc = build_graph(S);
-    if (rc) return rc;
-    for (int s = 0; s < nsteps; ++s) CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
+    for (int s = 0; s < nsteps; ++s)
+        if (cgl_status rc = run_step(S)) return rc;
     return CGL_OK;
 }
 
