@@ -1431,18 +1431,21 @@ static cgl_status build_graph(cgl_state* S) {
     return CGL_OK;
 }
 
-// One step: the step graph, or, for the first step of a problem, plain launches
-// behind which the graph is captured while they run (the capture costs about
-// as much as a step of 256^2 elements: a new state's first step of KPP 256^2 Q2
-// took 307 us with the graph built first, 274 us so).  The launches and the graph follow one another on S->st, to
-// which the side streams are joined.
+// One step: the step graph, or, for the first step of a problem, plain
+// launches behind which the graph is captured while they run (the capture
+// costs about as much as a step of 256^2 elements: a new state's first step of
+// KPP 256^2 Q2 took 307 us with the graph built first, 274 us so).  The
+// launches and the graph follow one another on S->st, to which the side
+// streams are joined.  On a caller's stream the graph comes first: where that
+// stream cannot be captured nothing has run.
 static cgl_status run_step(cgl_state* S) {
-    if (S->step_graph) {
-        CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
-        return CGL_OK;
+    if (!S->step_graph && S->own_stream) {
+        CUDA_TRY(enqueue_step(S));
+        return build_graph(S);
     }
-    CUDA_TRY(enqueue_step(S));
-    return build_graph(S);
+    if (cgl_status rc = build_graph(S)) return rc;
+    CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
+    return CGL_OK;
 }
 
 extern "C" cgl_status cgl_step(cgl_state* S, int32_t nsteps, double t_end, cgl_step_info* info) {
