@@ -123,44 +123,39 @@ def impl_algorithmic_bytes(kernel, mesh, nc, rsz, k_g, k_u):
     N2 = (mesh.p + 1) ** 2
     d = 8
     mixed = rsz == 4
+    EV = E * N2 * nc * rsz  # an element vector
     b = {
-        # reads u; writes u^e, dt_e (3), ubar^{e,L}, gamma, nu (float64), f^L
-        # (4 nc), the scalar capacities Q (2) and, mixed scalars, the float
-        # speed sum and the float-float mean
-        "k_pre": (nc * NN * rsz + (nc + 3 + nc + 2) * E * d + 4 * nc * E * rsz + (2 * E * rsz if nc == 1 else 0)
-                  + (3 * E * 4 if mixed else 0)),
-        "k_avg": nc * NN * 4 + 2 * nc * E * 4,
+        # scalars (k_lo): u -> u^e, dt_e (3), ubar^{e,L} (float64), f^L, the
+        # capacities Q (2) and, mixed, the float speed sum and float-float mean
+        "k_pre": NN * rsz + (1 + 3 + 1) * E * d + (4 + 2) * E * rsz + (3 * E * 4 if mixed else 0),
         "k_sens": nc * NN * rsz + 2 * E * d,
-        "k_res_ev": 3 * nc * NN * rsz + 2 * E * d + E * N2 * nc * rsz,
-        "k_res_w": nc * NN * rsz + E * N2 * nc * rsz,
-        "k_update_ev": 2 * nc * NN * rsz + (nc + 3 + nc) * E * d + (2 + 4 * nc) * E * rsz
-                       + 2 * E * N2 * nc * rsz + (nc + 1) * E * d,
-        "k_final": E * N2 * nc * rsz + 3 * nc * NN * rsz,
+        "k_res_w": nc * NN * rsz + EV,
+        # scalars (k_res_s): u, g, gamma, nu, W^e -> residual
+        "k_res_ev": 3 * nc * NN * rsz + 2 * E * d + 2 * EV,
+        # u, ubar^{e,L}, dt_e (2), Q or the certificate's copies, f^L -> ubar^e, facet terms
+        "k_facet": nc * NN * rsz + (nc + 2) * E * d + (2 * E * rsz if nc == 1 else (1 + nc) * E * 4)
+                   + 4 * nc * E * rsz + nc * E * d + nc * E * rsz,
+        # u, udot, residual, ubar^e, facet terms, speed sum and means (mixed)
+        # or u^e and dt_e (2) -> increments, beta
+        "k_update_ev": 2 * nc * NN * rsz + EV + nc * E * d + nc * E * rsz
+                       + ((1 + 2 * nc) * E * 4 if mixed else (nc + 2) * E * d) + EV + E * d,
+        "k_final": EV + 3 * nc * NN * rsz,
         "k_grad_rhs": nc * NN * rsz + 2 * 2 * nc * NN * rsz,
-        "k_gather_init": E * N2 * nc * rsz + 2 * nc * NN * rsz,
+        "k_gather_init": EV + 2 * nc * NN * rsz,
         "k_grad_sweep": nc * NN * rsz + 2 * nc * NN * rsz * (2 if k_g > 1 else 1),
-        "k_udot_sweep": E * N2 * nc * rsz + 2 * nc * NN * rsz,
+        "k_udot_sweep": EV + 2 * nc * NN * rsz,
         "k_mass_sweep": 3 * ((2 * nc * k_g + nc * k_u) / max(1, k_g + k_u)) * NN * rsz,
     }
-    if mixed and nc > 1:
-        # systems: k_avg also writes the flux of each mean and 5 speed parts
-        # (2 nc + 5 floats per cell); k_pre_lo reads those and the
-        # float-float means and writes u^e, dt_e (3), ubar^{e,L} (float64),
-        # f^L (4 nc), the float speed sum and ubar^{e,L} copies; k_sens reads
-        # u and writes gamma, nu
-        b["k_avg"] = nc * NN * 4 + 2 * nc * E * 4 + (2 * nc + 5) * E * 4
-        b["k_pre"] = ((2 * nc + 2 * nc + 5) * E * 4 + (nc + 3 + nc) * E * d + 4 * nc * E * 4
-                      + (1 + nc) * E * 4)
-    if mixed:
-        # k_res_s: u, g, gamma, nu, W^e -> element residual; k_facet: u,
-        # ubar^{e,L}, dt_e/h, Q, f^L -> ubar^e, facet terms; k_update_el: u,
-        # udot, residuals, ubar^e, facet terms, speed sum, means -> increments, beta
-        # (scalars from 2^20 nodes; systems keep the single k_res_ev)
-        b["k_res_ev"] = (3 * nc * NN * 4 + 2 * E * d + 2 * E * N2 * nc * 4 if (NN >= (1 << 20) and nc == 1)
-                         else b["k_res_ev"])
-        b["k_facet"] = nc * NN * 4 + (nc + 1) * E * d + (2 + 4 * nc) * E * 4 + nc * E * d + nc * E * 4
-        b["k_update_ev"] = (2 * nc * NN * 4 + E * N2 * nc * 4 + nc * E * d + nc * E * 4 + E * 4
-                            + 2 * nc * E * 4 + E * N2 * nc * 4 + E * d)
+    if nc > 1:
+        # k_avg: u -> the means (float-float, or float64 u^e), the flux of
+        # each and 6 speed parts per cell; k_lo_sys reads those and writes
+        # u^e (mixed), dt_e (3), ubar^{e,L} (float64), f^L, the float speed
+        # sum and ubar^{e,L} copies; k_res_sys: u, g, gamma, nu -> residual
+        means = 2 * nc * E * 4 if mixed else nc * E * d
+        cq = (2 * nc + 6) * E * rsz
+        b["k_avg"] = nc * NN * rsz + means + cq
+        b["k_pre"] = means + cq + ((nc if mixed else 0) + 3 + nc) * E * d + 4 * nc * E * rsz + (1 + nc) * E * 4
+        b["k_res_ev"] = 3 * nc * NN * rsz + 2 * E * d + EV
     return b.get(kernel)
 
 
@@ -178,18 +173,17 @@ def load_peaks():
 # dfma counted twice as flops) and DRAM bytes read + written.  None where the
 # kernel changed after the capture.
 NCU_PER_ELEMENT = {
-    # profiles/euler_blast_1024_q2_kernel_counts.md and, for the shared-memory wavefronts,
-    # profiles/euler_blast_1024_q2_shared_wavefronts.md (kernel names as cgl_profile reports them:
-    # k_pre is k_pre_lo and k_update_ev is k_update_el in this FP32-mixed Euler stage)
-    ("k_sens", HEADLINE): {"warp_inst": 195.41, "fp64_flops": 0.0, "dram_bytes": 69.6, "shared_wavefronts": 3.38},
-    ("k_grad_sweep", HEADLINE): {"warp_inst": 142.62, "fp64_flops": 0.0, "dram_bytes": 138.1, "shared_wavefronts": 46.82},
-    ("k_res_ev", HEADLINE): {"warp_inst": 146.29, "fp64_flops": 0.0, "dram_bytes": 403.1, "shared_wavefronts": 0.12},
-    ("k_update_ev", HEADLINE): {"warp_inst": 70.4, "fp64_flops": 4.024, "dram_bytes": 545.6, "shared_wavefronts": 0.16},
-    ("k_facet", HEADLINE): {"warp_inst": 79.32, "fp64_flops": 12.051, "dram_bytes": 248.4, "shared_wavefronts": 0.06},
-    ("k_pre", HEADLINE): {"warp_inst": 49.71, "fp64_flops": 22.0, "dram_bytes": 218.2, "shared_wavefronts": 0.15},
-    ("k_udot_sweep", HEADLINE): {"warp_inst": 81.14, "fp64_flops": 0.0, "dram_bytes": 233.1, "shared_wavefronts": 13.66},
-    ("k_final", HEADLINE): {"warp_inst": 37.17, "fp64_flops": 0.0, "dram_bytes": 316.9, "shared_wavefronts": 0.66},
-    ("k_avg", HEADLINE): {"warp_inst": 21.69, "fp64_flops": 0.0, "dram_bytes": 98.4, "shared_wavefronts": 0.06},
+    # profiles/euler_blast_1024_q2_stage_kernels.md (names as cgl_profile reports them: k_pre is k_lo_sys,
+    # k_res_ev k_res_sys, k_update_ev k_upd_sys and k_facet k_facet_sys in this Euler stage)
+    ("k_pre", HEADLINE): {"warp_inst": 48.34, "fp64_flops": 22.00, "dram_bytes": 206.6, "shared_wavefronts": 1.15},
+    ("k_facet", HEADLINE): {"warp_inst": 60.24, "fp64_flops": 13.26, "dram_bytes": 223.1, "shared_wavefronts": 2.88},
+    ("k_grad_sweep", HEADLINE): {"warp_inst": 80.05, "fp64_flops": 0.00, "dram_bytes": 140.0, "shared_wavefronts": 15.74},
+    ("k_res_ev", HEADLINE): {"warp_inst": 154.58, "fp64_flops": 0.00, "dram_bytes": 328.0, "shared_wavefronts": 19.25},
+    ("k_udot_sweep", HEADLINE): {"warp_inst": 44.19, "fp64_flops": 0.00, "dram_bytes": 230.3, "shared_wavefronts": 6.99},
+    ("k_update_ev", HEADLINE): {"warp_inst": 98.88, "fp64_flops": 0.03, "dram_bytes": 489.3, "shared_wavefronts": 5.60},
+    ("k_final", HEADLINE): {"warp_inst": 37.17, "fp64_flops": 0.00, "dram_bytes": 317.2, "shared_wavefronts": 0.66},
+    ("k_sens", HEADLINE): {"warp_inst": 82.78, "fp64_flops": 0.00, "dram_bytes": 67.0, "shared_wavefronts": 7.66},
+    ("k_avg", HEADLINE): {"warp_inst": 18.06, "fp64_flops": 0.00, "dram_bytes": 99.3, "shared_wavefronts": 0.06},
 }
 
 SM_COUNT_GB300 = 152

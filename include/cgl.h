@@ -111,18 +111,18 @@ typedef struct cgl_mesh_desc {
 /* Problem parameters. cgl_problem_defaults() fills the paper's defaults:
    q = 1 (Sec. 5), r = 2 (Sec. 2.2), w_lin = 1e-3 (Sec. 5.4), gamma = 1.4
    (Sec. 5.2), omega_CFL = 0.2, k_g = k_u = 1. */
-/* cgl_problem.options.  CGL_OPT_FP64_LIMITER: in the FP32-mixed form, evaluate
+/* cgl_problem.options.  CGL_OPT_FP64_LIMITER: evaluate
  * every Appendix-A positivity factor (facet and nodal limiter) with the float64
  * formula.  By default a float32 evaluation with a rigorous error bound first
  * certifies the factors that equal 1 and only the others are evaluated in
  * float64; the results are identical, the option exists to check that.
- * No effect in the FP64 form or for scalar fluxes. */
+ * No effect for scalar fluxes. */
 #define CGL_OPT_FP64_LIMITER 1
-/* cgl_problem.options.  CGL_OPT_UNFUSED_SWEEPS: in the FP32-mixed form on meshes
- * of 2^22 nodes or more, run the right-hand sides of the g_h and udot solves and
- * their first Richardson sweeps as separate kernels.  By default they are
- * fused there (one kernel each); the results are identical, the option exists
- * to check that. */
+/* cgl_problem.options.  CGL_OPT_UNFUSED_SWEEPS: run the
+ * right-hand sides of the g_h and udot solves and their first Richardson sweeps
+ * as separate kernels.  By default they are fused (one kernel each; in the FP64
+ * form the g_h one only on tiny meshes); the results are identical, the option
+ * exists to check that. */
 #define CGL_OPT_UNFUSED_SWEEPS 2
 /* cgl_problem.options.  CGL_OPT_SUBCELL_DT: the unlimited-flux variant of the
  * paper's Sec. 4.3 (step 4 with the flux limiter deactivated): the pseudo time

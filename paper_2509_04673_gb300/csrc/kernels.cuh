@@ -2,28 +2,35 @@
 // convex-limited CG-WENO scheme (Kuzmin, Hajduk, Vedral, arXiv 2509.04673),
 // following the order of the algorithm summary in Sec. 4.3:
 //
-//   k_pre          cell averages u^e of the element and its face neighbours
-//                  (eq. (ueold)), facet speeds, dt_e (eq. (dtmaxcell)), f^L,
-//                  ubar^{e,L} (eq. (uelowFCT)), WENO sensor gamma_e (eqs.
-//                  (WENO:alpha), (WENO:norm)), nu_e (eq. (stab:WENO)), block
-//                  minimum of dt_e
+//   k_lo           scalars: cell averages u^e (eq. (ueold)), facet speeds,
+//                  dt_e (eq. (dtmaxcell)), f^L, ubar^{e,L} (eq. (uelowFCT)),
+//                  block minimum of dt_e; systems: k_avg (averages, their
+//                  fluxes and speed parts), then k_lo_sys
 //   k_dt_final     global dt = omega_CFL min_e dt_e (eq. (cflglob), Sec. 5)
+//   k_sens         WENO sensor gamma_e (eqs. (WENO:alpha), (WENO:norm)), nu_e
+//                  (eq. (stab:WENO))
 //   k_grad_rhs     right-hand side of the g_h projection, int phi_i grad u_h,
 //                  as a tiled separable stencil, and its lumped iterate
 //   k_mass_sweep   lumped-preconditioned Richardson sweep with M_C applied
-//                  as a tiled separable stencil
-//   k_res_ev       element residual: Galerkin part of eq. (weak:stab2) with
+//                  as a tiled separable stencil; k_grad_sweep and
+//                  k_udot_sweep carry the first one (fused.cuh)
+//   k_res_w, k_res_s (scalars), k_res_sys (systems)
+//                  element residual: Galerkin part of eq. (weak:stab2) with
 //                  boundary terms (eqs. (aec), (aecb)) and s_h (eq. (stab:WENO))
 //   k_gather_init  node-centric sum over E_i of the element residuals in a
 //                  fixed order (deterministic), and its lumped iterate
-//   k_update_ev    facet fluxes f^H (eq. (hoflux)), flux limiter (eq. (fAlim),
-//                  Appendix A), ubar^e (eq. (uelim)), f_i^e (eq. (aec)),
-//                  beta_e (eqs. (slimit1), (slimit2), Appendix A), element
-//                  contributions of eq. (eq:SSPupdate)
+//   k_facet (scalars), k_facet_sys (systems)
+//                  facet fluxes f^H (eq. (hoflux)), flux limiter (eq. (fAlim),
+//                  Appendix A), ubar^e (eq. (uelim))
+//   k_update_el (scalars), k_upd_sys (systems)
+//                  f_i^e (eq. (aec)), beta_e (eqs. (slimit1), (slimit2),
+//                  Appendix A), element contributions of eq. (eq:SSPupdate)
 //   k_final        node gather, SSP-RK combination, invariant-domain check;
 //                  on the last stage of a step also t += dt
 //
-// One thread per element (or node; the stencils use 32 x 16 node tiles).
+// One thread per element or node; per element and component in k_res_sys and
+// k_upd_sys; the facets of systems once per facet; the stencils by segments
+// of p nodes.
 // Kernels are templated on the bulk precision R (double, or float in the
 // mixed form), the degree P and the physics policy Ph. Cell averages, dt_e,
 // the facet flux limiter, limiter bound gaps and positivity factors are
@@ -521,7 +528,7 @@ DEV void load_facet(const R* __restrict__ f, long long i, R (&v)[NC]) {
 }
 
 // ---------------------------------------------------------------------------
-// k_pre: dt_e, ubar^{e,L}, gamma_e, nu_e
+// the low-order part: dt_e, ubar^{e,L}
 // ---------------------------------------------------------------------------
 // block-wide minimum of positive doubles folded into *bits with an integer
 // atomicMin on the bit pattern (order independent, hence deterministic)
@@ -549,7 +556,7 @@ DEV void block_min_to(double v, unsigned long long* bits) {
 }
 
 // ---------------------------------------------------------------------------
-// k_pre: per element u^e and the face neighbours' u^{e'} (from their blocks,
+// per element u^e and the face neighbours' u^{e'} (from their blocks,
 // eq. (ueold)), f(u^e), lambda_e, the facet speeds and f^L, dt_e (eq.
 // (dtmaxcell)), ubar^{e,L} (eq. (uelowFCT)), the flux-limiter capacities,
 // gamma_e (eqs. (WENO:alpha), (WENO:norm)), nu_e, the element vectors of the
@@ -625,7 +632,7 @@ __device__ __noinline__ double subcell_dt(const R* __restrict__ u, const MeshDev
     return fmin(best, m0 / total) / sfac;
 }
 
-// low-order quantities of a boundary facet of the FP32-mixed k_pre: the
+// low-order quantities of a boundary facet of the FP32-mixed form: the
 // speed bound (inflated like the interior ones) and F(u^e, u_hat; n) in the
 // canonical orientation, u_hat of side d at the facet midpoint in float-float
 // (FIXED: the side's state; OUTFLOW: u^e; WALL: u^e with reversed normal
@@ -724,7 +731,7 @@ store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
             // (smaller magnitudes stay admissible)
             q_out[e] = __fmul_rz(s4, fmaxf(0.f, narrow(pr.umax - bl)));
             q_out[m.E + e] = __fmul_rz(s4, fminf(0.f, narrow(pr.umin - bl)));
-            // the float-float mean, for the element contributions of k_update_ev
+            // the float-float mean, for the element contributions of k_update_el
             avg[e] = uh[0];
             avg[m.E + e] = ul[0];
         } else {
@@ -732,7 +739,7 @@ store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
             cf_out[(1 + c) * m.E + e] = narrow(bl);
         }
     }
-    cf_out[e] = sf;  // the float speed sum (dt_e in float for k_update_ev)
+    cf_out[e] = sf;  // the float speed sum (dt_e in float for the update)
     return dte;
 }
 
@@ -1281,7 +1288,7 @@ __global__ void __launch_bounds__(K_TX * TY) k_sens(MeshDev m, ProbDev pr, const
     else nu_out[e] = lm * (m.h * (0.5 / P));
 }
 
-// global dt from the block minima folded into the bit pattern by k_pre
+// global dt from the block minima folded into the bit pattern by k_lo
 // dt = min(cfl * min_e dt_e, t_end - t), never negative
 static __global__ void k_dt_final(unsigned long long* bits, double cfl, const double* t,
                                   const double* t_end, double* dt) {
@@ -1481,7 +1488,7 @@ DEV NodeCands node_cands(const MeshDev& m, int gx, int gy) {
 }
 
 // ---------------------------------------------------------------------------
-// k_res_ev: R^e_i = W^e_i - s^e_i with
+// The element residual R^e_i = W^e_i - s^e_i with
 //   W^e_i = int grad phi_i . f(u_h) - sum_{interior faces} int phi_i f_h.n
 //           - sum_{faces on dOmega} int phi_i F(u_h, u_hat; n)
 //   s^e_i = nu_e int grad phi_i . (grad u_h - gamma_e g_h)      eq. (stab:WENO)
@@ -1881,7 +1888,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 6 : P 
 }
 
 // ---------------------------------------------------------------------------
-// k_update_ev: facet fluxes and flux limiter, ubar^e, f_i^e, beta_e and the
+// The update: facet fluxes and flux limiter, ubar^e, f_i^e, beta_e and the
 // element increments of eq. (eq:SSPupdate),
 //   m_i u_i^SSP = sum_e m_i^e [(1 - theta_e) u_i + theta_e ubar_i^e]
 //   <=> u_i^SSP = u_i + sum_e (m_i^e/m_i) theta_e (ubar^e - u_i + beta_e f_i^e/m_i^e),
@@ -2259,7 +2266,7 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
     const Tab<R>& T = tab_of<R>(m, P);
     const double me = m.me;
     // theta = dt / dt_e = dt s / h; FP32-mixed: in float from the float
-    // speed sum of k_pre (it weights float increments; the check counts only)
+    // speed sum of the low-order part (it weights float increments; the check counts only)
     R thR;
     if constexpr (sizeof(R) == 4) {
         thR = __fmul_rn((float)dt, __fmul_rn(cf[e], m.inv_h_f));
@@ -2310,7 +2317,7 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
         const R fh_term = fh[c];
         R ueh, uel;
         if constexpr (sizeof(R) == 4) {
-            // the float-float mean itself (k_pre for scalars, k_avg for systems)
+            // the float-float mean itself (k_lo for scalars, k_avg for systems)
             ueh = avg[(2 * c) * m.E + e];
             uel = avg[(2 * c + 1) * m.E + e];
         } else {

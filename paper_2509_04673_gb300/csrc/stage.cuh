@@ -24,10 +24,10 @@ struct Bufs {
     void* q;      // flux-limiter capacities [2][E] (scalar)  (R)
     void* fl;     // low-order facet fluxes [E][4][NC]         (R)
     float* cf;    // float copies for the Euler limiter certificate [1+NC][E]: s, ubar^{e,L}
-    float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_pre for scalars)
+    float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_lo for scalars)
     void* cq;     // systems: flux of the mean and speed parts per cell [2NC + 6][E]  (R) (k_avg)
     void* fht;    // facet terms of f_i^e [NC][E]  (R) (k_facet -> k_update_el, k_upd_sys)
-    cudaStream_t st2, st3, st4;            // second stream of a stage (k_facet)
+    cudaStream_t st2, st3, st4;  // side streams of a stage (run_stage)
     cudaEvent_t ev_fork0, ev_s, ev_w, ev_join;
     double *ue, *dte, *ubl, *gam, *nu, *ube, *beta;
     unsigned long long* cnt;     // CNT_N counters
