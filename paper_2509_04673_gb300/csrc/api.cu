@@ -784,7 +784,6 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
         {&B.EV, 16},                  {&B.ER, E * N2 * nc * r},    {&B.EW, E * N2 * nc * r},     {(void**)&B.q, 2 * E * r},
         {(void**)&B.ue, nc * E * 8},  {(void**)&B.cf, (1 + nc) * E * 4},  {(void**)&B.avg, 2 * nc * E * 4},
         {&B.fht, nc * E * r},
-        {&B.cq, nc > 1 ? (2 * nc + PhysEuler::NPART) * E * r : 16},
         {(void**)&B.dte, 3 * E * 8},  {(void**)&B.fl, 4 * nc * E * r},      {(void**)&B.ubl, nc * E * 8}, {(void**)&B.gam, E * 8},
         {(void**)&B.nu, E * 8},       {(void**)&B.ube, nc * E * 8}, {(void**)&B.beta, E * 8},
         {(void**)&B.cnt, CNT_N * 8},  {(void**)&B.dtbits, 8},      {(void**)&B.dt, 8},
@@ -797,6 +796,8 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
             return rc;
         }
     }
+    // cq: [2nc + 6][E] values in the nc (p + 1)^2 >= 16 of EW, free until the update
+    if (nc > 1) B.cq = B.EW;
     // the side streams of a stage and their fork/join events (run_stage)
     {
         cudaError_t e1 = cudaStreamCreateWithFlags(&B.st2, cudaStreamNonBlocking);
@@ -1436,12 +1437,17 @@ static cgl_status build_graph(cgl_state* S) {
 // costs about as much as a step of 256^2 elements: a new state's first step of
 // KPP 256^2 Q2 took 307 us with the graph built first, 274 us so).  The
 // launches and the graph follow one another on S->st, to which the side
-// streams are joined.  On a caller's stream the graph comes first: where that
-// stream cannot be captured nothing has run.
+// streams are joined.  Where a caller's stream cannot be captured (the legacy
+// stream, or one that is being captured) the graph comes first and fails before
+// anything has run.
 static cgl_status run_step(cgl_state* S) {
-    if (!S->step_graph && S->own_stream) {
-        CUDA_TRY(enqueue_step(S));
-        return build_graph(S);
+    if (!S->step_graph && S->st != cudaStreamLegacy) {
+        cudaStreamCaptureStatus cs;
+        CUDA_TRY(cudaStreamIsCapturing(S->st, &cs));
+        if (cs == cudaStreamCaptureStatusNone) {
+            CUDA_TRY(enqueue_step(S));
+            return build_graph(S);
+        }
     }
     if (cgl_status rc = build_graph(S)) return rc;
     CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));

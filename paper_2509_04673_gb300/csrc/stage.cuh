@@ -25,7 +25,7 @@ struct Bufs {
     void* fl;     // low-order facet fluxes [E][4][NC]         (R)
     float* cf;    // float copies for the Euler limiter certificate [1+NC][E]: s, ubar^{e,L}
     float* avg;   // float-float cell means [2NC][E] (FP32-mixed: k_avg for systems, k_lo for scalars)
-    void* cq;     // systems: flux of the mean and speed parts per cell [2NC + 6][E]  (R) (k_avg)
+    void* cq;     // systems: flux of the mean and speed parts per cell [2NC + 6][E]  (R) (k_avg), in EW
     void* fht;    // facet terms of f_i^e [NC][E]  (R) (k_facet -> k_update_el, k_upd_sys)
     cudaStream_t st2, st3, st4;  // side streams of a stage (run_stage)
     cudaEvent_t ev_fork0, ev_s, ev_w, ev_join;
