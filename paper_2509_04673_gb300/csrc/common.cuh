@@ -202,7 +202,8 @@ DEV int a2_base(const MeshDev& m) {
 // float64) refined by Newton-Raphson, one step in float, one third-order step
 // in float64, to within a unit in the last place; unlike the IEEE division it
 // has no slow path, and in float64 it takes 3 instructions of GB300's narrow
-// pipe instead of about 10
+// pipe instead of about 10.  For normal x with a normal reciprocal (1 / 0 is
+// NaN here, not infinity)
 DEV float rcp_nr(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -213,12 +214,6 @@ DEV double rcp_nr(double x) {
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = __fma_rn(-x, r, 1.0);
     return __fma_rn(r, __fma_rn(e, e, e), r);
-}
-// a double that is 0 or infinite (integer tests: a float64 comparison runs on
-// the float64 pipe too)
-DEV bool is_zero_or_inf(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    return hi == 0x7ff00000u || (hi | (unsigned)__double2loint(x)) == 0u;
 }
 DEV bool is_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
 DEV bool is_finite(float x) { return isfinite(x); }

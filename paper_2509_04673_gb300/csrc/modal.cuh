@@ -44,15 +44,22 @@ DEV double sub_r(double a, double b) { return __dsub_rn(a, b); }
 static __device__ __noinline__ float pow_rare(float x, float e) { return powf(x, e); }
 static __device__ __noinline__ double pow_rare(double x, double e) { return pow(x, e); }
 
-// 1 / x of a weight: float by the hardware's approximation (within one unit in
-// the last place), float64 by rcp_nr; an infinite norm gives 0, as the exact
-// operation does (x > 0 otherwise)
+// 1 / x, x >= 0, of a weight or a norm: float by the hardware's approximation
+// (within one unit in the last place), float64 by rcp_nr where x and 1 / x are
+// normal and by the division, out of line, elsewhere.  Both give infinity at 0
+// (a flat element's norm with gamma_eps = 0) and 0 at infinity, as the division
+// does.
+static __device__ __noinline__ double rcp_rare(double x) { return 1.0 / x; }
 DEV float recip(float x) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-DEV double recip(double x) { return is_zero_or_inf(x) ? 0.0 : rcp_nr(x); }
+DEV double recip(double x) {
+    // the biased exponent in 1 .. 2044: x < 2^1022
+    if ((((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 1u >= 2044u) return rcp_rare(x);
+    return rcp_nr(x);
+}
 
 // modal coefficients of one line
 template <class R, int P>

@@ -1,7 +1,7 @@
 """The arithmetic routines of the kernels that stand for hardware or library
-operations (common.cuh, modal.cuh), on the device: square roots at zero, at
-subnormals, at the ends of the range and at infinity, and over the normal
-range in units of the last place; and whole stages with values there."""
+operations (common.cuh, modal.cuh), on the device: square roots and reciprocals
+at zero, at subnormals, at the ends of the range and at infinity, and over the
+normal range in units of the last place; and whole stages with values there."""
 import json
 import math
 import os
@@ -75,3 +75,49 @@ def test_float64_gas_at_rest_with_a_narrow_velocity_pulse(cgl, p, basis):  # noq
     assert np.abs(nu - nu_ref).max() <= 1e-13 * nu_ref.max()
     assert np.abs(gam - S.sensor(om, om.blocks(u), d)).max() <= 1e-10
     assert _rel(out, ref, 4) <= TOL64
+
+
+@pytest.mark.parametrize("name,least", [("recip_d", 2.0 ** -1074), ("recip_f", 2.0 ** -149)])
+def test_reciprocal(arith, name, least):
+    """Within one unit in the last place over the normal range; infinity at zero, zero at infinity."""
+    assert arith[name] <= 1.0
+    u = 2.0 ** (-52 if name == "recip_d" else -23)
+    for x, y in _points(arith, name):
+        if name == "recip_f":
+            with np.errstate(over="ignore"):
+                x = float(np.float32(x))
+        if x == 0.0:
+            assert y == math.inf
+        elif math.isinf(x):
+            assert y == 0.0
+        elif 1.0 / x > 3.4e38 and name == "recip_f":
+            assert y == math.inf
+        else:
+            assert y == 1.0 / x or abs(y - 1.0 / x) <= max(u / x, least), (x, y)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("flux,p", [(1, 1), (1, 2), (2, 3), (1, 4), (3, 2)])
+def test_flat_element_without_gamma_eps(cgl, flux, p, prec):  # noqa: F811
+    """gamma_eps = 0: an element with constant coefficients among others that are not has the ratio
+    num / 0 and so gamma = 0, full dissipation at the foot of a jump, in both precisions."""
+    mesh = Mesh(9, 8, p, 0.0, 9 / 8, 0.0, 1.0)
+    prob = _problem(dict(flux=flux, mode=3, fl=1, gamma_eps=0.0))
+    make = inputs.random_euler_state if flux == 3 else (
+        lambda m, s: inputs.random_scalar_state(m, s, prob.umin, prob.umax, 0.4))
+    u = make(mesh, 5 + p).astype(np.float32).astype(np.float64)
+    for c in range(u.shape[0]):
+        u[c, 3 * p:4 * p + 1, 4 * p:5 * p + 1] = u[c, 3 * p, 4 * p]
+    om = S.OracleMesh(mesh)
+    with np.errstate(divide="ignore"):
+        ref = S.sensor(om, om.blocks(u), prob.as_dict())
+    assert ref[3 * 9 + 4] == 0.0
+    st = cgl.State(cgl.Mesh(mesh), u.shape[0], prec)
+    st.set_problem(prob)
+    st.set_state(u)
+    st.set_base_state(u)
+    st.stage(1e-4, 0.0, 1.0, raise_on_idp=False)
+    gam = st.get_field(cgl.FIELD_GAMMA)
+    st.close()
+    assert gam[3 * 9 + 4] == 0.0
+    assert np.abs(gam - ref).max() <= (5e-6 if prec else 1e-10)
