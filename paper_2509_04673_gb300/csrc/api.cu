@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/cgl.h"
+#include "modal_tables.h"
 #include "stage.cuh"
 #include "state.h"
 
@@ -318,59 +319,14 @@ static void build_lgl_tables(int p, Tab<double>& T, double* a2) {
         }
 }
 
-// Modal tables of degree p (modal.cuh).  With P_k the Legendre polynomials on
-// [0, 1] and L[k][a] the P_k coefficient of the basis function a, a line v
-// has the modal coefficients l_k = (sum_a L[k][a] v_a) / L[k][p], so that u =
-// sum_k l_k m_k with m_k = L[k][p] P_k.  mf holds the weights L[k][p - j] /
-// L[k][p] of the pairs (v_j, v_{p-j}), mc the expansion of m_j(x + 1) in m_k,
-// and m2 the semi-norm matrix of eq. (WENO:norm) over the products
-// m_k1 m_k2, off-diagonal entries doubled.  Gauss-Legendre with p + 2 points
-// (exact to degree 2p + 3).
-static void build_modal_tables(int p, Tab<double>& T, double* m2) {
-    const int n = p + 1, nq = p + 2, n2 = n * n;
-    double xg[NQMAX], wg[NQMAX];
-    gauss_legendre(nq, xg, wg);
-    // monomial coefficients of P_k(2x - 1): sum_i (-1)^(k+i) C(k,i) C(k+i,i) x^i
-    double P[N1MAX][N1MAX], L[N1MAX][N1MAX];
-    for (int k = 0; k < n; ++k)
-        for (int i = 0; i < N1MAX; ++i)
-            P[k][i] = i <= k ? ((k + i) % 2 ? -1.0 : 1.0) * binom(k, i) * binom(k + i, i) : 0.0;
-    for (int k = 0; k < n; ++k)
-        for (int a = 0; a < n; ++a) {
-            double s = 0.0;
-            for (int q = 0; q < nq; ++q) s += T.wq[q] * T.Bq[q][a] * poly_eval(p, P[k], T.xq[q]);
-            L[k][a] = (2 * k + 1) * s;
-        }
-    const int pairs = (p + 1) / 2;  // (v_j, v_{p-j}), j < pairs; an even p has the middle value too
-    for (int k = 0; k < n; ++k)
-        for (int j = 1; j < 3; ++j) {
-            const bool used = (k % 2 == 0) ? j < pairs + (p % 2 == 0) : j < pairs;
-            T.mf[k][j - 1] = used ? L[k][p - j] / L[k][p] : 0.0;
-        }
-    for (int k = 0; k < n; ++k)
-        for (int j = 0; j < n; ++j) {
-            double s = 0.0;
-            for (int q = 0; q < nq; ++q) s += T.wq[q] * poly_eval(p, P[j], T.xq[q] + 1.0) * poly_eval(p, P[k], T.xq[q]);
-            T.mc[k][j] = j > k ? (2 * k + 1) * s * L[j][p] / L[k][p] : (j == k ? 1.0 : 0.0);
-        }
-    double S[N1MAX][N1MAX][N1MAX];
-    for (int d = 0; d <= p; ++d)
-        for (int k = 0; k < n; ++k)
-            for (int l = 0; l < n; ++l) {
-                double dk[N1MAX], dl[N1MAX], s = 0.0;
-                poly_deriv(p, P[k], d, dk);
-                poly_deriv(p, P[l], d, dl);
-                for (int q = 0; q < nq; ++q) s += T.wq[q] * poly_eval(p, dk, T.xq[q]) * poly_eval(p, dl, T.xq[q]);
-                S[d][k][l] = s * L[k][p] * L[l][p];
-            }
-    for (int i = 0; i < n2; ++i)
-        for (int j = 0; j < n2; ++j) {
-            double s = 0.0;
-            for (int d1 = 0; d1 <= p; ++d1)
-                for (int d2 = 0; d2 <= p - d1; ++d2)
-                    if (d1 + d2 >= 1) s += S[d1][i % n][j % n] * S[d2][i / n][j / n];
-            m2[i * n2 + j] = i == j ? s : 2.0 * s;
-        }
+// the modal tables of degree p into T and m2
+static void build_modal_tables(int p, const double* xn, Tab<double>& T, double* m2) {
+    ModalTables t;
+    modal_tables(p, xn, t);
+    std::memcpy(T.mf, t.mf, sizeof(T.mf));
+    std::memcpy(T.mc, t.mc, sizeof(T.mc));
+    const int n2 = (p + 1) * (p + 1);
+    for (int i = 0; i < n2 * n2; ++i) m2[i] = t.m2[i];
 }
 
 // weighted quadrature tables and the derivative of the basis in itself: phi_k'
@@ -464,7 +420,7 @@ static void build_tables(HostTables& H) {
                                 H.a2d[off + (b * n + a) * n2 + d * n + c] +=
                                     S[k1][a * n + c] * S[k2][b * n + d];
             }
-        build_modal_tables(p, T, H.m2d + off);
+        build_modal_tables(p, nullptr, T, H.m2d + off);
         build_point_tables(p, false, T);
         // float copies
         Tab<float>& F = H.tf[p];
@@ -475,7 +431,7 @@ static void build_tables(HostTables& H) {
     for (int i = 0; i < A2_TOTAL; ++i) H.m2f[i] = (float)H.m2d[i];
     for (int p = 1; p <= PMAX; ++p) {
         build_lgl_tables(p, H.td[PMAX + 1 + p], H.a2d + A2_TOTAL + A2_OFF[p]);
-        build_modal_tables(p, H.td[PMAX + 1 + p], H.m2d + A2_TOTAL + A2_OFF[p]);
+        build_modal_tables(p, H.td[PMAX + 1 + p].xn, H.td[PMAX + 1 + p], H.m2d + A2_TOTAL + A2_OFF[p]);
         build_point_tables(p, true, H.td[PMAX + 1 + p]);
     }
 }
