@@ -218,22 +218,80 @@ DEV double rcp_nr(double x) {
 DEV bool is_finite(double x) { return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u; }
 DEV bool is_finite(float x) { return isfinite(x); }
 
+// the bits of a float, and the high and low word of a double
+HDEV int bits_of(float x) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(x);
+#else
+    int i;
+    std::memcpy(&i, &x, 4);
+    return i;
+#endif
+}
+HDEV float float_of(int i) {
+#ifdef __CUDA_ARCH__
+    return __int_as_float(i);
+#else
+    float x;
+    std::memcpy(&x, &i, 4);
+    return x;
+#endif
+}
+HDEV unsigned hi_word(double x) {
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2hiint(x);
+#else
+    uint64_t b;
+    std::memcpy(&b, &x, 8);
+    return (unsigned)(b >> 32);
+#endif
+}
+HDEV unsigned lo_word(double x) {
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2loint(x);
+#else
+    uint64_t b;
+    std::memcpy(&b, &x, 8);
+    return (unsigned)b;
+#endif
+}
+// d rounded toward zero
+HDEV float float_rz(double d) {
+#ifdef __CUDA_ARCH__
+    return __double2float_rz(d);
+#else
+    const float f = (float)d;
+    return std::fabs((double)f) > std::fabs(d) ? std::nextafter(f, 0.f) : f;
+#endif
+}
+
 // Conversions between float and float64 in integer arithmetic: the hardware's
 // run on the float64 pipe, 16 clocks a warp there, where they were half of the
 // float64 instructions of the FP32-mixed kernels.  widen is exact; narrow cuts
 // to 24 bits (exact for a widened float); split_ff gives a float pair hi + lo
 // that holds the leading 47 bits.  Zeros take the same path; subnormal,
-// infinite and out-of-range values the hardware's.
+// infinite and out-of-range values the hardware's (narrow: toward zero).
 DEV double widen(float f) {
     const unsigned b = (unsigned)__float_as_int(f), e = b & 0x7f800000u;
     if ((e == 0 && (b << 1) != 0) || e == 0x7f800000u) return (double)f;
     const unsigned hi = (b & 0x80000000u) | (e == 0 ? 0u : ((b & 0x7fffffffu) >> 3) + 0x38000000u);
     return __hiloint2double((int)hi, (int)(b << 29));
 }
-DEV float narrow(double d) {
-    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
-    if (a - 0x38100000u >= 0x0fe00000u) return (a | l) == 0u ? __int_as_float((int)h) : __double2float_rz(d);
-    return __int_as_float((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
+HDEV float narrow(double d) {
+    const unsigned h = hi_word(d), l = lo_word(d), a = h & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x0fe00000u) return (a | l) == 0u ? float_of((int)h) : float_rz(d);
+    return float_of((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
+}
+// the same for the certificate euler_alpha_is_one: infinite from 2^128 on (it
+// refuses infinities; the largest float, which narrow gives, it would take for
+// the value)
+HDEV float cert_float(double d) {
+    const unsigned h = hi_word(d), l = lo_word(d), a = h & 0x7fffffffu;
+    if (a - 0x38100000u >= 0x0fe00000u) {
+        if ((a | l) == 0u) return float_of((int)h);
+        return a >= 0x47f00000u ? float_of((int)((h & 0x80000000u) | 0x7f800000u)) : float_rz(d);
+    }
+    return float_of((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
 }
 DEV void split_ff(double d, float& hi, float& lo) {
     const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
@@ -540,24 +598,6 @@ HDEV T euler_alpha(const T* ub, const T* f, T m, T eps) {
 // 2^-109 and all of them together stay below 2^-100.  So T > 2^-16 A +
 // 2^-100 certifies T > 0 for both evaluations.  NaN, infinite, zero or
 // subnormal rho or m fail and are left to the float64 formula.
-HDEV int bits_of(float x) {
-#ifdef __CUDA_ARCH__
-    return __float_as_int(x);
-#else
-    int i;
-    std::memcpy(&i, &x, 4);
-    return i;
-#endif
-}
-HDEV float float_of(int i) {
-#ifdef __CUDA_ARCH__
-    return __int_as_float(i);
-#else
-    float x;
-    std::memcpy(&x, &i, 4);
-    return x;
-#endif
-}
 HDEV float pow2f(int k) { return float_of((127 + k) << 23); }  // 2^k, -126 <= k <= 127
 
 HDEV bool euler_alpha_is_one(const float* ub, const float* f, float m, float ome) {

@@ -736,7 +736,7 @@ store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
             avg[m.E + e] = ul[0];
         } else {
             // float copies for the certificate of the facet limiter (euler_alpha_is_one)
-            cf_out[(1 + c) * m.E + e] = narrow(bl);
+            cf_out[(1 + c) * m.E + e] = cert_float(bl);
         }
     }
     cf_out[e] = sf;  // the float speed sum (dt_e in float for the update)
@@ -858,10 +858,10 @@ store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
             q_out[e] = fmax(0.0, (0.25 * s) * (pr.umax - bl));
             q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
         } else {
-            cf_out[(1 + c) * m.E + e] = narrow(bl);  // for the certificate of the facet limiter
+            cf_out[(1 + c) * m.E + e] = cert_float(bl);  // for the certificate of the facet limiter
         }
     }
-    if (NC > 1) cf_out[e] = narrow(s);
+    if (NC > 1) cf_out[e] = cert_float(s);
     return dte;
 }
 
@@ -2156,7 +2156,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     float fAf[NC], fAm[NC], ub[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
-                        fAf[c] = sizeof(R) == 4 ? __fsub_rn((float)FLr[d][c], (float)FHr[d][c]) : narrow(fA[c]);
+                        fAf[c] = sizeof(R) == 4 ? __fsub_rn((float)FLr[d][c], (float)FHr[d][c]) : cert_float(fA[c]);
                         fAm[c] = -fAf[c];
                     }
                     bool one = true;
@@ -2783,7 +2783,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                 float fA[NC], ub[NC];
 #pragma unroll
                 for (int c = 0; c < NC; ++c)
-                    fA[c] = sizeof(R) == 4 ? __fsub_rn((float)FL[c], (float)FH[c]) : narrow((double)FL[c] - (double)FH[c]);
+                    fA[c] = sizeof(R) == 4 ? __fsub_rn((float)FL[c], (float)FH[c]) : cert_float((double)FL[c] - (double)FH[c]);
                 if (f.eL >= 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * E + f.eL];
@@ -3013,7 +3013,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
     if (pr.mode == MODE_WENO_L) {
 #pragma unroll
         for (int i = 0; i < N2; ++i) sF[i][c][tx] = F[i];
-        sU[c][tx] = narrow(ubd);
+        sU[c][tx] = cert_float(ubd);
         __syncthreads();
         float ubf[NC];
         const bool cert = !(pr.opts & OPT_FP64_LIMITER);
@@ -3026,7 +3026,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
             if (cert) {
                 float ff[NC];
 #pragma unroll
-                for (int k = 0; k < NC; ++k) ff[k] = sizeof(R) == 4 ? (float)sF[i][k][tx] : narrow((double)sF[i][k][tx]);
+                for (int k = 0; k < NC; ++k) ff[k] = sizeof(R) == 4 ? (float)sF[i][k][tx] : cert_float((double)sF[i][k][tx]);
                 float mi = m.me_f;
                 if (lgl) mi = (float)(m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]));
                 if (euler_alpha_is_one(ubf, ff, mi, pr.ome_f)) continue;
