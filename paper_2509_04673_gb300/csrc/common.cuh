@@ -593,24 +593,31 @@ HDEV T euler_alpha(const T* ub, const T* f, T m, T eps) {
 // evaluated in float together with A, the same expression with every
 // monomial in absolute value.  With n operations and k inputs off by 2^-23
 // (n + 2k < 60) the float error is below (n + 2k) 2^-24 A and the float64 one
-// below (n + k) 2^-53 A.  Scaled values are required to be at most 2^40, so
-// an underflowed input or product (error <= 2^-150) is amplified to at most
-// 2^-109 and all of them together stay below 2^-100.  So T > 2^-16 A +
-// 2^-100 certifies T > 0 for both evaluations.  NaN, infinite, zero or
+// below (n + k) 2^-53 A.  Inputs cut from float64 data (ub always, f in the
+// float64 form) are off by up to 2^-149 besides where they are subnormal in
+// float; the scaling multiplies that by 1/rho and 1/(rho m).  rho >= 2^-44 and,
+// in the float64 form, rho m >= 2^-44 (products of the powers of two) keep it
+// below 2^-105, and with the scaled |f_rho| <= 4 all terms that it enters, but
+// for those that 2^-16 A covers, stay below 2^-100.  Scaled values are required
+// to be at most 2^40 (no overflow); an underflowed product adds 2^-149.  So T >
+// 2^-16 A + 2^-100 certifies T > 0 for both evaluations.  NaN, infinite, zero or
 // subnormal rho or m fail and are left to the float64 formula.
 HDEV float pow2f(int k) { return float_of((127 + k) << 23); }  // 2^k, -126 <= k <= 127
 
+// R: the precision of the contributions f that the floats hold
+template <class R = float>
 HDEV bool euler_alpha_is_one(const float* ub, const float* f, float m, float ome) {
     const int brho = bits_of(ub[0]), bm = bits_of(m);
     const int erho = (brho >> 23) & 0xff, em = (bm >> 23) & 0xff;
-    // rho and m positive, normal and finite
-    if (brho <= 0 || bm <= 0 || erho == 0 || em == 0 || erho == 0xff || em == 0xff) return false;
+    // rho and m positive, normal and finite, rho and rho m as above
+    if (brho <= 0 || bm <= 0 || erho < 127 - 44 || em == 0 || erho == 0xff || em == 0xff) return false;
+    if (sizeof(R) == 8 && erho + em < 254 - 44) return false;
     const float sj = pow2f(127 - erho), sk = pow2f(127 - em);  // rho sj, m sk in [1, 2)
     const float rho = ub[0] * sj, mx = ub[1] * sj, my = ub[2] * sj, E = ub[3] * sj;
     const float fr = (f[0] * sj) * sk, fmx = (f[1] * sj) * sk, fmy = (f[2] * sj) * sk, fE = (f[3] * sj) * sk;
     const float ms = m * sk;
     const float big = 0x1p40f;
-    if (!(fabsf(mx) <= big && fabsf(my) <= big && fabsf(E) <= big && fabsf(fr) <= big && fabsf(fmx) <= big &&
+    if (!(fabsf(mx) <= big && fabsf(my) <= big && fabsf(E) <= big && fabsf(fr) <= 4.f && fabsf(fmx) <= big &&
           fabsf(fmy) <= big && fabsf(fE) <= big))
         return false;
     const float K = 0x1p-16f, A0 = 0x1p-100f;

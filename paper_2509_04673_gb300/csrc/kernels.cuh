@@ -2163,12 +2163,12 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     if (Lc >= 0) {
 #pragma unroll
                         for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Lc];
-                        one = euler_alpha_is_one(ub, fAf, 0.25f * cf[Lc], pr.ome_f);
+                        one = euler_alpha_is_one<R>(ub, fAf, 0.25f * cf[Lc], pr.ome_f);
                     }
                     if (one && Rc >= 0) {
 #pragma unroll
                         for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Rc];
-                        one = euler_alpha_is_one(ub, fAm, 0.25f * cf[Rc], pr.ome_f);
+                        one = euler_alpha_is_one<R>(ub, fAm, 0.25f * cf[Rc], pr.ome_f);
                     }
                     if (one) {
 #pragma unroll
@@ -2397,7 +2397,7 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
                     float ff[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) ff[c] = (float)F[c][i];
-                    if (euler_alpha_is_one(ubf, ff, m.me_f, pr.ome_f)) continue;
+                    if (euler_alpha_is_one<R>(ubf, ff, m.me_f, pr.ome_f)) continue;
                 }
                 double f[NC];
 #pragma unroll
@@ -2787,7 +2787,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                 if (f.eL >= 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * E + f.eL];
-                    one = euler_alpha_is_one(ub, fA, 0.25f * cf[f.eL], pr.ome_f);
+                    one = euler_alpha_is_one<R>(ub, fA, 0.25f * cf[f.eL], pr.ome_f);
                 }
                 if (one && f.eR >= 0) {
 #pragma unroll
@@ -2795,7 +2795,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                         ub[c] = cf[(1 + c) * E + f.eR];
                         fA[c] = -fA[c];
                     }
-                    one = euler_alpha_is_one(ub, fA, 0.25f * cf[f.eR], pr.ome_f);
+                    one = euler_alpha_is_one<R>(ub, fA, 0.25f * cf[f.eR], pr.ome_f);
                 }
             }
             if (!one) {
@@ -3029,7 +3029,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
                 for (int k = 0; k < NC; ++k) ff[k] = sizeof(R) == 4 ? (float)sF[i][k][tx] : cert_float((double)sF[i][k][tx]);
                 float mi = m.me_f;
                 if (lgl) mi = (float)(m.h * m.h * (TL.wl[i % N1] * TL.wl[i / N1]));
-                if (euler_alpha_is_one(ubf, ff, mi, pr.ome_f)) continue;
+                if (euler_alpha_is_one<R>(ubf, ff, mi, pr.ome_f)) continue;
             }
             double f[NC], ub[NC];
 #pragma unroll

@@ -50,7 +50,7 @@ int main(int argc, char** argv) {
             ubf[c] = cgl::cert_float(ub[c]);
             ff[c] = cgl::cert_float(f[c]);
         }
-        if (!cgl::euler_alpha_is_one(ubf, ff, t % 5 ? (float)m : cgl::cert_float(m), ome)) continue;
+        if (!cgl::euler_alpha_is_one<double>(ubf, ff, t % 5 ? (float)m : cgl::cert_float(m), ome)) continue;
         ++certified;
         if (cgl::euler_alpha<double>(ub, f, m, eps) != 1.0 && ++wrong < 5)
             std::fprintf(stderr, "wrong: ub %.9g %.9g %.9g %.9g f %.9g %.9g %.9g %.9g m %.9g\n", ub[0], ub[1], ub[2],

@@ -28,10 +28,13 @@ def check(tmp_path_factory):
     return run
 
 
-# decades of the density and of m: ordinary ones (most factors are certified there), and around and
-# beyond the largest float
+# decades of the density and of m: ordinary ones (most factors are certified there), around and beyond
+# the largest float, and where contributions or averages are subnormal or zero as floats
 @pytest.mark.parametrize("decades,least", [((-8, 3, -9, -1), 0.2), ((30, 45, -9, -1), 0.0), ((37, 39, -2, 2), 0.0),
-                                           ((38, 120, -20, 40), 0.0), ((20, 38, 0, 60), 0.0)])
+                                           ((38, 120, -20, 40), 0.0), ((20, 38, 0, 60), 0.0),
+                                           ((-38, -30, -12, -1), 0.0), ((-45, -20, -30, -5), 0.0),
+                                           ((-20, -5, -30, -1), 0.0), ((-8, 3, -40, -20), 0.0),
+                                           ((-60, -20, 0, 40), 0.0)])
 def test_certificate_on_float64_data(check, decades, least):
     out, err = check(*decades)
     assert out["wrong"] == 0, (out, err)
