@@ -48,6 +48,21 @@ namespace cgl {
 // element-vector layout: value v of local node i of element e, NV values
 DEV long long ev_at(long long E, int e, int i, int v, int NV) { return (long long)(i * NV + v) * E + e; }
 
+// Value k of element e in an array of several values per element, [k][e].  A
+// scalar state takes 192 bytes per element and more, so that three values of
+// every element that fits one GPU can exceed 2^32; a system 592, so that eight
+// cannot exceed 2^32 nor four 2^31 (those are indexed in 32 bits in place).
+// 64-bit offsets throughout cost 2 % per step (Euler blast 2048^2 Q2 10.27 ->
+// 10.49 ms).
+template <int NC>
+DEV auto off(int E, int k, int e) {
+    if constexpr (NC == 1) return (long long)k * E + e;
+    else return (unsigned)k * (unsigned)E + (unsigned)e;
+}
+// the values k of an array of more than eight
+template <class T>
+DEV T* field(T* p, int E, int k) { return p + (long long)k * E; }
+
 
 // Programmatic dependent launch: every kernel of a stage first lets the next
 // kernel of the stream be scheduled (it launches once all blocks of this one
@@ -710,8 +725,8 @@ DEV double lo_outputs_mixed(const MeshDev& m, const ProbDev& pr, const float* __
     }
     const double dte = m.h * rs;
     dte_out[e] = dte;
-    dte_out[m.E + e] = rs;
-    dte_out[2 * m.E + e] = s * m.inv_h;
+    dte_out[off<NC>(m.E, 1, e)] = rs;
+    dte_out[off<NC>(m.E, 2, e)] = s * m.inv_h;
 #pragma unroll
     for (int d = 0; d < 4; ++d)
 store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
@@ -730,13 +745,13 @@ store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
             // gaps in float64, both factors and the product rounded toward zero
             // (smaller magnitudes stay admissible)
             q_out[e] = __fmul_rz(s4, fmaxf(0.f, narrow(pr.umax - bl)));
-            q_out[m.E + e] = __fmul_rz(s4, fminf(0.f, narrow(pr.umin - bl)));
+            q_out[off<NC>(m.E, 1, e)] = __fmul_rz(s4, fminf(0.f, narrow(pr.umin - bl)));
             // the float-float mean, for the element contributions of k_update_el
             avg[e] = uh[0];
-            avg[m.E + e] = ul[0];
+            avg[off<NC>(m.E, 1, e)] = ul[0];
         } else {
             // float copies for the certificate of the facet limiter (euler_alpha_is_one)
-            cf_out[(1 + c) * m.E + e] = cert_float(bl);
+            cf_out[off<NC>(m.E, 1 + c, e)] = cert_float(bl);
         }
     }
     cf_out[e] = sf;  // the float speed sum (dt_e in float for the update)
@@ -841,8 +856,8 @@ DEV double lo_outputs_fp64(const MeshDev& m, const ProbDev& pr, const double* __
     }
     const double dte = m.h * rs;
     dte_out[e] = dte;
-    dte_out[m.E + e] = rs;              // dt_e / h
-    dte_out[2 * m.E + e] = s * m.inv_h; // 1 / dt_e
+    dte_out[off<NC>(m.E, 1, e)] = rs;              // dt_e / h
+    dte_out[off<NC>(m.E, 2, e)] = s * m.inv_h; // 1 / dt_e
 #pragma unroll
     for (int d = 0; d < 4; ++d)
 store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
@@ -856,9 +871,9 @@ store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
             // (|K|/|dK|)(umax - ubar^{e,L})/dt_e = (s/4)(umax - ubar^{e,L}) >= 0, and
             // (s/4)(umin - ubar^{e,L}) <= 0
             q_out[e] = fmax(0.0, (0.25 * s) * (pr.umax - bl));
-            q_out[m.E + e] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
+            q_out[off<NC>(m.E, 1, e)] = fmin(0.0, (0.25 * s) * (pr.umin - bl));
         } else {
-            cf_out[(1 + c) * m.E + e] = cert_float(bl);  // for the certificate of the facet limiter
+            cf_out[off<NC>(m.E, 1 + c, e)] = cert_float(bl);  // for the certificate of the facet limiter
         }
     }
     if (NC > 1) cf_out[e] = cert_float(s);
@@ -887,8 +902,8 @@ __global__ void k_avg(MeshDev m, ProbDev pr, const R* __restrict__ u, float* __r
         if constexpr (sizeof(R) == 4) {
             float hi, lo;
             ff_mean<N2>(U, hi, lo);
-            avg[(2 * c) * m.E + e] = hi;
-            avg[(2 * c + 1) * m.E + e] = lo;
+            avg[off<NC>(m.E, 2 * c, e)] = hi;
+            avg[off<NC>(m.E, 2 * c + 1, e)] = lo;
             uh[c] = hi;
         } else {
             uh[c] = cell_mean<R, P>(m, U);
@@ -900,11 +915,11 @@ __global__ void k_avg(MeshDev m, ProbDev pr, const R* __restrict__ u, float* __r
     Ph::speed_parts(uh, PV<R>::gam(pr), q);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        cq[c * m.E + e] = fx[c];
-        cq[(NC + c) * m.E + e] = fy[c];
+        field(cq, m.E, c)[e] = fx[c];
+        field(cq, m.E, NC + c)[e] = fy[c];
     }
 #pragma unroll
-    for (int k = 0; k < Ph::NPART; ++k) cq[(2 * NC + k) * m.E + e] = q[k];
+    for (int k = 0; k < Ph::NPART; ++k) field(cq, m.E, 2 * NC + k)[e] = q[k];
 }
 
 // element of position i of a tile's halo rows (tiles of K_TX x TY elements, one
@@ -1107,18 +1122,17 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? (SUB ? 5 : 6) : (SUB ? 
         FacetItem f;
         if (!facet_item(m, ex0, ey0, axis, f)) continue;
         R F[NC], lam;
-        const R* __restrict__ fa = cq + (long long)(f.axis * NC) * E;  // the means' fluxes along the facet's axis
+        const R* __restrict__ fa = field(cq, E, f.axis * NC);  // the means' fluxes along the facet's axis
         if (f.eL >= 0 && f.eR >= 0) {
-            const R* __restrict__ q = cq + (long long)(2 * NC) * E;
-            const R* __restrict__ qv = q + (long long)f.axis * E;
-            const R l = Ph::facet_speed_parts(qv[f.eL], q[2 * E + f.eL], q[3 * E + f.eL], q[4 * E + f.eL], q[5 * E + f.eL],
-                                              qv[f.eR], q[2 * E + f.eR], q[3 * E + f.eR], q[4 * E + f.eR], q[5 * E + f.eR],
-                                              g);
+            const R* __restrict__ q = field(cq, E, 2 * NC + 2);
+            const R* __restrict__ qv = field(cq, E, 2 * NC + f.axis);
+            const R l = Ph::facet_speed_parts(qv[f.eL], q[f.eL], q[E + f.eL], q[2 * E + f.eL], q[3 * E + f.eL], qv[f.eR],
+                                              q[f.eR], q[E + f.eR], q[2 * E + f.eR], q[3 * E + f.eR], g);
             if constexpr (sizeof(R) == 4) {
                 lam = __fmul_rn(l, 1.0f + 0x1p-20f);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    const float* __restrict__ ah = avg + (long long)(2 * c) * E;
+                    const float* __restrict__ ah = field(avg, E, 2 * c);
                     F[c] = llf_value(fa[c * E + f.eL], fa[c * E + f.eR], lam,
                                      ff_diff(ah[f.eR], ah[E + f.eR], ah[f.eL], ah[E + f.eL]));
                 }
@@ -1136,8 +1150,8 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? (SUB ? 5 : 6) : (SUB ? 
                 CompVec<float, NC> vh, vl, vf;
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    vh.v[c] = avg[(long long)(2 * c) * E + e];
-                    vl.v[c] = avg[(long long)(2 * c + 1) * E + e];
+                    vh.v[c] = avg[off<NC>(E, 2 * c, e)];
+                    vl.v[c] = avg[off<NC>(E, 2 * c + 1, e)];
                     vf.v[c] = fa[c * E + e];
                 }
                 const CompVec<float, NC + 1> o =
@@ -1179,8 +1193,8 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? (SUB ? 5 : 6) : (SUB ? 
             float ul[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                us[c] = avg[(long long)(2 * c) * E + e];
-                ul[c] = avg[(long long)(2 * c + 1) * E + e];
+                us[c] = avg[off<NC>(E, 2 * c, e)];
+                ul[c] = avg[off<NC>(E, 2 * c + 1, e)];
             }
             dte = lo_outputs_mixed<P, Ph, SUB>(m, pr, u, lam, F, us, ul, ue_io, dte_out, ubl_out, nullptr, fl_out, cf_out,
                                                nullptr, ex, ey, e);
@@ -2007,8 +2021,8 @@ __device__ __noinline__ CompVec<double, Ph::NC + 1> reduce_pseudo_step(const Pro
 DEV void store_reduced_step(const MeshDev& m, double* dte_a, float* cf, double rs2, int e) {
     const double dte2 = m.h * rs2;
     dte_a[e] = dte2;
-    dte_a[m.E + e] = rs2;
-    dte_a[2 * m.E + e] = 1.0 / dte2;
+    dte_a[off<1>(m.E, 1, e)] = rs2;
+    dte_a[off<1>(m.E, 2, e)] = 1.0 / dte2;
     cf[e] = __double2float_ru(1.0 / rs2);
 }
 
@@ -2136,10 +2150,10 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                 R fmaxv = inf, fminv = -inf;
                 if (Lc >= 0) {
                     fmaxv = fmin(fmaxv, qcap[Lc]);
-                    fminv = fmax(fminv, qcap[m.E + Lc]);
+                    fminv = fmax(fminv, qcap[off<NC>(m.E, 1, Lc)]);
                 }
                 if (Rc >= 0) {
-                    fmaxv = fmin(fmaxv, -qcap[m.E + Rc]);
+                    fmaxv = fmin(fmaxv, -qcap[off<NC>(m.E, 1, Rc)]);
                     fminv = fmax(fminv, -qcap[Rc]);
                 }
                 FBr[d] = (fA >= R(0)) ? fmin(fA, fmaxv) : fmax(fA, fminv);
@@ -2162,12 +2176,12 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     bool one = true;
                     if (Lc >= 0) {
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Lc];
+                        for (int c = 0; c < NC; ++c) ub[c] = cf[off<NC>(m.E, 1 + c, Lc)];
                         one = euler_alpha_is_one<R>(ub, fAf, 0.25f * cf[Lc], pr.ome_f);
                     }
                     if (one && Rc >= 0) {
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * m.E + Rc];
+                        for (int c = 0; c < NC; ++c) ub[c] = cf[off<NC>(m.E, 1 + c, Rc)];
                         one = euler_alpha_is_one<R>(ub, fAm, 0.25f * cf[Rc], pr.ome_f);
                     }
                     if (one) {
@@ -2188,7 +2202,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                     double ub[NC];
 #pragma unroll
                     for (int c = 0; c < NC; ++c) ub[c] = ubl[c * m.E + Lc];
-                    double mL = (0.25 * h) * dte_a[2 * m.E + Lc];
+                    double mL = (0.25 * h) * dte_a[off<NC>(m.E, 2, Lc)];
                     alpha = fmin(alpha, euler_alpha<double>(ub, fA, mL, pr.pos_eps));
                 }
                 if (Rc >= 0) {
@@ -2198,7 +2212,7 @@ DEV void facet_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][Di
                         ub[c] = ubl[c * m.E + Rc];
                         fm[c] = -fA[c];
                     }
-                    double mR = (0.25 * h) * dte_a[2 * m.E + Rc];
+                    double mR = (0.25 * h) * dte_a[off<NC>(m.E, 2, Rc)];
                     alpha = fmin(alpha, euler_alpha<double>(ub, fm, mR, pr.pos_eps));
                 }
                 if constexpr (mixed_sys) {
@@ -2318,8 +2332,8 @@ DEV void element_part(const MeshDev& m, const ProbDev& pr, const R (&U)[Ph::NC][
         R ueh, uel;
         if constexpr (sizeof(R) == 4) {
             // the float-float mean itself (k_lo for scalars, k_avg for systems)
-            ueh = avg[(2 * c) * m.E + e];
-            uel = avg[(2 * c + 1) * m.E + e];
+            ueh = avg[off<NC>(m.E, 2 * c, e)];
+            uel = avg[off<NC>(m.E, 2 * c + 1, e)];
         } else {
             split<R>(uec[c], ueh, uel);
         }
@@ -2435,8 +2449,8 @@ DEV void update_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
     const double me = m.me;
     const double dt = *dtp;
     const double dte = dte_a[e];
-    const double rs = dte_a[m.E + e];       // dt_e / h
-    const double rdte = dte_a[2 * m.E + e]; // 1 / dt_e
+    const double rs = dte_a[off<NC>(m.E, 1, e)];       // dt_e / h
+    const double rdte = dte_a[off<NC>(m.E, 2, e)]; // 1 / dt_e
     int nb[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) nb[d] = neighbour(m, ex, ey, d);
@@ -2458,8 +2472,8 @@ DEV void update_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ u,
         // a pseudo time step decreased by the remark after eq. (dtmaxcell)
         const double dte2 = h * rs2;
         dte_a[e] = dte2;
-        dte_a[m.E + e] = rs2;
-        dte_a[2 * m.E + e] = 1.0 / dte2;
+        dte_a[off<NC>(m.E, 1, e)] = rs2;
+        dte_a[off<NC>(m.E, 2, e)] = 1.0 / dte2;
         element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, dt, dte2, 1.0 / dte2, ubec, fh, EW, beta_out, cnt, ex,
                                ey, e);
         return;
@@ -2502,7 +2516,7 @@ __global__ void __launch_bounds__(128) k_q1_facet(MeshDev m, ProbDev pr, const R
     double ubec[NC];
     R fh[NC];
     double rs2;  // eq. (aecQ1) is not combined with the pseudo-time-step reduction
-    facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, dte_a[m.E + e], dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2,
+    facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, dte_a[off<NC>(m.E, 1, e)], dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2,
                          cnt);
 #pragma unroll
     for (int c = 0; c < NC; ++c) ube_out[c * m.E + e] = ubec[c];
@@ -2584,7 +2598,7 @@ __global__ void k_udl(MeshDev m, const R* __restrict__ u, const double* __restri
                 for (int i = 0; i < 2; ++i) {
                     if (i < c.nxc) {
                         const int e = ey * m.nx + (i ? c.ex1 : c.ex0);
-                        s += (ube[k * m.E + e] - ui) * dte_a[2 * m.E + e];
+                        s += (ube[k * m.E + e] - ui) * dte_a[off<NC>(m.E, 2, e)];
                     }
                 }
             }
@@ -2615,7 +2629,7 @@ __global__ void __launch_bounds__(128) k_q1_update(MeshDev m, ProbDev pr, const 
         ubec[c] = ube[c * m.E + e];
         fh[c] = R(0);
     }
-    element_part<R, P, Ph, true>(m, pr, U, udl, ER, cf, avg, uec, *dtp, dte_a[e], dte_a[2 * m.E + e], ubec, fh, EW,
+    element_part<R, P, Ph, true>(m, pr, U, udl, ER, cf, avg, uec, *dtp, dte_a[e], dte_a[off<NC>(m.E, 2, e)], ubec, fh, EW,
                                  beta_out, cnt, ex, ey, e, gam[e]);
 }
 
@@ -2639,7 +2653,7 @@ DEV void facet_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__ 
     R fh[1];
     uec[0] = pr.fl == FL_NONE ? ue[e] : 0.0;  // u^e enters ubar^e only without the flux limiter
     ublc[0] = ubl[e];
-    const double rs = dte_a[m.E + e];
+    const double rs = dte_a[off<1>(m.E, 1, e)];
     double rs2;
     facet_part<R, P, Ph>(m, pr, U, nb, uec, ublc, rs, dte_a, ubl, qcap, fl_in, cf, e, ubec, fh, rs2, cnt);
     ube_out[e] = ubec[0];
@@ -2666,7 +2680,7 @@ DEV void update_el_at(const MeshDev& m, const ProbDev& pr, const R* __restrict__
         element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, 0.0, 0.0, ubec, fh, EW, beta_out, cnt, ex, ey, e);
     } else {
         const double uec[1] = {ue[e]};
-        element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, dte_a[e], dte_a[2 * m.E + e], ubec, fh, EW, beta_out,
+        element_part<R, P, Ph>(m, pr, U, ud, ER, cf, avg, uec, *dtp, dte_a[e], dte_a[off<1>(m.E, 2, e)], ubec, fh, EW, beta_out,
                                cnt, ex, ey, e);
     }
 }
@@ -2786,13 +2800,13 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                     fA[c] = sizeof(R) == 4 ? __fsub_rn((float)FL[c], (float)FH[c]) : cert_float((double)FL[c] - (double)FH[c]);
                 if (f.eL >= 0) {
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) ub[c] = cf[(1 + c) * E + f.eL];
+                    for (int c = 0; c < NC; ++c) ub[c] = cf[off<NC>(E, 1 + c, f.eL)];
                     one = euler_alpha_is_one<R>(ub, fA, 0.25f * cf[f.eL], pr.ome_f);
                 }
                 if (one && f.eR >= 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
-                        ub[c] = cf[(1 + c) * E + f.eR];
+                        ub[c] = cf[off<NC>(E, 1 + c, f.eR)];
                         fA[c] = -fA[c];
                     }
                     one = euler_alpha_is_one<R>(ub, fA, 0.25f * cf[f.eR], pr.ome_f);
@@ -2805,7 +2819,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                 if (f.eL >= 0) {
 #pragma unroll
                     for (int c = 0; c < NC; ++c) ub[c] = ubl[c * E + f.eL];
-                    alpha = fmin(alpha, euler_alpha_rare(ub, fA, (0.25 * m.h) * dte_a[2 * E + f.eL], pr.pos_eps));
+                    alpha = fmin(alpha, euler_alpha_rare(ub, fA, (0.25 * m.h) * dte_a[off<NC>(E, 2, f.eL)], pr.pos_eps));
                 }
                 if (f.eR >= 0) {
                     double fm[NC];
@@ -2814,7 +2828,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
                         ub[c] = ubl[c * E + f.eR];
                         fm[c] = -fA[c];
                     }
-                    alpha = fmin(alpha, euler_alpha_rare(ub, fm, (0.25 * m.h) * dte_a[2 * E + f.eR], pr.pos_eps));
+                    alpha = fmin(alpha, euler_alpha_rare(ub, fm, (0.25 * m.h) * dte_a[off<NC>(E, 2, f.eR)], pr.pos_eps));
                 }
                 if (alpha != 1.0) {
 #pragma unroll
@@ -2847,7 +2861,7 @@ __global__ void __launch_bounds__(F_NT, sizeof(R) == 4 ? 6 : 3)
     int at[4];
 #pragma unroll
     for (int d = 0; d < 4; ++d) at[d] = facet_of(tx, ty, d);
-    const double rs = dte_a[E + e];
+    const double rs = dte_a[off<NC>(E, 1, e)];
     double rs2 = rs, ub[NC];
     R fh[NC];
     // (m_i^e / |K_e|) |S| times the outward sum of f^H, the facet term of eq.
@@ -2946,7 +2960,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
         thR = __fmul_rn(__fadd_rn(dth, dtl), __fmul_rn(s, m.inv_h_f));
         dteR = __fmul_rn(m.h_f, __frcp_rn(s));
     } else {
-        thR = *dtp * dte_a[2 * m.E + e];
+        thR = *dtp * dte_a[off<NC>(m.E, 2, e)];
         dteR = dte_a[e];
     }
     if (valid && c == 0 && thR > R(1)) atomicAdd(&cnt[CNT_CFL], 1ull);
@@ -2975,8 +2989,8 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
         for (int i = 0; i < N2; ++i) F[i] = r[(long long)(i * NC) * m.E];
         R ueh, uel;
         if constexpr (sizeof(R) == 4) {
-            ueh = avg[(2 * c) * m.E + e];
-            uel = avg[(2 * c + 1) * m.E + e];
+            ueh = avg[off<NC>(m.E, 2 * c, e)];
+            uel = avg[off<NC>(m.E, 2 * c + 1, e)];
         } else {
             split<R>(ue[c * m.E + e], ueh, uel);
         }
