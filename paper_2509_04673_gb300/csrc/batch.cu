@@ -186,10 +186,10 @@ DEV void node_phase_body(int phase, const InstDev& D, const MeshDev& m, int gx0,
         case PH_GRADF:
             // right-hand side and first sweep in one pass (k carries k_g: b is
             // kept only when more sweeps follow)
-            grad_sweep_seg<float, P, 1, BatchTile<P, NT, true>>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tid, ws);
+            grad_sweep_seg<float, P, 1, 1, BatchTile<P, NT, true>>(m, D.u, k > 1 ? D.bg : nullptr, D.g2, gx0, gy0, tid, ws);
             break;
-        case PH_GATHERF: udot_sweep_seg<float, P, 1, TL>(m, D.ER, D.r, D.ud2, gx0, gy0, tid, ws); break;
-        case PH_GRAD: grad_rhs_seg<float, P, 1, TL>(m, D.u, D.bg, D.g, gx0, gy0, tid, ws); break;
+        case PH_GATHERF: udot_sweep_seg<float, P, 1, 1, TL>(m, D.ER, D.r, D.ud2, gx0, gy0, tid, ws); break;
+        case PH_GRAD: grad_rhs_seg<float, P, 1, 1, TL>(m, D.u, D.bg, D.g, gx0, gy0, tid, ws); break;
         case PH_SWEEP_G:
             if (k & 1) mass_sweep_seg<float, P, 2, TL>(m, D.g2, D.bg, D.g, gx0, gy0, tid, ws);
             else mass_sweep_seg<float, P, 2, TL>(m, D.g, D.bg, D.g2, gx0, gy0, tid, ws);

@@ -273,7 +273,7 @@ DEV bool tile_full(const MeshDev& m, int gx0, int gy0) {
 // x pass with the derivative and the mass operator, y pass to b and g0 on the
 // one-element halo, then the sweep's x and y passes.  A thread keeps b and g0
 // of its own nodes in registers from the first y pass to the second.
-template <class R, int P, int NC, class TL, bool FULL>
+template <class R, int P, int NC, int NF, class TL, bool FULL>
 DEV void grad_sweep_body(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
                          int gy0, int tid, R* ws) {
     constexpr int TEY = TL::TEY, S1 = TL::S1, KY = TL::KY, RY = TL::RY, RX = TL::RX;
@@ -289,10 +289,10 @@ DEV void grad_sweep_body(const MeshDev& m, const R* __restrict__ u, R* __restric
     Stage<R, P, TL, 2, TL::W2, TL::H2, TL::PU, TL::S2, FULL> in(m, gx0, gy0, tid);
     in.template load<true>(m, u, tid);
 #pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
+    for (int c = 0; c < NF; ++c) {
         in.store(A, tid);
         __syncthreads();
-        if (c + 1 < NC) in.template load<true>(m, u + (c + 1) * m.NN, tid);
+        if (c + 1 < NF) in.template load<true>(m, u + (c + 1) * m.NN, tid);
         if (feeds_seg) {
             const R* X = A + t.xr * TL::S2 + t.xs + 1;
             R* Y = B + t.xr * S1 + t.xs;
@@ -369,7 +369,7 @@ DEV void grad_sweep_body(const MeshDev& m, const R* __restrict__ u, R* __restric
 }
 
 // b and g0 alone, from u on a one-element halo
-template <class R, int P, int NC, class TL, bool FULL>
+template <class R, int P, int NC, int NF, class TL, bool FULL>
 DEV void grad_rhs_body(const MeshDev& m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout, int gx0,
                        int gy0, int tid, R* ws) {
     constexpr int TEY = TL::TEY, S1 = TL::S1, RX = TL::RX, RY = TL::RY;
@@ -382,10 +382,10 @@ DEV void grad_rhs_body(const MeshDev& m, const R* __restrict__ u, R* __restrict_
     Stage<R, P, TL, 1, TL::W1, TL::H1, TL::PG, S1, FULL> in(m, gx0, gy0, tid);
     in.template load<true>(m, u, tid);
 #pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
+    for (int c = 0; c < NF; ++c) {
         in.store(A, tid);
         __syncthreads();
-        if (c + 1 < NC) in.template load<true>(m, u + (c + 1) * m.NN, tid);
+        if (c + 1 < NF) in.template load<true>(m, u + (c + 1) * m.NN, tid);
         if (t.own_seg) {
             const R* X = A + t.xr * S1 + t.xs;
             R* Y = B + t.xr * S1 + t.xs;
@@ -479,7 +479,7 @@ DEV void mass_sweep_body(const MeshDev& m, const R* __restrict__ xin, const R* _
 // value are consecutive in the element index, and no lane branches on its
 // node's position in the element.  r = sum over E_i (stored for further sweeps
 // and diagnostics), udot0 = r / m_i, udot1 = udot0 + (r - M_C udot0) / m_i.
-template <class R, int P, int NC, class TL, bool FULL>
+template <class R, int P, int NC, int NF, class TL, bool FULL>
 DEV void udot_sweep_body(const MeshDev& m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout,
                          int gx0, int gy0, int tid, R* ws) {
     constexpr int TEX = TL::TEX, TEY = TL::TEY, S1 = TL::S1, RY = TL::RY, N1 = P + 1;
@@ -493,7 +493,7 @@ DEV void udot_sweep_body(const MeshDev& m, const R* __restrict__ ER, R* __restri
     const SegThread<R, P, TL, FULL> t(m, gx0, tid);
     const R w0 = vertex_weight<R, P, 0>(T, t.xkind);
 #pragma unroll 1
-    for (int v0 = 0; v0 < NC; v0 += FB) {
+    for (int v0 = 0; v0 < NF; v0 += FB) {
         if (v0 > 0) __syncthreads();  // the previous fields are consumed
 #pragma unroll 1
         for (int it = tid; it < NI && t.act; it += TL::NT) {
@@ -578,28 +578,29 @@ DEV void udot_sweep_body(const MeshDev& m, const R* __restrict__ ER, R* __restri
     }
 }
 
-// The same on any tile: inside the mesh or at its edge.  ws: TL::grad_ws,
-// rhs_ws, sweep_ws or udot_ws(NC) values.  All threads of the block call them
-// together.
-template <class R, int P, int NC, class TL>
+// The same on any tile, inside the mesh or at its edge, for NF of the fields
+// (pointers to the first of them; of the udot sweep a multiple of
+// udot_fields(NC)).  ws: TL::grad_ws, rhs_ws, sweep_ws or udot_ws(NC) values.
+// All threads of the block call them together.
+template <class R, int P, int NC, int NF, class TL>
 DEV void grad_sweep_seg(const MeshDev& m, const R* u, R* bout, R* gout, int gx0, int gy0, int tid, R* ws) {
-    if (tile_full<P, TL, 2>(m, gx0, gy0)) grad_sweep_body<R, P, NC, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
-    else grad_sweep_body<R, P, NC, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
+    if (tile_full<P, TL, 2>(m, gx0, gy0)) grad_sweep_body<R, P, NC, NF, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
+    else grad_sweep_body<R, P, NC, NF, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
 }
-template <class R, int P, int NC, class TL>
+template <class R, int P, int NC, int NF, class TL>
 DEV void grad_rhs_seg(const MeshDev& m, const R* u, R* bout, R* gout, int gx0, int gy0, int tid, R* ws) {
-    if (tile_full<P, TL, 1>(m, gx0, gy0)) grad_rhs_body<R, P, NC, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
-    else grad_rhs_body<R, P, NC, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
+    if (tile_full<P, TL, 1>(m, gx0, gy0)) grad_rhs_body<R, P, NC, NF, TL, true>(m, u, bout, gout, gx0, gy0, tid, ws);
+    else grad_rhs_body<R, P, NC, NF, TL, false>(m, u, bout, gout, gx0, gy0, tid, ws);
 }
 template <class R, int P, int NV, class TL>
 DEV void mass_sweep_seg(const MeshDev& m, const R* xin, const R* b, R* xout, int gx0, int gy0, int tid, R* ws) {
     if (tile_full<P, TL, 1>(m, gx0, gy0)) mass_sweep_body<R, P, NV, TL, true>(m, xin, b, xout, gx0, gy0, tid, ws);
     else mass_sweep_body<R, P, NV, TL, false>(m, xin, b, xout, gx0, gy0, tid, ws);
 }
-template <class R, int P, int NC, class TL>
+template <class R, int P, int NC, int NF, class TL>
 DEV void udot_sweep_seg(const MeshDev& m, const R* ER, R* rout, R* xout, int gx0, int gy0, int tid, R* ws) {
-    if (tile_full<P, TL, 2>(m, gx0, gy0)) udot_sweep_body<R, P, NC, TL, true>(m, ER, rout, xout, gx0, gy0, tid, ws);
-    else udot_sweep_body<R, P, NC, TL, false>(m, ER, rout, xout, gx0, gy0, tid, ws);
+    if (tile_full<P, TL, 2>(m, gx0, gy0)) udot_sweep_body<R, P, NC, NF, TL, true>(m, ER, rout, xout, gx0, gy0, tid, ws);
+    else udot_sweep_body<R, P, NC, NF, TL, false>(m, ER, rout, xout, gx0, gy0, tid, ws);
 }
 
 // The tiles of the single-state kernels (HALO: of the fused g_h kernel, by two
@@ -630,39 +631,54 @@ DEV R* dyn_shared() {
     return reinterpret_cast<R*>(dyn_smem);
 }
 
-template <class R, int P, int NC, int SIZE>
+// The stencil kernels.  A block takes NF of the fields: all of them, one after
+// the other with the next one's loads under the passes of this one, where the
+// tiles alone fill the GPU; else one (of the udot sweep udot_fields(NC)), and
+// the grid has a layer for each.
+template <int NF, int N>
+DEV long long first_field(const MeshDev& m) {
+    return NF == N ? 0 : (long long)(blockIdx.z * NF) * m.NN;
+}
+
+template <class R, int P, int NC, int NF, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT, SIZE ? 1 : (P == 3 ? 4 : 3))
     k_grad_sweep(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
     using TL = stage_tile_t<R, P, SIZE, true>;
     pdl_begin();
-    grad_sweep_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
-                                 dyn_shared<R>());
+    const long long at = first_field<NF, NC>(m);
+    grad_sweep_seg<R, P, NC, NF, TL>(m, u + at, bout ? bout + at : bout, gout + at, blockIdx.x * TL::NX, blockIdx.y * TL::NY,
+                                     threadIdx.x, dyn_shared<R>());
 }
 
-template <class R, int P, int NC, int SIZE>
+template <class R, int P, int NC, int NF, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_grad_rhs(MeshDev m, const R* __restrict__ u, R* __restrict__ bout, R* __restrict__ gout) {
     using TL = stage_tile_t<R, P, SIZE>;
     pdl_begin();
-    grad_rhs_seg<R, P, NC, TL>(m, u, bout, gout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
-                               dyn_shared<R>());
+    const long long at = first_field<NF, NC>(m);
+    grad_rhs_seg<R, P, NC, NF, TL>(m, u + at, bout + at, gout + at, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                                   dyn_shared<R>());
 }
 
-template <class R, int P, int NC, int SIZE>
+template <class R, int P, int NC, int NF, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_udot_sweep(MeshDev m, const R* __restrict__ ER, R* __restrict__ rout, R* __restrict__ xout) {
     using TL = stage_tile_t<R, P, SIZE>;
     pdl_begin();
-    udot_sweep_seg<R, P, NC, TL>(m, ER, rout, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
-                                 dyn_shared<R>());
+    const long long at = first_field<NF, NC>(m);
+    const R* __restrict__ er = ER + (NF == NC ? 0 : (long long)(blockIdx.z * NF) * m.E);
+    udot_sweep_seg<R, P, NC, NF, TL>(m, er, rout + at, xout + at, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+                                     dyn_shared<R>());
 }
 
-template <class R, int P, int NV, int SIZE>
+// (NV: the fields of a launch)
+template <class R, int P, int NV, int NF, int SIZE>
 __global__ void __launch_bounds__(stage_tile_t<R, P, SIZE>::NT)
     k_mass_sweep(MeshDev m, const R* __restrict__ xin, const R* __restrict__ b, R* __restrict__ xout) {
     using TL = stage_tile_t<R, P, SIZE>;
     pdl_begin();
-    mass_sweep_seg<R, P, NV, TL>(m, xin, b, xout, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
+    const long long at = first_field<NF, NV>(m);
+    mass_sweep_seg<R, P, NF, TL>(m, xin + at, b + at, xout + at, blockIdx.x * TL::NX, blockIdx.y * TL::NY, threadIdx.x,
                                  dyn_shared<R>());
 }
 

@@ -147,22 +147,33 @@ struct Stencils {
     void (*udot)(MeshDev, const R*, R*, R*);
     void (*sweep_g)(MeshDev, const R*, const R*, R*);
     void (*sweep_u)(MeshDev, const R*, const R*, R*);
-    dim3 grid, grid_halo, block;
+    dim3 grid_rhs, grid_grad, grid_udot, grid_g, grid_u, block;
     int ws_grad, ws_rhs, ws_udot, ws_sweep;
 };
 template <class R, int P, int NC, int SIZE>
 Stencils<R, P, NC> stencils_of(const MeshDev& m) {
     using T = stage_tile_t<R, P, SIZE>;
     using H = stage_tile_t<R, P, SIZE, true>;
+    // fields of a block: float launches over small tiles, which leave the GPU
+    // partly idle, have a layer of the grid for each field (the udot sweep for
+    // each udot_fields).  FP32-mixed Euler 60^2 Q3 with two sweeps: k_mass_sweep
+    // 25 -> 10 us, the step 365 -> 199; with one sweep 208 -> 167.  In float64
+    // the layers take the pipe from the sensor beside them (Euler 60^2 Q3 FP64
+    // 0.8 of the speed with them).
+    constexpr bool ONE = sizeof(R) == 4 && SIZE == 1;
+    constexpr int FB = T::udot_fields(NC);
+    const unsigned gx = nblk(m.nnx, T::NX), gy = nblk(m.nny, T::NY);
     Stencils<R, P, NC> s;
-    s.grad = k_grad_rhs<R, P, NC, SIZE>;
+    s.grad = k_grad_rhs<R, P, NC, ONE ? 1 : NC, SIZE>;
     s.grad_sweep = nullptr;
-    if constexpr (sizeof(R) == 4 || SIZE == 2) s.grad_sweep = k_grad_sweep<R, P, NC, SIZE>;
-    s.udot = k_udot_sweep<R, P, NC, SIZE>;
-    s.sweep_g = k_mass_sweep<R, P, 2 * NC, SIZE>;
-    s.sweep_u = k_mass_sweep<R, P, NC, SIZE>;
-    s.grid = dim3(nblk(m.nnx, T::NX), nblk(m.nny, T::NY));
-    s.grid_halo = dim3(nblk(m.nnx, H::NX), nblk(m.nny, H::NY));
+    if constexpr (sizeof(R) == 4 || SIZE == 2) s.grad_sweep = k_grad_sweep<R, P, NC, ONE ? 1 : NC, SIZE>;
+    s.udot = k_udot_sweep<R, P, NC, ONE ? FB : NC, SIZE>;
+    s.sweep_g = k_mass_sweep<R, P, 2 * NC, ONE ? 1 : 2 * NC, SIZE>;
+    s.sweep_u = k_mass_sweep<R, P, NC, ONE ? 1 : NC, SIZE>;
+    s.grid_rhs = s.grid_u = dim3(gx, gy, ONE ? NC : 1);
+    s.grid_grad = dim3(nblk(m.nnx, H::NX), nblk(m.nny, H::NY), ONE ? NC : 1);
+    s.grid_udot = dim3(gx, gy, ONE ? NC / FB : 1);
+    s.grid_g = dim3(gx, gy, ONE ? 2 * NC : 1);
     s.block = dim3(T::NT);
     s.ws_grad = (int)sizeof(R) * H::grad_ws;
     s.ws_rhs = (int)sizeof(R) * T::rhs_ws;
@@ -303,17 +314,17 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         int k0 = 0;
         if (fuse_g && pr.k_g >= 1) {
             CGL_LAUNCH(prof, KID_GRADF, st,
-                       chk(launch_shared(pdl, S.grad_sweep, S.grid_halo, S.block, S.ws_grad, st, m, (const R*)u,
+                       chk(launch_shared(pdl, S.grad_sweep, S.grid_grad, S.block, S.ws_grad, st, m, (const R*)u,
                                          pr.k_g > 1 ? bg : (R*)nullptr, g2)));
             std::swap(g, g2);
             k0 = 1;
         } else {
             CGL_LAUNCH(prof, KID_GRAD, st,
-                       chk(launch_shared(pdl, S.grad, S.grid, S.block, S.ws_rhs, st, m, (const R*)u, bg, g)));
+                       chk(launch_shared(pdl, S.grad, S.grid_rhs, S.block, S.ws_rhs, st, m, (const R*)u, bg, g)));
         }
         for (int k = k0; k < pr.k_g; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch_shared(pdl, S.sweep_g, S.grid, S.block, S.ws_sweep, st, m, (const R*)g, (const R*)bg, g2)));
+                       chk(launch_shared(pdl, S.sweep_g, S.grid_g, S.block, S.ws_sweep, st, m, (const R*)g, (const R*)bg, g2)));
             std::swap(g, g2);
         }
         R* ER = (R*)B.ER;
@@ -332,7 +343,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         int k1 = 0;
         if (fuse && pr.k_u >= 1) {
             CGL_LAUNCH(prof, KID_UDOTF, st,
-                       chk(launch_shared(pdl, S.udot, S.grid, S.block, S.ws_udot, st, m, (const R*)ER, r, ud2)));
+                       chk(launch_shared(pdl, S.udot, S.grid_udot, S.block, S.ws_udot, st, m, (const R*)ER, r, ud2)));
             std::swap(ud, ud2);
             k1 = 1;
         } else {
@@ -341,7 +352,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         }
         for (int k = k1; k < pr.k_u; ++k) {
             CGL_LAUNCH(prof, KID_SWEEP, st,
-                       chk(launch_shared(pdl, S.sweep_u, S.grid, S.block, S.ws_sweep, st, m, (const R*)ud, (const R*)r, ud2)));
+                       chk(launch_shared(pdl, S.sweep_u, S.grid_u, S.block, S.ws_sweep, st, m, (const R*)ud, (const R*)r, ud2)));
             std::swap(ud, ud2);
         }
     }
