@@ -22,6 +22,7 @@
 #include "modal_tables.h"
 #include "stage.cuh"
 #include "state.h"
+#include "step_order.h"
 
 using namespace cgl;
 
@@ -1363,16 +1364,18 @@ static cudaError_t enqueue_step(cgl_state* S, Prof* prof = nullptr) {
     if (e != cudaSuccess) return e;
     e = S->stage(B, m, p2, 0.75, 0.25, false, false, S->st, prof);
     if (e != cudaSuccess) return e;
-    e = S->stage(B, m, p3, 1.0 / 3.0, 2.0 / 3.0, false, false, S->st, prof);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return S->stage(B, m, p3, 1.0 / 3.0, 2.0 / 3.0, false, false, S->st, prof);
 }
 
 static cgl_status build_graph(cgl_state* S) {
     if (S->step_graph) return CGL_OK;
     cudaGraph_t g = nullptr;
-    CUDA_TRY(cudaStreamBeginCapture(S->st, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_step(S);
+    cudaError_t e = cudaStreamBeginCapture(S->st, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(CGL_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
+    }
+    e = enqueue_step(S);
     cudaError_t e2 = cudaStreamEndCapture(S->st, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -1382,32 +1385,35 @@ static cgl_status build_graph(cgl_state* S) {
     e = cudaGraphInstantiate(&S->step_graph, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         S->step_graph = nullptr;
         return fail(CGL_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
     }
     return CGL_OK;
 }
 
-// One step: the step graph, or, for the first step of a problem, plain
-// launches behind which the graph is captured while they run (the capture
-// costs about as much as a step of 256^2 elements: a new state's first step of
-// KPP 256^2 Q2 took 307 us with the graph built first, 274 us so).  The
-// launches and the graph follow one another on S->st, to which the side
-// streams are joined.  Where a caller's stream cannot be captured (the legacy
-// stream, or one that is being captured) the graph comes first and fails before
-// anything has run.
+// One step (step_order.h).  A new state's first step of KPP 256^2 Q2 took 307 us
+// with the graph built first, 274 us with plain launches first.  The launches and
+// the graph follow one another on S->st, to which the side streams are joined.
+// The legacy stream and one that is being captured cannot be captured.
 static cgl_status run_step(cgl_state* S) {
+    bool capturable = false;
     if (!S->step_graph && S->st != cudaStreamLegacy) {
         cudaStreamCaptureStatus cs;
         CUDA_TRY(cudaStreamIsCapturing(S->st, &cs));
-        if (cs == cudaStreamCaptureStatusNone) {
-            CUDA_TRY(enqueue_step(S));
-            return build_graph(S);
-        }
+        capturable = cs == cudaStreamCaptureStatusNone;
     }
-    if (cgl_status rc = build_graph(S)) return rc;
-    CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
-    return CGL_OK;
+    return one_step(
+        S->step_graph != nullptr, capturable,
+        [&]() -> cgl_status {
+            CUDA_TRY(enqueue_step(S));
+            return CGL_OK;
+        },
+        [&] { return build_graph(S); },
+        [&]() -> cgl_status {
+            CUDA_TRY(cudaGraphLaunch(S->step_graph, S->st));
+            return CGL_OK;
+        });
 }
 
 extern "C" cgl_status cgl_step(cgl_state* S, int32_t nsteps, double t_end, cgl_step_info* info) {

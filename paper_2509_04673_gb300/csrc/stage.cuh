@@ -58,8 +58,11 @@ struct Prof {
     }
 };
 
+// (in run_stage: nothing is launched once a launch has failed, so that k_final
+// never gathers what the others have left out)
 #define CGL_LAUNCH(PROF, ID, ST, ...)             \
     do {                                          \
+        if (err != cudaSuccess) break;            \
         if (PROF) (PROF)->begin((ID), (ST));      \
         __VA_ARGS__;                              \
         if (PROF) (PROF)->end((ST));              \
@@ -226,6 +229,11 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     auto chk = [&](cudaError_t e) {
         if (e != cudaSuccess && err == cudaSuccess) err = e;
     };
+    // the stage's own first error, and none left behind for the thread's next call
+    auto done = [&] {
+        if (err != cudaSuccess) cudaGetLastError();
+        return err;
+    };
     R* u = (R*)B.u;
     // the Q1 variant of eq. (aecQ1) needs neither g_h, nor the residual, nor udot
     const bool lo = pr.mode == MODE_LO, q1 = (pr.opts & OPT_AEC_Q1) != 0 && !lo;
@@ -274,7 +282,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         CGL_LAUNCH(prof, KID_DT, s2,
                    chk(launch(pdl, k_dt_final, dim3(1), dim3(1), s2, B.dtbits, pr.cfl, (const double*)B.t,
                               (const double*)B.t_end, B.dt)));
-    if (dt_only) return err != cudaSuccess ? err : cudaGetLastError();
+    if (dt_only) return done();
     if (q1) {
         CGL_LAUNCH(prof, KID_Q1F, st,
                    chk(launch(pdl, k_q1_facet<R, P, Ph>, ge, be, st, m, pr, (const R*)u, (const double*)B.ue,
@@ -292,7 +300,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
         CGL_LAUNCH(prof, KID_FINAL, st,
                    chk(launch(pdl, k_final<R, P, NC>, gn, bn, st, m, pr, (const R*)B.EW, (R*)B.un, u, R(a), R(b),
                               B.cnt, pr.last_stage ? B.t : (double*)nullptr, (const double*)B.dt)));
-        return err != cudaSuccess ? err : cudaGetLastError();
+        return done();
     }
     // the facet part of the update
     if constexpr (NC > 1)
@@ -373,7 +381,7 @@ cudaError_t run_stage(const Bufs& B, const MeshDev& m, const ProbDev& pr_in, dou
     CGL_LAUNCH(prof, KID_FINAL, st,
                chk(launch(pdl, k_final<R, P, NC>, gn, bn, st, m, pr, (const R*)B.EW, (R*)B.un, u, R(a), R(b),
                           B.cnt, pr.last_stage ? B.t : (double*)nullptr, (const double*)B.dt)));
-    return err != cudaSuccess ? err : cudaGetLastError();
+    return done();
 }
 
 // stage of one precision R (float64: the FP64 form; float: FP32-mixed) for
