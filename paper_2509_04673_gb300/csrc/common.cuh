@@ -313,10 +313,10 @@ DEV void split_ff(double d, float& hi, float& lo) {
 // the reciprocal square root's approximation y (20 bits) refined by one
 // third-order Newton-Raphson step: with d = 1 - x y^2, sqrt(x) = x y (1 + d/2
 // + 3 d^2/8 + O(d^3)), 5 float64 instructions.  The approximation takes a
-// subnormal argument for 0 (y infinite): zeros, subnormal and infinite values
-// and NaN go to sqrt, out of line.  A squared speed is subnormal for 1.5e-162
-// < |v| < 1.5e-154, which every smooth pulse in a gas at rest passes through
-// in its tail.
+// subnormal argument for 0 (y infinite): subnormal values go to sqrt, out of
+// line; zeros (flat elements, gas at rest) return at once.  A squared speed is
+// subnormal for 1.5e-162 < |v| < 1.5e-154, which every smooth pulse in a gas at
+// rest passes through in its tail.
 static __device__ __noinline__ double sqrt_rare(double x) { return sqrt(x); }
 DEV float root(float x) {
     float r;
@@ -324,13 +324,15 @@ DEV float root(float x) {
     return r;
 }
 DEV double root(double x) {
-    // the biased exponent in 1 .. 0x7fe: normal and finite (an integer test: a
+    // by the biased exponent, 1 .. 0x7fe for normal values (integer tests: a
     // float64 comparison runs on the float64 pipe too)
-    if ((((unsigned)__double2hiint(x) >> 20) & 0x7ffu) - 1u >= 0x7feu) return sqrt_rare(x);
+    const unsigned h = hi_word(x), e = (h >> 20) & 0x7ffu;
+    if (e == 0u && ((h << 12) | lo_word(x)) != 0u) return sqrt_rare(x);
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double t = __dmul_rn(x, y), d = __fma_rn(-t, y, 1.0);
-    return __fma_rn(__dmul_rn(t, d), __fma_rn(0.375, d, 0.5), t);
+    const double s = __fma_rn(__dmul_rn(t, d), __fma_rn(0.375, d, 0.5), t);
+    return e - 1u < 0x7feu ? s : x;
 }
 
 // ---------------------------------------------------------------------------
