@@ -269,7 +269,7 @@ HDEV float float_rz(double d) {
 // run on the float64 pipe, 16 clocks a warp there, where they were half of the
 // float64 instructions of the FP32-mixed kernels.  widen is exact; narrow cuts
 // to 24 bits (exact for a widened float); split_ff gives a float pair hi + lo
-// that holds the leading 47 bits.  Zeros take the same path; subnormal,
+// that holds 48 bits, as (float)d and (float)(d - hi) do.  Zeros take the same path; subnormal,
 // infinite and out-of-range values the hardware's (narrow: toward zero).
 DEV double widen(float f) {
     const unsigned b = (unsigned)__float_as_int(f), e = b & 0x7f800000u;
@@ -294,18 +294,20 @@ HDEV float cert_float(double d) {
     return float_of((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
 }
 DEV void split_ff(double d, float& hi, float& lo) {
-    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d), a = h & 0x7fffffffu;
+    const unsigned h = hi_word(d), l = lo_word(d), a = h & 0x7fffffffu;
     // 2^-74 <= |d| < 2^127, so that the unit of the low part is normal
     if (a - 0x3b500000u >= 0x0c900000u) {
         const bool zero = (a | l) == 0u;
-        hi = zero ? 0.f : __double2float_rz(d);
+        hi = zero ? 0.f : __double2float_rn(d);
         lo = zero ? 0.f : __double2float_rn(d - (double)hi);
         return;
     }
-    hi = __int_as_float((int)((h & 0x80000000u) | ((a - 0x38000000u) << 3) | (l >> 29)));
-    // the 29 bits left, in units of 2^(exponent - 52)
+    // 24 bits, rounded up where the rest is half a unit or more; the rest, 28
+    // bits and a sign, in units of 2^(exponent - 52)
+    const unsigned up = (l >> 28) & 1u;
+    hi = __int_as_float((int)((h & 0x80000000u) | ((((a - 0x38000000u) << 3) | (l >> 29)) + up)));
     const float s = __int_as_float((int)((h & 0x80000000u) | (((a >> 20) - 896u - 52u) << 23)));
-    lo = __fmul_rn((float)(l & 0x1fffffffu), s);
+    lo = __fmul_rn((float)((int)(l & 0x1fffffffu) - (int)(up << 29)), s);
 }
 
 // sqrt of a squared speed or norm, x >= 0: in float the hardware's

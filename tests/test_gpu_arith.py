@@ -47,6 +47,15 @@ def test_square_root(arith):
             assert abs(y - math.sqrt(x)) <= 2.0 ** -52 * math.sqrt(x), (x, y)
 
 
+def test_conversions(arith):
+    """widen is exact, narrow cuts to 24 bits; split_ff's pair rounds the high part to nearest and the
+    rest, 28 bits, to 24: half a unit of 2^-24 and 8 of 2^-53 of the value's power of two."""
+    assert arith["widen"] == 0.0
+    assert arith["narrow"] <= 1.0
+    assert arith["split_hi"] <= 0.5
+    assert arith["split_pair"] <= 8.0
+
+
 @pytest.mark.parametrize("p,basis", [(1, 0), (2, 0), (3, 0), (4, 0), (2, 1)])
 def test_float64_gas_at_rest_with_a_narrow_velocity_pulse(cgl, p, basis):  # noqa: F811
     """exp(-r^2 / s^2) passes through every scale down to the smallest subnormal: the squares of the
