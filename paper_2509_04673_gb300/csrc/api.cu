@@ -755,18 +755,15 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
     }
     // cq: [2nc + 6][E] values in the nc (p + 1)^2 >= 16 of EW, free until the update
     if (nc > 1) B.cq = B.EW;
-    // the side streams of a stage and their fork/join events (run_stage)
+    // the first side stream of a stage and its fork/join events (run_stage); the
+    // others at the state's own first stage (ensure_side_streams)
     {
-        cudaError_t e1 = cudaStreamCreateWithFlags(&B.st2, cudaStreamNonBlocking);
-        if (e1 == cudaSuccess) e1 = cudaStreamCreateWithFlags(&B.st3, cudaStreamNonBlocking);
-        if (e1 == cudaSuccess && nc == 1) e1 = cudaStreamCreateWithFlags(&B.st4, cudaStreamNonBlocking);
-        cudaError_t e2 = e1 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_s, cudaEventDisableTiming) : e1;
-        if (e2 == cudaSuccess) e2 = cudaEventCreateWithFlags(&B.ev_fork0, cudaEventDisableTiming);
-        if (e2 == cudaSuccess && nc == 1) e2 = cudaEventCreateWithFlags(&B.ev_w, cudaEventDisableTiming);
-        cudaError_t e3 = e2 == cudaSuccess ? cudaEventCreateWithFlags(&B.ev_join, cudaEventDisableTiming) : e2;
-        if (e3 != cudaSuccess) {
+        cudaError_t e = cudaStreamCreateWithFlags(&B.st2, cudaStreamNonBlocking);
+        for (cudaEvent_t* ev : {&B.ev_fork0, &B.ev_s, &B.ev_join})
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) {
             cgl_state_destroy(S);
-            return fail(CGL_ECUDA, "stream/event creation: %s", cudaGetErrorString(e3));
+            return fail(CGL_ECUDA, "stream/event creation: %s", cudaGetErrorString(e));
         }
     }
     // zero everything once so that fields read before the first stage are defined
@@ -1351,6 +1348,17 @@ static cgl_status read_info(cgl_state* S, cgl_step_info* info, long long steps, 
     return CGL_OK;
 }
 
+// The side streams that only a state stepped by itself uses (the states of a
+// batch share the batch's): at its first stage, since a stream takes 4 to 17 us
+// to create.
+static cgl_status ensure_side_streams(cgl_state* S) {
+    Bufs& B = S->B;
+    if (!B.st3) CUDA_TRY(cudaStreamCreateWithFlags(&B.st3, cudaStreamNonBlocking));
+    if (S->nc == 1 && !B.st4) CUDA_TRY(cudaStreamCreateWithFlags(&B.st4, cudaStreamNonBlocking));
+    if (S->nc == 1 && !B.ev_w) CUDA_TRY(cudaEventCreateWithFlags(&B.ev_w, cudaEventDisableTiming));
+    return CGL_OK;
+}
+
 static cudaError_t enqueue_step(cgl_state* S, Prof* prof = nullptr) {
     const MeshDev& m = S->mesh->m;
     const Bufs& B = S->B;
@@ -1406,6 +1414,7 @@ static cgl_status run_step(cgl_state* S) {
     return one_step(
         S->step_graph != nullptr, capturable,
         [&]() -> cgl_status {
+            if (const cgl_status rc = ensure_side_streams(S)) return rc;
             CUDA_TRY(enqueue_step(S));
             return CGL_OK;
         },
@@ -1444,6 +1453,7 @@ extern "C" cgl_status cgl_stage(cgl_state* S, double dt, double a, double b, cgl
     if (!S) return fail(CGL_EINVAL, "null state");
     if (!S->has_problem) return fail(CGL_EINVAL, "cgl_set_problem first");
     if (!(dt >= 0.0) || !std::isfinite(dt)) return fail(CGL_EINVAL, "dt must be finite and >= 0");
+    if (const cgl_status rc = ensure_side_streams(S)) return rc;
     unsigned long long c0[CNT_N];
     CUDA_TRY(cudaMemcpyAsync(c0, S->B.cnt, sizeof(c0), cudaMemcpyDeviceToHost, S->st));
     CUDA_TRY(cudaMemcpyAsync(S->B.dt, &dt, 8, cudaMemcpyHostToDevice, S->st));
