@@ -472,7 +472,7 @@ cgl_status cgl_gradient_noalloc(const cgl_mesh *mesh, const double *u, double *g
 const char *cgl_kernel_name(int32_t id);
 
 /* Run nsteps (1..1000) SSP-RK3 steps launch by launch (no graph, every
-   kernel on the state's stream, the second stream's kernels included, so
+   kernel on the state's stream, the side streams' kernels included, so
    that no two kernels overlap) with CUDA events around every kernel; ms[id] and
    launches[id] receive the summed device time and the launch count per
    kernel identifier (nk >= 32). The state is advanced like cgl_step. */

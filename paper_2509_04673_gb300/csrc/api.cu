@@ -738,7 +738,7 @@ extern "C" cgl_status cgl_state_create(const cgl_mesh* mesh, int32_t ncomp, int3
         {&B.u, nc * NN * r},          {&B.un, nc * NN * r},        {&B.g, 2 * nc * NN * r},
         {&B.g2, 2 * nc * NN * r},     {&B.ud2, nc * NN * r},
         {&B.bg, 2 * nc * NN * r},     {&B.r, nc * NN * r},         {&B.ud, nc * NN * r},
-        {&B.EV, 16},                  {&B.ER, E * N2 * nc * r},    {&B.EW, E * N2 * nc * r},     {(void**)&B.q, 2 * E * r},
+        {&B.ER, E * N2 * nc * r},     {&B.EW, E * N2 * nc * r},    {(void**)&B.q, 2 * E * r},
         {(void**)&B.ue, nc * E * 8},  {(void**)&B.cf, (1 + nc) * E * 4},  {(void**)&B.avg, 2 * nc * E * 4},
         {&B.fht, nc * E * r},
         {(void**)&B.dte, 3 * E * 8},  {(void**)&B.fl, 4 * nc * E * r},      {(void**)&B.ubl, nc * E * 8}, {(void**)&B.gam, E * 8},

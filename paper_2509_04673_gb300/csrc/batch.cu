@@ -250,11 +250,13 @@ DEV void node_loop(int phase, const InstDev* __restrict__ I, const Tile* __restr
 // A kernel that carries only one degree's code keeps the instruction working
 // set small: measured on the 256-instance batch, the four degrees launched
 // apart took 7.0 ms per step against 10.3 ms for one kernel over all
-// degrees.  7 blocks of 128 threads per SM (a 72-register cap) for every
-// degree: the tile loops are latency-bound, and the register budgets the
-// element phases would take at p = 3 and 4 (4 and 3 blocks per SM) measured
-// slower, 2.34 and 3.94 ms against 2.19 and 3.17 ms per step for those
-// degrees' instances.
+// degrees.  A 72-register cap for every degree (7 blocks of 128 threads per
+// SM by registers): the tile loops are latency-bound, and the register budgets
+// that the element phases would take at p = 3 and 4 (4 and 3 blocks per SM)
+// measured slower, 2.34 and 3.94 ms against 2.19 and 3.17 ms per step for those
+// degrees' instances (both with the node tiles before the present ones).  The
+// workspace of the present tiles lets 6 blocks of p = 4 run on an SM (8832
+// floats each); at p <= 3 the registers decide.
 constexpr int batch_min_blocks(int) { return 7; }
 
 template <int P>

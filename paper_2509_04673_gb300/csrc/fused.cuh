@@ -39,17 +39,6 @@
 
 namespace cgl {
 
-// wrap (gx, gy) on periodic directions (wrap_periodic: any number of
-// periods); false outside a non-periodic mesh
-DEV bool wrap_node(const MeshDev& m, int& gx, int& gy) {
-    bool in = true;
-    if (m.py) gy = wrap_periodic(gy, m.nny);
-    else in = gy >= 0 && gy < m.nny;
-    if (m.px) gx = wrap_periodic(gx, m.nnx);
-    else in = in && gx >= 0 && gx < m.nnx;
-    return in;
-}
-
 // A tile of TEX x TEY elements (NX x NY nodes) worked by NT threads: LX
 // segments wide in the x passes, RX rows of them per step; LY node columns
 // wide in the y passes, RY y segments per step, KY steps.  HALO: the passes
@@ -176,7 +165,8 @@ struct SegThread {
 // RY-th row, the few columns beyond the block's width go round the block.
 // load() reads into registers, so that it can run ahead of the barrier that
 // frees the planes, store() writes them.  Values outside a non-periodic mesh
-// are 0 (every weight that reaches them is 0).
+// are 0, and the 1D operators rely on it: they give a vertex at the end of the
+// mesh the same weights beyond it as any other.
 template <class R, int P, class TL, int HALO, int W, int H, int PL, int S, bool FULL>
 struct Stage {
     static constexpr int K = (H + TL::RY - 1) / TL::RY;
@@ -199,8 +189,10 @@ struct Stage {
         if (periodic) g = wrap_periodic(g, n);
         return g >= 0 && g < n;
     }
-    // CG: through L2 (ld.global.cg), where the kernel launched just before may
-    // still run
+    // CG: through L2 (ld.global.cg).  u, which k_final reads and writes: it may
+    // still run when the kernel behind it starts (and waits), so that lines of u
+    // in an SM's L1 can be older than the other SMs' writes.  The fields that the
+    // kernel before has only written are read the ordinary way
     template <bool CG>
     static DEV R get(const R* __restrict__ p) {
         if constexpr (CG) return __ldcg(p);

@@ -407,13 +407,11 @@ DEV void lo_facets(const MeshDev& m, const ProbDev& pr, const int (&nb)[4], int 
     }
 }
 
-// the float64 Appendix-A factor where the float32 certificate of the
-// FP32-mixed form could not show alpha = 1 (rare): out of line, so that the
-// unrolled node loop of the slope limiter carries a call per node instead of
-// a copy of the float64 formula (measured: k_update_el 5.52 -> 5.41 ms per
-// three blast steps; in k_facet, at its 73-register cap, the call measured
-// slower, 4.66 -> 5.80 ms, so the facet limiter keeps it inline, as does the
-// FP64 form, where it runs everywhere)
+// the float64 Appendix-A factor where the float32 certificate could not show
+// alpha = 1 (rare): out of line in the facet and slope limiters of systems, so
+// that their loops carry a call instead of a copy of the float64 formula.  Only
+// the eq. (aecQ1) variant has it inline: k_q1_facet behind the certificate,
+// k_q1_update in float64, where it runs without one
 static __device__ __noinline__ double euler_alpha_rare(const double* ub, const double* f, double m, double eps) {
     return euler_alpha<double>(ub, f, m, eps);
 }
@@ -570,19 +568,16 @@ DEV void block_min_to(double v, unsigned long long* bits) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// per element u^e and the face neighbours' u^{e'} (from their blocks,
-// eq. (ueold)), f(u^e), lambda_e, the facet speeds and f^L, dt_e (eq.
-// (dtmaxcell)), ubar^{e,L} (eq. (uelowFCT)), the flux-limiter capacities,
-// gamma_e (eqs. (WENO:alpha), (WENO:norm)), nu_e, the element vectors of the
-// g_h right-hand side, and (stage 1) the block minimum of dt_e.
-// ---------------------------------------------------------------------------
-// FP32-mixed form of pre_at: cell means as float-float pairs, low-order
-// facet fluxes formed in float (their flux part is float-accurate anyway,
-// the jump term comes from float-float differences), float facet fluxes and
-// flux-limiter capacities (rounded toward zero, so they stay admissible)
-// stored for the update pass; float64 for u^e, the speed-sum reciprocal,
-// dt_e, ubar^{e,L} and the bound gaps.
+// The low-order part of a stage: u^e of an element and its face neighbours (eq.
+// (ueold)), the facet speeds and f^L, dt_e (eq. (dtmaxcell)), ubar^{e,L} (eq.
+// (uelowFCT)), the flux-limiter capacities and, in stage 1, the block minimum of
+// dt_e.  In the FP32-mixed form the cell means are float-float pairs and the
+// low-order facet fluxes float (their flux part is float-accurate anyway, the
+// jump comes from float-float differences), as are the capacities (rounded
+// toward zero, so they stay admissible); u^e, the reciprocal of the speed sum,
+// dt_e, ubar^{e,L} and the bound gaps are float64.
+
+// values passed to and from the out-of-line functions
 template <class R, int NC>
 struct CompVec {
     R v[NC];
@@ -729,7 +724,7 @@ DEV double lo_outputs_mixed(const MeshDev& m, const ProbDev& pr, const float* __
     dte_out[off<NC>(m.E, 2, e)] = s * m.inv_h;
 #pragma unroll
     for (int d = 0; d < 4; ++d)
-store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
+        store_facet<float, NC>(fl_out, (long long)e * 4 + d, F[d]);
     const float s4 = 0.25f * sf;  // |K| / (|dK| dt_e), exact
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -860,7 +855,7 @@ DEV double lo_outputs_fp64(const MeshDev& m, const ProbDev& pr, const double* __
     dte_out[off<NC>(m.E, 2, e)] = s * m.inv_h; // 1 / dt_e
 #pragma unroll
     for (int d = 0; d < 4; ++d)
-store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
+        store_facet<double, NC>(fl_out, (long long)e * 4 + d, FL[d]);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const double os = ((FL[1][c] - FL[0][c]) + FL[3][c]) - FL[2][c];
@@ -947,7 +942,8 @@ DEV int halo_pos(int tx, int ty, int d) {
 // dt_e, ubar^{e,L}, the flux-limiter capacities); gamma_e and nu_e come from
 // k_sens, which runs beside it.  The means and their fluxes of a tile of 32 x
 // TY elements and its halo are formed once in shared memory, instead of five
-// times per element.  The arithmetic of pre_at.
+// times per element.  pre_at_mixed is the same arithmetic for one element of a
+// batch.
 template <class R, int P, class Ph, int TY, bool SUB = false>
 __global__ void __launch_bounds__(K_TX * TY) k_lo(MeshDev m, ProbDev pr, const R* __restrict__ u,
                                                   double* __restrict__ ue_out, double* __restrict__ dte_out,
@@ -2026,7 +2022,8 @@ DEV void store_reduced_step(const MeshDev& m, double* dte_a, float* cf, double r
     cf[e] = __double2float_ru(1.0 / rs2);
 }
 
-// facet part of the element update: canonical f^H, the flux limiter and
+// facet part of the element update (scalars, and systems in the eq. (aecQ1)
+// variant; k_facet_sys holds that of systems): canonical f^H, the flux limiter and
 // ubar^e (eqs. (hoflux), (fAlim)/(uelim), Appendix A), and the facet term
 // (h/(p+1)^2) sum_d +-f^H_d of the element contributions f_i^e (eq. (aec))
 template <class R, int P, class Ph>
@@ -2634,7 +2631,7 @@ __global__ void __launch_bounds__(128) k_q1_update(MeshDev m, ProbDev pr, const 
 }
 
 // Scalars: the update in two kernels.  k_facet needs only u and the outputs of
-// k_lo, so it runs on a second stream beside the g_h and udot kernels;
+// k_lo, so it runs on the low-order stream beside the g_h and udot kernels;
 // k_update_el then reads its ubar^e and facet terms.  The bodies are
 // device functions of one element, also run by the batched stage.
 template <class R, int P, class Ph>
@@ -3073,7 +3070,7 @@ __global__ void __launch_bounds__(32 * Ph::NC, sizeof(R) == 4 ? (P <= 2 ? 8 : P 
 }
 
 // Scalars: the residual in two kernels.  k_res_w (the Galerkin part W^e, needs
-// only u) runs on the second stream from the start of the stage, beside k_lo
+// only u) runs on a stream of its own from the start of the stage, beside k_lo
 // and the g_h kernels; k_res_s adds the stabilisation, which needs g_h,
 // gamma_e and nu_e.  W^e passes through the increment buffer, which is free
 // until k_update_el.

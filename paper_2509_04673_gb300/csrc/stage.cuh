@@ -18,7 +18,6 @@ struct Bufs {
     void* bg;     // rhs of g_h       [2NC][NN] (R)
     void* r;      // target residual  [NC][NN]  (R)
     void* ud;     // udot             [NC][NN]  (R)
-    void* EV;     // unused (16 bytes)
     void* ER;     // element residual [N2][NC][E]  (R)
     void* EW;     // SSP increments   [N2][NC][E]  (R)
     void* q;      // flux-limiter capacities [2][E] (scalar)  (R)
