@@ -175,15 +175,15 @@ def load_peaks():
 NCU_PER_ELEMENT = {
     # profiles/euler_blast_1024_q2_stage_kernels.md (names as cgl_profile reports them: k_pre is k_lo_sys,
     # k_res_ev k_res_sys, k_update_ev k_upd_sys and k_facet k_facet_sys in this Euler stage)
-    ("k_pre", HEADLINE): {"warp_inst": 48.34, "fp64_flops": 22.00, "dram_bytes": 206.6, "shared_wavefronts": 1.15},
-    ("k_facet", HEADLINE): {"warp_inst": 60.24, "fp64_flops": 13.26, "dram_bytes": 223.1, "shared_wavefronts": 2.88},
-    ("k_grad_sweep", HEADLINE): {"warp_inst": 80.05, "fp64_flops": 0.00, "dram_bytes": 140.0, "shared_wavefronts": 15.74},
-    ("k_res_ev", HEADLINE): {"warp_inst": 154.58, "fp64_flops": 0.00, "dram_bytes": 328.0, "shared_wavefronts": 19.25},
-    ("k_udot_sweep", HEADLINE): {"warp_inst": 44.19, "fp64_flops": 0.00, "dram_bytes": 230.3, "shared_wavefronts": 6.99},
-    ("k_update_ev", HEADLINE): {"warp_inst": 98.88, "fp64_flops": 0.03, "dram_bytes": 489.3, "shared_wavefronts": 5.60},
-    ("k_final", HEADLINE): {"warp_inst": 37.17, "fp64_flops": 0.00, "dram_bytes": 317.2, "shared_wavefronts": 0.66},
-    ("k_sens", HEADLINE): {"warp_inst": 82.78, "fp64_flops": 0.00, "dram_bytes": 67.0, "shared_wavefronts": 7.66},
-    ("k_avg", HEADLINE): {"warp_inst": 18.06, "fp64_flops": 0.00, "dram_bytes": 99.3, "shared_wavefronts": 0.06},
+    ("k_pre", HEADLINE): {"warp_inst": 48.29, "fp64_flops": 22.00, "dram_bytes": 206.2, "shared_wavefronts": 1.23},
+    ("k_facet", HEADLINE): {"warp_inst": 60.55, "fp64_flops": 13.26, "dram_bytes": 222.0, "shared_wavefronts": 2.88},
+    ("k_grad_sweep", HEADLINE): {"warp_inst": 80.05, "fp64_flops": 0.00, "dram_bytes": 139.8, "shared_wavefronts": 15.74},
+    ("k_res_ev", HEADLINE): {"warp_inst": 154.59, "fp64_flops": 0.00, "dram_bytes": 328.0, "shared_wavefronts": 19.26},
+    ("k_udot_sweep", HEADLINE): {"warp_inst": 44.19, "fp64_flops": 0.00, "dram_bytes": 230.7, "shared_wavefronts": 7.00},
+    ("k_update_ev", HEADLINE): {"warp_inst": 96.07, "fp64_flops": 0.03, "dram_bytes": 489.5, "shared_wavefronts": 5.60},
+    ("k_final", HEADLINE): {"warp_inst": 37.17, "fp64_flops": 0.00, "dram_bytes": 316.7, "shared_wavefronts": 0.66},
+    ("k_sens", HEADLINE): {"warp_inst": 82.78, "fp64_flops": 0.00, "dram_bytes": 67.6, "shared_wavefronts": 7.66},
+    ("k_avg", HEADLINE): {"warp_inst": 18.22, "fp64_flops": 0.00, "dram_bytes": 98.9, "shared_wavefronts": 0.06},
 }
 
 SM_COUNT_GB300 = 152
