@@ -310,20 +310,21 @@ DEV void split_ff(double d, float& hi, float& lo) {
     lo = __fmul_rn((float)((int)(l & 0x1fffffffu) - (int)(up << 29)), s);
 }
 
-// sqrt of a squared speed or norm, x >= 0: in float the hardware's
-// approximation (within a unit in the last place, no slow path); in float64
-// the reciprocal square root's approximation y (20 bits) refined by one
-// third-order Newton-Raphson step: with d = 1 - x y^2, sqrt(x) = x y (1 + d/2
-// + 3 d^2/8 + O(d^3)), 5 float64 instructions.  The approximation takes a
-// subnormal argument for 0 (y infinite): subnormal values go to sqrt, out of
-// line; zeros (flat elements, gas at rest) return at once.  A squared speed is
+// sqrt of a squared speed, x >= 0: in float x y, y the hardware's reciprocal
+// square root (no slow path), corrected by its residual: half a unit in the last
+// place and a little, as sqrtf; the approximation alone made nu_e 1.2 to 1.7
+// times less exact.  In float64 the approximation y (20 bits) refined by one
+// third-order Newton-Raphson step: with d = 1 - x y^2, sqrt(x) = x y (1 + d/2 +
+// 3 d^2/8 + O(d^3)), 5 float64 instructions.  It takes a subnormal argument for 0
+// (y infinite): subnormal values go to sqrt, out of line.  A squared speed is
 // subnormal for 1.5e-162 < |v| < 1.5e-154, which every smooth pulse in a gas at
 // rest passes through in its tail.
 static __device__ __noinline__ double sqrt_rare(double x) { return sqrt(x); }
 DEV float root(float x) {
-    float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
+    float y;
+    asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    const float t = __fmul_rn(x, y), s = __fmaf_rn(__fmaf_rn(-t, t, x), __fmul_rn(0.5f, y), t);
+    return x == 0.f || x == __int_as_float(0x7f800000) ? x : s;
 }
 DEV double root(double x) {
     // by the biased exponent, 1 .. 0x7fe for normal values (integer tests: a

@@ -61,6 +61,15 @@ DEV double recip(double x) {
     return rcp_nr(x);
 }
 
+// square root of a squared norm, x >= 0: float by the hardware's approximation
+// (within one unit in the last place; gamma_e is as exact with it as without)
+DEV float norm_root(float x) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+DEV double norm_root(double x) { return root(x); }
+
 // modal coefficients of one line
 template <class R, int P>
 DEV void modal_line(const Tab<R>& T, const R (&v)[P + 1], R (&l)[P + 1]) {
@@ -223,8 +232,8 @@ DEV R modal_sensor(const Tab<R>& T, int a2b, const ProbDev& pr, const R (&own)[(
             for (int i = 1; i < N2; ++i) D[i] = fma_r(wd, sub_r(own[i], W[KEEP ? d : 0][i]), D[i]);
         }
     });
-    const R num = root(fmax(modal_norm<R, P>(D, a2b), R(0)));
-    const R den = root(sig0);
+    const R num = norm_root(fmax(modal_norm<R, P>(D, a2b), R(0)));
+    const R den = norm_root(sig0);
     const R ratio = num * recip(den + geps);
     return R(1) - (pr.q1 ? fmin(R(1), ratio) : pow_rare(fmin(R(1), ratio), PV<R>::q(pr)));
 }
