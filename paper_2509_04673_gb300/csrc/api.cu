@@ -1401,7 +1401,7 @@ static cgl_status build_graph(cgl_state* S) {
 }
 
 // One step (step_order.h).  A new state's first step of KPP 256^2 Q2 took 307 us
-// with the graph built first, 274 us with plain launches first.  The launches and
+// with the graph built first, 260 us with plain launches first.  The launches and
 // the graph follow one another on S->st, to which the side streams are joined.
 // The legacy stream and one that is being captured cannot be captured.
 static cgl_status run_step(cgl_state* S) {

@@ -76,9 +76,9 @@ inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs)
 
 // Size of the stencils' tiles (StageTile): large ones unless they make fewer
 // than four (p <= 2) or two blocks per SM, tiny ones (float64) where the small
-// ones make fewer than one.  Euler 768 x 192 Q2 FP32-mixed, 325 large tiles: 569
-// us/step with them, 557 with small ones; Burgers 301 x 199 Q4, 475 large
-// tiles: 259 and 273.
+// ones make fewer than one.  Euler 768 x 192 Q2 FP32-mixed, 325 large tiles: 548
+// us/step with them, 531 with small ones; Burgers 301 x 199 Q4, 475 large
+// tiles: 257 and 260.
 template <class R, int P>
 inline int tile_size(const MeshDev& m) {
     using TL = stage_tile_t<R, P, 0>;
